@@ -68,29 +68,23 @@ int sum_nreg(const TileBatch& tb, cudaStream_t s) {
     return t;
 }
 
-// Dense (pseudo-)inverse of every factorised problem of a tile batch:
-// out[ooff[i] + r * ld[i] + c] = (K_i^+)[r][c] for r, c < n[i].  The identity
-// columns are solved in blocks of 32 columns, one CTA per (problem, block),
-// so the whole GPU works on it.
+// Dense (pseudo-)inverse of every factorised FP64 problem of a tile batch:
+// out[ooff[i] + r * ld[i] + c] = (K_i^+)[r][c] for r, c < n[i].  The lower
+// triangle is solved for, one CTA per (problem, few columns), so the whole
+// GPU works on it, and mirrored.
 void dense_inverse(const TileBatch& tb, double* out, const std::vector<long long>& ooff, const std::vector<int>& ld,
                    cudaStream_t st) {
     int maxn = 0;
     for (int v : tb.n) maxn = std::max(maxn, v);
     const int lde = tb.max_K * NB;
     DevBuf<double> E((size_t)tb.total_rows * lde);
-    tile_identity(tb, E.p, lde, st);
-    tile_solve(tb, E.p, lde, maxn, nullptr, st);
-    std::vector<CopyItem> ci(tb.P);
-    for (int i = 0; i < tb.P; ++i) {
-        ci[i].soff = tb.roff[i] * lde;
-        ci[i].lds = lde;
-        ci[i].doff = ooff[i];
-        ci[i].ldd = ld[i];
-        ci[i].rows = tb.n[i];
-        ci[i].cols = tb.n[i];
+    if (!tile_inverse_f64(tb, E.p, lde, maxn, st)) {
+        tile_identity(tb, E.p, lde, st);
+        tile_solve(tb, E.p, lde, maxn, nullptr, st);
     }
-    DevBuf<CopyItem> d_ci = upload_vec(ci, st);
-    copy_blocks(d_ci.p, tb.P, E.p, out, st);
+    DevBuf<long long> d_ooff = upload_vec(ooff, st);
+    DevBuf<int> d_ld = upload_vec(ld, st);
+    mirror_lower(tb, E.p, lde, maxn, d_ooff.p, d_ld.p, out, st);
     MSDD_CUDA(cudaStreamSynchronize(st));
 }
 

@@ -14,10 +14,6 @@ namespace {
 constexpr int TPB = 256;     // threads per CTA; each owns 4 entries of a 32 x 32 tile
 constexpr int LDS = NB + 1;  // padded shared-memory row stride
 
-__device__ __forceinline__ long long tile_index(long long toff, int kb, int R, int C) {
-    return toff + ((long long)R * (kb + 1) + (R - C)) * NB2;
-}
-
 template <typename T>
 __device__ __forceinline__ void load_tile(T (*dst)[LDS], const T* __restrict__ src) {
     for (int e = threadIdx.x; e < NB2; e += TPB) dst[e / NB][e % NB] = src[e];
@@ -277,15 +273,6 @@ __global__ void __launch_bounds__(TPB) k_tile_solve(
     }
 }
 
-
-// cp.async (16-byte global -> shared copies, completion by groups)
-__device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
-    unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(sa), "l"(gmem));
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::); }
-template <int N>
-__device__ __forceinline__ void cp_async_wait_n() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N)); }
 
 // ------------------------------------------------------------------ solve, one right-hand side
 // The PCG local solves.  One CTA of 128 threads per matrix; the whole local
@@ -825,13 +812,6 @@ __device__ __forceinline__ void band_load4<float>(const float* tile, int r, int 
     const float4 x = *reinterpret_cast<const float4*>(tile + r * NB + ((g ^ band_swz(r)) << 2));
     v[0] = x.x; v[1] = x.y; v[2] = x.z; v[3] = x.w;
 }
-template <>
-__device__ __forceinline__ void band_load4<double>(const double* tile, int r, int g, double (&v)[4]) {
-    const double2* p = reinterpret_cast<const double2*>(tile + r * NB + ((g ^ band_swz(r)) << 2));
-    const double2 a = p[0], b = p[1];
-    v[0] = a.x; v[1] = a.y; v[2] = b.x; v[3] = b.y;
-}
-
 template <typename T, int CPT, int CG>
 struct BandSmem {
     static constexpr int ZLD = CG * CPT;                // columns held in the ring and Acc
@@ -2326,6 +2306,7 @@ void tile_solve(const TileBatch& tb, double* X, int ldx, int ncols, const int* s
             return;
         }
     }
+    if (!tb.prec && tile_solve_f64(tb, X, ldx, ncols, skip, s, gdone)) return;
     int maxkb = 0;
     for (int v : tb.kb) maxkb = std::max(maxkb, v);
     // the band kernels stage blocks of X with 16-byte copies
@@ -2345,9 +2326,8 @@ void tile_solve(const TileBatch& tb, double* X, int ldx, int ncols, const int* s
         launch_band_ws<12, 10, 2, 2, 4>(tb, *tm, X, ldx, ncols, skip, s, gdone);
         return;
     }
-    if (maxkb <= 2 && ncols <= NB && aligned) {
-        if (tb.prec) launch_band_cols<float>(tb, tb.tiles_f.p, tb.dinv_f.p, X, ldx, ncols, skip, s, gdone);
-        else launch_band_cols<double>(tb, tb.tiles_d.p, tb.dinv_d.p, X, ldx, ncols, skip, s, gdone);
+    if (tb.prec && maxkb <= 2 && ncols <= NB && aligned) {
+        launch_band_cols<float>(tb, tb.tiles_f.p, tb.dinv_f.p, X, ldx, ncols, skip, s, gdone);
         return;
     }
     const dim3 grid(tb.P, (ncols + NB - 1) / NB);

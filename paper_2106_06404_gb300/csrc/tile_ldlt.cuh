@@ -18,6 +18,21 @@
 
 namespace msdd {
 
+#ifdef __CUDACC__
+// first element of tile (R, C) of a problem
+__device__ __forceinline__ long long tile_index(long long toff, int kb, int R, int C) {
+    return toff + ((long long)R * (kb + 1) + (R - C)) * NB2;
+}
+// cp.async (16-byte global -> shared copies, completion by groups)
+__device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
+    unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(sa), "l"(gmem));
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::); }
+template <int N>
+__device__ __forceinline__ void cp_async_wait_n() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N)); }
+#endif
+
 struct TileBatch {
     int P = 0;
     int prec = 0;                 // 0: double tiles, 1: float tiles
@@ -52,6 +67,18 @@ void tile_from_dense(TileBatch& tb, const double* src, const long long* d_soff, 
                      cudaStream_t s);
 // In-place LDL^T of every problem; fills d_status (0 ok, k+1 = failing row) and d_nreg.
 void tile_factor(TileBatch& tb, double reg_tol, cudaStream_t s);
+// FP64 batches (tile_solve_f64.cu): tile_solve for prec == 0; false, with
+// nothing launched, where shared memory cannot hold a problem's solution ring
+// (dense problems beyond 21,000 rows: tile_solve takes the generic kernel).
+bool tile_solve_f64(const TileBatch& tb, double* X, int ldx, int ncols, const int* skip, cudaStream_t s,
+                    const int* gdone);
+// E (total_rows x lde, lde >= ncols) <- columns 0 .. ncols - 1 of every
+// problem's inverse, the tile rows from each column's own on (the lower
+// triangle and the diagonal tiles); false as above.
+bool tile_inverse_f64(const TileBatch& tb, double* E, int lde, int ncols, cudaStream_t s);
+// out[ooff[i] + r * ld[i] + c] for r, c < n[i] from the lower triangle of E.
+void mirror_lower(const TileBatch& tb, const double* E, int lde, int maxn, const long long* d_ooff, const int* d_ld,
+                  double* out, cudaStream_t s);
 // E (total_rows x lde) <- per problem the identity of order n[i] (zero elsewhere).
 void tile_identity(const TileBatch& tb, double* E, int lde, cudaStream_t s);
 // Solve K X = B in place.  X is double, row-major, problem i rows at
