@@ -41,7 +41,10 @@ __global__ void k_init(double* __restrict__ X, const int* __restrict__ n_, const
     }
 }
 
-__global__ void k_form_rhs(double* __restrict__ W, const double* __restrict__ AX, const double* __restrict__ BX,
+// W is FP64, or FP32 beside FP32 factors (whose solve rounds its right-hand
+// side to FP32 in any case), with a leading dimension of its own
+template <typename WT>
+__global__ void k_form_rhs(WT* __restrict__ W, int ldw, const double* __restrict__ AX, const double* __restrict__ BX,
                            const double* __restrict__ theta, const int* __restrict__ n_, const int* __restrict__ K_,
                            const long long* __restrict__ roff_, const int* __restrict__ p_, int ldx, double sigma,
                            int first, const int* __restrict__ done) {
@@ -52,20 +55,21 @@ __global__ void k_form_rhs(double* __restrict__ W, const double* __restrict__ AX
     const long long rows = (long long)K_[i] * NB;
     if (threadIdx.x < p) smu[threadIdx.x] = first ? 0.0 : 1.0 / (theta[i * PMAX + threadIdx.x] + sigma);
     __syncthreads();
-    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < rows * ldx;
+    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < rows * ldw;
          e += (long long)gridDim.x * blockDim.x) {
-        int r = (int)(e / ldx), c = (int)(e % ldx);
+        int r = (int)(e / ldw), c = (int)(e % ldw);
         long long idx = (roff_[i] + r) * ldx + c;
         double v = 0.0;
         if (r < n && c < p) {
             double bx = BX[idx];
             v = first ? bx : bx - (AX[idx] + sigma * bx) * smu[c];
         }
-        W[idx] = v;
+        W[(roff_[i] + r) * ldw + c] = from_f64<WT>(v);
     }
 }
 
-__global__ void k_form_y(double* __restrict__ Y, const double* __restrict__ X, const double* __restrict__ W,
+template <typename WT>
+__global__ void k_form_y(double* __restrict__ Y, const double* __restrict__ X, const WT* __restrict__ W, int ldw,
                          const double* __restrict__ theta, const int* __restrict__ n_, const int* __restrict__ K_,
                          const long long* __restrict__ roff_, const int* __restrict__ p_, int ldx, double sigma,
                          int first, const int* __restrict__ done) {
@@ -81,7 +85,10 @@ __global__ void k_form_y(double* __restrict__ Y, const double* __restrict__ X, c
         int r = (int)(e / ldx), c = (int)(e % ldx);
         long long idx = (roff_[i] + r) * ldx + c;
         double v = 0.0;
-        if (r < n && c < p) v = first ? W[idx] : fma(X[idx], smu[c], W[idx]);
+        if (r < n && c < p) {
+            const double w = to_f64(W[(roff_[i] + r) * ldw + c]);
+            v = first ? w : fma(X[idx], smu[c], w);
+        }
         Y[idx] = v;
     }
 }
@@ -1034,128 +1041,142 @@ __global__ void k_check_knorm(const double* __restrict__ partial, const double* 
         decide(i, sres, theta, p, sigma, tol, eta, nev_max, it, maxit, true, done, m_, iters, n_active, best, best_it);
 }
 
-// ---- FP32 start phase: Euclidean CholQR of the block W (W = Q R, X <- Q).
-// G = W^T W with FP32 products, one CTA per problem.
-// Partial Grams over `gsplit` row ranges of each problem (grid: problems x
-// splits), written to Gp[(i gsplit + s) PMAX^2]; k_cholqr sums them.
-__global__ void __launch_bounds__(TPB) k_gram32(const double* __restrict__ W, double* __restrict__ Gp,
-                                                const int* __restrict__ n_, const long long* __restrict__ roff_,
-                                                const int* __restrict__ p_, int ldx, int gsplit) {
-    __shared__ float sW[ROWBLK][LD];
-    const int i = blockIdx.x, sp = blockIdx.y;
-    const int n = n_[i], p = p_[i];
-    const long long roff = roff_[i];
-    const int rows_per = (n + gsplit - 1) / gsplit;
-    const int r_lo = sp * rows_per, r_hi = min(n, r_lo + rows_per);
-    const int npair = p * (p + 1) / 2;
-    int pa[3], pb[3];
-    float acc[3] = {0.f, 0.f, 0.f};
-    for (int q = 0; q < 3; ++q) {
-        int e = threadIdx.x + q * TPB;
-        pa[q] = -1;
-        if (e < npair) {
-            int a = 0, rem = e;
-            while (rem >= p - a) { rem -= p - a; ++a; }
-            pa[q] = a;
-            pb[q] = a + rem;
-        }
-    }
-    for (int r0 = r_lo; r0 < r_hi; r0 += ROWBLK) {
-        __syncthreads();
-        for (int e = threadIdx.x; e < ROWBLK * p; e += TPB) {
-            int rr = e / p, c = e % p;
-            int r = r0 + rr;
-            sW[rr][c] = r < r_hi ? f64_to_f32(W[(roff + r) * ldx + c]) : 0.f;
-        }
-        __syncthreads();
-        for (int q = 0; q < 3; ++q) {
-            if (pa[q] < 0) continue;
-            float s = 0.f;
-#pragma unroll 8
-            for (int rr = 0; rr < ROWBLK; ++rr) s += sW[rr][pa[q]] * sW[rr][pb[q]];
-            acc[q] += s;
-        }
-    }
-    double* G = Gp + ((long long)i * gsplit + sp) * PMAX * PMAX;
-    for (int q = 0; q < 3; ++q) {
-        if (pa[q] < 0) continue;
-        G[pa[q] * PMAX + pb[q]] = f32_to_f64(acc[q]);
-        G[pb[q] * PMAX + pa[q]] = f32_to_f64(acc[q]);
-    }
-}
+// ---- FP32 start phase: block inverse iteration W <- K~^{-1} B (W C) with
+// C = D R^{-1} from the Euclidean CholQR of W (D W^T W D = R^T R, D =
+// diag(W^T W)^{-1/2}).  The blocks are FP32 with ldw = p rounded up to 4
+// columns a row, so a row is one to two whole 32-byte sectors of each group
+// of columns and nothing is converted; the orthonormal block W C itself is
+// only formed at the end: the next right-hand side is (B W) C, B applied to
+// the rows of W and C to the result.
 
-// C = D R^{-1} with D = diag(G)^{-1/2} and D G D = R^T R (FP32 Cholesky, one
-// warp per problem: G holds FP32 products and X = W C is formed in FP32, so
-// FP64 here would only lengthen the serial chain).  A column whose pivot
-// falls below 1e-10 of its scaled diagonal is dependent on the previous
-// ones: it is reset to its scaled self (R row e_k) so that the basis stays
-// finite; the FP64 phase removes it.
+// Partial Gram matrices of row range blockIdx.y: a thread owns a 4 x 4 tile of
+// the upper triangle and every `lanes`-th row (two 16-byte loads and 16 FMA a
+// row); the tiles are summed over the row lanes in shared memory.  The last
+// block of a problem (ticket) sums the row ranges in order and factorises, in
+// one warp: column b of the scaled Gram in the registers of lane b, a row of
+// R exchanged through shared memory per step.  A column whose pivot falls
+// below 1e-10 of its scaled diagonal is dependent on the previous ones: it is
+// reset to its scaled self (R row e_k) so that the basis stays finite; the
+// FP64 phase removes it.
 __device__ __forceinline__ float rsqrt_f32(float x) {
     const float r = rsqrtf(x);
     return r * fmaf(-0.5f * x * r, r, 1.5f);
 }
-__global__ void k_cholqr(const double* __restrict__ Gp, int gsplit, double* __restrict__ C,
-                         const int* __restrict__ p_) {
-    __shared__ float R[PMAX][LD], Ri[PMAX][LD], d[PMAX], d_inv[PMAX];
-    const int i = blockIdx.x;
-    const int p = p_[i];
-    const int t = threadIdx.x;
-    const double* Gi = Gp + (long long)i * gsplit * PMAX * PMAX;
-    // G = sum of the row-range partials, by the whole block (their loads are
-    // the long part); the factorisation below is one warp's
-    for (int e = t; e < PMAX * PMAX; e += blockDim.x) {
-        int a = e / PMAX, b = e % PMAX;
-        float g = 0.f;
-        if (a < p && b < p)
-            for (int sp = 0; sp < gsplit; ++sp) g += f64_to_f32(Gi[(long long)sp * PMAX * PMAX + e]);
-        R[a][b] = g;
-        Ri[a][b] = 0.f;
-    }
-    __syncthreads();
-    if (t >= 32) return;
-    if (t < PMAX) {
-        const float g = t < p ? R[t][t] : 0.f;
-        d[t] = g > 0.f ? rsqrt_f32(g) : 0.f;
-    }
+
+template <int PB>
+__device__ void cholqr_warp(float (*G)[PMAX + 4], float* dinv, int p, float* __restrict__ C) {
+    const int b = threadIdx.x & 31;
+    const float gbb = b < p ? G[b][b] : 0.f;
+    const float db = gbb > 0.f ? rsqrt_f32(gbb) : 0.f;      // column scale
+    dinv[b] = db;
     __syncwarp();
-    for (int e = t; e < PMAX * PMAX; e += 32) {
-        int a = e / PMAX, b = e % PMAX;
-        R[a][b] = (a < p && b < p) ? d[a] * R[a][b] * d[b] : 0.f;
-    }
+    float g[PB];
+#pragma unroll
+    for (int a = 0; a < PB; ++a) g[a] = a < p && b < p ? dinv[a] * G[min(a, b)][max(a, b)] * db : 0.f;
     __syncwarp();
-    // upper Cholesky in place: R <- U with D G D = U^T U
-    for (int k = 0; k < p; ++k) {
-        const float piv = R[k][k];
+    float rinv[PB];
+#pragma unroll
+    for (int k = 0; k < PB; ++k) {
+        const float piv = __shfl_sync(0xffffffffu, g[k], k);
         const bool ok = piv > 1e-10f;
         const float ru = ok ? rsqrt_f32(piv) : 1.f;
+        rinv[k] = ru;
+        const float u = b == k ? (ok ? piv * ru : 1.f) : (ok && b > k ? g[k] * ru : 0.f);   // R[k][b]
+        G[k][b] = u;
         __syncwarp();
-        if (t == 0) { R[k][k] = ok ? piv * ru : 1.f; d_inv[k] = ru; }
-        for (int j = k + 1 + t; j < p; j += 32) R[k][j] = ok ? R[k][j] * ru : 0.f;
-        __syncwarp();
-        for (int e = t; e < p * p; e += 32) {
-            int a = e / p, b = e % p;
-            if (a > k && b >= a) R[a][b] -= R[k][a] * R[k][b];
-        }
-        __syncwarp();
+#pragma unroll
+        for (int a = k + 1; a < PB; ++a) g[a] = fmaf(-G[k][a], u, g[a]);
     }
-    // Ri = U^{-1} (upper), column-parallel back substitution
-    if (t < p) {
-        for (int r = t; r >= 0; --r) {
-            float v = (r == t) ? 1.f : 0.f;
-            for (int j = r + 1; j <= t; ++j) v -= R[r][j] * Ri[j][t];
-            Ri[r][t] = v * d_inv[r];
-        }
+    // column b of R^{-1}, from the last row up
+    float x[PB];
+#pragma unroll
+    for (int a = 0; a < PB; ++a) x[a] = a == b ? 1.f : 0.f;
+#pragma unroll
+    for (int j = PB - 1; j >= 0; --j) {
+        x[j] *= rinv[j];
+#pragma unroll
+        for (int a = 0; a < j; ++a) x[a] = fmaf(-G[a][j], x[j], x[a]);
     }
-    __syncwarp();
-    for (int e = t; e < PMAX * PMAX; e += 32) {
-        int a = e / PMAX, b = e % PMAX;
-        C[(long long)i * PMAX * PMAX + e] = (a < p && b < p) ? f32_to_f64(d[a] * Ri[a][b]) : 0.0;
-    }
+#pragma unroll
+    for (int a = 0; a < PB; ++a)
+        if (b < PMAX) C[a * PMAX + b] = a < p && b < p && a <= b ? dinv[a] * x[a] : 0.f;
 }
 
-// X = W C in FP32 arithmetic, on blocks of 32 rows.
-__global__ void __launch_bounds__(TPB) k_update32(const double* __restrict__ W, double* __restrict__ X,
-                                                  const double* __restrict__ C, const int* __restrict__ n_,
+constexpr int G32_T = 256;
+__global__ void __launch_bounds__(G32_T) k_gram_cholqr32(const float* __restrict__ W, int ldw, float* __restrict__ Gp,
+                                                         float* __restrict__ C, const int* __restrict__ n_,
+                                                         const long long* __restrict__ roff_,
+                                                         const int* __restrict__ p_, int gsplit,
+                                                         unsigned* __restrict__ ticket) {
+    __shared__ float red[G32_T][17];
+    __shared__ float G[PMAX][PMAX + 4];
+    __shared__ float dinv[PMAX];
+    __shared__ int s_last;
+    const int i = blockIdx.x, sp = blockIdx.y, t = threadIdx.x;
+    const int n = n_[i], p = p_[i], q = (p + 3) / 4;
+    if (p == 0) return;
+    const int ntile = q * (q + 1) / 2, lanes = G32_T / ntile;
+    const int rows_per = (n + gsplit - 1) / gsplit;
+    const int r_lo = sp * rows_per, r_hi = min(n, r_lo + rows_per);
+    const int tile = t % ntile, rl = t / ntile;
+    int a = 0, rem = tile;
+    while (rem >= q - a) { rem -= q - a; ++a; }
+    const int b = a + rem;
+    float acc[4][4] = {};
+    if (rl < lanes) {
+        const float* base = W + roff_[i] * ldw;
+#pragma unroll 4
+        for (int r = r_lo + rl; r < r_hi; r += lanes) {
+            const float4 u = *reinterpret_cast<const float4*>(base + (long long)r * ldw + 4 * a);
+            const float4 v = *reinterpret_cast<const float4*>(base + (long long)r * ldw + 4 * b);
+            const float uu[4] = {u.x, u.y, u.z, u.w}, vv[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+            for (int x = 0; x < 4; ++x)
+#pragma unroll
+                for (int y = 0; y < 4; ++y) acc[x][y] = fmaf(uu[x], vv[y], acc[x][y]);
+        }
+    }
+#pragma unroll
+    for (int x = 0; x < 4; ++x)
+#pragma unroll
+        for (int y = 0; y < 4; ++y) red[t][4 * x + y] = acc[x][y];
+    __syncthreads();
+    float* Gs = Gp + ((long long)i * gsplit + sp) * PMAX * PMAX;
+    for (int e = t; e < ntile * 16; e += G32_T) {
+        const int tl = e >> 4, xy = e & 15;
+        float s = 0.f;
+        for (int l = 0; l < lanes; ++l) s += red[l * ntile + tl][xy];
+        int ta = 0, tr = tl;
+        while (tr >= q - ta) { tr -= q - ta; ++ta; }
+        Gs[(4 * ta + (xy >> 2)) * PMAX + 4 * (ta + tr) + (xy & 3)] = s;
+    }
+    __threadfence();
+    __syncthreads();
+    if (t == 0) s_last = atomicAdd(&ticket[i], 1u) == (unsigned)gsplit - 1;
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    for (int e = t; e < 16 * q * q; e += G32_T) {
+        const int x = e / (4 * q), y = e % (4 * q);
+        float s = 0.f;
+        if (x <= y && y < p)
+            for (int k = 0; k < gsplit; ++k) s += __ldcg(Gp + ((long long)i * gsplit + k) * PMAX * PMAX + x * PMAX + y);
+        G[x][y] = s;
+    }
+    if (t == 0) ticket[i] = 0;
+    __syncthreads();
+    if (t >= 32) return;
+    float* Ci = C + (long long)i * PMAX * PMAX;
+    if (ldw <= 12) cholqr_warp<12>(G, dinv, p, Ci);
+    else if (ldw <= 16) cholqr_warp<16>(G, dinv, p, Ci);
+    else if (ldw <= 20) cholqr_warp<20>(G, dinv, p, Ci);
+    else cholqr_warp<32>(G, dinv, p, Ci);
+}
+
+// X = W C on blocks of 32 rows (FP32 products, stored as FP64): the end of
+// the start phase.  Columns >= p stay as they are.
+__global__ void __launch_bounds__(TPB) k_update32(const float* __restrict__ W, int ldw, double* __restrict__ X,
+                                                  const float* __restrict__ C, const int* __restrict__ n_,
                                                   const int* __restrict__ K_, const long long* __restrict__ roff_,
                                                   const int* __restrict__ p_, int ldx) {
     __shared__ float sC[PMAX][LD], sW[ROWBLK][LD];
@@ -1166,11 +1187,11 @@ __global__ void __launch_bounds__(TPB) k_update32(const double* __restrict__ W, 
     if (r0 >= rows) return;
     const long long roff = roff_[i];
     const int t = threadIdx.x;
-    for (int e = t; e < p * p; e += TPB) sC[e / p][e % p] = f64_to_f32(C[(long long)i * PMAX * PMAX + (e / p) * PMAX + e % p]);
+    for (int e = t; e < p * p; e += TPB) sC[e / p][e % p] = C[(long long)i * PMAX * PMAX + (e / p) * PMAX + e % p];
     for (int e = t; e < ROWBLK * p; e += TPB) {
         int rr = e / p, c = e % p;
         int r = r0 + rr;
-        sW[rr][c] = r < n ? f64_to_f32(W[(roff + r) * ldx + c]) : 0.f;
+        sW[rr][c] = r < n ? W[(roff + r) * ldw + c] : 0.f;
     }
     __syncthreads();
     for (int e = t; e < ROWBLK * p; e += TPB) {
@@ -1179,6 +1200,19 @@ __global__ void __launch_bounds__(TPB) k_update32(const double* __restrict__ W, 
         float x = 0.f;
         for (int j = 0; j < p; ++j) x += sW[rr][j] * sC[j][c];
         X[(roff + r0 + rr) * ldx + c] = f32_to_f64(x);
+    }
+}
+
+// W = X rounded to FP32 (columns >= p_i are zero in X): the start phase's first block
+__global__ void k_start32(const double* __restrict__ X, int ldx, float* __restrict__ W, int ldw,
+                          const int* __restrict__ K_, const long long* __restrict__ roff_) {
+    const int i = blockIdx.y;
+    const long long rows = (long long)K_[i] * NB;
+    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < rows * ldw;
+         e += (long long)gridDim.x * blockDim.x) {
+        const long long r = e / ldw;
+        const int c = (int)(e % ldw);
+        W[(roff_[i] + r) * ldw + c] = f64_to_f32(X[(roff_[i] + r) * ldx + c]);
     }
 }
 
@@ -1275,7 +1309,21 @@ void GevpBatch::alloc(cudaStream_t s) {
     P = K.P;
     d_p.upload(p, s);
     size_t rows = (size_t)K.total_rows;
-    for (DevBuf<double>* b : {&X, &AX, &BX, &Y, &AY, &BY, &W}) { b->alloc(rows * ldx); b->zero(s); }
+    for (DevBuf<double>* b : {&X, &AX, &BX, &Y, &AY, &BY}) { b->alloc(rows * ldx); b->zero(s); }
+    if (K.prec) {
+        int pm = 1;
+        for (int v : p) pm = std::max(pm, v);
+        ldw = (pm + 3) / 4 * 4;
+        W32.alloc(rows * ldw);
+        W32.zero(s);
+        W.release();
+        ticket.alloc(P);
+        ticket.zero(s);
+    } else {
+        ldw = ldx;
+        W.alloc(rows * ldx);
+        W.zero(s);
+    }
     H.alloc((size_t)P * PMAX * PMAX);
     M.alloc((size_t)P * PMAX * PMAX);
     // row splits: about 2048 CTAs in total, at least 64 rows per split (the
@@ -1309,6 +1357,9 @@ GevpBatch GevpBatch::slice(int p0, int np, int group) const {
                     std::make_pair(&v.Y, &Y), std::make_pair(&v.AY, &AY), std::make_pair(&v.BY, &BY),
                     std::make_pair(&v.W, &W)})
         *pr.first = pr.second->view(0, pr.second->n);
+    v.ldw = ldw;
+    v.W32 = W32.view(0, W32.n);
+    v.ticket = ticket.view(p0, ticket.n ? np : 0);
     const size_t q2 = (size_t)PMAX * PMAX;
     v.H = H.view(p0 * q2, np * q2); v.M = M.view(p0 * q2, np * q2); v.C = C.view(p0 * q2, np * q2);
     v.theta = theta.view((size_t)p0 * PMAX, (size_t)np * PMAX);
@@ -1342,15 +1393,23 @@ void eig_init(GevpBatch& g, unsigned long long seed, cudaStream_t s) {
 
 void eig_form_rhs(GevpBatch& g, double sigma, bool first, cudaStream_t s) {
     dim3 grid(32, g.P);
-    k_form_rhs<<<grid, 256, 0, s>>>(g.W.p, g.AX.p, g.BX.p, g.theta.p, g.K.d_n.p, g.K.d_K.p, g.K.d_roff.p, g.d_p.p,
-                                    g.ldx, sigma, first ? 1 : 0, g.done.p);
+    if (g.K.prec)
+        k_form_rhs<float><<<grid, 256, 0, s>>>(g.W32.p, g.ldw, g.AX.p, g.BX.p, g.theta.p, g.K.d_n.p, g.K.d_K.p,
+                                               g.K.d_roff.p, g.d_p.p, g.ldx, sigma, first ? 1 : 0, g.done.p);
+    else
+        k_form_rhs<double><<<grid, 256, 0, s>>>(g.W.p, g.ldw, g.AX.p, g.BX.p, g.theta.p, g.K.d_n.p, g.K.d_K.p,
+                                                g.K.d_roff.p, g.d_p.p, g.ldx, sigma, first ? 1 : 0, g.done.p);
     MSDD_LAUNCH_CHECK();
 }
 
 void eig_form_y(GevpBatch& g, double sigma, bool first, cudaStream_t s) {
     dim3 grid(32, g.P);
-    k_form_y<<<grid, 256, 0, s>>>(g.Y.p, g.X.p, g.W.p, g.theta.p, g.K.d_n.p, g.K.d_K.p, g.K.d_roff.p, g.d_p.p, g.ldx,
-                                  sigma, first ? 1 : 0, g.done.p);
+    if (g.K.prec)
+        k_form_y<float><<<grid, 256, 0, s>>>(g.Y.p, g.X.p, g.W32.p, g.ldw, g.theta.p, g.K.d_n.p, g.K.d_K.p,
+                                             g.K.d_roff.p, g.d_p.p, g.ldx, sigma, first ? 1 : 0, g.done.p);
+    else
+        k_form_y<double><<<grid, 256, 0, s>>>(g.Y.p, g.X.p, g.W.p, g.ldw, g.theta.p, g.K.d_n.p, g.K.d_K.p,
+                                              g.K.d_roff.p, g.d_p.p, g.ldx, sigma, first ? 1 : 0, g.done.p);
     MSDD_LAUNCH_CHECK();
 }
 
@@ -1368,13 +1427,23 @@ void eig_check_knorm(GevpBatch& g, const EigParams& ep, int it, cudaStream_t s) 
     MSDD_LAUNCH_CHECK();
 }
 
-void eig_cholqr32(GevpBatch& g, cudaStream_t s) {
-    k_gram32<<<dim3(g.P, g.gsplit), TPB, 0, s>>>(g.W.p, g.Hp.p, g.K.d_n.p, g.K.d_roff.p, g.d_p.p, g.ldx, g.gsplit);
+void eig_start32(GevpBatch& g, float* W, cudaStream_t s) {
+    k_start32<<<dim3(32, g.P), 256, 0, s>>>(g.X.p, g.ldx, W, g.ldw, g.K.d_K.p, g.K.d_roff.p);
     MSDD_LAUNCH_CHECK();
-    k_cholqr<<<g.P, 256, 0, s>>>(g.Hp.p, g.gsplit, g.C.p, g.d_p.p);
+}
+
+void eig_cholqr32(GevpBatch& g, const float* W, cudaStream_t s) {
+    // the FP64 Gram partials and coefficients are free in this phase and hold the FP32 ones
+    k_gram_cholqr32<<<dim3(g.P, g.gsplit), G32_T, 0, s>>>(W, g.ldw, reinterpret_cast<float*>(g.Hp.p),
+                                                          reinterpret_cast<float*>(g.C.p), g.K.d_n.p, g.K.d_roff.p,
+                                                          g.d_p.p, g.gsplit, g.ticket.p);
     MSDD_LAUNCH_CHECK();
+}
+
+void eig_update32(GevpBatch& g, const float* W, cudaStream_t s) {
     dim3 grid(g.nblk_max, g.P);
-    k_update32<<<grid, TPB, 0, s>>>(g.W.p, g.X.p, g.C.p, g.K.d_n.p, g.K.d_K.p, g.K.d_roff.p, g.d_p.p, g.ldx);
+    k_update32<<<grid, TPB, 0, s>>>(W, g.ldw, g.X.p, reinterpret_cast<const float*>(g.C.p), g.K.d_n.p, g.K.d_K.p,
+                                    g.K.d_roff.p, g.d_p.p, g.ldx);
     MSDD_LAUNCH_CHECK();
 }
 

@@ -26,7 +26,13 @@ struct GevpBatch {
     std::vector<int> p;               // block size per problem (<= PMAX)
     DevBuf<int> d_p;
     TileBatch K;                      // factor of Abar + sigma B (rows = problem size)
-    DevBuf<double> X, AX, BX, Y, AY, BY, W;        // (total_rows x ldx)
+    DevBuf<double> X, AX, BX, Y, AY, BY, W;        // (total_rows x ldx); W with FP64 factors only
+    // right-hand sides and solutions beside FP32 factors (total_rows x ldw,
+    // ldw = the largest p rounded up to 4): the solves round them to FP32
+    // either way, so FP32 storage halves their traffic at the same results
+    DevBuf<float> W32;
+    int ldw = PMAX;
+    DevBuf<unsigned> ticket;          // per problem: row ranges of the FP32 Gram that are done
     DevBuf<double> H, M, C, theta, res;            // per problem PMAX^2 / PMAX
     int gsplit = 1;                                // row splits of the Gram products
     DevBuf<double> Hp, Mp;                         // per (problem, split) PMAX^2 partial Grams
@@ -67,9 +73,11 @@ void eig_form_y(GevpBatch& g, double sigma, bool first, cudaStream_t s);
 void eig_form_y_knorm(GevpBatch& g, double sigma, cudaStream_t s);
 // Convergence test on the K^+-norm residuals (regularised coarse pencils).
 void eig_check_knorm(GevpBatch& g, const EigParams& ep, int it, cudaStream_t s);
-// FP32 start phase: X <- orthonormal basis of span(W) by Euclidean CholQR
-// (Gram with FP32 products, FP64 Cholesky of the scaled p x p Gram).
-void eig_cholqr32(GevpBatch& g, cudaStream_t s);
+// FP32 start phase: W <- X in FP32; C (FP32, in the buffer of g.C) with W C an
+// orthonormal basis of span(W) by Euclidean CholQR; X <- W C.
+void eig_start32(GevpBatch& g, float* W, cudaStream_t s);
+void eig_cholqr32(GevpBatch& g, const float* W, cudaStream_t s);
+void eig_update32(GevpBatch& g, const float* W, cudaStream_t s);
 // H = Y^T AY, M = Y^T BY.
 void eig_gram(GevpBatch& g, cudaStream_t s);
 // Rayleigh-Ritz: theta ascending, C with C^T M C = I.

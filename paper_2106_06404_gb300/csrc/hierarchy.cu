@@ -90,8 +90,8 @@ void dense_inverse(const TileBatch& tb, double* out, const std::vector<long long
 
 // Subspace iteration driver.  apply(v, p0, X, AX, BX, skip, s) applies Abar
 // and B to the problems of batch view v (first problem p0 of the whole
-// batch), solve(v, p0, ncols, s) applies K^{-1} to v.W, bapply32(v, p0, X, W, s)
-// is the FP32 B apply.  `tag` names the kernel families for profiling;
+// batch), solve(v, p0, ncols, W32, s) applies K^{-1} to W32 (FP32 factors) or
+// v.W, bapply32(v, p0, W, Wout, C, s) is Wout = (B W) C in FP32.  `tag` names the kernel families for profiling;
 // `apply_bytes`/`apply_flops` are the algorithmic amounts of one operator
 // application per problem.
 //
@@ -154,24 +154,29 @@ void run_eig(GevpBatch& g, const EigParams& ep, Apply apply, Solve solve, BApply
         am[k].solve_b = am[k].sb0;
         am[k].solve_f = am[k].sf0;
     }
-    // FP32 start phase: block inverse iteration Y = K~^{-1} B X with Euclidean
-    // CholQR, all in FP32 arithmetic; the FP64 phase below starts from its
-    // subspace and alone decides convergence.
+    // FP32 start phase: block inverse iteration W <- K~^{-1} B (W C), C from
+    // the Euclidean CholQR of W, all in FP32; the FP64 phase below starts from
+    // its subspace and alone decides convergence.  The blocks alternate
+    // between W32 and a second buffer (B reads neighbouring rows).
+    DevBuf<float> wb(fp32_iters > 0 ? g.W32.n : 0);
+    for (int k = 0; k < G && fp32_iters > 0; ++k) eig_start32(gv[k], wb.p, gs[k]);
     for (int it = 0; it < fp32_iters; ++it)
         for (int k = 0; k < G; ++k) {
             GevpBatch& v = gv[k];
+            float *src = it % 2 == 0 ? wb.p : v.W32.p, *dst = it % 2 == 0 ? v.W32.p : wb.p;
             prof.begin(tag + "_fp32_start_other", gs[k]);
-            bapply32(v, gp0[k], v.X.p, v.W.p, gs[k]);
+            bapply32(v, gp0[k], src, dst, it == 0 ? nullptr : reinterpret_cast<const float*>(v.C.p), gs[k]);
             prof.end(gs[k], 0.0, 0.0);
             prof.begin(tag + "_solve", gs[k]);
-            solve(v, gp0[k], am[k].pm, gs[k]);
+            solve(v, gp0[k], am[k].pm, dst, gs[k]);
             prof.end(gs[k], am[k].sb0, am[k].sf0);
             if (G == 2 && k == 0 && it == 0) {
                 MSDD_CUDA(cudaEventRecord(ev_off, gs[0]));        // the second half starts one solve later
                 MSDD_CUDA(cudaStreamWaitEvent(gs[1], ev_off, 0));
             }
             prof.begin(tag + "_fp32_start_other", gs[k]);
-            eig_cholqr32(v, gs[k]);
+            eig_cholqr32(v, dst, gs[k]);
+            if (it + 1 == fp32_iters) eig_update32(v, dst, gs[k]);
             prof.end(gs[k], 0.0, 0.0);
         }
     std::vector<int> active(G), iter(G, 0);
@@ -187,7 +192,7 @@ void run_eig(GevpBatch& g, const EigParams& ep, Apply apply, Solve solve, BApply
         const double fr = (double)active[k] / v.P;
         if (!fused || first) eig_form_rhs(v, ep.sigma, first, s);
         prof.begin(tag + "_solve", s);
-        solve(v, gp0[k], am[k].pm, s);
+        solve(v, gp0[k], am[k].pm, v.W32.p, s);
         prof.end(s, am[k].solve_b * fr, am[k].solve_f * fr);
         if (offset) {
             MSDD_CUDA(cudaEventRecord(ev_off, s));
@@ -356,7 +361,7 @@ std::vector<ProbBox> make_fine_boxes(const Geom& g, const msdd_decomp& dec) {
 size_t Hierarchy::device_bytes() const {
     size_t b = 0;
     b += fdir.bytes() + fge.K.bytes() + cdir.bytes() + mdir.bytes() + mge.K.bytes();
-    b += (fge.X.n + fge.AX.n + fge.BX.n + fge.Y.n + fge.AY.n + fge.BY.n + fge.W.n) * 8;
+    b += (fge.X.n + fge.AX.n + fge.BX.n + fge.Y.n + fge.AY.n + fge.BY.n + fge.W.n) * 8 + fge.W32.n * 4;
     b += (mge.X.n + mge.AX.n + mge.BX.n + mge.Y.n + mge.AY.n + mge.BY.n + mge.W.n) * 8;
     b += (Phi.n + A1.n + Abar_m.n + K_m.n + Zb.n + Tm.n + A0.n + frhs.n + v1.n + r0buf.n) * 8;
     b += (Minv.n + A0inv.n + y0buf.n + z1t.n) * 8;
@@ -581,12 +586,15 @@ void Hierarchy::build_fine() {
             [=](GevpBatch& v, int p0, const double* X, double* AX, double* BX, const int* skip, cudaStream_t s) {
                 apply_local(*ls, bx + p0, dim, v.K, X, AX, BX, v.ldx, block_p, skip, s);
             },
-            [=](GevpBatch& v, int, int pmax, cudaStream_t s) { tile_solve(v.K, v.W.p, v.ldx, pmax, v.done.p, s); },
-            [=](GevpBatch& v, int p0, const double* X, double* W, cudaStream_t s) {
-                apply_local_b32(*ls, bx + p0, dim, v.K, X, W, v.ldx, block_p, s);
+            [=](GevpBatch& v, int, int pmax, float* W32, cudaStream_t s) {
+                if (v.K.prec) tile_solve(v.K, W32, v.ldw, pmax, v.done.p, s);
+                else tile_solve(v.K, v.W.p, v.ldw, pmax, v.done.p, s);
+            },
+            [=](GevpBatch& v, int p0, const float* W, float* Wout, const float* C, cudaStream_t s) {
+                apply_local_b32(*ls, bx + p0, dim, v.K, W, Wout, v.ldw, C, s);
             },
             [=](GevpBatch& v, int p0, cudaStream_t s) {
-                apply_local_rhs(*ls, bx + p0, dim, v.K, v.X.p, v.W.p, v.ldx, v.d_p.p, v.theta.p, ep.sigma,
+                apply_local_rhs(*ls, bx + p0, dim, v.K, v.X.p, v.W.p, v.W32.p, v.ldw, v.ldx, v.d_p.p, v.theta.p, ep.sigma,
                                 v.partial.p, v.nblk_max, v.done.p, s);
             },
             true, opt.precision == 1 ? opt.fp32_start_iters : 0,
@@ -967,14 +975,14 @@ void Hierarchy::build_coarse() {
                     apply_dense_pencil(Ab, dao + p0, dng + p0, dno + p0, v.K, X, AX, BX, v.ldx, block_p, skip, v.P,
                                        ngen_max, s);
                 },
-                [=](GevpBatch& v, int p0, int, cudaStream_t s) {
+                [=](GevpBatch& v, int p0, int, float*, cudaStream_t s) {
                     gemm_batched(dki + p0, v.P, 0, 0, 1.0, Kinv, v.W.p, 0.0, Wtp, ngen_max, pmax_m, s, nullptr,
                                  v.done.p);
                     const long long e0 = mrow[p0], e1 = mrow[p0 + v.P];
                     MSDD_CUDA(cudaMemcpyAsync(v.W.p + e0, Wtp + e0, (e1 - e0) * sizeof(double),
                                               cudaMemcpyDeviceToDevice, s));
                 },
-                [=](GevpBatch&, int, const double*, double*, cudaStream_t) {},
+                [=](GevpBatch&, int, const float*, float*, const float*, cudaStream_t) {},
                 [=](GevpBatch&, int, cudaStream_t) {}, false, 0,
                 st, nullptr, prof, "coarse_gevp", (double)ngen_max * ngen_max * 8.0, 2.0 * ngen_max * ngen_max * block_p,
                 static_cast<int*>(pinned));

@@ -3,6 +3,7 @@
 #include "pcg.cuh"
 
 #include <cstring>
+#include <type_traits>
 #include <mutex>
 
 #include <cmath>
@@ -428,9 +429,10 @@ template <bool DF>
 __global__ void __launch_bounds__(128) k_apply_rhs(const ProbBox* __restrict__ boxes, int dim,
                                                    const long long* __restrict__ roff_, const int* __restrict__ K_,
                                                    const double* __restrict__ A, const double* __restrict__ B,
-                                                   const double* __restrict__ X, double* __restrict__ W, int ldx,
-                                                   const int* __restrict__ p_, const double* __restrict__ theta,
-                                                   double sigma, double* __restrict__ partial, int nblk_max,
+                                                   const double* __restrict__ X,
+                                                   std::conditional_t<DF, float, double>* __restrict__ W, int ldw,
+                                                   int ldx, const int* __restrict__ p_,
+                                                   const double* __restrict__ theta, double sigma, double* __restrict__ partial, int nblk_max,
                                                    const int* __restrict__ done) {
     static_assert(EIG_ROWBLK == NB, "row blocks are tile rows");
     __shared__ float sn[EIG_ROWBLK][PMAX + 1], sd[EIG_ROWBLK][PMAX + 1];
@@ -492,12 +494,12 @@ __global__ void __launch_bounds__(128) k_apply_rhs(const ProbBox* __restrict__ b
                 for (int c = 0; c < 4; ++c) { ax[c] = df_to_f64(axh[c], axl[c]); bx[c] = df_to_f64(bxh[c], bxl[c]); }
             }
         }
-        double* wr = W + (roff + r) * ldx + cb;
+        auto* wr = W + (roff + r) * ldw + cb;
 #pragma unroll
         for (int c = 0; c < 4; ++c)
             if (cb + c < p) {
                 const double rv = ax[c] - sth[cb + c] * bx[c];
-                wr[c] = r < n ? -rv * smu[cb + c] : 0.0;
+                wr[c] = from_f64<std::conditional_t<DF, float, double>>(r < n ? -rv * smu[cb + c] : 0.0);
                 const float rf = f64_to_f32(rv), bf = f64_to_f32(bx[c]);
                 sn[rr][cb + c] = rf * rf;
                 sd[rr][cb + c] = bf * bf;
@@ -516,42 +518,54 @@ __global__ void __launch_bounds__(128) k_apply_rhs(const ProbBox* __restrict__ b
     }
 }
 
-// FP32 arithmetic, conversions on the integer pipe; padding rows zeroed.
-__global__ void __launch_bounds__(128) k_apply_local_b32(const ProbBox* __restrict__ boxes, int dim,
-                                                         const long long* __restrict__ roff_, const int* __restrict__ K_,
-                                                         const float* __restrict__ B32, const double* __restrict__ X,
-                                                         double* __restrict__ W, int ldx, int ncols) {
-    const int i = blockIdx.y;
+// Wout = (B32 W) C in FP32 (padding rows zeroed; C null: the identity), on
+// blocks of 32 rows; a thread owns a row and four columns.  C (PMAX columns,
+// upper triangular) comes from the CholQR of W.  Bound by the loads of the
+// 3^d neighbour rows (L1/L2 hits mostly), 16 bytes each.
+template <int D>
+__global__ void __launch_bounds__(256) k_b32_cholqr(const ProbBox* __restrict__ boxes,
+                                                    const long long* __restrict__ roff_, const int* __restrict__ K_,
+                                                    const float* __restrict__ B32, const float* __restrict__ W,
+                                                    float* __restrict__ Wout, int ldw, const float* __restrict__ C) {
+    constexpr int NOFF = D == 3 ? 27 : 9;
+    __shared__ __align__(16) float sC[PMAX][PMAX], sT[NB][PMAX + 4];
+    const int i = blockIdx.y, r0 = blockIdx.x * NB;
+    if (r0 >= K_[i] * NB) return;
     const ProbBox pb = boxes[i];
-    const int n = box_size(pb.nlo, pb.nhi, dim);
-    const int rows = K_[i] * NB;
-    const int w0 = pb.nhi[0] - pb.nlo[0] + 1, w1 = dim >= 2 ? pb.nhi[1] - pb.nlo[1] + 1 : 1;
-    const int noff = dim == 3 ? 27 : 9;
-    const int nchunk = (ncols + 7) / 8;
+    const int n = box_size(pb.nlo, pb.nhi, D);
+    const int w0 = pb.nhi[0] - pb.nlo[0] + 1, w1 = pb.nhi[1] - pb.nlo[1] + 1;
     const long long roff = roff_[i];
-    for (long long w = blockIdx.x * (long long)blockDim.x + threadIdx.x; w < (long long)rows * nchunk;
-         w += (long long)gridDim.x * blockDim.x) {
-        const int r = (int)(w / nchunk), c0 = (int)(w % nchunk) * 8;
-        const int c1 = min(ncols, c0 + 8);
-        float acc[8];
+    const int cg = threadIdx.x, rr = threadIdx.y, r = r0 + rr, t = rr * blockDim.x + cg;
+    if (C)
+        for (int e = t; e < ldw * ldw; e += blockDim.x * NB)
+            sC[e / ldw][e % ldw] = C[(long long)i * PMAX * PMAX + (e / ldw) * PMAX + e % ldw];
+    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (r < n) {
+        const float* br = B32 + (roff + r) * NOFF;
+        const float* xr = W + (roff + r) * ldw + 4 * cg;
 #pragma unroll
-        for (int c = 0; c < 8; ++c) acc[c] = 0.f;
-        if (r < n) {
-            const float* br = B32 + (roff + r) * noff;
-            for (int oi = 0; oi < noff; ++oi) {
-                const float b = br[oi];
-                if (b == 0.f) continue;
-                const double* xr = X + (roff + r + nbr_offset(oi, w0, w1, dim)) * ldx;
-#pragma unroll
-                for (int c = 0; c < 8; ++c)
-                    if (c0 + c < c1) acc[c] += b * f64_to_f32(xr[c0 + c]);
-            }
+        for (int oi = 0; oi < NOFF; ++oi) {
+            const float b = br[oi];
+            if (b == 0.f) continue;                  // also: the neighbour is outside the box
+            const int o = (oi % 3 - 1) + w0 * ((oi / 3) % 3 - 1) + (D == 3 ? w0 * w1 * (oi / 9 - 1) : 0);
+            const float4 x = *reinterpret_cast<const float4*>(xr + (long long)o * ldw);
+            acc.x = fmaf(b, x.x, acc.x); acc.y = fmaf(b, x.y, acc.y);
+            acc.z = fmaf(b, x.z, acc.z); acc.w = fmaf(b, x.w, acc.w);
         }
-        double* wr = W + (roff + r) * ldx;
-#pragma unroll
-        for (int c = 0; c < 8; ++c)
-            if (c0 + c < c1) wr[c0 + c] = f32_to_f64(acc[c]);
     }
+    if (C) {
+        *reinterpret_cast<float4*>(&sT[rr][4 * cg]) = acc;
+        __syncthreads();
+        acc = make_float4(0.f, 0.f, 0.f, 0.f);
+        const int kmax = 4 * cg + 4;                 // C is upper triangular
+        for (int k = 0; k < kmax; ++k) {
+            const float v = sT[rr][k];
+            const float4 c = *reinterpret_cast<const float4*>(&sC[k][4 * cg]);
+            acc.x = fmaf(v, c.x, acc.x); acc.y = fmaf(v, c.y, acc.y);
+            acc.z = fmaf(v, c.z, acc.z); acc.w = fmaf(v, c.w, acc.w);
+        }
+    }
+    *reinterpret_cast<float4*>(Wout + (roff + r) * ldw + 4 * cg) = acc;
 }
 
 // Stencil coefficients of the global operator: S[o * nun + u] = A(u, u + o)
@@ -742,24 +756,27 @@ void apply_local(const LocalStencil& ls, const ProbBox* d_boxes, int dim, const 
 }
 
 void apply_local_rhs(const LocalStencil& ls, const ProbBox* d_boxes, int dim, const TileBatch& layout,
-                     const double* X, double* W, int ldx, const int* d_p, const double* theta, double sigma,
-                     double* partial, int nblk_max, const int* done, cudaStream_t s) {
+                     const double* X, double* W, float* W32, int ldw, int ldx, const int* d_p, const double* theta,
+                     double sigma, double* partial, int nblk_max, const int* done, cudaStream_t s) {
     if (layout.P == 0) return;
     dim3 grid(nblk_max, layout.P);
     if (layout.prec)
-        k_apply_rhs<true><<<grid, 128, 0, s>>>(d_boxes, dim, layout.d_roff.p, layout.d_K.p, ls.a.p, ls.b.p, X, W, ldx,
-                                               d_p, theta, sigma, partial, nblk_max, done);
+        k_apply_rhs<true><<<grid, 128, 0, s>>>(d_boxes, dim, layout.d_roff.p, layout.d_K.p, ls.a.p, ls.b.p, X, W32,
+                                               ldw, ldx, d_p, theta, sigma, partial, nblk_max, done);
     else
-        k_apply_rhs<false><<<grid, 128, 0, s>>>(d_boxes, dim, layout.d_roff.p, layout.d_K.p, ls.a.p, ls.b.p, X, W, ldx,
-                                                d_p, theta, sigma, partial, nblk_max, done);
+        k_apply_rhs<false><<<grid, 128, 0, s>>>(d_boxes, dim, layout.d_roff.p, layout.d_K.p, ls.a.p, ls.b.p, X, W,
+                                                ldw, ldx, d_p, theta, sigma, partial, nblk_max, done);
     MSDD_LAUNCH_CHECK();
 }
 
 void apply_local_b32(const LocalStencil& ls, const ProbBox* d_boxes, int dim, const TileBatch& layout,
-                     const double* X, double* W, int ldx, int ncols, cudaStream_t s) {
+                     const float* W, float* Wout, int ldw, const float* C, cudaStream_t s) {
     if (layout.P == 0) return;
-    dim3 grid(64, layout.P);
-    k_apply_local_b32<<<grid, 128, 0, s>>>(d_boxes, dim, layout.d_roff.p, layout.d_K.p, ls.b32.p, X, W, ldx, ncols);
+    const dim3 grid(layout.max_K, layout.P), block(ldw / 4, NB);
+    if (dim == 3)
+        k_b32_cholqr<3><<<grid, block, 0, s>>>(d_boxes, layout.d_roff.p, layout.d_K.p, ls.b32.p, W, Wout, ldw, C);
+    else
+        k_b32_cholqr<2><<<grid, block, 0, s>>>(d_boxes, layout.d_roff.p, layout.d_K.p, ls.b32.p, W, Wout, ldw, C);
     MSDD_LAUNCH_CHECK();
 }
 

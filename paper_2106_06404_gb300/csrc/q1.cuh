@@ -118,13 +118,16 @@ void apply_local(const LocalStencil& ls, const ProbBox* d_boxes, int dim, const 
 // W = BX - (AX + sigma BX) diag(1 / (theta + sigma)) with AX, BX from the
 // stored stencils (zero on padding rows, columns < p_i), and the residual
 // partial sums of X (layout of EIG_ROWBLK) for the problems with done == 0;
-// theta is PMAX per problem, partial (P * nblk_max * 2 PMAX).
+// theta is PMAX per problem, partial (P * nblk_max * 2 PMAX).  The result goes
+// to W32 beside FP32 factors, to W otherwise (leading dimension ldw).
 void apply_local_rhs(const LocalStencil& ls, const ProbBox* d_boxes, int dim, const TileBatch& layout,
-                     const double* X, double* W, int ldx, const int* d_p, const double* theta, double sigma,
-                     double* partial, int nblk_max, const int* done, cudaStream_t s);
-// W = X Abar X X in FP32 arithmetic from b32 (same contract as apply_b32).
+                     const double* X, double* W, float* W32, int ldw, int ldx, const int* d_p, const double* theta,
+                     double sigma, double* partial, int nblk_max, const int* done, cudaStream_t s);
+// Wout = (B W) C in FP32 arithmetic from b32 (blocks of ldw columns, a multiple
+// of 4; zero on padding rows); C is PMAX x PMAX per problem and upper
+// triangular, null for the identity.
 void apply_local_b32(const LocalStencil& ls, const ProbBox* d_boxes, int dim, const TileBatch& layout,
-                     const double* X, double* W, int ldx, int ncols, cudaStream_t s);
+                     const float* W, float* Wout, int ldw, const float* C, cudaStream_t s);
 
 // Stored 3^d-point stencil of the global operator: S[o * n + u] = A(u, u + o),
 // offsets o lexicographic (x fastest) in {-1, 0, 1}^d, zero where u + o is

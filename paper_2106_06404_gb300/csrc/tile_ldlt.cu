@@ -158,11 +158,11 @@ __global__ void __launch_bounds__(TPB) k_tile_factor(
 // ------------------------------------------------------------------ solve
 // acc[r][c] for the 4 (row, column) pairs owned by a thread: row r = t>>3,
 // columns c0 + 8q.
-template <typename T>
+template <typename T, typename XT>
 __global__ void __launch_bounds__(TPB) k_tile_solve(
     const T* __restrict__ tiles, const T* __restrict__ dinv, const int* __restrict__ n_,
     const int* __restrict__ kb_, const int* __restrict__ K_, const long long* __restrict__ toff_,
-    const long long* __restrict__ roff_, double* __restrict__ X, int ldx, int ncols,
+    const long long* __restrict__ roff_, XT* __restrict__ X, int ldx, int ncols,
     const int* __restrict__ skip, const int* __restrict__ gdone)
 {
     __shared__ T Sa[NB][LDS];
@@ -186,7 +186,7 @@ __global__ void __launch_bounds__(TPB) k_tile_solve(
     // forward: z_R = T_R (x_R - sum_J L_RJ z_J)
     for (int R = 0; R < K; ++R) {
         T acc[4];
-        double* xr = X + (roff + (long long)R * NB) * ldx;
+        XT* xr = X + (roff + (long long)R * NB) * ldx;
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
             int c = c0 + 8 * q;
@@ -196,7 +196,7 @@ __global__ void __launch_bounds__(TPB) k_tile_solve(
         for (int J = Jmin; J < R; ++J) {
             __syncthreads();
             load_tile(Sa, tiles + tile_index(toff, kb, R, J));
-            const double* xj = X + (roff + (long long)J * NB) * ldx;
+            const XT* xj = X + (roff + (long long)J * NB) * ldx;
             for (int e = t; e < NB * NB; e += TPB) {
                 int a = e / NB, c = e % NB;
                 Sx[a][c] = c < ncols ? T(xj[(long long)a * ldx + c]) : T(0);
@@ -223,14 +223,14 @@ __global__ void __launch_bounds__(TPB) k_tile_solve(
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
             int c = c0 + 8 * q;
-            if (c < ncols) xr[(long long)r * ldx + c] = (double)out[q];
+            if (c < ncols) xr[(long long)r * ldx + c] = XT(out[q]);
         }
     }
     // backward: x_R = T_R^T (D_R^{-1} z_R - sum_I L_IR^T x_I)
     for (int R = K - 1; R >= 0; --R) {
         __syncthreads();
         T acc[4];
-        double* xr = X + (roff + (long long)R * NB) * ldx;
+        XT* xr = X + (roff + (long long)R * NB) * ldx;
         const T dr = dinv[roff + (long long)R * NB + r];
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
@@ -241,7 +241,7 @@ __global__ void __launch_bounds__(TPB) k_tile_solve(
         for (int I = R + 1; I <= Imax; ++I) {
             __syncthreads();
             load_tile(Sa, tiles + tile_index(toff, kb, I, R));
-            const double* xi = X + (roff + (long long)I * NB) * ldx;
+            const XT* xi = X + (roff + (long long)I * NB) * ldx;
             for (int e = t; e < NB * NB; e += TPB) {
                 int a = e / NB, c = e % NB;
                 Sx[a][c] = c < ncols ? T(xi[(long long)a * ldx + c]) : T(0);
@@ -268,7 +268,7 @@ __global__ void __launch_bounds__(TPB) k_tile_solve(
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
             int c = c0 + 8 * q;
-            if (c < ncols) xr[(long long)r * ldx + c] = (double)out[q];
+            if (c < ncols) xr[(long long)r * ldx + c] = XT(out[q]);
         }
     }
 }
@@ -776,237 +776,6 @@ __global__ void __launch_bounds__(S1T) k_tile_solve1_dense(
 }
 
 
-// ------------------------------------------------------------------ solve, several right-hand sides, band
-// For kb <= 2, one 64-thread CTA per problem.  Step R needs the diagonal
-// tile, the kb off-diagonal tiles of block row (forward) or block column
-// (backward) R, the 32 x ncols block R of X and D_R^{-1}; these are copied
-// into shared memory with cp.async BAND_STAGES - 1 steps ahead.  The last kb
-// solution blocks stay in a shared ring.  Thread t owns the register block
-// rows 4 (t >> 3) + i, i < 4, columns CPT (t & 7) + j, j < CPT.
-//
-// Tiles are stored in shared memory as 32 x 32 with the 4-element groups of
-// a row permuted: group g of row r sits at position g ^ ((r >> 2) & 7).  The
-// four rows 4 rg + i a warp reads together for one group (forward), and the
-// four groups rg of one row (backward), then fall in distinct banks.
-constexpr int BAND_STAGES = 3;
-constexpr int BAND_SLOTS = 3;      // diagonal tile + at most 2 off-diagonal tiles per step
-
-__device__ __forceinline__ int band_swz(int row) { return (row >> 2) & 7; }
-
-// copy one 32 x 32 tile (row-major in global memory) into the permuted layout
-template <typename T, int NT>
-__device__ __forceinline__ void band_async_tile(T* dst, const T* __restrict__ src) {
-    constexpr int PER = 16 / (int)sizeof(T);           // elements per 16-byte chunk
-    for (int ch = threadIdx.x; ch < NB2 / PER; ch += NT) {
-        const int e = ch * PER, r = e / NB, c = e % NB;
-        const int g = c >> 2, within = c & 3;
-        cp_async16(dst + r * NB + ((g ^ band_swz(r)) << 2) + within, src + e);
-    }
-}
-
-// four consecutive elements of a permuted tile: row r, group g
-template <typename T>
-__device__ __forceinline__ void band_load4(const T* tile, int r, int g, T (&v)[4]);
-template <>
-__device__ __forceinline__ void band_load4<float>(const float* tile, int r, int g, float (&v)[4]) {
-    const float4 x = *reinterpret_cast<const float4*>(tile + r * NB + ((g ^ band_swz(r)) << 2));
-    v[0] = x.x; v[1] = x.y; v[2] = x.z; v[3] = x.w;
-}
-template <typename T, int CPT, int CG>
-struct BandSmem {
-    static constexpr int ZLD = CG * CPT;                // columns held in the ring and Acc
-    static size_t bytes(int sxld) {
-        return sizeof(T) * ((size_t)BAND_STAGES * BAND_SLOTS * NB2 + (size_t)BAND_STAGES * NB + (size_t)(BAND_SLOTS + 1) * NB * ZLD) +
-               sizeof(double) * (size_t)BAND_STAGES * NB * sxld;
-    }
-};
-
-template <typename T, int CPT, int CG>
-__global__ void __launch_bounds__(8 * CG) k_tile_solve_band(
-    const T* __restrict__ tiles, const T* __restrict__ dinv, const int* __restrict__ kb_, const int* __restrict__ K_,
-    const long long* __restrict__ toff_, const long long* __restrict__ roff_, double* __restrict__ Xall, int ldx,
-    int ncols_all, const int* __restrict__ skip, const int* __restrict__ gdone)
-{
-    // blockIdx.y selects a chunk of ZLD columns (an independent set of
-    // right-hand sides solved by its own CTA)
-    constexpr int NST = BAND_STAGES, ZLD = BandSmem<T, CPT, CG>::ZLD, NT = 8 * CG;
-    const int cbase = blockIdx.y * ZLD;
-    const int ncols = min(ZLD, ncols_all - cbase);
-    double* __restrict__ X = Xall + cbase;
-    const int sxld = ((ncols + 1) / 2) * 2;             // staged columns of X (whole 16-byte chunks)
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    T* St = reinterpret_cast<T*>(smem_raw);                                   // [NST][SLOTS][32*32]
-    T* Sd = St + (size_t)NST * BAND_SLOTS * NB2;                              // [NST][32]   D^{-1}
-    T* Zr = Sd + (size_t)NST * NB;                                            // [SLOTS][32][ZLD]
-    T* Acc = Zr + (size_t)BAND_SLOTS * NB * ZLD;                              // [32][ZLD]
-    double* Sx = reinterpret_cast<double*>(Acc + (size_t)NB * ZLD);           // [NST][32][sxld]
-    const int i = blockIdx.x;
-    if (skip && skip[i]) return;
-    if (gdone && *gdone) return;
-    const int kb = kb_[i], K = K_[i];
-    const long long toff = toff_[i], roff = roff_[i];
-    const int t = threadIdx.x;
-    const int rg = t / CG, cg = t % CG, warp = t >> 5;
-    const int r0 = 4 * rg, c0 = CPT * cg;
-    // rows of this warp: 4 * (32 warp / CG) ... 4 * ((32 warp + 31) / CG) + 3
-    const int wrow_lo = 4 * ((32 * warp) / CG), wgrp_hi = (32 * warp + 31) / CG;
-    auto stile = [&](int st, int slot) { return St + (size_t)(st * BAND_SLOTS + slot) * NB2; };
-    auto issue = [&](int st, int R, bool fwd) {
-        if (R >= 0 && R < K) {
-            band_async_tile<T, NT>(stile(st, 0), tiles + tile_index(toff, kb, R, R));
-            for (int d = 1; d <= kb; ++d) {
-                const int o = fwd ? R - d : R + d;
-                if (o < 0 || o >= K) continue;
-                band_async_tile<T, NT>(stile(st, d), tiles + (fwd ? tile_index(toff, kb, R, o) : tile_index(toff, kb, o, R)));
-            }
-            if (!fwd) {
-                constexpr int PER = 16 / (int)sizeof(T);
-                for (int ch = t; ch < NB / PER; ch += NT)
-                    cp_async16(Sd + st * NB + ch * PER, dinv + roff + (long long)R * NB + ch * PER);
-            }
-            const int cpr = sxld / 2;                    // 16-byte chunks per row
-            const double* src = X + (roff + (long long)R * NB) * ldx;
-            double* dst = Sx + (size_t)st * NB * sxld;
-            for (int ch = t; ch < NB * cpr; ch += NT) {
-                const int r = ch / cpr, c = (ch % cpr) * 2;
-                cp_async16(dst + r * sxld + c, src + (long long)r * ldx + c);
-            }
-        }
-        cp_async_commit();
-    };
-    auto finish = [&](T (&acc)[4][CPT], int R, const T* Tt, bool fwd) {
-        // Acc <- acc; out = T_R acc (forward) or T_R^T acc (backward)
-#pragma unroll
-        for (int a = 0; a < 4; ++a)
-#pragma unroll
-            for (int j = 0; j < CPT; ++j) Acc[(r0 + a) * ZLD + c0 + j] = acc[a][j];
-        __syncthreads();
-        T out[4][CPT];
-#pragma unroll
-        for (int a = 0; a < 4; ++a)
-#pragma unroll
-            for (int j = 0; j < CPT; ++j) out[a][j] = T(0);
-        if (fwd) {
-            // T_R is lower triangular with zeros above the diagonal: the
-            // groups up to the warp's last row suffice
-            const int gmax = wgrp_hi + 1;
-#pragma unroll 4
-            for (int g = 0; g < gmax; ++g) {
-                T l[4][4];
-#pragma unroll
-                for (int a = 0; a < 4; ++a) band_load4<T>(Tt, r0 + a, g, l[a]);
-#pragma unroll
-                for (int kk = 0; kk < 4; ++kk) {
-                    const T* z = Acc + (4 * g + kk) * ZLD + c0;
-#pragma unroll
-                    for (int j = 0; j < CPT; ++j) {
-                        const T zv = z[j];
-#pragma unroll
-                        for (int a = 0; a < 4; ++a) out[a][j] += l[a][kk] * zv;
-                    }
-                }
-            }
-        } else {
-#pragma unroll 4
-            for (int k = wrow_lo; k < NB; ++k) {
-                T l[4];
-                band_load4<T>(Tt, k, rg, l);
-                const T* z = Acc + k * ZLD + c0;
-#pragma unroll
-                for (int j = 0; j < CPT; ++j) {
-                    const T zv = z[j];
-#pragma unroll
-                    for (int a = 0; a < 4; ++a) out[a][j] += l[a] * zv;
-                }
-            }
-        }
-        T* Zw = Zr + (size_t)(R % BAND_SLOTS) * NB * ZLD;
-#pragma unroll
-        for (int a = 0; a < 4; ++a) {
-            double* xw = X + (roff + (long long)R * NB + r0 + a) * ldx;
-#pragma unroll
-            for (int j = 0; j < CPT; ++j) {
-                Zw[(r0 + a) * ZLD + c0 + j] = out[a][j];
-                if (c0 + j < ncols) xw[c0 + j] = to_f64(out[a][j]);
-            }
-        }
-    };
-
-    // forward: z_R = T_R (x_R - sum_J L_RJ z_J)
-    for (int k = 0; k < NST - 1; ++k) issue(k, k, true);
-    for (int R = 0; R < K; ++R) {
-        const int st = R % NST;
-        cp_async_wait_n<NST - 2>();
-        __syncthreads();
-        issue((R + NST - 1) % NST, R + NST - 1, true);
-        T acc[4][CPT];
-        const double* xs = Sx + (size_t)st * NB * sxld;
-#pragma unroll
-        for (int a = 0; a < 4; ++a)
-#pragma unroll
-            for (int j = 0; j < CPT; ++j) acc[a][j] = (c0 + j < ncols) ? from_f64<T>(xs[(r0 + a) * sxld + c0 + j]) : T(0);
-        for (int d = 1; d <= kb; ++d) {
-            if (R - d < 0) break;
-            const T* L = stile(st, d);
-            const T* Z = Zr + (size_t)((R - d) % BAND_SLOTS) * NB * ZLD;
-#pragma unroll
-            for (int g = 0; g < NB / 4; ++g) {
-                T l[4][4];
-#pragma unroll
-                for (int a = 0; a < 4; ++a) band_load4<T>(L, r0 + a, g, l[a]);
-#pragma unroll
-                for (int kk = 0; kk < 4; ++kk) {
-                    const T* z = Z + (4 * g + kk) * ZLD + c0;
-#pragma unroll
-                    for (int j = 0; j < CPT; ++j) {
-                        const T zv = z[j];
-#pragma unroll
-                        for (int a = 0; a < 4; ++a) acc[a][j] -= l[a][kk] * zv;
-                    }
-                }
-            }
-        }
-        finish(acc, R, stile(st, 0), true);
-    }
-    cp_async_wait_n<0>();
-    __syncthreads();
-    // backward: x_R = T_R^T (D_R^{-1} z_R - sum_I L_IR^T x_I)
-    for (int k = 0; k < NST - 1; ++k) issue(k, K - 1 - k, false);
-    for (int R = K - 1, it = 0; R >= 0; --R, ++it) {
-        const int st = it % NST;
-        cp_async_wait_n<NST - 2>();
-        __syncthreads();
-        issue((it + NST - 1) % NST, R - (NST - 1), false);
-        T acc[4][CPT];
-        const double* xs = Sx + (size_t)st * NB * sxld;
-        const T* dv = Sd + st * NB;
-#pragma unroll
-        for (int a = 0; a < 4; ++a)
-#pragma unroll
-            for (int j = 0; j < CPT; ++j)
-                acc[a][j] = (c0 + j < ncols) ? dv[r0 + a] * from_f64<T>(xs[(r0 + a) * sxld + c0 + j]) : T(0);
-        for (int d = 1; d <= kb; ++d) {
-            if (R + d >= K) break;
-            const T* L = stile(st, d);
-            const T* Z = Zr + (size_t)((R + d) % BAND_SLOTS) * NB * ZLD;
-#pragma unroll 8
-            for (int k = 0; k < NB; ++k) {
-                T l[4];
-                band_load4<T>(L, k, rg, l);
-                const T* z = Z + k * ZLD + c0;
-#pragma unroll
-                for (int j = 0; j < CPT; ++j) {
-                    const T zv = z[j];
-#pragma unroll
-                    for (int a = 0; a < 4; ++a) acc[a][j] -= l[a] * zv;
-                }
-            }
-        }
-        finish(acc, R, stile(st, 0), false);
-    }
-    cp_async_wait_n<0>();
-}
-
 // ---- TMA / mbarrier helpers of the FP32 band solve.  Every mbarrier wait is
 // bounded; a kernel whose wait runs out records it in g_wait_timeouts.
 __device__ int g_wait_timeouts;
@@ -1433,41 +1202,6 @@ __global__ void __launch_bounds__(TF_NT) k_tile_factor_tc(
     if (t == 0) { status[i] = s_status; nreg[i] = s_nreg; }
 }
 
-// ---- the FP32 band solve with TMA tile loads, warp-specialised (kb <= 2)
-// The steps and expressions of k_tile_solve_band<float> (forward z_R = T_R
-// (x_R - sum_J L_RJ z_J), backward x_R = T_R^T (D_R^{-1} z_R - sum_I L_IR^T
-// x_I), products summed in the same order), arranged so that no block
-// barrier sits on the sweeps' chain: each
-// of W consumer warps owns C right-hand-side columns and all 32 rows of a
-// tile row (lane = row), so a step's data exchange is warp-internal
-// (__syncwarp); a producer warp streams the tiles of each step and D^{-1}
-// with TMA into an NST-stage ring ("full" mbarriers completed by the copies'
-// byte counts, "empty" mbarriers released by each consumer warp after its
-// last read of the stage).  Each lane prefetches its own row of the
-// right-hand sides with cp.async, XD steps ahead.  Column k of tile
-// L_{R,R-d} can be nonzero only where 32 d + r - k <= b (the band), so the
-// forward products start at k = 32 d - b and the backward ones stop at
-// k = b - 32 d + 31.  Every wait is bounded; on a timeout the CTA records it
-// (g_wait_timeouts), the producer waits (bounded) for the copies it still
-// has in flight, and the CTA returns.
-template <int C>
-__device__ __forceinline__ void ws_ld(const float* p, float (&v)[C]) {
-    if constexpr (C == 4) {
-        const float4 x = *reinterpret_cast<const float4*>(p);
-        v[0] = x.x; v[1] = x.y; v[2] = x.z; v[3] = x.w;
-    } else if constexpr (C == 2) {
-        const float2 x = *reinterpret_cast<const float2*>(p);
-        v[0] = x.x; v[1] = x.y;
-    } else {
-        v[0] = *p;
-    }
-}
-template <int C>
-__device__ __forceinline__ void ws_st(float* p, const float (&v)[C]) {
-    if constexpr (C == 4) *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]);
-    else if constexpr (C == 2) *reinterpret_cast<float2*>(p) = make_float2(v[0], v[1]);
-    else *p = v[0];
-}
 // element (row, col) of a 128-byte-swizzled 32 x 32 FP32 tile
 __device__ __forceinline__ int swz(int row, int col) { return row * NB + ((((col >> 2) ^ (row & 7))) << 2) + (col & 3); }
 
@@ -1484,12 +1218,10 @@ __device__ __forceinline__ void ws_row_product(const float* tile, const float* V
     }
 #pragma unroll
     for (int k = K0; k < K1; ++k) {
-        float v[C];
-        ws_ld<C>(V + k * C, v);
 #pragma unroll
         for (int c = 0; c < C; ++c) {
-            if (SIGN > 0) acc[c] += l[k - K0] * v[c];
-            else acc[c] -= l[k - K0] * v[c];
+            if (SIGN > 0) acc[c] += l[k - K0] * V[k * C + c];
+            else acc[c] -= l[k - K0] * V[k * C + c];
         }
     }
 }
@@ -1501,322 +1233,356 @@ __device__ __forceinline__ void ws_col_product(const float* tile, const float* V
     for (int k = 0; k < K1; ++k) l[k] = tile[swz(k, lane)];
 #pragma unroll
     for (int k = 0; k < K1; ++k) {
-        float v[C];
-        ws_ld<C>(V + k * C, v);
 #pragma unroll
         for (int c = 0; c < C; ++c) {
-            if (SIGN > 0) acc[c] += l[k] * v[c];
-            else acc[c] -= l[k] * v[c];
+            if (SIGN > 0) acc[c] += l[k] * V[k * C + c];
+            else acc[c] -= l[k] * V[k * C + c];
         }
     }
-}
-
-// Wide-band forms of the two products: the loads are volatile shared
-// loads issued eight k at a time ahead of their products (the compiler keeps
-// their order), with two partial sums per column.  With 13 tiles a step the
-// products dominate and this ordering is 2-12% faster; with 3 tiles the
-// plain forms above are.
-__device__ __forceinline__ float4 lds4_ordered(const float* p) {
-    float4 r;
-    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];\n"
-                 : "=f"(r.x), "=f"(r.y), "=f"(r.z), "=f"(r.w)
-                 : "r"(smem_u32(p)));
-    return r;
-}
-__device__ __forceinline__ float lds1_ordered(const float* p) {
-    float r;
-    asm volatile("ld.shared.f32 %0, [%1];\n" : "=f"(r) : "r"(smem_u32(p)));
-    return r;
-}
-__device__ __forceinline__ float2 lds2_ordered(const float* p) {
-    float2 r;
-    asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];\n" : "=f"(r.x), "=f"(r.y) : "r"(smem_u32(p)));
-    return r;
-}
-template <int C>
-__device__ __forceinline__ void ws_ld_ordered(const float* p, float (&v)[C]) {
-    if constexpr (C == 4) {
-        const float4 x = lds4_ordered(p);
-        v[0] = x.x; v[1] = x.y; v[2] = x.z; v[3] = x.w;
-    } else if constexpr (C == 2) {
-        const float2 x = lds2_ordered(p);
-        v[0] = x.x; v[1] = x.y;
-    } else {
-        ws_ld<C>(p, v);
-    }
-}
-template <int C, int K0, int K1, int SIGN>
-__device__ __forceinline__ void ws_row_product_wide(const float* tile, const float* V, int lane, float (&acc)[C]) {
-    constexpr int NK = K1 - K0;
-    static_assert(NK % 8 == 0, "k range in multiples of 8");
-    float l[NK];
-#pragma unroll
-    for (int g = K0 / 4; g < K1 / 4; ++g) {
-        const float4 x = lds4_ordered(tile + lane * NB + ((g ^ (lane & 7)) << 2));
-        l[4 * g - K0] = x.x; l[4 * g - K0 + 1] = x.y; l[4 * g - K0 + 2] = x.z; l[4 * g - K0 + 3] = x.w;
-    }
-    float a0[C], a1[C];
-#pragma unroll
-    for (int c = 0; c < C; ++c) { a0[c] = acc[c]; a1[c] = 0.f; }
-#pragma unroll
-    for (int k8 = 0; k8 < NK; k8 += 8) {
-        float v[8][C];
-#pragma unroll
-        for (int k = 0; k < 8; ++k) ws_ld_ordered<C>(V + (K0 + k8 + k) * C, v[k]);
-#pragma unroll
-        for (int k = 0; k < 8; k += 2)
-#pragma unroll
-            for (int c = 0; c < C; ++c) {
-                if (SIGN > 0) { a0[c] += l[k8 + k] * v[k][c]; a1[c] += l[k8 + k + 1] * v[k + 1][c]; }
-                else { a0[c] -= l[k8 + k] * v[k][c]; a1[c] -= l[k8 + k + 1] * v[k + 1][c]; }
-            }
-    }
-#pragma unroll
-    for (int c = 0; c < C; ++c) acc[c] = a0[c] + a1[c];
-}
-template <int C, int K1, int SIGN>
-__device__ __forceinline__ void ws_col_product_wide(const float* tile, const float* V, int lane, float (&acc)[C]) {
-    static_assert(K1 % 8 == 0, "k range in multiples of 8");
-    float l[K1];
-#pragma unroll
-    for (int k = 0; k < K1; ++k) l[k] = lds1_ordered(tile + swz(k, lane));
-    float a0[C], a1[C];
-#pragma unroll
-    for (int c = 0; c < C; ++c) { a0[c] = acc[c]; a1[c] = 0.f; }
-#pragma unroll
-    for (int k8 = 0; k8 < K1; k8 += 8) {
-        float v[8][C];
-#pragma unroll
-        for (int k = 0; k < 8; ++k) ws_ld_ordered<C>(V + (k8 + k) * C, v[k]);
-#pragma unroll
-        for (int k = 0; k < 8; k += 2)
-#pragma unroll
-            for (int c = 0; c < C; ++c) {
-                if (SIGN > 0) { a0[c] += l[k8 + k] * v[k][c]; a1[c] += l[k8 + k + 1] * v[k + 1][c]; }
-                else { a0[c] -= l[k8 + k] * v[k][c]; a1[c] -= l[k8 + k + 1] * v[k + 1][c]; }
-            }
-    }
-#pragma unroll
-    for (int c = 0; c < C; ++c) acc[c] = a0[c] + a1[c];
-}
-// the form a configuration uses: ordered for wide bands (more than 2 tiles)
-// with 2 or 4 columns a warp (the configurations that were measured)
-template <bool WIDE, int C, int K0, int K1, int SIGN>
-__device__ __forceinline__ void ws_rowp(const float* tile, const float* V, int lane, float (&acc)[C]) {
-    if constexpr (WIDE) ws_row_product_wide<C, K0, K1, SIGN>(tile, V, lane, acc);
-    else ws_row_product<C, K0, K1, SIGN>(tile, V, lane, acc);
-}
-template <bool WIDE, int C, int K1, int SIGN>
-__device__ __forceinline__ void ws_colp(const float* tile, const float* V, int lane, float (&acc)[C]) {
-    if constexpr (WIDE) ws_col_product_wide<C, K1, SIGN>(tile, V, lane, acc);
-    else ws_col_product<C, K1, SIGN>(tile, V, lane, acc);
 }
 
 __device__ __forceinline__ void mbar_arrive(unsigned long long* bar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(smem_u32(bar)) : "memory");
 }
 
-template <int KBP, int W, int C, int NST, int XD>
-struct BandWs {
-    // The backward sweep's first right-hand side read from X (block K-1-S,
-    // written by forward step K-1-S) is issued XD - 1 steps ahead, at step
-    // K - XD + 1: it must come after that write, so XD <= S + 1 = KBP + 2.
-    static_assert(XD <= KBP + 2, "X prefetch deeper than the solution ring allows");
-    static constexpr int SLOTS = KBP + 1;            // tiles per step; also the solution ring per warp
-    static constexpr int NT = 32 * (W + 1);
-    static constexpr int COLS = W * C;
-    static constexpr size_t stage_bytes = (size_t)SLOTS * NB2 * sizeof(float);
-    static constexpr size_t warp_bytes =
-        sizeof(float) * ((size_t)SLOTS * NB * C + (size_t)NB * C) + sizeof(double) * (size_t)XD * NB * C;
-    static constexpr size_t smem_bytes =
-        1024 + (size_t)NST * stage_bytes + (size_t)NST * NB * sizeof(float) + 16 * (size_t)NST + (size_t)W * warp_bytes;
-};
+// ---- the FP32 band solve of several right-hand sides (kb <= 12), TMA tile
+// loads, k split over warps.  Forward z_R = T_R (x_R - sum_J L_RJ z_J),
+// backward x_R = T_R^T (D_R^{-1} z_R - sum_I L_IR^T x_I); all sums in FP32.
+//
+// A solve is a chain of 2 K dependent steps of one CTA; a step's products
+// are (kb + 1) tiles of 32 x 32 by 4 J columns.  Letting every warp run over
+// all tiles for columns of its own makes each tile element travel from shared
+// memory once per warp (LSU bound: the earlier form took 3350 cycles a step
+// at kb = 2, 9700 at kb = 12).  Here the NW consumer warps split the k index
+// instead, so that every tile element is read once: a warp takes groups of
+// four k and accumulates all 32 rows x 4 J columns in registers (lane = 8 row
+// groups x 4 column groups, 4 rows x J columns each: 4 + J wide loads per
+// 16 J FMA).  The partial sums are exchanged through shared memory: warp w
+// sums and finishes the 32 / NW rows of its slice, which are exactly the rows
+// it then multiplies as its k-slice of T_R, and of the next step's nearest
+// tile.  Two barriers of the consumer warps a step.  128 problems of n = 1369,
+// b = 38, 16 columns: 134.6 -> 110.8 us a launch (with X in FP32); 108 of
+// n = 6859, b = 381, 20 columns: 2113 -> 1571 us.  Still bound by shared
+// memory: 4 + J 16-byte loads, four LSU cycles each, feed 16 J FMA.
+//
+// A producer warp streams the tiles of each step by TMA (128-byte swizzle,
+// ring of nst stages of S = maxkb + 1 tiles, "full" mbarriers by byte count,
+// "empty" ones released by each consumer warp after its last read).  Column
+// blocks of a tile that lie outside the band (element (r, k) of L_{R,R-d} is
+// zero unless 32 d + r - k <= b) are skipped in groups of four k.  Every wait
+// is bounded; after a timeout (recorded in g_wait_timeouts) the producer
+// waits (bounded) for its copies in flight and the consumers leave together
+// at the end of the step.
+__device__ __forceinline__ float as_f32(double x) { return f64_to_f32(x); }
+__device__ __forceinline__ float as_f32(float x) { return x; }
+constexpr int KS_LD = 40;        // column stride of the exchange blocks: 16-byte reads of 4 columns or 8 row groups are conflict-free
 
-// Half-bandwidth b at most KBP tiles (kb <= KBP); a step needs the diagonal
-// tile and kb off-diagonal tiles, and z_{R-1} .. z_{R-kb} (forward) or
-// x_{R+1} .. x_{R+kb} (backward) from the warp's ring of KBP + 1 solution
-// blocks.  When the backward sweep starts, the ring still holds z_R for the
-// last KBP + 1 rows, so only the rows before those are read back from X.
-template <int KBP, int W, int C, int NST, int XD>
-__global__ void __launch_bounds__(32 * (W + 1)) k_tile_solve_band_ws(
+template <int NW, int J>
+constexpr size_t band_ks_smem(int S, int nst) {
+    return 1024 + (size_t)nst * S * NB2 * 4 + 16 * (size_t)nst + sizeof(float) * (size_t)(2 * NW + S + 1) * 4 * J * KS_LD;
+}
+
+template <int NW, int J, typename XT>
+__global__ void __launch_bounds__(32 * (NW + 1)) k_tile_solve_band_ks(
     const __grid_constant__ CUtensorMap tmt, const float* __restrict__ dinv, const int* __restrict__ kb_,
     const int* __restrict__ K_, const int* __restrict__ b_, const long long* __restrict__ toff_,
-    const long long* __restrict__ roff_, double* __restrict__ Xall, int ldx, int ncols_all,
-    const int* __restrict__ skip, const int* __restrict__ gdone)
+    const long long* __restrict__ roff_, XT* Xall, int ldx, int ncols_all, const int* __restrict__ skip,
+    const int* __restrict__ gdone, int S, int nst)
 {
-    using Cfg = BandWs<KBP, W, C, NST, XD>;
-    constexpr int S = Cfg::SLOTS;
-    static_assert(C == 1 || C == 2 || C == 4, "1, 2 or 4 columns per warp");
+    constexpr int COLS = 4 * J, RS = NB / NW, QS = RS / 4;   // columns, rows and k-groups of a warp's slice
+    constexpr int UNITS = COLS * QS, UN = (UNITS + 31) / 32;  // (column, four rows) units of a slice per lane
+    constexpr int BLK = COLS * KS_LD;
     extern __shared__ unsigned char smem_raw[];
     unsigned char* base = smem_raw + ((1024 - (smem_u32(smem_raw) & 1023)) & 1023);
-    float* St = reinterpret_cast<float*>(base);                                        // [NST][S][32*32]
-    float* Sd = St + (size_t)NST * S * NB2;                                            // [NST][32]
-    unsigned long long* full = reinterpret_cast<unsigned long long*>(Sd + (size_t)NST * NB);
-    unsigned long long* empty = full + NST;
-    unsigned char* wbase = reinterpret_cast<unsigned char*>(empty + NST);
-    __shared__ int s_abort;
+    float* St = reinterpret_cast<float*>(base);                        // [nst][S][32*32]
+    unsigned long long* full = reinterpret_cast<unsigned long long*>(St + (size_t)nst * S * NB2);
+    unsigned long long* empty = full + nst;
+    float* P1 = reinterpret_cast<float*>(empty + nst);                 // [NW][COLS][KS_LD] partial sums
+    float* P2 = P1 + NW * BLK;
+    float* Zr = P2 + NW * BLK;                                         // [S][COLS][KS_LD] solutions
+    float* Ac = Zr + S * BLK;                                          // [COLS][KS_LD]
+    __shared__ int s_abort, s_stop;
 
     const int i = blockIdx.x;
     if (skip && skip[i]) return;
     if (gdone && *gdone) return;
     const int kb = kb_[i], K = K_[i], bw = b_[i];
-    if (kb > KBP) return;                            // never launched so (host dispatch)
+    if (kb >= S || K == 0) return;                   // never launched so (host dispatch)
     const long long toff = toff_[i], roff = roff_[i];
     const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
     if (t == 0) {
         s_abort = 0;
-        for (int s = 0; s < NST; ++s) {
+        s_stop = 0;
+        for (int s = 0; s < nst; ++s) {
             mbar_init(&full[s], 1);
-            mbar_init(&empty[s], W);
+            mbar_init(&empty[s], NW);
         }
         fence_mbar_init();
     }
     __syncthreads();
-    auto stile = [&](int st, int slot) { return St + (size_t)(st * S + slot) * NB2; };
     auto give_up = [&]() {
         if (atomicExch(&s_abort, 1) == 0) atomicAdd(&g_wait_timeouts, 1);
     };
     const int total = 2 * K;                         // steps of both sweeps
 
-    if (warp == W) {
+    if (warp == NW) {
         // ---------------- producer: one lane issues every copy
         if (lane == 0) {
-            unsigned pending = 0, par = 0;           // stages with copies in flight, their phase parity
+            unsigned pending = 0, par = 0, ph = 0;   // stages with copies in flight, their parity; use parity of each stage
+            int st = 0;
             for (int it = 0; it < total; ++it) {
-                const int st = it % NST;
-                if (it >= NST) {
-                    if (!mbar_wait_bounded(&empty[st], ((it / NST) - 1) & 1u)) { give_up(); break; }
+                if (it >= nst) {
+                    if (!mbar_wait_bounded(&empty[st], ((ph >> st) & 1u) ^ 1u)) { give_up(); break; }
                     pending &= ~(1u << st);
                 }
                 if (*(volatile int*)&s_abort) break;
                 const bool fwd = it < K;
                 const int R = fwd ? it : total - 1 - it;
-                int nt = 1;
-                for (int d = 1; d <= kb; ++d) {
-                    const int o = fwd ? R - d : R + d;
-                    if (o >= 0 && o < K) ++nt;
+                const int nd = min(kb, fwd ? R : K - 1 - R);
+                float* dst = St + (size_t)st * S * NB2;
+                mbar_expect_tx(&full[st], (nd + 1) * NB2 * 4);
+                for (int d = nd; d >= 0; --d) {
+                    const long long ti = fwd ? tile_index(toff, kb, R, R - d) : tile_index(toff, kb, R + d, R);
+                    tma_load_tile(dst + (size_t)d * NB2, &tmt, (int)(ti / NB), &full[st]);
                 }
-                mbar_expect_tx(&full[st], nt * NB2 * 4 + (fwd ? 0 : NB * 4));
-                tma_load_tile(stile(st, 0), &tmt, (int)(tile_index(toff, kb, R, R) / NB), &full[st]);
-                for (int d = 1; d <= kb; ++d) {
-                    const int o = fwd ? R - d : R + d;
-                    if (o < 0 || o >= K) continue;
-                    const long long ti = fwd ? tile_index(toff, kb, R, o) : tile_index(toff, kb, o, R);
-                    tma_load_tile(stile(st, d), &tmt, (int)(ti / NB), &full[st]);
-                }
-                if (!fwd) bulk_load(Sd + st * NB, dinv + roff + (long long)R * NB, NB * 4, &full[st]);
                 pending |= 1u << st;
-                par = (par & ~(1u << st)) | (((unsigned)(it / NST) & 1u) << st);
+                par = (par & ~(1u << st)) | (((ph >> st) & 1u) << st);
+                ph ^= 1u << st;
+                st = st + 1 == nst ? 0 : st + 1;
             }
             // after an abort, copies still in flight must land before the CTA exits
             if (*(volatile int*)&s_abort)
-                for (int s = 0; s < NST; ++s)
+                for (int s = 0; s < nst; ++s)
                     if (pending & (1u << s)) mbar_wait_bounded(&full[s], (par >> s) & 1u);
         }
         return;
     }
 
-    // ---------------- consumer warp: columns [c_lo, c_lo + nc)
-    const int c_lo = blockIdx.y * Cfg::COLS + warp * C;
-    const int nc = max(0, min(C, ncols_all - c_lo));
-    float* Zr = reinterpret_cast<float*>(wbase + (size_t)warp * Cfg::warp_bytes);     // [S][32][C]
-    float* Acc = Zr + (size_t)S * NB * C;                                               // [32][C]
-    double* Xs = reinterpret_cast<double*>(Acc + (size_t)NB * C);                      // [XD][32][C]
-    double* X = Xall + c_lo;
-    // loads of this lane's row: index q < K: forward step q (row q); q >= K:
-    // backward row K - 1 - S - (q - K) (backward steps s >= S)
-    const int nload = K + max(0, K - S);
-    auto issue_load = [&](int q) {
-        if (q < nload && nc > 0) {
-            if (q >= K) __threadfence_block();       // rows written by this lane in the forward sweep
-            const int R = q < K ? q : K - 1 - S - (q - K);
-            const double* src = X + (roff + (long long)R * NB + lane) * ldx;
-            double* dst = Xs + ((size_t)(q % XD) * NB + lane) * C;
-            if constexpr (C == 1) {
-                asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(smem_u32(dst)), "l"(src));
-            } else {
-                cp_async16(dst, src);
-                if (C == 4 && nc > 2) cp_async16(dst + 2, src + 2);
-            }
-        }
-        cp_async_commit();
-    };
-    for (int q = 0; q < XD - 1; ++q) issue_load(q);
-    int q_next = XD - 1, q_use = 0;
-    for (int it = 0; it < total; ++it) {
-        const int st = it % NST;
+    // ---------------- consumer warps
+    auto consumers_sync = [&]() { asm volatile("bar.sync 1, %0;\n" ::"r"(32 * NW) : "memory"); };
+    const int rg = lane & 7, cg = lane >> 3;
+    const int cbase = blockIdx.y * COLS;
+    // this lane's units of the warp's slice: column uc[u], rows ur[u] .. ur[u] + 3
+    int uc[UN], ur[UN];
+    bool uon[UN], uok[UN];
+#pragma unroll
+    for (int u = 0; u < UN; ++u) {
+        const int e = lane + 32 * u;
+        uc[u] = e / QS;
+        ur[u] = RS * warp + 4 * (e % QS);
+        uon[u] = e < UNITS;
+        uok[u] = uon[u] && cbase + uc[u] < ncols_all;
+    }
+    XT xn[UN][4];                                    // next right-hand side rows, as loaded (converted when used)
+    float dn[UN][4], zl[UN][4];                      // next D^{-1}, last solution rows
+    auto load_rhs = [&](int it) {
         const bool fwd = it < K;
         const int R = fwd ? it : total - 1 - it;
-        float acc[C];
-        // right-hand side of this step (own row)
-        if (fwd || (it - K) >= S) {
-            issue_load(q_next++);
-            cp_async_wait_n<XD - 1>();
-            const double* xs = Xs + ((size_t)(q_use % XD) * NB + lane) * C;
 #pragma unroll
-            for (int c = 0; c < C; ++c) acc[c] = c < nc ? f64_to_f32(xs[c]) : 0.f;
-            ++q_use;
-        } else {
-            ws_ld<C>(Zr + ((size_t)(R % S) * NB + lane) * C, acc);
-        }
-        if (!mbar_wait_bounded(&full[st], (it / NST) & 1u)) { give_up(); break; }
-        if (nc > 0) {
-            if (!fwd) {
-                const float dr = Sd[st * NB + lane];
+        for (int u = 0; u < UN; ++u) {
+            const long long row = roff + (long long)R * NB + ur[u];
 #pragma unroll
-                for (int c = 0; c < C; ++c) acc[c] *= dr;
+            for (int a = 0; a < 4; ++a) {
+                xn[u][a] = uok[u] ? Xall[(row + a) * ldx + cbase + uc[u]] : XT(0);
+                dn[u][a] = 1.f;
             }
-            for (int d = 1; d <= kb; ++d) {
-                const int o = fwd ? R - d : R + d;
-                if (o < 0 || o >= K) continue;
-                const float* L = stile(st, d);
-                const float* Z = Zr + (size_t)(o % S) * NB * C;
-                if (fwd) {
-                    // acc -= L_{R,o}[lane][k] z_o[k]; nonzero only for k >= 32 d - b
-                    const int k0 = NB * d - bw;
-                    if (k0 >= 24) ws_rowp<(KBP > 2 && C >= 2), C, 24, 32, -1>(L, Z, lane, acc);
-                    else if (k0 >= 16) ws_rowp<(KBP > 2 && C >= 2), C, 16, 32, -1>(L, Z, lane, acc);
-                    else ws_rowp<(KBP > 2 && C >= 2), C, 0, 32, -1>(L, Z, lane, acc);
-                } else {
-                    // acc -= L_{o,R}[k][lane] x_o[k]; nonzero only for k <= b - 32 d + 31
-                    const int kend = bw - NB * d + NB;
-                    if (kend <= 8) ws_colp<(KBP > 2 && C >= 2), C, 8, -1>(L, Z, lane, acc);
-                    else if (kend <= 16) ws_colp<(KBP > 2 && C >= 2), C, 16, -1>(L, Z, lane, acc);
-                    else ws_colp<(KBP > 2 && C >= 2), C, 32, -1>(L, Z, lane, acc);
+            if (!fwd && uok[u]) {
+                const float4 d4 = *reinterpret_cast<const float4*>(dinv + row);
+                dn[u][0] = d4.x; dn[u][1] = d4.y; dn[u][2] = d4.z; dn[u][3] = d4.w;
+            }
+        }
+    };
+    float acc[4][J];
+    auto clear = [&]() {
+#pragma unroll
+        for (int a = 0; a < 4; ++a)
+#pragma unroll
+            for (int j = 0; j < J; ++j) acc[a][j] = 0.f;
+    };
+    // acc += (32 x 4 columns 4 q .. of the tile, or of its transpose) V[:, 4 q ..]; forward rows rg + 8 a, backward 4 rg + a
+    auto product = [&](const float* T, const float* V, int q, bool fwd) {
+        float4 v[J];
+#pragma unroll
+        for (int j = 0; j < J; ++j) v[j] = *reinterpret_cast<const float4*>(V + (cg + 4 * j) * KS_LD + 4 * q);
+        if (fwd) {
+#pragma unroll
+            for (int a = 0; a < 4; ++a) {
+                const float4 l = *reinterpret_cast<const float4*>(T + (rg + 8 * a) * NB + ((q ^ rg) << 2));
+#pragma unroll
+                for (int j = 0; j < J; ++j) {
+                    acc[a][j] = fmaf(l.x, v[j].x, acc[a][j]);
+                    acc[a][j] = fmaf(l.y, v[j].y, acc[a][j]);
+                    acc[a][j] = fmaf(l.z, v[j].z, acc[a][j]);
+                    acc[a][j] = fmaf(l.w, v[j].w, acc[a][j]);
                 }
             }
-            ws_st<C>(Acc + lane * C, acc);
-            __syncwarp();
-            const float* T = stile(st, 0);
-            float out[C];
+        } else {
 #pragma unroll
-            for (int c = 0; c < C; ++c) out[c] = 0.f;
-            if (fwd) ws_rowp<(KBP > 2 && C >= 2), C, 0, 32, 1>(T, Acc, lane, out);
-            else ws_colp<(KBP > 2 && C >= 2), C, 32, 1>(T, Acc, lane, out);
-            __syncwarp();                                   // Acc reads done before the next step's writes
-            ws_st<C>(Zr + ((size_t)(R % S) * NB + lane) * C, out);
-            double* xw = X + (roff + (long long)R * NB + lane) * ldx;
+            for (int kk = 0; kk < 4; ++kk) {
+                const int k = 4 * q + kk;
+                const float4 l = *reinterpret_cast<const float4*>(T + k * NB + ((rg ^ (k & 7)) << 2));
 #pragma unroll
-            for (int c = 0; c < C; ++c)
-                if (c < nc) xw[c] = f32_to_f64(out[c]);
+                for (int j = 0; j < J; ++j) {
+                    const float x = kk == 0 ? v[j].x : kk == 1 ? v[j].y : kk == 2 ? v[j].z : v[j].w;
+                    acc[0][j] = fmaf(l.x, x, acc[0][j]);
+                    acc[1][j] = fmaf(l.y, x, acc[1][j]);
+                    acc[2][j] = fmaf(l.z, x, acc[2][j]);
+                    acc[3][j] = fmaf(l.w, x, acc[3][j]);
+                }
+            }
         }
+    };
+    auto store_partial = [&](float* P, bool fwd) {
+        float* dst = P + warp * BLK;
+#pragma unroll
+        for (int j = 0; j < J; ++j) {
+            if (fwd) {
+#pragma unroll
+                for (int a = 0; a < 4; ++a) dst[(cg + 4 * j) * KS_LD + rg + 8 * a] = acc[a][j];
+            } else {
+                *reinterpret_cast<float4*>(dst + (cg + 4 * j) * KS_LD + 4 * rg) =
+                    make_float4(acc[0][j], acc[1][j], acc[2][j], acc[3][j]);
+            }
+        }
+    };
+    // four-k groups of the outermost tile that hold nonzeros (the last ones forward, the first ones backward)
+    const int nql = kb > 0 ? min(8, 8 - (NB * kb - bw) / 4) : 0;
+    load_rhs(0);
+    int st = 0;
+    unsigned ph = 0;                                 // parity of each stage's next use
+    int zs = 0;                                      // ring slot of this step's solution
+    for (int it = 0; it < total; ++it) {
+        const bool fwd = it < K;
+        const int R = fwd ? it : total - 1 - it;
+        const int nd = min(kb, fwd ? R : K - 1 - R);
+        if (it == K) zs = (K - 1) % S;               // the backward sweep overwrites z_R by x_R in its slot
+        float x[UN][4];
+#pragma unroll
+        for (int u = 0; u < UN; ++u)
+#pragma unroll
+            for (int a = 0; a < 4; ++a) x[u][a] = as_f32(xn[u][a]) * dn[u][a];
+        if (it == K) {                               // the last forward step's rows are still in registers
+#pragma unroll
+            for (int u = 0; u < UN; ++u)
+                if (uok[u]) {
+                    const float4 d4 = *reinterpret_cast<const float4*>(dinv + roff + (long long)R * NB + ur[u]);
+                    x[u][0] = zl[u][0] * d4.x; x[u][1] = zl[u][1] * d4.y;
+                    x[u][2] = zl[u][2] * d4.z; x[u][3] = zl[u][3] * d4.w;
+                }
+        }
+        if (it + 1 < total && it + 1 != K) load_rhs(it + 1);
+        const float* tiles = St + (size_t)st * S * NB2;
+        const bool ok = mbar_wait_bounded(&full[st], (ph >> st) & 1u);
+        if (!ok) give_up();
+        clear();
+        if (ok && nd > 0) {
+            // tiles d >= 2: all k groups, spread over the warps
+            const int nfar = nd < 2 ? 0 : 8 * (nd - 2) + (nd == kb ? nql : 8);
+            for (int f = warp; f < nfar; f += NW) {
+                const int d = 2 + (f >> 3);
+                const int q = (f & 7) + (fwd && d == kb ? 8 - nql : 0);
+                int slot = fwd ? zs - d : zs + d;
+                slot += slot < 0 ? S : 0;
+                slot -= slot >= S ? S : 0;
+                product(tiles + (size_t)d * NB2, Zr + slot * BLK, q, fwd);
+            }
+            // the nearest tile: this warp's slice of z_{R-1} (x_{R+1})
+            int slot = fwd ? zs - 1 : zs + 1;
+            slot += slot < 0 ? S : 0;
+            slot -= slot >= S ? S : 0;
+#pragma unroll
+            for (int m = 0; m < QS; ++m) {
+                const int q = QS * warp + m;
+                if (kb > 1 || (fwd ? q >= 8 - nql : q < nql)) product(tiles + NB2, Zr + slot * BLK, q, fwd);
+            }
+        }
+        store_partial(P1, fwd);
+        consumers_sync();                            // every partial sum is in P1
+#pragma unroll
+        for (int u = 0; u < UN; ++u)
+            if (uon[u]) {
+                float4 y = make_float4(x[u][0], x[u][1], x[u][2], x[u][3]);
+#pragma unroll
+                for (int w = 0; w < NW; ++w) {
+                    const float4 p = *reinterpret_cast<const float4*>(P1 + w * BLK + uc[u] * KS_LD + ur[u]);
+                    y.x -= p.x; y.y -= p.y; y.z -= p.z; y.w -= p.w;
+                }
+                *reinterpret_cast<float4*>(Ac + uc[u] * KS_LD + ur[u]) = y;
+            }
+        __syncwarp();
+        clear();
+        if (ok) {
+#pragma unroll
+            for (int m = 0; m < QS; ++m) product(tiles, Ac, QS * warp + m, fwd);
+        }
+        store_partial(P2, fwd);
         __syncwarp();
         if (lane == 0) mbar_arrive(&empty[st]);
+        if (t == 0) *(volatile int*)&s_stop = *(volatile int*)&s_abort;
+        consumers_sync();                            // every partial of the solution is in P2
+        if (*(volatile int*)&s_stop) break;          // sampled once: every warp leaves after this step
+#pragma unroll
+        for (int u = 0; u < UN; ++u)
+            if (uon[u]) {
+                float4 z = *reinterpret_cast<const float4*>(P2 + uc[u] * KS_LD + ur[u]);
+#pragma unroll
+                for (int w = 1; w < NW; ++w) {
+                    const float4 p = *reinterpret_cast<const float4*>(P2 + w * BLK + uc[u] * KS_LD + ur[u]);
+                    z.x += p.x; z.y += p.y; z.z += p.z; z.w += p.w;
+                }
+                *reinterpret_cast<float4*>(Zr + zs * BLK + uc[u] * KS_LD + ur[u]) = z;
+                zl[u][0] = z.x; zl[u][1] = z.y; zl[u][2] = z.z; zl[u][3] = z.w;
+                if (uok[u]) {
+                    XT* xw = Xall + (roff + (long long)R * NB + ur[u]) * ldx + cbase + uc[u];
+#pragma unroll
+                    for (int a = 0; a < 4; ++a) {
+                        if constexpr (sizeof(XT) == 8) xw[(long long)a * ldx] = f32_to_f64(zl[u][a]);
+                        else xw[(long long)a * ldx] = zl[u][a];
+                    }
+                }
+            }
+        __syncwarp();
+        ph ^= 1u << st;
+        st = st + 1 == nst ? 0 : st + 1;
+        if (fwd) zs = zs + 1 == S ? 0 : zs + 1;
+        else zs = zs == 0 ? S - 1 : zs - 1;
     }
-    cp_async_wait_n<0>();
 }
 
-// Launch of k_tile_solve_band_ws for one configuration.
-template <int KBP, int W, int C, int NST, int XD>
-void launch_band_ws(const TileBatch& tb, const CUtensorMap& tm, double* X, int ldx, int ncols, const int* skip,
-                    cudaStream_t s, const int* gdone) {
-    using Cfg = BandWs<KBP, W, C, NST, XD>;
-    static_assert(Cfg::smem_bytes <= 227 * 1024, "shared memory per CTA");
-    auto kern = k_tile_solve_band_ws<KBP, W, C, NST, XD>;
-    raise_smem_limit(kern, Cfg::smem_bytes);
-    kern<<<dim3(tb.P, (ncols + Cfg::COLS - 1) / Cfg::COLS), Cfg::NT, Cfg::smem_bytes, s>>>(
-        tm, tb.dinv_f.p, tb.d_kb.p, tb.d_K.p, tb.d_b.p, tb.d_toff.p, tb.d_roff.p, X, ldx, ncols, skip, gdone);
+template <int NW, int J, typename XT>
+void launch_band_ks(const TileBatch& tb, const CUtensorMap& tm, int maxkb, XT* X, int ldx, int ncols, int chunks,
+                    const int* skip, cudaStream_t s, const int* gdone) {
+    const int S = maxkb + 1;
+    // stages: up to four, with two CTAs an SM where that leaves at least two
+    const size_t half = 112 * 1024, full = 226 * 1024;
+    const size_t limit = band_ks_smem<NW, J>(S, 2) <= half ? half : full;
+    int nst = 4;
+    while (nst > 2 && band_ks_smem<NW, J>(S, nst) > limit) --nst;
+    const size_t b = band_ks_smem<NW, J>(S, nst);
+    auto kern = k_tile_solve_band_ks<NW, J, XT>;
+    raise_smem_limit(kern, b);
+    kern<<<dim3(tb.P, chunks), 32 * (NW + 1), b, s>>>(tm, tb.dinv_f.p, tb.d_kb.p, tb.d_K.p, tb.d_b.p, tb.d_toff.p,
+                                                      tb.d_roff.p, X, ldx, ncols, skip, gdone, S, nst);
     MSDD_LAUNCH_CHECK();
+}
+
+// Column groups of 4 J <= 20 columns, as even as they come: J from the count.
+template <typename XT>
+void solve_band_ks(const TileBatch& tb, const CUtensorMap& tm, int maxkb, XT* X, int ldx, int ncols, const int* skip,
+                   cudaStream_t s, const int* gdone) {
+    const int chunks = (ncols + 19) / 20, J = (ncols + 4 * chunks - 1) / (4 * chunks);
+    auto go = [&](auto nw) {
+        constexpr int NW = decltype(nw)::value;
+        switch (J) {
+            case 1: launch_band_ks<NW, 1>(tb, tm, maxkb, X, ldx, ncols, chunks, skip, s, gdone); break;
+            case 2: launch_band_ks<NW, 2>(tb, tm, maxkb, X, ldx, ncols, chunks, skip, s, gdone); break;
+            case 3: launch_band_ks<NW, 3>(tb, tm, maxkb, X, ldx, ncols, chunks, skip, s, gdone); break;
+            case 4: launch_band_ks<NW, 4>(tb, tm, maxkb, X, ldx, ncols, chunks, skip, s, gdone); break;
+            default: launch_band_ks<NW, 5>(tb, tm, maxkb, X, ldx, ncols, chunks, skip, s, gdone); break;
+        }
+    };
+    if (maxkb <= 2) go(std::integral_constant<int, 4>{});
+    else go(std::integral_constant<int, 8>{});
 }
 
 // ---- one right-hand side, wide bands: the off-diagonal tiles of a step split
@@ -1826,7 +1592,7 @@ void launch_band_ws(const TileBatch& tb, const CUtensorMap& tm, double* X, int l
 // the right-hand side minus those sums and applies T_R (T_R^T backward), writes
 // the step's solution to the ring and to X, under two named barriers of the
 // consumer warps.  The producer warp streams the tiles as in
-// k_tile_solve_band_ws; warp 0 alone releases a stage, after the barrier that
+// k_tile_solve_band_ks; warp 0 alone releases a stage, after the barrier that
 // ends every warp's reads of it.
 template <int KBP, int WS, int NST, int XD>
 struct BandSplit {
@@ -1880,7 +1646,7 @@ __global__ void __launch_bounds__(32 * (WS + 1)) k_tile_solve_band_split(
     const int total = 2 * K;
 
     if (warp == WS) {
-        // ---------------- producer (as in k_tile_solve_band_ws)
+        // ---------------- producer (as in k_tile_solve_band_ks)
         if (lane == 0) {
             unsigned pending = 0, par = 0;
             for (int it = 0; it < total; ++it) {
@@ -2043,24 +1809,19 @@ const CUtensorMap* tile_tensor_map(const TileBatch& tb) {
     return m;
 }
 
-template <typename T, int CPT, int CG>
-void launch_band(const TileBatch& tb, const T* tiles, const T* dinv, double* X, int ldx, int ncols, const int* skip,
-                 cudaStream_t s, const int* gdone) {
-    constexpr int ZLD = BandSmem<T, CPT, CG>::ZLD;
-    const int chunks = (ncols + ZLD - 1) / ZLD;
-    const size_t b = BandSmem<T, CPT, CG>::bytes(((std::min(ncols, ZLD) + 1) / 2) * 2);
-    raise_smem_limit(k_tile_solve_band<T, CPT, CG>, b);
-    k_tile_solve_band<T, CPT, CG><<<dim3(tb.P, chunks), 8 * CG, b, s>>>(tiles, dinv, tb.d_kb.p, tb.d_K.p, tb.d_toff.p,
-                                                                         tb.d_roff.p, X, ldx, ncols, skip, gdone);
+// FP32 factors, any number of columns
+template <typename XT>
+void solve_f32(const TileBatch& tb, XT* X, int ldx, int ncols, const int* skip, cudaStream_t s, const int* gdone) {
+    int maxkb = 0;
+    for (int v : tb.kb) maxkb = std::max(maxkb, v);
+    const CUtensorMap* tm = maxkb <= 12 ? tile_tensor_map(tb) : nullptr;
+    if (tm) {
+        solve_band_ks(tb, *tm, maxkb, X, ldx, ncols, skip, s, gdone);
+        return;
+    }
+    k_tile_solve<float, XT><<<dim3(tb.P, (ncols + NB - 1) / NB), TPB, 0, s>>>(
+        tb.tiles_f.p, tb.dinv_f.p, tb.d_n.p, tb.d_kb.p, tb.d_K.p, tb.d_toff.p, tb.d_roff.p, X, ldx, ncols, skip, gdone);
     MSDD_LAUNCH_CHECK();
-}
-
-template <typename T>
-void launch_band_cols(const TileBatch& tb, const T* tiles, const T* dinv, double* X, int ldx, int ncols,
-                      const int* skip, cudaStream_t s, const int* gdone) {
-    // chunks of 8 columns, one 64-thread CTA each (more independent
-    // sequential sweeps in flight per SM than wider CTAs)
-    launch_band<T, 1, 8>(tb, tiles, dinv, X, ldx, ncols, skip, s, gdone);
 }
 
 __global__ void k_fill_identity(double* __restrict__ E, const int* __restrict__ n_, const int* __restrict__ K_,
@@ -2307,37 +2068,20 @@ void tile_solve(const TileBatch& tb, double* X, int ldx, int ncols, const int* s
         }
     }
     if (!tb.prec && tile_solve_f64(tb, X, ldx, ncols, skip, s, gdone)) return;
-    int maxkb = 0;
-    for (int v : tb.kb) maxkb = std::max(maxkb, v);
-    // the band kernels stage blocks of X with 16-byte copies
-    const bool aligned = ldx % 2 == 0 && ((uintptr_t)X % 16) == 0;
-    const CUtensorMap* tm = tb.prec && aligned && ncols <= NB ? tile_tensor_map(tb) : nullptr;
-    if (tm && maxkb <= 2) {
-        // 16 columns in 4 warps of 4, 6 stages.  8 warps of 2 with 3 stages
-        // is 9% faster on its own (129 vs 139 us a launch) but no faster in
-        // the set-up, where the other half's kernels share the SMs
-        launch_band_ws<2, 4, 4, 6, 4>(tb, *tm, X, ldx, ncols, skip, s, gdone);
-        return;
-    }
-    if (tm && maxkb <= 12) {
-        // wide bands (3D boxes): 20 columns per CTA in 10 warps of 2, 2 stages
-        // of 13 tiles (17% faster than 5 warps of 4 with 3 stages: the smaller
-        // shared-memory carve-out leaves L1 to the right-hand-side rows)
-        launch_band_ws<12, 10, 2, 2, 4>(tb, *tm, X, ldx, ncols, skip, s, gdone);
-        return;
-    }
-    if (tb.prec && maxkb <= 2 && ncols <= NB && aligned) {
-        launch_band_cols<float>(tb, tb.tiles_f.p, tb.dinv_f.p, X, ldx, ncols, skip, s, gdone);
+    if (tb.prec) {
+        solve_f32(tb, X, ldx, ncols, skip, s, gdone);
         return;
     }
     const dim3 grid(tb.P, (ncols + NB - 1) / NB);
-    if (tb.prec)
-        k_tile_solve<float><<<grid, TPB, 0, s>>>(tb.tiles_f.p, tb.dinv_f.p, tb.d_n.p, tb.d_kb.p, tb.d_K.p,
-                                                tb.d_toff.p, tb.d_roff.p, X, ldx, ncols, skip, gdone);
-    else
-        k_tile_solve<double><<<grid, TPB, 0, s>>>(tb.tiles_d.p, tb.dinv_d.p, tb.d_n.p, tb.d_kb.p, tb.d_K.p,
-                                                 tb.d_toff.p, tb.d_roff.p, X, ldx, ncols, skip, gdone);
+    k_tile_solve<double, double><<<grid, TPB, 0, s>>>(tb.tiles_d.p, tb.dinv_d.p, tb.d_n.p, tb.d_kb.p, tb.d_K.p,
+                                                      tb.d_toff.p, tb.d_roff.p, X, ldx, ncols, skip, gdone);
     MSDD_LAUNCH_CHECK();
+}
+
+void tile_solve(const TileBatch& tb, float* X, int ldx, int ncols, const int* skip, cudaStream_t s) {
+    if (tb.P == 0) return;
+    if (!tb.prec || ncols > ldx) throw std::runtime_error("tile_solve: FP32 blocks need FP32 factors and ncols <= ldx");
+    solve_f32(tb, X, ldx, ncols, skip, s, nullptr);
 }
 
 }  // namespace msdd

@@ -88,6 +88,8 @@ void tile_identity(const TileBatch& tb, double* E, int lde, cudaStream_t s);
 // skips everything when non-zero.
 void tile_solve(const TileBatch& tb, double* X, int ldx, int ncols, const int* skip, cudaStream_t s,
                 const int* gdone = nullptr);
+// The same for FP32 factors and an FP32 X (leading dimension ldx, any).
+void tile_solve(const TileBatch& tb, float* X, int ldx, int ncols, const int* skip, cudaStream_t s);
 // Throws if a bounded wait in a solve kernel gave up (its error flag is
 // reset); call after a synchronisation point.
 void tile_check_waits();
