@@ -12,6 +12,15 @@ namespace {
 constexpr int TPB = 256;
 constexpr int LD = PMAX + 1;
 constexpr int ROWBLK = EIG_ROWBLK;
+// The unwanted part of the spectrum, [0, mu_{p+1}], is not known; the smallest
+// Ritz value mu_p of the block bounds it from above once the block has settled
+// and is below mu_p's limit before that (Ritz values grow), where a smaller
+// interval only damps less.  0.95 of it rather than all of it, so that the
+// last wanted pair still grows against the interval when the block holds no
+// guard columns (block_p = nev_max): 12 pairs of a 1400-point model spectrum
+// in a block of 12 took 95 plain steps, 31 at 0.95, over 100 at 1; in a block
+// of 16, 48, 19 and 17.
+constexpr double CHEB_CUT = 0.95;
 
 __global__ void k_init(double* __restrict__ X, const int* __restrict__ n_, const int* __restrict__ K_,
                        const long long* __restrict__ roff_, const int* __restrict__ p_, int ldx,
@@ -68,49 +77,79 @@ __global__ void k_form_rhs(WT* __restrict__ W, int ldw, const double* __restrict
     }
 }
 
+// The accelerated step of column c: with S = K^{-1} B and S X = X diag(mu) + W,
+// the Chebyshev recurrence in x = (S - e) / e on the damped interval [0, 2 e],
+//   Y = 2 x X - Q  (FORM_CHEB), the first step of it Y = x X  (FORM_CHEB1),
+// where Q is the block before X in the basis of X.  FORM_FIRST: Y = W (the
+// block W = S X itself).  2 e = cheb[i] (0: no interval known, plain step).
+__device__ __forceinline__ void cheb_coef(int mode, double cc, double mu, double& a, double& w, double& q) {
+    if (mode == FORM_FIRST) { a = 0.0; w = 1.0; q = 0.0; return; }
+    if (!(cc > 0.0)) { a = mu; w = 1.0; q = 0.0; return; }
+    const double e = 0.5 * cc;
+    w = (mode == FORM_CHEB ? 2.0 : 1.0) / e;
+    a = w * (mu - e);
+    q = mode == FORM_CHEB ? -1.0 : 0.0;
+}
+
 template <typename WT>
 __global__ void k_form_y(double* __restrict__ Y, const double* __restrict__ X, const WT* __restrict__ W, int ldw,
+                         const double* __restrict__ Q, const double* __restrict__ cheb,
                          const double* __restrict__ theta, const int* __restrict__ n_, const int* __restrict__ K_,
                          const long long* __restrict__ roff_, const int* __restrict__ p_, int ldx, double sigma,
-                         int first, const int* __restrict__ done) {
-    __shared__ double smu[PMAX];                       // 1 / (theta + sigma): one division per column
+                         int mode, const int* __restrict__ done) {
+    __shared__ double sa[PMAX], sw, sq;                // one division per column
     const int i = blockIdx.y;
     if (done[i]) return;
     const int n = n_[i], p = p_[i];
     const long long rows = (long long)K_[i] * NB;
-    if (threadIdx.x < p) smu[threadIdx.x] = first ? 0.0 : 1.0 / (theta[i * PMAX + threadIdx.x] + sigma);
+    if (threadIdx.x < p) {
+        double a, w, q;
+        cheb_coef(mode, cheb[i], mode == FORM_FIRST ? 0.0 : 1.0 / (theta[i * PMAX + threadIdx.x] + sigma), a, w, q);
+        sa[threadIdx.x] = a;
+        if (threadIdx.x == 0) { sw = w; sq = q; }
+    }
     __syncthreads();
-    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < rows * ldx;
+    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < rows * ldw;
          e += (long long)gridDim.x * blockDim.x) {
-        int r = (int)(e / ldx), c = (int)(e % ldx);
+        int r = (int)(e / ldw), c = (int)(e % ldw);
         long long idx = (roff_[i] + r) * ldx + c;
         double v = 0.0;
         if (r < n && c < p) {
-            const double w = to_f64(W[(roff_[i] + r) * ldw + c]);
-            v = first ? w : fma(X[idx], smu[c], w);
+            v = sw * to_f64(W[(roff_[i] + r) * ldw + c]);
+            if (mode != FORM_FIRST) v = fma(X[idx], sa[c], v);
+            if (sq != 0.0) v = fma(sq, Q[idx], v);
         }
         Y[idx] = v;
     }
 }
 
-// Y = X diag(mu) + W on a block of 32 rows, and per column the partial sums
+// Y (as k_form_y) on a block of 32 rows, and per column the partial sums
 // of W . R with R = BX - (AX + sigma BX) diag(mu) recomputed: W = K^+ R, so
 // sum W.R = R^T K^+ R, the squared K^+-norm of the transformed residual.
 __global__ void __launch_bounds__(TPB) k_form_y_knorm(double* __restrict__ Y, const double* __restrict__ X,
                                                       const double* __restrict__ W, const double* __restrict__ AX,
-                                                      const double* __restrict__ BX, const double* __restrict__ theta,
+                                                      const double* __restrict__ BX, const double* __restrict__ Q,
+                                                      const double* __restrict__ cheb, int mode,
+                                                      const double* __restrict__ theta,
                                                       const int* __restrict__ n_, const int* __restrict__ K_,
                                                       const long long* __restrict__ roff_, const int* __restrict__ p_,
                                                       int ldx, double sigma, double* __restrict__ partial,
                                                       int nblk_max, const int* __restrict__ done) {
-    __shared__ double red[ROWBLK][LD], smu[PMAX];
+    __shared__ double red[ROWBLK][LD], smu[PMAX], sa[PMAX], sw, sq;
     const int i = blockIdx.y, blk = blockIdx.x;
     if (done[i]) return;
     const int n = n_[i], p = p_[i];
     const long long rows = (long long)K_[i] * NB;
     const int r0 = blk * ROWBLK;
     if (r0 >= rows) return;
-    if (threadIdx.x < p) smu[threadIdx.x] = 1.0 / (theta[i * PMAX + threadIdx.x] + sigma);
+    if (threadIdx.x < p) {
+        const double mu = 1.0 / (theta[i * PMAX + threadIdx.x] + sigma);
+        double a, w, q;
+        cheb_coef(mode, cheb[i], mu, a, w, q);
+        smu[threadIdx.x] = mu;
+        sa[threadIdx.x] = a;
+        if (threadIdx.x == 0) { sw = w; sq = q; }
+    }
     __syncthreads();
     const long long roff = roff_[i];
     const int t = threadIdx.x;
@@ -126,7 +165,8 @@ __global__ void __launch_bounds__(TPB) k_form_y_knorm(double* __restrict__ Y, co
                 double w = W[idx];
                 double bx = BX[idx];
                 double R = bx - (AX[idx] + sigma * bx) * mu;
-                v = X[idx] * mu + w;
+                v = fma(X[idx], sa[c], sw * w);
+                if (sq != 0.0) v = fma(sq, Q[idx], v);
                 wr = w * R;
             }
             Y[idx] = v;
@@ -672,6 +712,7 @@ __device__ bool rr_fast(double (*S)[LD], double (*V)[LD], double (*L)[LD], doubl
 __global__ void __launch_bounds__(TPB) k_rayleigh_ritz(const double* __restrict__ Hp, const double* __restrict__ Mp,
                                                        int gsplit, double* __restrict__ H, double* __restrict__ M,
                                                        double* __restrict__ C, double* __restrict__ theta,
+                                                       double* __restrict__ cheb, double sigma,
                                                        const int* __restrict__ p_, int* __restrict__ rank,
                                                        const int* __restrict__ done) {
     __shared__ double S[PMAX][LD], V[PMAX][LD], L[PMAX][LD], T[PMAX][LD], U[PMAX][LD];
@@ -836,11 +877,20 @@ sorted_output:
         if (k < p && S[perm[k]][perm[k]] >= 1e299) v = 0.0;
         C[(long long)i * PMAX * PMAX + e] = v;
     }
-    if (t == 0) rank[i] = r;
+    if (t == 0) {
+        rank[i] = r;
+        // damped interval [0, CHEB_CUT mu_min]: mu_min the smallest finite Ritz value of S = K^{-1} B in the block
+        int k = p - 1;
+        while (k > 0 && !(S[perm[k]][perm[k]] < 1e299)) --k;
+        const double th = S[perm[k]][perm[k]] + sigma;
+        cheb[i] = th > 0.0 && th < 1e299 ? CHEB_CUT / th : 0.0;
+    }
 }
 
 // X = Y C, AX = AY C, BX = BY C on a block of 32 rows; residual partial sums.
 // Outputs (row, column < p) are spread over the threads, at most 4 each.
+// Q (null: not wanted) receives the old X times C: the block before the new X
+// in the new basis, for the Chebyshev recurrence.
 // FULL = false: X = Y C only (AX, BX, partial untouched).
 // DF (with FULL = false, the chosen form's X-only update): the products in
 // double-float (split_f64 while staging, df_fma), X stored as FP64.
@@ -848,12 +898,13 @@ template <bool FULL, bool DF = false>
 __global__ void __launch_bounds__(TPB) k_update(const double* __restrict__ Y, const double* __restrict__ AY,
                                                 const double* __restrict__ BY, double* __restrict__ X,
                                                 double* __restrict__ AX, double* __restrict__ BX,
-                                                const double* __restrict__ C, const double* __restrict__ theta,
-                                                const int* __restrict__ n_, const int* __restrict__ K_,
+                                                double* __restrict__ Q, const double* __restrict__ C,
+                                                const double* __restrict__ theta, const int* __restrict__ n_, const int* __restrict__ K_,
                                                 const long long* __restrict__ roff_, const int* __restrict__ p_,
                                                 int ldx, double* __restrict__ partial, int nblk_max,
                                                 const int* __restrict__ done) {
-    __shared__ double sC[PMAX][LD], sY[ROWBLK][LD], sA[ROWBLK][LD], sB[ROWBLK][LD];
+    __shared__ double sC[PMAX][LD], sY[ROWBLK][LD], sX[ROWBLK][LD];
+    __shared__ double sA[FULL ? ROWBLK : 1][LD], sB[FULL ? ROWBLK : 1][LD];
     const int i = blockIdx.y, blk = blockIdx.x;
     if (done[i]) return;
     const int n = n_[i], p = p_[i];
@@ -868,11 +919,14 @@ __global__ void __launch_bounds__(TPB) k_update(const double* __restrict__ Y, co
         float (*cL)[LD] = cH + PMAX;
         float (*yH)[LD] = reinterpret_cast<float (*)[LD]>(&sY[0][0]);
         float (*yL)[LD] = yH + ROWBLK;
+        float (*qH)[LD] = reinterpret_cast<float (*)[LD]>(&sX[0][0]);
+        float (*qL)[LD] = qH + ROWBLK;
         for (int e = t; e < p * p; e += TPB)
             split_f64(C[(long long)i * PMAX * PMAX + (e / p) * PMAX + e % p], cH[e / p][e % p], cL[e / p][e % p]);
         for (int e = t; e < ROWBLK * p; e += TPB) {
             const int rr = e / p, c = e % p, r = r0 + rr;
             split_f64(r < n ? Y[(roff + r) * ldx + c] : 0.0, yH[rr][c], yL[rr][c]);
+            if (Q) split_f64(r < n ? X[(roff + r) * ldx + c] : 0.0, qH[rr][c], qL[rr][c]);
         }
         __syncthreads();
 #pragma unroll
@@ -884,6 +938,11 @@ __global__ void __launch_bounds__(TPB) k_update(const double* __restrict__ Y, co
             for (int j = 0; j < p; ++j) df_fma(xh, xl, yH[rr][j], yL[rr][j], cH[j][c], cL[j][c]);
             const int r = r0 + rr;
             if (r < rows) X[(roff + r) * ldx + c] = df_to_f64(xh, xl);
+            if (Q && r < rows) {
+                float ph = 0.f, pl = 0.f;
+                for (int j = 0; j < p; ++j) df_fma(ph, pl, qH[rr][j], qL[rr][j], cH[j][c], cL[j][c]);
+                Q[(roff + r) * ldx + c] = df_to_f64(ph, pl);
+            }
         }
         return;
     }
@@ -894,6 +953,7 @@ __global__ void __launch_bounds__(TPB) k_update(const double* __restrict__ Y, co
         bool ok = r < n;
         long long idx = (roff + r) * ldx + c;
         sY[rr][c] = ok ? Y[idx] : 0.0;
+        if (Q) sX[rr][c] = ok ? X[idx] : 0.0;
         if (FULL) {
             sA[rr][c] = ok ? AY[idx] : 0.0;
             sB[rr][c] = ok ? BY[idx] : 0.0;
@@ -910,6 +970,11 @@ __global__ void __launch_bounds__(TPB) k_update(const double* __restrict__ Y, co
             for (int j = 0; j < p; ++j) x += sY[rr][j] * sC[j][c];
             int r = r0 + rr;
             if (r < rows) X[(roff + r) * ldx + c] = x;
+            if (Q && r < rows) {
+                double v = 0.0;
+                for (int j = 0; j < p; ++j) v += sX[rr][j] * sC[j][c];
+                Q[(roff + r) * ldx + c] = v;
+            }
         }
         return;
     }
@@ -932,6 +997,11 @@ __global__ void __launch_bounds__(TPB) k_update(const double* __restrict__ Y, co
             X[idx] = x;
             AX[idx] = ax;
             BX[idx] = bx;
+            if (Q) {
+                double v = 0.0;
+                for (int j = 0; j < p; ++j) v += sX[rr][j] * sC[j][c];
+                Q[idx] = v;
+            }
         }
         double rv = ax - theta[i * PMAX + c] * bx;
         vnum[k] = rv * rv;
@@ -1041,30 +1111,31 @@ __global__ void k_check_knorm(const double* __restrict__ partial, const double* 
         decide(i, sres, theta, p, sigma, tol, eta, nev_max, it, maxit, true, done, m_, iters, n_active, best, best_it);
 }
 
-// ---- FP32 start phase: block inverse iteration W <- K~^{-1} B (W C) with
-// C = D R^{-1} from the Euclidean CholQR of W (D W^T W D = R^T R, D =
-// diag(W^T W)^{-1/2}).  The blocks are FP32 with ldw = p rounded up to 4
-// columns a row, so a row is one to two whole 32-byte sectors of each group
-// of columns and nothing is converted; the orthonormal block W C itself is
-// only formed at the end: the next right-hand side is (B W) C, B applied to
-// the rows of W and C to the result.
+// ---- FP32 start phase on X = V C, C = D R^{-1} from the Euclidean CholQR of
+// V (D V^T V D = R^T R, D = diag(V^T V)^{-1/2}): V <- S X, S = K~^{-1} B, in the
+// power steps, V <- w (S X - e X) [- Q] in the steps of the Chebyshev recurrence
+// (as k_form_y; Q the X before it times C).  The blocks are FP32 with ldw = p
+// rounded up to 4 columns a row, so nothing is converted; the right-hand side
+// is (B V) C, B applied to the rows of V and C to the result.
 
-// Partial Gram matrices of row range blockIdx.y: a thread owns a 4 x 4 tile of
-// the upper triangle and every `lanes`-th row (two 16-byte loads and 16 FMA a
-// row); the tiles are summed over the row lanes in shared memory.  The last
+// Partial Gram matrices of row range blockIdx.y, staged through shared memory
+// (V formed from S X, X and Q on the way in the Chebyshev steps): a thread owns
+// a 4 x 4 tile of the upper triangle and every `lanes`-th row; the tiles are
+// summed over the row lanes in shared memory.  The last
 // block of a problem (ticket) sums the row ranges in order and factorises, in
 // one warp: column b of the scaled Gram in the registers of lane b, a row of
 // R exchanged through shared memory per step.  A column whose pivot falls
 // below 1e-10 of its scaled diagonal is dependent on the previous ones: it is
 // reset to its scaled self (R row e_k) so that the basis stays finite; the
-// FP64 phase removes it.
+// FP64 phase removes it.  After a power step |R_kk| estimates the eigenvalues
+// of S (orthogonal iteration); the damped interval is taken from the smallest.
 __device__ __forceinline__ float rsqrt_f32(float x) {
     const float r = rsqrtf(x);
     return r * fmaf(-0.5f * x * r, r, 1.5f);
 }
 
 template <int PB>
-__device__ void cholqr_warp(float (*G)[PMAX + 4], float* dinv, int p, float* __restrict__ C) {
+__device__ float cholqr_warp(float (*G)[PMAX + 4], float* dinv, int p, float* __restrict__ C) {
     const int b = threadIdx.x & 31;
     const float gbb = b < p ? G[b][b] : 0.f;
     const float db = gbb > 0.f ? rsqrt_f32(gbb) : 0.f;      // column scale
@@ -1075,10 +1146,12 @@ __device__ void cholqr_warp(float (*G)[PMAX + 4], float* dinv, int p, float* __r
     for (int a = 0; a < PB; ++a) g[a] = a < p && b < p ? dinv[a] * G[min(a, b)][max(a, b)] * db : 0.f;
     __syncwarp();
     float rinv[PB];
+    float rmin = 3e38f;                              // lane k: |R_kk| of the unscaled factor, 0 if it was reset
 #pragma unroll
     for (int k = 0; k < PB; ++k) {
         const float piv = __shfl_sync(0xffffffffu, g[k], k);
         const bool ok = piv > 1e-10f;
+        if (b == k && k < p) rmin = ok && db > 0.f ? sqrtf(piv) / db : 0.f;
         const float ru = ok ? rsqrt_f32(piv) : 1.f;
         rinv[k] = ru;
         const float u = b == k ? (ok ? piv * ru : 1.f) : (ok && b > k ? g[k] * ru : 0.f);   // R[k][b]
@@ -1100,20 +1173,26 @@ __device__ void cholqr_warp(float (*G)[PMAX + 4], float* dinv, int p, float* __r
 #pragma unroll
     for (int a = 0; a < PB; ++a)
         if (b < PMAX) C[a * PMAX + b] = a < p && b < p && a <= b ? dinv[a] * x[a] : 0.f;
+    for (int o = 16; o > 0; o >>= 1) rmin = fminf(rmin, __shfl_xor_sync(0xffffffffu, rmin, o));
+    return rmin;
 }
 
-constexpr int G32_T = 256;
-__global__ void __launch_bounds__(G32_T) k_gram_cholqr32(const float* __restrict__ W, int ldw, float* __restrict__ Gp,
-                                                         float* __restrict__ C, const int* __restrict__ n_,
+constexpr int G32_T = 256, G32_ROWS = 64;
+// mode FORM_FIRST: V = SX (a power step); else V (written) = w (SX - e X) [- Q]
+__global__ void __launch_bounds__(G32_T) k_gram_cholqr32(const float* __restrict__ SX, const float* __restrict__ X,
+                                                         const float* __restrict__ Q, float* __restrict__ V, int mode,
+                                                         int ldw, float* __restrict__ Gp, float* __restrict__ C,
+                                                         double* __restrict__ cheb, const int* __restrict__ n_,
                                                          const long long* __restrict__ roff_,
                                                          const int* __restrict__ p_, int gsplit,
                                                          unsigned* __restrict__ ticket) {
     __shared__ float red[G32_T][17];
+    __shared__ __align__(16) float sV[G32_ROWS][PMAX + 4];
     __shared__ float G[PMAX][PMAX + 4];
     __shared__ float dinv[PMAX];
     __shared__ int s_last;
     const int i = blockIdx.x, sp = blockIdx.y, t = threadIdx.x;
-    const int n = n_[i], p = p_[i], q = (p + 3) / 4;
+    const int n = n_[i], p = p_[i], q = (p + 3) / 4, qw = ldw / 4;
     if (p == 0) return;
     const int ntile = q * (q + 1) / 2, lanes = G32_T / ntile;
     const int rows_per = (n + gsplit - 1) / gsplit;
@@ -1122,19 +1201,42 @@ __global__ void __launch_bounds__(G32_T) k_gram_cholqr32(const float* __restrict
     int a = 0, rem = tile;
     while (rem >= q - a) { rem -= q - a; ++a; }
     const int b = a + rem;
+    double cw = 1.0, ca = 0.0, cq = 0.0;
+    if (mode != FORM_FIRST) cheb_coef(mode, cheb[i], 0.0, ca, cw, cq);
+    // cheb_coef at mu = 0: a = -w e (0 in a plain step, whose V is SX)
+    const float fw = (float)cw, fa = (float)ca, fq = (float)cq;
     float acc[4][4] = {};
-    if (rl < lanes) {
-        const float* base = W + roff_[i] * ldw;
-#pragma unroll 4
-        for (int r = r_lo + rl; r < r_hi; r += lanes) {
-            const float4 u = *reinterpret_cast<const float4*>(base + (long long)r * ldw + 4 * a);
-            const float4 v = *reinterpret_cast<const float4*>(base + (long long)r * ldw + 4 * b);
-            const float uu[4] = {u.x, u.y, u.z, u.w}, vv[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-            for (int x = 0; x < 4; ++x)
-#pragma unroll
-                for (int y = 0; y < 4; ++y) acc[x][y] = fmaf(uu[x], vv[y], acc[x][y]);
+    const long long base = roff_[i] * ldw;
+    for (int r0 = r_lo; r0 < r_hi; r0 += G32_ROWS) {
+        const int nr = min(G32_ROWS, r_hi - r0);
+        __syncthreads();
+        for (int e = t; e < nr * qw; e += G32_T) {
+            const int rr = e / qw, g4 = 4 * (e % qw);
+            const long long o = base + (long long)(r0 + rr) * ldw + g4;
+            float4 v = *reinterpret_cast<const float4*>(SX + o);
+            if (mode != FORM_FIRST) {
+                const float4 x = *reinterpret_cast<const float4*>(X + o);
+                v.x = fmaf(fa, x.x, fw * v.x); v.y = fmaf(fa, x.y, fw * v.y);
+                v.z = fmaf(fa, x.z, fw * v.z); v.w = fmaf(fa, x.w, fw * v.w);
+                if (fq != 0.f) {
+                    const float4 u = *reinterpret_cast<const float4*>(Q + o);
+                    v.x -= u.x; v.y -= u.y; v.z -= u.z; v.w -= u.w;
+                }
+                *reinterpret_cast<float4*>(V + o) = v;
+            }
+            *reinterpret_cast<float4*>(&sV[rr][g4]) = v;
         }
+        __syncthreads();
+        if (rl < lanes)
+            for (int r = rl; r < nr; r += lanes) {
+                const float4 u = *reinterpret_cast<const float4*>(&sV[r][4 * a]);
+                const float4 v = *reinterpret_cast<const float4*>(&sV[r][4 * b]);
+                const float uu[4] = {u.x, u.y, u.z, u.w}, vv[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+                for (int x = 0; x < 4; ++x)
+#pragma unroll
+                    for (int y = 0; y < 4; ++y) acc[x][y] = fmaf(uu[x], vv[y], acc[x][y]);
+            }
     }
 #pragma unroll
     for (int x = 0; x < 4; ++x)
@@ -1167,10 +1269,12 @@ __global__ void __launch_bounds__(G32_T) k_gram_cholqr32(const float* __restrict
     __syncthreads();
     if (t >= 32) return;
     float* Ci = C + (long long)i * PMAX * PMAX;
-    if (ldw <= 12) cholqr_warp<12>(G, dinv, p, Ci);
-    else if (ldw <= 16) cholqr_warp<16>(G, dinv, p, Ci);
-    else if (ldw <= 20) cholqr_warp<20>(G, dinv, p, Ci);
-    else cholqr_warp<32>(G, dinv, p, Ci);
+    float rmin;
+    if (ldw <= 12) rmin = cholqr_warp<12>(G, dinv, p, Ci);
+    else if (ldw <= 16) rmin = cholqr_warp<16>(G, dinv, p, Ci);
+    else if (ldw <= 20) rmin = cholqr_warp<20>(G, dinv, p, Ci);
+    else rmin = cholqr_warp<32>(G, dinv, p, Ci);
+    if (mode == FORM_FIRST && t == 0) cheb[i] = CHEB_CUT * (double)rmin;
 }
 
 // X = W C on blocks of 32 rows (FP32 products, stored as FP64): the end of
@@ -1309,7 +1413,7 @@ void GevpBatch::alloc(cudaStream_t s) {
     P = K.P;
     d_p.upload(p, s);
     size_t rows = (size_t)K.total_rows;
-    for (DevBuf<double>* b : {&X, &AX, &BX, &Y, &AY, &BY}) { b->alloc(rows * ldx); b->zero(s); }
+    for (DevBuf<double>* b : {&X, &AX, &BX, &Y, &AY, &BY, &Q}) { b->alloc(rows * ldx); b->zero(s); }
     if (K.prec) {
         int pm = 1;
         for (int v : p) pm = std::max(pm, v);
@@ -1338,6 +1442,8 @@ void GevpBatch::alloc(cudaStream_t s) {
     nblk_max = (int)ceil_div((long long)K.max_K * NB, ROWBLK);
     partial.alloc((size_t)P * nblk_max * 2 * PMAX);
     done.alloc(P);
+    cheb.alloc(P);
+    cheb.zero(s);
     best.alloc(P);
     best_it.alloc(P);
     m.alloc(P);
@@ -1355,7 +1461,7 @@ GevpBatch GevpBatch::slice(int p0, int np, int group) const {
     v.K = K.slice(p0, np);
     for (auto pr : {std::make_pair(&v.X, &X), std::make_pair(&v.AX, &AX), std::make_pair(&v.BX, &BX),
                     std::make_pair(&v.Y, &Y), std::make_pair(&v.AY, &AY), std::make_pair(&v.BY, &BY),
-                    std::make_pair(&v.W, &W)})
+                    std::make_pair(&v.W, &W), std::make_pair(&v.Q, &Q)})
         *pr.first = pr.second->view(0, pr.second->n);
     v.ldw = ldw;
     v.W32 = W32.view(0, W32.n);
@@ -1370,6 +1476,7 @@ GevpBatch GevpBatch::slice(int p0, int np, int group) const {
     v.nblk_max = nblk_max;
     v.partial = partial.view((size_t)p0 * nblk_max * 2 * PMAX, (size_t)np * nblk_max * 2 * PMAX);
     v.done = done.view(p0, np); v.m = m.view(p0, np); v.rank = rank.view(p0, np); v.iters = iters.view(p0, np);
+    v.cheb = cheb.view(p0, np);
     v.best = best.view(p0, np); v.best_it = best_it.view(p0, np);
     v.n_active = n_active.view(group, 1);
     v.knorm = knorm;
@@ -1402,20 +1509,20 @@ void eig_form_rhs(GevpBatch& g, double sigma, bool first, cudaStream_t s) {
     MSDD_LAUNCH_CHECK();
 }
 
-void eig_form_y(GevpBatch& g, double sigma, bool first, cudaStream_t s) {
+void eig_form_y(GevpBatch& g, double sigma, EigForm mode, cudaStream_t s) {
     dim3 grid(32, g.P);
     if (g.K.prec)
-        k_form_y<float><<<grid, 256, 0, s>>>(g.Y.p, g.X.p, g.W32.p, g.ldw, g.theta.p, g.K.d_n.p, g.K.d_K.p,
-                                             g.K.d_roff.p, g.d_p.p, g.ldx, sigma, first ? 1 : 0, g.done.p);
+        k_form_y<float><<<grid, 256, 0, s>>>(g.Y.p, g.X.p, g.W32.p, g.ldw, g.Q.p, g.cheb.p, g.theta.p, g.K.d_n.p,
+                                             g.K.d_K.p, g.K.d_roff.p, g.d_p.p, g.ldx, sigma, mode, g.done.p);
     else
-        k_form_y<double><<<grid, 256, 0, s>>>(g.Y.p, g.X.p, g.W.p, g.ldw, g.theta.p, g.K.d_n.p, g.K.d_K.p,
-                                              g.K.d_roff.p, g.d_p.p, g.ldx, sigma, first ? 1 : 0, g.done.p);
+        k_form_y<double><<<grid, 256, 0, s>>>(g.Y.p, g.X.p, g.W.p, g.ldw, g.Q.p, g.cheb.p, g.theta.p, g.K.d_n.p,
+                                              g.K.d_K.p, g.K.d_roff.p, g.d_p.p, g.ldx, sigma, mode, g.done.p);
     MSDD_LAUNCH_CHECK();
 }
 
-void eig_form_y_knorm(GevpBatch& g, double sigma, cudaStream_t s) {
+void eig_form_y_knorm(GevpBatch& g, double sigma, EigForm mode, cudaStream_t s) {
     dim3 grid(g.nblk_max, g.P);
-    k_form_y_knorm<<<grid, TPB, 0, s>>>(g.Y.p, g.X.p, g.W.p, g.AX.p, g.BX.p, g.theta.p, g.K.d_n.p, g.K.d_K.p,
+    k_form_y_knorm<<<grid, TPB, 0, s>>>(g.Y.p, g.X.p, g.W.p, g.AX.p, g.BX.p, g.Q.p, g.cheb.p, mode, g.theta.p, g.K.d_n.p, g.K.d_K.p,
                                         g.K.d_roff.p, g.d_p.p, g.ldx, sigma, g.partial.p, g.nblk_max, g.done.p);
     MSDD_LAUNCH_CHECK();
 }
@@ -1432,11 +1539,12 @@ void eig_start32(GevpBatch& g, float* W, cudaStream_t s) {
     MSDD_LAUNCH_CHECK();
 }
 
-void eig_cholqr32(GevpBatch& g, const float* W, cudaStream_t s) {
+void eig_cholqr32(GevpBatch& g, EigForm mode, const float* SX, const float* X, const float* Q, float* V,
+                  cudaStream_t s) {
     // the FP64 Gram partials and coefficients are free in this phase and hold the FP32 ones
-    k_gram_cholqr32<<<dim3(g.P, g.gsplit), G32_T, 0, s>>>(W, g.ldw, reinterpret_cast<float*>(g.Hp.p),
-                                                          reinterpret_cast<float*>(g.C.p), g.K.d_n.p, g.K.d_roff.p,
-                                                          g.d_p.p, g.gsplit, g.ticket.p);
+    k_gram_cholqr32<<<dim3(g.P, g.gsplit), G32_T, 0, s>>>(SX, X, Q, V, mode, g.ldw, reinterpret_cast<float*>(g.Hp.p),
+                                                          reinterpret_cast<float*>(g.C.p), g.cheb.p, g.K.d_n.p,
+                                                          g.K.d_roff.p, g.d_p.p, g.gsplit, g.ticket.p);
     MSDD_LAUNCH_CHECK();
 }
 
@@ -1458,27 +1566,28 @@ void eig_gram(GevpBatch& g, cudaStream_t s) {
     MSDD_LAUNCH_CHECK();
 }
 
-void eig_rayleigh_ritz(GevpBatch& g, cudaStream_t s) {
-    k_rayleigh_ritz<<<g.P, TPB, 0, s>>>(g.Hp.p, g.Mp.p, g.gsplit, g.H.p, g.M.p, g.C.p, g.theta.p, g.d_p.p, g.rank.p,
-                                        g.done.p);
+void eig_rayleigh_ritz(GevpBatch& g, double sigma, cudaStream_t s) {
+    k_rayleigh_ritz<<<g.P, TPB, 0, s>>>(g.Hp.p, g.Mp.p, g.gsplit, g.H.p, g.M.p, g.C.p, g.theta.p, g.cheb.p, sigma,
+                                        g.d_p.p, g.rank.p, g.done.p);
     MSDD_LAUNCH_CHECK();
 }
 
-void eig_update(GevpBatch& g, cudaStream_t s) {
+void eig_update(GevpBatch& g, bool want_q, cudaStream_t s) {
     dim3 grid(g.nblk_max, g.P);
-    k_update<true><<<grid, TPB, 0, s>>>(g.Y.p, g.AY.p, g.BY.p, g.X.p, g.AX.p, g.BX.p, g.C.p, g.theta.p, g.K.d_n.p,
-                                        g.K.d_K.p, g.K.d_roff.p, g.d_p.p, g.ldx, g.partial.p, g.nblk_max, g.done.p);
+    k_update<true><<<grid, TPB, 0, s>>>(g.Y.p, g.AY.p, g.BY.p, g.X.p, g.AX.p, g.BX.p, want_q ? g.Q.p : nullptr,
+                                        g.C.p, g.theta.p, g.K.d_n.p, g.K.d_K.p, g.K.d_roff.p, g.d_p.p, g.ldx, g.partial.p, g.nblk_max, g.done.p);
     MSDD_LAUNCH_CHECK();
 }
 
-void eig_update_x(GevpBatch& g, cudaStream_t s) {
+void eig_update_x(GevpBatch& g, bool want_q, cudaStream_t s) {
+    double* q = want_q ? g.Q.p : nullptr;
     dim3 grid(g.nblk_max, g.P);
     if (g.K.prec)
-        k_update<false, true><<<grid, TPB, 0, s>>>(g.Y.p, nullptr, nullptr, g.X.p, nullptr, nullptr, g.C.p, g.theta.p,
+        k_update<false, true><<<grid, TPB, 0, s>>>(g.Y.p, nullptr, nullptr, g.X.p, nullptr, nullptr, q, g.C.p, g.theta.p,
                                                    g.K.d_n.p, g.K.d_K.p, g.K.d_roff.p, g.d_p.p, g.ldx, nullptr,
                                                    g.nblk_max, g.done.p);
     else
-        k_update<false><<<grid, TPB, 0, s>>>(g.Y.p, nullptr, nullptr, g.X.p, nullptr, nullptr, g.C.p, g.theta.p,
+        k_update<false><<<grid, TPB, 0, s>>>(g.Y.p, nullptr, nullptr, g.X.p, nullptr, nullptr, q, g.C.p, g.theta.p,
                                              g.K.d_n.p, g.K.d_K.p, g.K.d_roff.p, g.d_p.p, g.ldx, nullptr, g.nblk_max,
                                              g.done.p);
     MSDD_LAUNCH_CHECK();

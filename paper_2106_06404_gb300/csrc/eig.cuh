@@ -33,6 +33,8 @@ struct GevpBatch {
     DevBuf<float> W32;
     int ldw = PMAX;
     DevBuf<unsigned> ticket;          // per problem: row ranges of the FP32 Gram that are done
+    DevBuf<double> Q;                              // the block before X in its basis (Chebyshev recurrence)
+    DevBuf<double> cheb;                           // per problem: end of the damped interval of S = K^{-1} B, 0 unknown
     DevBuf<double> H, M, C, theta, res;            // per problem PMAX^2 / PMAX
     int gsplit = 1;                                // row splits of the Gram products
     DevBuf<double> Hp, Mp;                         // per (problem, split) PMAX^2 partial Grams
@@ -67,26 +69,33 @@ void eig_init(GevpBatch& g, unsigned long long seed, cudaStream_t s);
 void eig_load_start(GevpBatch& g, const double* Wst, int wc, const long long* d_woff, cudaStream_t s);
 // W = BX - (AX + sigma BX) diag(mu) (first == true: W = BX).
 void eig_form_rhs(GevpBatch& g, double sigma, bool first, cudaStream_t s);
-// Y = X diag(mu) + W (first == true: Y = W).
-void eig_form_y(GevpBatch& g, double sigma, bool first, cudaStream_t s);
-// Y = X diag(mu) + W with the K^+-norm residual partial sums of X.
-void eig_form_y_knorm(GevpBatch& g, double sigma, cudaStream_t s);
+// The next block from X, W = S X - X diag(mu) (S = K^{-1} B) and Q, the block
+// before X: FORM_FIRST Y = W (which then is S X), FORM_CHEB1 the first and
+// FORM_CHEB every further step of the Chebyshev recurrence that damps
+// [0, cheb[i]] (plain S X where cheb[i] is 0).
+enum EigForm { FORM_FIRST = 0, FORM_CHEB1 = 1, FORM_CHEB = 2 };
+void eig_form_y(GevpBatch& g, double sigma, EigForm mode, cudaStream_t s);
+// FP32 start phase: W <- X in FP32; V = S X (FORM_FIRST: V is SX and the
+// damped interval is set) or the Chebyshev step of SX, X and Q (V written),
+// and C (FP32, in the buffer of g.C) with V C an orthonormal basis of span(V)
+// by Euclidean CholQR; X <- W C.
+void eig_start32(GevpBatch& g, float* W, cudaStream_t s);
+void eig_cholqr32(GevpBatch& g, EigForm mode, const float* SX, const float* X, const float* Q, float* V,
+                  cudaStream_t s);
+void eig_update32(GevpBatch& g, const float* W, cudaStream_t s);
+// The same with the K^+-norm residual partial sums of X.
+void eig_form_y_knorm(GevpBatch& g, double sigma, EigForm mode, cudaStream_t s);
 // Convergence test on the K^+-norm residuals (regularised coarse pencils).
 void eig_check_knorm(GevpBatch& g, const EigParams& ep, int it, cudaStream_t s);
-// FP32 start phase: W <- X in FP32; C (FP32, in the buffer of g.C) with W C an
-// orthonormal basis of span(W) by Euclidean CholQR; X <- W C.
-void eig_start32(GevpBatch& g, float* W, cudaStream_t s);
-void eig_cholqr32(GevpBatch& g, const float* W, cudaStream_t s);
-void eig_update32(GevpBatch& g, const float* W, cudaStream_t s);
 // H = Y^T AY, M = Y^T BY.
 void eig_gram(GevpBatch& g, cudaStream_t s);
-// Rayleigh-Ritz: theta ascending, C with C^T M C = I.
-void eig_rayleigh_ritz(GevpBatch& g, cudaStream_t s);
-// X = Y C, AX = AY C, BX = BY C, residual partial sums.
-void eig_update(GevpBatch& g, cudaStream_t s);
+// Rayleigh-Ritz: theta ascending, C with C^T M C = I; the next damped interval.
+void eig_rayleigh_ritz(GevpBatch& g, double sigma, cudaStream_t s);
+// X = Y C, AX = AY C, BX = BY C, residual partial sums; want_q: Q = (old X) C.
+void eig_update(GevpBatch& g, bool want_q, cudaStream_t s);
 // X = Y C only: with a cheap operator (stored stencils) AX and BX are applied
 // afresh, together with the next right-hand side (apply_local_rhs).
-void eig_update_x(GevpBatch& g, cudaStream_t s);
+void eig_update_x(GevpBatch& g, bool want_q, cudaStream_t s);
 // Residuals, selection count m = min(nev_max, #{theta < eta}), convergence flags.
 void eig_check(GevpBatch& g, const EigParams& ep, int it, cudaStream_t s);
 

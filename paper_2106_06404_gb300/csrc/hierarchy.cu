@@ -12,6 +12,7 @@
 #include "hierarchy.cuh"
 
 #include <algorithm>
+#include <array>
 #include <chrono>
 #include <cmath>
 #include <cstring>
@@ -91,7 +92,8 @@ void dense_inverse(const TileBatch& tb, double* out, const std::vector<long long
 // Subspace iteration driver.  apply(v, p0, X, AX, BX, skip, s) applies Abar
 // and B to the problems of batch view v (first problem p0 of the whole
 // batch), solve(v, p0, ncols, W32, s) applies K^{-1} to W32 (FP32 factors) or
-// v.W, bapply32(v, p0, W, Wout, C, s) is Wout = (B W) C in FP32.  `tag` names the kernel families for profiling;
+// v.W, bapply32(v, p0, W, Wout, C, X, Q, s) is Wout = (B W) C in FP32, Q = X C
+// and X = W C.  `tag` names the kernel families for profiling;
 // `apply_bytes`/`apply_flops` are the algorithmic amounts of one operator
 // application per problem.
 //
@@ -99,9 +101,7 @@ void dense_inverse(const TileBatch& tb, double* out, const std::vector<long long
 // whose iterations are offset by about one band solve: the latency-bound
 // kernels of one half (band solve, Rayleigh-Ritz) then run beside the
 // FP64-bound kernels of the other (operators, Gram products, updates).
-// Convergence is read back every `batch` = 4 iterations (a host round trip
-// per iteration would drain the stream); a group that converged inside a
-// batch only launches kernels that skip its (done) problems.
+// Convergence is read back one iteration behind.
 //
 // With `fused` (operators cheaper than the p x p update: stored stencils),
 // the update forms X = Y C only and apply_rhs(v, p0, s) applies Abar and B
@@ -116,7 +116,6 @@ void run_eig(GevpBatch& g, const EigParams& ep, Apply apply, Solve solve, BApply
     eig_init(g, ep.seed, st);
     eig_load_start(g, start, start_cols, d_start_off, st);
     const int G = (groups == 2 && g.P >= 2 && st_b) ? 2 : 1;
-    const int batch = 4;
     std::vector<GevpBatch> gv;
     std::vector<int> gp0;
     std::vector<cudaStream_t> gs;
@@ -154,31 +153,42 @@ void run_eig(GevpBatch& g, const EigParams& ep, Apply apply, Solve solve, BApply
         am[k].solve_b = am[k].sb0;
         am[k].solve_f = am[k].sf0;
     }
-    // FP32 start phase: block inverse iteration W <- K~^{-1} B (W C), C from
-    // the Euclidean CholQR of W, all in FP32; the FP64 phase below starts from
-    // its subspace and alone decides convergence.  The blocks alternate
-    // between W32 and a second buffer (B reads neighbouring rows).
-    DevBuf<float> wb(fp32_iters > 0 ? g.W32.n : 0);
-    for (int k = 0; k < G && fp32_iters > 0; ++k) eig_start32(gv[k], wb.p, gs[k]);
-    for (int it = 0; it < fp32_iters; ++it)
+    // FP32 start phase: X = V C orthonormal (Euclidean CholQR), V <- S X with
+    // S = K~^{-1} B in the power steps and the Chebyshev recurrence on S in the
+    // others, all in FP32; the FP64 phase below starts from its subspace and
+    // alone decides convergence.  The damped interval comes from the last power
+    // step, so the first six are power steps (the block has to settle) and
+    // every eighth after them renews it: 20 such steps leave a 1400-point model
+    // spectrum 2-5 FP64 iterations, 20 power steps 9-14.
+    DevBuf<float> wb(fp32_iters > 0 ? 3 * g.W32.n : 0);
+    float *vb = wb.p, *sb = g.W32.p, *xb = wb.p + g.W32.n, *qb = wb.p + 2 * g.W32.n;    // V, S X, X, Q
+    auto start_mode = [](int it) {
+        const int j = (it - 6) % 8;
+        return it < 6 || j == 7 ? FORM_FIRST : j == 0 ? FORM_CHEB1 : FORM_CHEB;
+    };
+    for (int k = 0; k < G && fp32_iters > 0; ++k) eig_start32(gv[k], vb, gs[k]);
+    for (int it = 0; it < fp32_iters; ++it) {
+        const EigForm mode = start_mode(it);
         for (int k = 0; k < G; ++k) {
             GevpBatch& v = gv[k];
-            float *src = it % 2 == 0 ? wb.p : v.W32.p, *dst = it % 2 == 0 ? v.W32.p : wb.p;
             prof.begin(tag + "_fp32_start_other", gs[k]);
-            bapply32(v, gp0[k], src, dst, it == 0 ? nullptr : reinterpret_cast<const float*>(v.C.p), gs[k]);
+            bapply32(v, gp0[k], vb, sb, it == 0 ? nullptr : reinterpret_cast<const float*>(v.C.p),
+                     mode == FORM_FIRST ? nullptr : xb, mode == FORM_CHEB ? qb : nullptr, gs[k]);
             prof.end(gs[k], 0.0, 0.0);
             prof.begin(tag + "_solve", gs[k]);
-            solve(v, gp0[k], am[k].pm, dst, gs[k]);
+            solve(v, gp0[k], am[k].pm, sb, gs[k]);
             prof.end(gs[k], am[k].sb0, am[k].sf0);
             if (G == 2 && k == 0 && it == 0) {
                 MSDD_CUDA(cudaEventRecord(ev_off, gs[0]));        // the second half starts one solve later
                 MSDD_CUDA(cudaStreamWaitEvent(gs[1], ev_off, 0));
             }
             prof.begin(tag + "_fp32_start_other", gs[k]);
-            eig_cholqr32(v, dst, gs[k]);
-            if (it + 1 == fp32_iters) eig_update32(v, dst, gs[k]);
+            eig_cholqr32(v, mode, sb, xb, qb, vb, gs[k]);
+            if (it + 1 == fp32_iters) eig_update32(v, mode == FORM_FIRST ? sb : vb, gs[k]);
             prof.end(gs[k], 0.0, 0.0);
         }
+        if (mode == FORM_FIRST) std::swap(vb, sb);                // V is S X itself
+    }
     std::vector<int> active(G), iter(G, 0);
     for (int k = 0; k < G; ++k) {
         active[k] = gv[k].P;
@@ -189,6 +199,7 @@ void run_eig(GevpBatch& g, const EigParams& ep, Apply apply, Solve solve, BApply
         GevpBatch& v = gv[k];
         cudaStream_t s = gs[k];
         const bool first = it == 0;
+        const EigForm mode = first ? FORM_FIRST : it == 1 ? FORM_CHEB1 : FORM_CHEB;
         const double fr = (double)active[k] / v.P;
         if (!fused || first) eig_form_rhs(v, ep.sigma, first, s);
         prof.begin(tag + "_solve", s);
@@ -200,11 +211,11 @@ void run_eig(GevpBatch& g, const EigParams& ep, Apply apply, Solve solve, BApply
         }
         if (v.knorm && !first) {
             // test the current Ritz pairs before updating them
-            eig_form_y_knorm(v, ep.sigma, s);
+            eig_form_y_knorm(v, ep.sigma, mode, s);
             MSDD_CUDA(cudaMemsetAsync(v.n_active.p, 0, sizeof(int), s));
             eig_check_knorm(v, ep, it, s);
         } else {
-            eig_form_y(v, ep.sigma, first, s);
+            eig_form_y(v, ep.sigma, mode, s);
         }
         prof.begin(tag + "_apply", s);
         apply(v, gp0[k], v.Y.p, v.AY.p, v.BY.p, (const int*)v.done.p, s);
@@ -213,18 +224,18 @@ void run_eig(GevpBatch& g, const EigParams& ep, Apply apply, Solve solve, BApply
         eig_gram(v, s);
         prof.end(s, 3.0 * am[k].vec_n * 8.0 * fr, 2.0 * am[k].vec_n * (am[k].pm + 1) * fr);
         prof.begin(tag + "_rayleigh_ritz", s);
-        eig_rayleigh_ritz(v, s);
+        eig_rayleigh_ritz(v, ep.sigma, s);
         prof.end(s, 0.0, 0.0);
         if (fused) {
             prof.begin(tag + "_update", s);
-            eig_update_x(v, s);
+            eig_update_x(v, !first, s);
             prof.end(s, 2.0 * am[k].vec_n * 8.0 * fr, 2.0 * am[k].vec_n * am[k].pm * fr);
             prof.begin(tag + "_apply", s);
             apply_rhs(v, gp0[k], s);
             prof.end(s, (apply_bytes + 8.0 * am[k].vec_n / std::max(1, v.P)) * active[k], apply_flops * active[k]);
         } else {
             prof.begin(tag + "_update", s);
-            eig_update(v, s);
+            eig_update(v, !first, s);
             prof.end(s, 6.0 * am[k].vec_n * 8.0 * fr, 6.0 * am[k].vec_n * am[k].pm * fr);
         }
         if (v.knorm) {
@@ -233,29 +244,42 @@ void run_eig(GevpBatch& g, const EigParams& ep, Apply apply, Solve solve, BApply
             MSDD_CUDA(cudaMemsetAsync(v.n_active.p, 0, sizeof(int), s));
             eig_check(v, ep, it, s);
         }
-        MSDD_CUDA(cudaMemcpyAsync(&h_act[k], v.n_active.p, sizeof(int), cudaMemcpyDeviceToHost, s));
+        MSDD_CUDA(cudaMemcpyAsync(&h_act[2 * k + (it & 1)], v.n_active.p, sizeof(int), cudaMemcpyDeviceToHost, s));
         return true;
     };
-    for (;;) {
-        bool any = false;
-        std::vector<bool> checked(G, false);
-        for (int b = 0; b < batch; ++b)
-            for (int k = 0; k < G; ++k) {
-                if (active[k] == 0 || iter[k] >= ep.maxit) continue;
-                const bool offset = G == 2 && k == 0 && b == 0 && active[1] > 0 && iter[1] < ep.maxit;
-                if (iteration(k, iter[k], offset)) checked[k] = true;
-                ++iter[k];
-                any = true;
-            }
-        if (!any) break;
+    // the host reads the active count of iteration it while it + 1 is already
+    // enqueued: the stream does not drain, at the price of one iteration whose
+    // kernels find every problem done
+    cudaEvent_t ev_it[2][2];
+    for (auto& e : ev_it)
+        for (cudaEvent_t& x : e) MSDD_CUDA(cudaEventCreateWithFlags(&x, cudaEventDisableTiming));
+    std::vector<std::array<bool, 2>> checked(G, {false, false});
+    for (bool any = true; any;) {
+        any = false;
         for (int k = 0; k < G; ++k) {
-            MSDD_CUDA(cudaStreamSynchronize(gs[k]));
-            if (checked[k]) active[k] = h_act[k];
+            if (active[k] == 0 || iter[k] >= ep.maxit) continue;
+            const int it = iter[k]++;
+            const bool offset = G == 2 && k == 0 && it == 0 && active[1] > 0;
+            checked[k][it & 1] = iteration(k, it, offset);
+            MSDD_CUDA(cudaEventRecord(ev_it[k][it & 1], gs[k]));
+            any = true;
         }
-        bool more = false;
-        for (int k = 0; k < G; ++k) more = more || (active[k] > 0 && iter[k] < ep.maxit);
-        if (!more) break;
+        for (int k = 0; k < G; ++k) {
+            if (active[k] == 0 || iter[k] < 2) continue;
+            const bool last = iter[k] >= ep.maxit;               // then the last iteration is read too
+            for (int it = iter[k] - 2; it < iter[k] - (last ? 0 : 1); ++it) {
+                MSDD_CUDA(cudaEventSynchronize(ev_it[k][it & 1]));
+                if (checked[k][it & 1]) active[k] = h_act[2 * k + (it & 1)];
+            }
+        }
     }
+    for (int k = 0; k < G; ++k)
+        if (iter[k] == 1) {                                       // eig_maxit = 1
+            MSDD_CUDA(cudaEventSynchronize(ev_it[k][0]));
+            if (checked[k][0]) active[k] = h_act[2 * k];
+        }
+    for (auto& e : ev_it)
+        for (cudaEvent_t& x : e) cudaEventDestroy(x);
     for (int k = 1; k < G; ++k) {
         MSDD_CUDA(cudaEventRecord(ev_end, gs[k]));
         MSDD_CUDA(cudaStreamWaitEvent(st, ev_end, 0));
@@ -361,8 +385,8 @@ std::vector<ProbBox> make_fine_boxes(const Geom& g, const msdd_decomp& dec) {
 size_t Hierarchy::device_bytes() const {
     size_t b = 0;
     b += fdir.bytes() + fge.K.bytes() + cdir.bytes() + mdir.bytes() + mge.K.bytes();
-    b += (fge.X.n + fge.AX.n + fge.BX.n + fge.Y.n + fge.AY.n + fge.BY.n + fge.W.n) * 8 + fge.W32.n * 4;
-    b += (mge.X.n + mge.AX.n + mge.BX.n + mge.Y.n + mge.AY.n + mge.BY.n + mge.W.n) * 8;
+    b += (fge.X.n + fge.AX.n + fge.BX.n + fge.Y.n + fge.AY.n + fge.BY.n + fge.W.n + fge.Q.n) * 8 + fge.W32.n * 4;
+    b += (mge.X.n + mge.AX.n + mge.BX.n + mge.Y.n + mge.AY.n + mge.BY.n + mge.W.n + mge.Q.n) * 8;
     b += (Phi.n + A1.n + Abar_m.n + K_m.n + Zb.n + Tm.n + A0.n + frhs.n + v1.n + r0buf.n) * 8;
     b += (Minv.n + A0inv.n + y0buf.n + z1t.n) * 8;
     b += (x.n + r.n + p.n + q.n + z.n + stencil.n + coeff_own.n) * 8;
@@ -590,8 +614,8 @@ void Hierarchy::build_fine() {
                 if (v.K.prec) tile_solve(v.K, W32, v.ldw, pmax, v.done.p, s);
                 else tile_solve(v.K, v.W.p, v.ldw, pmax, v.done.p, s);
             },
-            [=](GevpBatch& v, int p0, const float* W, float* Wout, const float* C, cudaStream_t s) {
-                apply_local_b32(*ls, bx + p0, dim, v.K, W, Wout, v.ldw, C, s);
+            [=](GevpBatch& v, int p0, const float* W, float* Wout, const float* C, float* X, float* Q, cudaStream_t s) {
+                apply_local_b32(*ls, bx + p0, dim, v.K, W, Wout, v.ldw, C, X, Q, s);
             },
             [=](GevpBatch& v, int p0, cudaStream_t s) {
                 apply_local_rhs(*ls, bx + p0, dim, v.K, v.X.p, v.W.p, v.W32.p, v.ldw, v.ldx, v.d_p.p, v.theta.p, ep.sigma,
@@ -982,7 +1006,7 @@ void Hierarchy::build_coarse() {
                     MSDD_CUDA(cudaMemcpyAsync(v.W.p + e0, Wtp + e0, (e1 - e0) * sizeof(double),
                                               cudaMemcpyDeviceToDevice, s));
                 },
-                [=](GevpBatch&, int, const float*, float*, const float*, cudaStream_t) {},
+                [=](GevpBatch&, int, const float*, float*, const float*, float*, float*, cudaStream_t) {},
                 [=](GevpBatch&, int, cudaStream_t) {}, false, 0,
                 st, nullptr, prof, "coarse_gevp", (double)ngen_max * ngen_max * 8.0, 2.0 * ngen_max * ngen_max * block_p,
                 static_cast<int*>(pinned));

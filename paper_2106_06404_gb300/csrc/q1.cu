@@ -519,16 +519,18 @@ __global__ void __launch_bounds__(128) k_apply_rhs(const ProbBox* __restrict__ b
 }
 
 // Wout = (B32 W) C in FP32 (padding rows zeroed; C null: the identity), on
-// blocks of 32 rows; a thread owns a row and four columns.  C (PMAX columns,
+// blocks of 32 rows; a thread owns a row and four columns.  X (may be null)
+// receives W C, and Q (may be null) the old X times C.  C (PMAX columns,
 // upper triangular) comes from the CholQR of W.  Bound by the loads of the
 // 3^d neighbour rows (L1/L2 hits mostly), 16 bytes each.
 template <int D>
 __global__ void __launch_bounds__(256) k_b32_cholqr(const ProbBox* __restrict__ boxes,
                                                     const long long* __restrict__ roff_, const int* __restrict__ K_,
                                                     const float* __restrict__ B32, const float* __restrict__ W,
-                                                    float* __restrict__ Wout, int ldw, const float* __restrict__ C) {
+                                                    float* __restrict__ Wout, int ldw, const float* __restrict__ C,
+                                                    float* __restrict__ X, float* __restrict__ Q) {
     constexpr int NOFF = D == 3 ? 27 : 9;
-    __shared__ __align__(16) float sC[PMAX][PMAX], sT[NB][PMAX + 4];
+    __shared__ __align__(16) float sC[PMAX][PMAX], sT[3][NB][PMAX + 4];
     const int i = blockIdx.y, r0 = blockIdx.x * NB;
     if (r0 >= K_[i] * NB) return;
     const ProbBox pb = boxes[i];
@@ -554,16 +556,24 @@ __global__ void __launch_bounds__(256) k_b32_cholqr(const ProbBox* __restrict__ 
         }
     }
     if (C) {
-        *reinterpret_cast<float4*>(&sT[rr][4 * cg]) = acc;
+        const long long own = (roff + r) * ldw + 4 * cg;
+        *reinterpret_cast<float4*>(&sT[0][rr][4 * cg]) = acc;
+        if (X) *reinterpret_cast<float4*>(&sT[1][rr][4 * cg]) = *reinterpret_cast<const float4*>(W + own);
+        if (Q) *reinterpret_cast<float4*>(&sT[2][rr][4 * cg]) = *reinterpret_cast<const float4*>(X + own);
         __syncthreads();
-        acc = make_float4(0.f, 0.f, 0.f, 0.f);
-        const int kmax = 4 * cg + 4;                 // C is upper triangular
-        for (int k = 0; k < kmax; ++k) {
-            const float v = sT[rr][k];
-            const float4 c = *reinterpret_cast<const float4*>(&sC[k][4 * cg]);
-            acc.x = fmaf(v, c.x, acc.x); acc.y = fmaf(v, c.y, acc.y);
-            acc.z = fmaf(v, c.z, acc.z); acc.w = fmaf(v, c.w, acc.w);
-        }
+        auto times_c = [&](const float* v) {
+            float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
+            const int kmax = 4 * cg + 4;             // C is upper triangular
+            for (int k = 0; k < kmax; ++k) {
+                const float4 c = *reinterpret_cast<const float4*>(&sC[k][4 * cg]);
+                o.x = fmaf(v[k], c.x, o.x); o.y = fmaf(v[k], c.y, o.y);
+                o.z = fmaf(v[k], c.z, o.z); o.w = fmaf(v[k], c.w, o.w);
+            }
+            return o;
+        };
+        acc = times_c(sT[0][rr]);
+        if (X) *reinterpret_cast<float4*>(X + own) = times_c(sT[1][rr]);
+        if (Q) *reinterpret_cast<float4*>(Q + own) = times_c(sT[2][rr]);
     }
     *reinterpret_cast<float4*>(Wout + (roff + r) * ldw + 4 * cg) = acc;
 }
@@ -770,13 +780,15 @@ void apply_local_rhs(const LocalStencil& ls, const ProbBox* d_boxes, int dim, co
 }
 
 void apply_local_b32(const LocalStencil& ls, const ProbBox* d_boxes, int dim, const TileBatch& layout,
-                     const float* W, float* Wout, int ldw, const float* C, cudaStream_t s) {
+                     const float* W, float* Wout, int ldw, const float* C, float* X, float* Q, cudaStream_t s) {
     if (layout.P == 0) return;
     const dim3 grid(layout.max_K, layout.P), block(ldw / 4, NB);
     if (dim == 3)
-        k_b32_cholqr<3><<<grid, block, 0, s>>>(d_boxes, layout.d_roff.p, layout.d_K.p, ls.b32.p, W, Wout, ldw, C);
+        k_b32_cholqr<3><<<grid, block, 0, s>>>(d_boxes, layout.d_roff.p, layout.d_K.p, ls.b32.p, W, Wout, ldw, C,
+                                              X, Q);
     else
-        k_b32_cholqr<2><<<grid, block, 0, s>>>(d_boxes, layout.d_roff.p, layout.d_K.p, ls.b32.p, W, Wout, ldw, C);
+        k_b32_cholqr<2><<<grid, block, 0, s>>>(d_boxes, layout.d_roff.p, layout.d_K.p, ls.b32.p, W, Wout, ldw, C,
+                                              X, Q);
     MSDD_LAUNCH_CHECK();
 }
 

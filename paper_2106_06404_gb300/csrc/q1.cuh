@@ -125,9 +125,10 @@ void apply_local_rhs(const LocalStencil& ls, const ProbBox* d_boxes, int dim, co
                      double sigma, double* partial, int nblk_max, const int* done, cudaStream_t s);
 // Wout = (B W) C in FP32 arithmetic from b32 (blocks of ldw columns, a multiple
 // of 4; zero on padding rows); C is PMAX x PMAX per problem and upper
-// triangular, null for the identity.
+// triangular, null for the identity.  With C: X (may be null) <- W C, and
+// before that Q (may be null) <- X C.
 void apply_local_b32(const LocalStencil& ls, const ProbBox* d_boxes, int dim, const TileBatch& layout,
-                     const float* W, float* Wout, int ldw, const float* C, cudaStream_t s);
+                     const float* W, float* Wout, int ldw, const float* C, float* X, float* Q, cudaStream_t s);
 
 // Stored 3^d-point stencil of the global operator: S[o * n + u] = A(u, u + o),
 // offsets o lexicographic (x fastest) in {-1, 0, 1}^d, zero where u + o is
