@@ -113,8 +113,9 @@ typedef struct msdd_options {
     int profile;         /* 1: time every kernel family with CUDA events (see msdd_stats.prof);
                             2: only the band-solve families (*_solve): two events per band solve
                             instead of ~500 intervals per set-up, for timing runs */
-    int fp32_start_iters;/* precision 1: fine-level FP32 subspace iterations (FP32 B apply and
-                            solve, Euclidean CholQR) before the FP64 iterations (default 20) */
+    int fp32_start_iters;/* precision 1: most fine-level FP32 subspace iterations (FP32 B apply
+                            and solve, Euclidean CholQR) before the FP64 iterations (default
+                            20); a subdomain ends earlier where its spectrum needs fewer */
     const double* warm_start; /* device, may be NULL (default): start vectors of the fine-level
                             subspace iteration, rows = the fine subdomains' Neumann-box nodes
                             (subdomain order, each box lexicographic, x fastest) and warm_cols
@@ -166,7 +167,7 @@ typedef struct msdd_stats {
     msdd_kernel_prof prof[MSDD_MAX_PROF];     /* accumulated over set-up and solves */
     long long eig_iters_total[MSDD_MAX_LEVELS]; /* subspace iterations summed over the level's
                                                  subdomains (FP64 phase; the fine FP32 start
-                                                 phase adds fp32_start_iters per subdomain) */
+                                                 phase adds up to fp32_start_iters each) */
 } msdd_stats;
 
 typedef struct msdd_hierarchy msdd_hierarchy;   /* opaque, library-owned */

@@ -25,7 +25,8 @@ constexpr double CHEB_CUT = 0.95;
 __global__ void k_init(double* __restrict__ X, const int* __restrict__ n_, const int* __restrict__ K_,
                        const long long* __restrict__ roff_, const int* __restrict__ p_, int ldx,
                        unsigned long long seed, int* __restrict__ done, int* __restrict__ iters,
-                       double* __restrict__ theta, double* __restrict__ best, int* __restrict__ best_it) {
+                       double* __restrict__ theta, double* __restrict__ best, int* __restrict__ best_it,
+                       int* __restrict__ sdone, int* __restrict__ sstop, int* __restrict__ smax) {
     const int i = blockIdx.y;
     const int n = n_[i], p = p_[i];
     const long long rows = (long long)K_[i] * NB;
@@ -44,6 +45,9 @@ __global__ void k_init(double* __restrict__ X, const int* __restrict__ n_, const
         if (threadIdx.x == 0) {
             done[i] = (n == 0 || p == 0) ? 1 : 0;
             iters[i] = 0;
+            sdone[i] = done[i];
+            sstop[i] = 1 << 20;
+            if (i < 2) smax[i] = 0;
             best[i] = 1e300;
             best_it[i] = 0;
         }
@@ -1146,12 +1150,12 @@ __device__ float cholqr_warp(float (*G)[PMAX + 4], float* dinv, int p, float* __
     for (int a = 0; a < PB; ++a) g[a] = a < p && b < p ? dinv[a] * G[min(a, b)][max(a, b)] * db : 0.f;
     __syncwarp();
     float rinv[PB];
-    float rmin = 3e38f;                              // lane k: |R_kk| of the unscaled factor, 0 if it was reset
+    float rkk = 3e38f;                               // lane k: |R_kk| of the unscaled factor, 0 if it was reset
 #pragma unroll
     for (int k = 0; k < PB; ++k) {
         const float piv = __shfl_sync(0xffffffffu, g[k], k);
         const bool ok = piv > 1e-10f;
-        if (b == k && k < p) rmin = ok && db > 0.f ? sqrtf(piv) / db : 0.f;
+        if (b == k && k < p) rkk = ok && db > 0.f ? sqrtf(piv) / db : 0.f;
         const float ru = ok ? rsqrt_f32(piv) : 1.f;
         rinv[k] = ru;
         const float u = b == k ? (ok ? piv * ru : 1.f) : (ok && b > k ? g[k] * ru : 0.f);   // R[k][b]
@@ -1173,8 +1177,34 @@ __device__ float cholqr_warp(float (*G)[PMAX + 4], float* dinv, int p, float* __
 #pragma unroll
     for (int a = 0; a < PB; ++a)
         if (b < PMAX) C[a * PMAX + b] = a < p && b < p && a <= b ? dinv[a] * x[a] : 0.f;
-    for (int o = 16; o > 0; o >>= 1) rmin = fminf(rmin, __shfl_xor_sync(0xffffffffu, rmin, o));
-    return rmin;
+    return rkk;
+}
+
+// Iterations of the start phase that a problem needs, from the |R_kk| of the
+// power step that ends the settling part (mu_w: the smallest wanted
+// eigenvalue, either the one at eta or the nev-th; c: the damped interval): a
+// Chebyshev step grows mu_w by x + sqrt(x^2 - 1), x = 2 mu_w / c - 1, against
+// the damped ones; START_GAIN in all takes the block to FP32 accuracy, where
+// further FP32 steps no longer save FP64 ones.  Rounded up to a few stops
+// (start_stop); at most the caller's number.  Fine eigensolve at 20 and at the
+// chosen steps: 512^2 8.8 and 7.0 ms (10-13 steps, the same five FP64
+// iterations), 1000^2 26.8 and 20.7, 50x44x38 22.1 and 16.4 ms; the 96^3
+// composite keeps its 20 (147 ms), where 13 cost six more FP64 iterations
+// (165 ms) and a stop at 17 10 ms.
+constexpr float START_GAIN = 1e4f;
+__device__ int start_steps(float rkk, float c, int p, int nev, float mu_eta) {
+    const int lane = threadIdx.x & 31;
+    const float v = lane < p ? rkk : -1.f;
+    int rank = 0;
+    for (int k = 0; k < 32; ++k) {
+        const float w = __shfl_sync(0xffffffffu, v, k);
+        rank += w > v || (w == v && k < lane) ? 1 : 0;
+    }
+    const unsigned m = __ballot_sync(0xffffffffu, rank == min(nev, p) - 1);
+    const float mu_w = fmaxf(mu_eta, __shfl_sync(0xffffffffu, v, __ffs(m) - 1));
+    const float x = 2.f * mu_w / c - 1.f;
+    if (!(c > 0.f) || !(x > 1.01f)) return 1 << 20;
+    return START_SETTLE + (int)ceilf(logf(START_GAIN) / logf(x + sqrtf(x * x - 1.f)));
 }
 
 constexpr int G32_T = 256, G32_ROWS = 64;
@@ -1185,7 +1215,9 @@ __global__ void __launch_bounds__(G32_T) k_gram_cholqr32(const float* __restrict
                                                          double* __restrict__ cheb, const int* __restrict__ n_,
                                                          const long long* __restrict__ roff_,
                                                          const int* __restrict__ p_, int gsplit,
-                                                         unsigned* __restrict__ ticket) {
+                                                         unsigned* __restrict__ ticket, int it, float mu_eta, int nev,
+                                                         int* __restrict__ sdone, int* __restrict__ sstop,
+                                                         int* __restrict__ smax) {
     __shared__ float red[G32_T][17];
     __shared__ __align__(16) float sV[G32_ROWS][PMAX + 4];
     __shared__ float G[PMAX][PMAX + 4];
@@ -1193,7 +1225,7 @@ __global__ void __launch_bounds__(G32_T) k_gram_cholqr32(const float* __restrict
     __shared__ int s_last;
     const int i = blockIdx.x, sp = blockIdx.y, t = threadIdx.x;
     const int n = n_[i], p = p_[i], q = (p + 3) / 4, qw = ldw / 4;
-    if (p == 0) return;
+    if (p == 0 || sdone[i]) return;
     const int ntile = q * (q + 1) / 2, lanes = G32_T / ntile;
     const int rows_per = (n + gsplit - 1) / gsplit;
     const int r_lo = sp * rows_per, r_hi = min(n, r_lo + rows_per);
@@ -1269,22 +1301,40 @@ __global__ void __launch_bounds__(G32_T) k_gram_cholqr32(const float* __restrict
     __syncthreads();
     if (t >= 32) return;
     float* Ci = C + (long long)i * PMAX * PMAX;
-    float rmin;
-    if (ldw <= 12) rmin = cholqr_warp<12>(G, dinv, p, Ci);
-    else if (ldw <= 16) rmin = cholqr_warp<16>(G, dinv, p, Ci);
-    else if (ldw <= 20) rmin = cholqr_warp<20>(G, dinv, p, Ci);
-    else rmin = cholqr_warp<32>(G, dinv, p, Ci);
-    if (mode == FORM_FIRST && t == 0) cheb[i] = CHEB_CUT * (double)rmin;
+    float rkk;
+    if (ldw <= 12) rkk = cholqr_warp<12>(G, dinv, p, Ci);
+    else if (ldw <= 16) rkk = cholqr_warp<16>(G, dinv, p, Ci);
+    else if (ldw <= 20) rkk = cholqr_warp<20>(G, dinv, p, Ci);
+    else rkk = cholqr_warp<32>(G, dinv, p, Ci);
+    if (mode == FORM_FIRST) {
+        float rmin = rkk;
+        for (int o = 16; o > 0; o >>= 1) rmin = fminf(rmin, __shfl_xor_sync(0xffffffffu, rmin, o));
+        const float c = (float)CHEB_CUT * rmin;
+        if (t == 0) cheb[i] = c;
+        if (it == START_SETTLE - 1) {
+            const int stop = start_stop(start_steps(rkk, c, p, nev, mu_eta));
+            if (t == 0) {
+                sstop[i] = stop;
+                atomicMax(smax, stop);
+            }
+        }
+    }
+    __syncwarp();
+    if (t == 0 && it + 1 >= sstop[i]) sdone[i] = 1;
 }
 
 // X = W C on blocks of 32 rows (FP32 products, stored as FP64): the end of
 // the start phase.  Columns >= p stay as they are.
+// X of the problems whose start phase ends after `steps` iterations (last: of
+// those that have not ended before, too)
 __global__ void __launch_bounds__(TPB) k_update32(const float* __restrict__ W, int ldw, double* __restrict__ X,
                                                   const float* __restrict__ C, const int* __restrict__ n_,
                                                   const int* __restrict__ K_, const long long* __restrict__ roff_,
-                                                  const int* __restrict__ p_, int ldx) {
+                                                  const int* __restrict__ p_, int ldx, const int* __restrict__ sstop,
+                                                  int steps, int last) {
     __shared__ float sC[PMAX][LD], sW[ROWBLK][LD];
     const int i = blockIdx.y, blk = blockIdx.x;
+    if (sstop[i] != steps && !(last && sstop[i] > steps)) return;
     const int n = n_[i], p = p_[i];
     const long long rows = (long long)K_[i] * NB;
     const int r0 = blk * ROWBLK;
@@ -1450,6 +1500,9 @@ void GevpBatch::alloc(cudaStream_t s) {
     rank.alloc(P);
     iters.alloc(P);
     n_active.alloc(2);
+    sdone.alloc(P);
+    sstop.alloc(P);
+    smax.alloc(2);
 }
 
 GevpBatch GevpBatch::slice(int p0, int np, int group) const {
@@ -1477,6 +1530,8 @@ GevpBatch GevpBatch::slice(int p0, int np, int group) const {
     v.partial = partial.view((size_t)p0 * nblk_max * 2 * PMAX, (size_t)np * nblk_max * 2 * PMAX);
     v.done = done.view(p0, np); v.m = m.view(p0, np); v.rank = rank.view(p0, np); v.iters = iters.view(p0, np);
     v.cheb = cheb.view(p0, np);
+    v.sdone = sdone.view(p0, np); v.sstop = sstop.view(p0, np);
+    v.smax = smax.view(group, 1);
     v.best = best.view(p0, np); v.best_it = best_it.view(p0, np);
     v.n_active = n_active.view(group, 1);
     v.knorm = knorm;
@@ -1494,7 +1549,7 @@ void eig_init(GevpBatch& g, unsigned long long seed, cudaStream_t s) {
     if (g.P == 0) return;
     dim3 grid(32, g.P);
     k_init<<<grid, 256, 0, s>>>(g.X.p, g.K.d_n.p, g.K.d_K.p, g.K.d_roff.p, g.d_p.p, g.ldx, seed, g.done.p, g.iters.p,
-                                g.theta.p, g.best.p, g.best_it.p);
+                                g.theta.p, g.best.p, g.best_it.p, g.sdone.p, g.sstop.p, g.smax.p);
     MSDD_LAUNCH_CHECK();
 }
 
@@ -1539,19 +1594,21 @@ void eig_start32(GevpBatch& g, float* W, cudaStream_t s) {
     MSDD_LAUNCH_CHECK();
 }
 
-void eig_cholqr32(GevpBatch& g, EigForm mode, const float* SX, const float* X, const float* Q, float* V,
-                  cudaStream_t s) {
+void eig_cholqr32(GevpBatch& g, const EigParams& ep, int it, EigForm mode, const float* SX, const float* X,
+                  const float* Q, float* V, cudaStream_t s) {
     // the FP64 Gram partials and coefficients are free in this phase and hold the FP32 ones
     k_gram_cholqr32<<<dim3(g.P, g.gsplit), G32_T, 0, s>>>(SX, X, Q, V, mode, g.ldw, reinterpret_cast<float*>(g.Hp.p),
                                                           reinterpret_cast<float*>(g.C.p), g.cheb.p, g.K.d_n.p,
-                                                          g.K.d_roff.p, g.d_p.p, g.gsplit, g.ticket.p);
+                                                          g.K.d_roff.p, g.d_p.p, g.gsplit, g.ticket.p, it,
+                                                          (float)(1.0 / (ep.eta + ep.sigma)), ep.nev_max, g.sdone.p,
+                                                          g.sstop.p, g.smax.p);
     MSDD_LAUNCH_CHECK();
 }
 
-void eig_update32(GevpBatch& g, const float* W, cudaStream_t s) {
+void eig_update32(GevpBatch& g, const float* W, int steps, bool last, cudaStream_t s) {
     dim3 grid(g.nblk_max, g.P);
     k_update32<<<grid, TPB, 0, s>>>(W, g.ldw, g.X.p, reinterpret_cast<const float*>(g.C.p), g.K.d_n.p, g.K.d_K.p,
-                                    g.K.d_roff.p, g.d_p.p, g.ldx);
+                                    g.K.d_roff.p, g.d_p.p, g.ldx, g.sstop.p, steps, last ? 1 : 0);
     MSDD_LAUNCH_CHECK();
 }
 

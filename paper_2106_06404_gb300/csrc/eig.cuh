@@ -32,6 +32,7 @@ struct GevpBatch {
     // either way, so FP32 storage halves their traffic at the same results
     DevBuf<float> W32;
     int ldw = PMAX;
+    DevBuf<int> sdone, sstop, smax;   // FP32 start phase: ended, its iterations; per group the largest of them
     DevBuf<unsigned> ticket;          // per problem: row ranges of the FP32 Gram that are done
     DevBuf<double> Q;                              // the block before X in its basis (Chebyshev recurrence)
     DevBuf<double> cheb;                           // per problem: end of the damped interval of S = K^{-1} B, 0 unknown
@@ -78,11 +79,18 @@ void eig_form_y(GevpBatch& g, double sigma, EigForm mode, cudaStream_t s);
 // FP32 start phase: W <- X in FP32; V = S X (FORM_FIRST: V is SX and the
 // damped interval is set) or the Chebyshev step of SX, X and Q (V written),
 // and C (FP32, in the buffer of g.C) with V C an orthonormal basis of span(V)
-// by Euclidean CholQR; X <- W C.
+// by Euclidean CholQR; X <- W C of the problems that end after `steps`
+// iterations (last: or later).  The first START_SETTLE iterations are power
+// steps and every eighth after them; after the settling part sstop holds each
+// problem's number of iterations, one of the stops of start_stop.
+constexpr int START_SETTLE = 6;
+__host__ __device__ inline int start_stop(int steps) {
+    return steps <= 10 ? 10 : steps <= 13 ? 13 : 1 << 20;
+}
 void eig_start32(GevpBatch& g, float* W, cudaStream_t s);
-void eig_cholqr32(GevpBatch& g, EigForm mode, const float* SX, const float* X, const float* Q, float* V,
-                  cudaStream_t s);
-void eig_update32(GevpBatch& g, const float* W, cudaStream_t s);
+void eig_cholqr32(GevpBatch& g, const EigParams& ep, int it, EigForm mode, const float* SX, const float* X,
+                  const float* Q, float* V, cudaStream_t s);
+void eig_update32(GevpBatch& g, const float* W, int steps, bool last, cudaStream_t s);
 // The same with the K^+-norm residual partial sums of X.
 void eig_form_y_knorm(GevpBatch& g, double sigma, EigForm mode, cudaStream_t s);
 // Convergence test on the K^+-norm residuals (regularised coarse pencils).

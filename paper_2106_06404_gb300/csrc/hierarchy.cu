@@ -91,7 +91,7 @@ void dense_inverse(const TileBatch& tb, double* out, const std::vector<long long
 
 // Subspace iteration driver.  apply(v, p0, X, AX, BX, skip, s) applies Abar
 // and B to the problems of batch view v (first problem p0 of the whole
-// batch), solve(v, p0, ncols, W32, s) applies K^{-1} to W32 (FP32 factors) or
+// batch), solve(v, p0, ncols, W32, skip, s) applies K^{-1} to W32 (FP32 factors) or
 // v.W, bapply32(v, p0, W, Wout, C, X, Q, s) is Wout = (B W) C in FP32, Q = X C
 // and X = W C.  `tag` names the kernel families for profiling;
 // `apply_bytes`/`apply_flops` are the algorithmic amounts of one operator
@@ -130,7 +130,8 @@ void run_eig(GevpBatch& g, const EigParams& ep, Apply apply, Solve solve, BApply
         gp0 = {0, h};
         gs = {st, st_b};
     }
-    cudaEvent_t ev_start, ev_off, ev_end;
+    cudaEvent_t ev_start, ev_off, ev_end, ev_smax[2];
+    for (cudaEvent_t& e : ev_smax) MSDD_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
     MSDD_CUDA(cudaEventCreateWithFlags(&ev_start, cudaEventDisableTiming));
     MSDD_CUDA(cudaEventCreateWithFlags(&ev_off, cudaEventDisableTiming));
     MSDD_CUDA(cudaEventCreateWithFlags(&ev_end, cudaEventDisableTiming));
@@ -159,16 +160,28 @@ void run_eig(GevpBatch& g, const EigParams& ep, Apply apply, Solve solve, BApply
     // alone decides convergence.  The damped interval comes from the last power
     // step, so the first six are power steps (the block has to settle) and
     // every eighth after them renews it: 20 such steps leave a 1400-point model
-    // spectrum 2-5 FP64 iterations, 20 power steps 9-14.
+    // spectrum 2-5 FP64 iterations, 20 power steps 9-14.  Each problem ends
+    // after the iterations that its spectrum needs (start_steps); the host
+    // reads the largest number while the iterations up to the first stop are
+    // still running.
     DevBuf<float> wb(fp32_iters > 0 ? 3 * g.W32.n : 0);
     float *vb = wb.p, *sb = g.W32.p, *xb = wb.p + g.W32.n, *qb = wb.p + 2 * g.W32.n;    // V, S X, X, Q
     auto start_mode = [](int it) {
-        const int j = (it - 6) % 8;
-        return it < 6 || j == 7 ? FORM_FIRST : j == 0 ? FORM_CHEB1 : FORM_CHEB;
+        const int j = (it - START_SETTLE) % 8;
+        return it < START_SETTLE || j == 7 ? FORM_FIRST : j == 0 ? FORM_CHEB1 : FORM_CHEB;
     };
     for (int k = 0; k < G && fp32_iters > 0; ++k) eig_start32(gv[k], vb, gs[k]);
     for (int it = 0; it < fp32_iters; ++it) {
         const EigForm mode = start_mode(it);
+        if (it == start_stop(0)) {
+            int most = 0;
+            for (int k = 0; k < G; ++k) {
+                MSDD_CUDA(cudaEventSynchronize(ev_smax[k]));
+                most = std::max(most, h_act[4 + k]);
+            }
+            fp32_iters = std::min(fp32_iters, most);
+            if (it >= fp32_iters) break;
+        }
         for (int k = 0; k < G; ++k) {
             GevpBatch& v = gv[k];
             prof.begin(tag + "_fp32_start_other", gs[k]);
@@ -176,15 +189,20 @@ void run_eig(GevpBatch& g, const EigParams& ep, Apply apply, Solve solve, BApply
                      mode == FORM_FIRST ? nullptr : xb, mode == FORM_CHEB ? qb : nullptr, gs[k]);
             prof.end(gs[k], 0.0, 0.0);
             prof.begin(tag + "_solve", gs[k]);
-            solve(v, gp0[k], am[k].pm, sb, gs[k]);
+            solve(v, gp0[k], am[k].pm, sb, (const int*)v.sdone.p, gs[k]);
             prof.end(gs[k], am[k].sb0, am[k].sf0);
             if (G == 2 && k == 0 && it == 0) {
                 MSDD_CUDA(cudaEventRecord(ev_off, gs[0]));        // the second half starts one solve later
                 MSDD_CUDA(cudaStreamWaitEvent(gs[1], ev_off, 0));
             }
             prof.begin(tag + "_fp32_start_other", gs[k]);
-            eig_cholqr32(v, mode, sb, xb, qb, vb, gs[k]);
-            if (it + 1 == fp32_iters) eig_update32(v, mode == FORM_FIRST ? sb : vb, gs[k]);
+            eig_cholqr32(v, ep, it, mode, sb, xb, qb, vb, gs[k]);
+            if (it + 1 == fp32_iters || it + 1 == start_stop(it + 1))
+                eig_update32(v, mode == FORM_FIRST ? sb : vb, it + 1, it + 1 == fp32_iters, gs[k]);
+            if (it + 1 == START_SETTLE && fp32_iters > START_SETTLE) {
+                MSDD_CUDA(cudaMemcpyAsync(&h_act[4 + k], v.smax.p, sizeof(int), cudaMemcpyDeviceToHost, gs[k]));
+                MSDD_CUDA(cudaEventRecord(ev_smax[k], gs[k]));
+            }
             prof.end(gs[k], 0.0, 0.0);
         }
         if (mode == FORM_FIRST) std::swap(vb, sb);                // V is S X itself
@@ -203,7 +221,7 @@ void run_eig(GevpBatch& g, const EigParams& ep, Apply apply, Solve solve, BApply
         const double fr = (double)active[k] / v.P;
         if (!fused || first) eig_form_rhs(v, ep.sigma, first, s);
         prof.begin(tag + "_solve", s);
-        solve(v, gp0[k], am[k].pm, v.W32.p, s);
+        solve(v, gp0[k], am[k].pm, v.W32.p, (const int*)v.done.p, s);
         prof.end(s, am[k].solve_b * fr, am[k].solve_f * fr);
         if (offset) {
             MSDD_CUDA(cudaEventRecord(ev_off, s));
@@ -285,6 +303,7 @@ void run_eig(GevpBatch& g, const EigParams& ep, Apply apply, Solve solve, BApply
         MSDD_CUDA(cudaStreamWaitEvent(st, ev_end, 0));
     }
     MSDD_CUDA(cudaStreamSynchronize(st));
+    for (cudaEvent_t& e : ev_smax) cudaEventDestroy(e);
     cudaEventDestroy(ev_start);
     cudaEventDestroy(ev_off);
     cudaEventDestroy(ev_end);
@@ -610,12 +629,12 @@ void Hierarchy::build_fine() {
             [=](GevpBatch& v, int p0, const double* X, double* AX, double* BX, const int* skip, cudaStream_t s) {
                 apply_local(*ls, bx + p0, dim, v.K, X, AX, BX, v.ldx, block_p, skip, s);
             },
-            [=](GevpBatch& v, int, int pmax, float* W32, cudaStream_t s) {
-                if (v.K.prec) tile_solve(v.K, W32, v.ldw, pmax, v.done.p, s);
-                else tile_solve(v.K, v.W.p, v.ldw, pmax, v.done.p, s);
+            [=](GevpBatch& v, int, int pmax, float* W32, const int* skip, cudaStream_t s) {
+                if (v.K.prec) tile_solve(v.K, W32, v.ldw, pmax, skip, s);
+                else tile_solve(v.K, v.W.p, v.ldw, pmax, skip, s);
             },
             [=](GevpBatch& v, int p0, const float* W, float* Wout, const float* C, float* X, float* Q, cudaStream_t s) {
-                apply_local_b32(*ls, bx + p0, dim, v.K, W, Wout, v.ldw, C, X, Q, s);
+                apply_local_b32(*ls, bx + p0, dim, v.K, W, Wout, v.ldw, C, X, Q, v.sdone.p, s);
             },
             [=](GevpBatch& v, int p0, cudaStream_t s) {
                 apply_local_rhs(*ls, bx + p0, dim, v.K, v.X.p, v.W.p, v.W32.p, v.ldw, v.ldx, v.d_p.p, v.theta.p, ep.sigma,
@@ -999,7 +1018,7 @@ void Hierarchy::build_coarse() {
                     apply_dense_pencil(Ab, dao + p0, dng + p0, dno + p0, v.K, X, AX, BX, v.ldx, block_p, skip, v.P,
                                        ngen_max, s);
                 },
-                [=](GevpBatch& v, int p0, int, float*, cudaStream_t s) {
+                [=](GevpBatch& v, int p0, int, float*, const int*, cudaStream_t s) {
                     gemm_batched(dki + p0, v.P, 0, 0, 1.0, Kinv, v.W.p, 0.0, Wtp, ngen_max, pmax_m, s, nullptr,
                                  v.done.p);
                     const long long e0 = mrow[p0], e1 = mrow[p0 + v.P];

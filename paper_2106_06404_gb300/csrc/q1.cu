@@ -528,11 +528,12 @@ __global__ void __launch_bounds__(256) k_b32_cholqr(const ProbBox* __restrict__ 
                                                     const long long* __restrict__ roff_, const int* __restrict__ K_,
                                                     const float* __restrict__ B32, const float* __restrict__ W,
                                                     float* __restrict__ Wout, int ldw, const float* __restrict__ C,
-                                                    float* __restrict__ X, float* __restrict__ Q) {
+                                                    float* __restrict__ X, float* __restrict__ Q,
+                                                    const int* __restrict__ skip) {
     constexpr int NOFF = D == 3 ? 27 : 9;
     __shared__ __align__(16) float sC[PMAX][PMAX], sT[3][NB][PMAX + 4];
     const int i = blockIdx.y, r0 = blockIdx.x * NB;
-    if (r0 >= K_[i] * NB) return;
+    if (r0 >= K_[i] * NB || skip[i]) return;
     const ProbBox pb = boxes[i];
     const int n = box_size(pb.nlo, pb.nhi, D);
     const int w0 = pb.nhi[0] - pb.nlo[0] + 1, w1 = pb.nhi[1] - pb.nlo[1] + 1;
@@ -780,15 +781,16 @@ void apply_local_rhs(const LocalStencil& ls, const ProbBox* d_boxes, int dim, co
 }
 
 void apply_local_b32(const LocalStencil& ls, const ProbBox* d_boxes, int dim, const TileBatch& layout,
-                     const float* W, float* Wout, int ldw, const float* C, float* X, float* Q, cudaStream_t s) {
+                     const float* W, float* Wout, int ldw, const float* C, float* X, float* Q,
+                     const int* skip, cudaStream_t s) {
     if (layout.P == 0) return;
     const dim3 grid(layout.max_K, layout.P), block(ldw / 4, NB);
     if (dim == 3)
         k_b32_cholqr<3><<<grid, block, 0, s>>>(d_boxes, layout.d_roff.p, layout.d_K.p, ls.b32.p, W, Wout, ldw, C,
-                                              X, Q);
+                                              X, Q, skip);
     else
         k_b32_cholqr<2><<<grid, block, 0, s>>>(d_boxes, layout.d_roff.p, layout.d_K.p, ls.b32.p, W, Wout, ldw, C,
-                                              X, Q);
+                                              X, Q, skip);
     MSDD_LAUNCH_CHECK();
 }
 

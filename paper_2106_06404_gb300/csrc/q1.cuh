@@ -126,9 +126,10 @@ void apply_local_rhs(const LocalStencil& ls, const ProbBox* d_boxes, int dim, co
 // Wout = (B W) C in FP32 arithmetic from b32 (blocks of ldw columns, a multiple
 // of 4; zero on padding rows); C is PMAX x PMAX per problem and upper
 // triangular, null for the identity.  With C: X (may be null) <- W C, and
-// before that Q (may be null) <- X C.
+// before that Q (may be null) <- X C.  Problems with skip != 0 are left alone.
 void apply_local_b32(const LocalStencil& ls, const ProbBox* d_boxes, int dim, const TileBatch& layout,
-                     const float* W, float* Wout, int ldw, const float* C, float* X, float* Q, cudaStream_t s);
+                     const float* W, float* Wout, int ldw, const float* C, float* X, float* Q,
+                     const int* skip, cudaStream_t s);
 
 // Stored 3^d-point stencil of the global operator: S[o * n + u] = A(u, u + o),
 // offsets o lexicographic (x fastest) in {-1, 0, 1}^d, zero where u + o is
