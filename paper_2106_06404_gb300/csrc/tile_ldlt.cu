@@ -283,15 +283,19 @@ __global__ void __launch_bounds__(TPB) k_tile_solve(
 // rows contiguously across the warp, partial sums of the 4 warps are combined
 // in shared memory.  For band matrices (kb <= KBP) the tiles of step R+1 are
 // loaded into registers while step R computes.
-// ------------------------------------------------------------------ factor, dense, right-looking
-// Dense batches (kb >= K - 1: coarse-level matrices) are factored one tile
+// ------------------------------------------------------------------ factor, right-looking
+// Dense batches (coarse-level matrices) and FP64 bands are factored one tile
 // column k per launch triple, so that many CTAs share each step instead of
 // one CTA per matrix: the diagonal tile (one CTA per problem), the panel
 // L_ik = A_ik T_k^T D_k^{-1} (one CTA per tile), and the trailing update
-// A_ij -= L_ik D_k L_jk^T for k < j <= i (one CTA per tile).  Every tile sees
-// the subtractions of k_tile_factor in the same order and in the same
-// precision, so the factors are the same.  k_save_diag first parks the
-// original diagonal (the null-pivot reference) in dinv and clears the status.
+// A_ij -= L_ik D_k L_jk^T for k < j <= i <= k + kb (one CTA per tile).  In
+// FP64 the pipe bounds the panel and the update, so both skip the zeros: T_k
+// is lower triangular, and columns below 32 (i - k) - b of tile (i, k) lie
+// outside the band.  k_save_diag first parks the original diagonal (the
+// null-pivot reference) in dinv and clears the status.
+// Measured (GB300, Dirichlet and Neumann batches side by side): 27 FP64
+// matrices of n = 1452..1872, b = 133..157 17.1 -> 4.5 ms a factorisation
+// against one CTA per matrix, 144 of n ~ 1300, b = 36 6.0 -> 3.7 ms.
 template <typename T>
 __global__ void __launch_bounds__(TPB) k_save_diag(const T* __restrict__ tiles, T* __restrict__ dinv,
                                                    const int* __restrict__ kb_, const int* __restrict__ K_,
@@ -308,96 +312,156 @@ __global__ void __launch_bounds__(TPB) k_save_diag(const T* __restrict__ tiles, 
     if (threadIdx.x == 0) { status[i] = 0; nreg[i] = 0; }
 }
 
+// LDL^T of the diagonal tile and T = L^{-1} in one elimination of [A | I]:
+// lane = row, warp w holds columns w + 4 j of both in registers.  Step k: the
+// warp that owns column k publishes it and the reciprocal pivot (shared
+// memory, one barrier); with m_a = A_ak / d_k, entry (a, b) of A takes off
+// A_ak m_b (columns b > k, m_b by shuffle from lane b) and of T m_a T_kb
+// (columns b <= k, T_kb by shuffle from lane k).  The 32 pivots are the chain (a division, a barrier and
+// about eight FP64 operations of every warp each), so one barrier a pivot
+// instead of three, and the inverse in the same pass instead of a second one.
 template <typename T>
-__global__ void __launch_bounds__(TPB) k_rl_diag(T* __restrict__ tiles, T* __restrict__ dinv,
+__global__ void __launch_bounds__(128) k_rl_diag(T* __restrict__ tiles, T* __restrict__ dinv,
                                                  const int* __restrict__ n_, const int* __restrict__ kb_,
                                                  const int* __restrict__ K_, const long long* __restrict__ toff_,
                                                  const long long* __restrict__ roff_, int* __restrict__ status,
-                                                 int* __restrict__ nreg, double reg_tol, int k) {
-    __shared__ T W[NB][LDS];
-    __shared__ T Sa[NB][LDS];
-    __shared__ T sd[NB];
-    __shared__ T od[NB];
-    __shared__ T piv_inv;
+                                                 int* __restrict__ nreg, double reg_tol, int k0) {
+    __shared__ T S[NB][LDS];
+    __shared__ T col[2][NB], piv[2], sd[NB], od[NB];
     __shared__ int s_status, s_nreg;
     const int i = blockIdx.x;
-    const int K = K_[i];
-    if (k >= K) return;
-    const int kb = kb_[i], t = threadIdx.x;
-    const long long toff = toff_[i], roff = roff_[i];
+    if (k0 >= K_[i]) return;
+    const int kb = kb_[i], t = threadIdx.x, a = t & 31, w = t >> 5;
+    T* tile = tiles + tile_index(toff_[i], kb, k0, k0);
+    T* dv = dinv + roff_[i] + (long long)k0 * NB;
+    const int valid = n_[i] - k0 * NB;                 // rows from here on are padding
     if (t == 0) { s_status = status[i]; s_nreg = nreg[i]; }
-    load_tile(W, tiles + tile_index(toff, kb, k, k));
-    if (t < NB) od[t] = dinv[roff + (long long)k * NB + t];
+    for (int e = t; e < NB2; e += 128) S[e / NB][e % NB] = tile[e];
+    if (t < NB) od[t] = dv[t];
     __syncthreads();
-    factor_diag_tile<T>(W, Sa, sd, od, piv_inv, n_[i] - k * NB, reg_tol, k, s_status, s_nreg,
-                        tiles + tile_index(toff, kb, k, k), dinv + roff + (long long)k * NB);
+    T A[NB / 4], L[NB / 4];
+#pragma unroll
+    for (int j = 0; j < NB / 4; ++j) {
+        const int b = w + 4 * j;
+        A[j] = S[a][b];
+        L[j] = a == b ? T(1) : T(0);
+    }
+#pragma unroll
+    for (int k = 0; k < NB; ++k) {
+        const int buf = k & 1;
+        if (w == (k & 3)) {
+            const T v = A[k >> 2];
+            col[buf][a] = v;
+            if (a == k) {
+                T r;
+                if (k >= valid) r = T(1);
+                else if (reg_tol > 0.0 && !(v > T(reg_tol) * od[k])) { r = T(0); ++s_nreg; }
+                else if (!(v > T(0))) { r = T(0); if (s_status == 0) s_status = k0 * NB + k + 1; }
+                else r = T(1) / v;
+                piv[buf] = r;
+                sd[k] = r;
+            }
+        }
+        __syncthreads();
+        const T m = a > k && a < valid && k < valid ? col[buf][a] * piv[buf] : T(0);
+#pragma unroll
+        for (int j = 0; j < NB / 4; ++j) {
+            const int b = w + 4 * j;                   // (the same side of k for the whole warp)
+            if (4 * j + 3 > k && b > k) A[j] -= col[buf][a] * __shfl_sync(0xffffffffu, m, b);
+            if (4 * j <= k && b <= k) L[j] -= m * __shfl_sync(0xffffffffu, L[j], k);
+        }
+    }
     __syncthreads();
+#pragma unroll
+    for (int j = 0; j < NB / 4; ++j) S[a][w + 4 * j] = L[j];
+    __syncthreads();
+    for (int e = t; e < NB2; e += 128) tile[e] = S[e / NB][e % NB];
+    if (t < NB) dv[t] = sd[t];
     if (t == 0) { status[i] = s_status; nreg[i] = s_nreg; }
 }
 
-// grid.y: i = k + 1 + blockIdx.y
+// grid.y: tile row k + 1 + blockIdx.y
 template <typename T>
 __global__ void __launch_bounds__(TPB) k_rl_panel(T* __restrict__ tiles, const T* __restrict__ dinv,
                                                   const int* __restrict__ kb_, const int* __restrict__ K_,
-                                                  const long long* __restrict__ toff_,
+                                                  const int* __restrict__ b_, const long long* __restrict__ toff_,
                                                   const long long* __restrict__ roff_, int k) {
     __shared__ T W[NB][LDS];
     __shared__ T Sb[NB][LDS];
     __shared__ T sd[NB];
-    const int i = blockIdx.x, R = k + 1 + blockIdx.y;
-    const int K = K_[i];
-    if (R >= K) return;
-    const int kb = kb_[i], t = threadIdx.x, r = t >> 3, c0 = t & 7;
+    const int i = blockIdx.x, d = 1 + blockIdx.y, R = k + d;
+    const int kb = kb_[i];
+    if (R >= K_[i] || d > kb) return;
+    const int t = threadIdx.x, r = t >> 3, c0 = t & 7;
     const long long toff = toff_[i], roff = roff_[i];
     T* dst = tiles + tile_index(toff, kb, R, k);
     load_tile(W, dst);
     load_tile(Sb, tiles + tile_index(toff, kb, k, k));
     if (t < NB) sd[t] = dinv[roff + (long long)k * NB + t];
     __syncthreads();
+    const int kk0 = max(0, NB * d - b_[i]) & ~7;       // columns of A_Rk before it are zero
     T out[4] = {0, 0, 0, 0};
-#pragma unroll 8
-    for (int kk = 0; kk < NB; ++kk) {
-        T w = W[r][kk];
 #pragma unroll
-        for (int q = 0; q < 4; ++q) out[q] += w * Sb[c0 + 8 * q][kk];
+    for (int g = 0; g < 4; ++g) {                      // columns 8 g .. 8 g + 7 of A reach the rows >= 8 g of T
+        if (8 * g < kk0) continue;
+#pragma unroll
+        for (int kk = 8 * g; kk < 8 * g + 8; ++kk) {
+            const T w = W[r][kk];
+#pragma unroll
+            for (int q = g; q < 4; ++q) out[q] += w * Sb[c0 + 8 * q][kk];
+        }
     }
 #pragma unroll
     for (int q = 0; q < 4; ++q) dst[r * NB + c0 + 8 * q] = out[q] * sd[c0 + 8 * q];
 }
 
-// grid.y enumerates the tiles (i, j), k < j <= i < K, row by row
+// grid.y enumerates the tiles (R, C), k < C <= R <= k + kb, row by row
 template <typename T>
 __global__ void __launch_bounds__(TPB) k_rl_update(T* __restrict__ tiles, const T* __restrict__ dinv,
                                                    const int* __restrict__ kb_, const int* __restrict__ K_,
-                                                   const long long* __restrict__ toff_,
+                                                   const int* __restrict__ b_, const long long* __restrict__ toff_,
                                                    const long long* __restrict__ roff_, int k) {
     __shared__ T Sa[NB][LDS];
     __shared__ T Sb[NB][LDS];
     __shared__ T sd[NB];
     const int i = blockIdx.x;
-    const int K = K_[i];
+    const int K = K_[i], kb = kb_[i];
     int e = blockIdx.y, R = k + 1;
     while (R < K && e >= R - k) { e -= R - k; ++R; }
-    if (R >= K) return;
+    if (R >= K || R - k > kb) return;
     const int C = k + 1 + e;
-    const int kb = kb_[i], t = threadIdx.x, r = t >> 3, c0 = t & 7;
+    const int t = threadIdx.x, r = t >> 3, c0 = t & 7;
     const long long toff = toff_[i], roff = roff_[i];
     T* dst = tiles + tile_index(toff, kb, R, C);
     T acc[4];
 #pragma unroll
     for (int q = 0; q < 4; ++q) acc[q] = dst[r * NB + c0 + 8 * q];
-    load_tile(Sa, tiles + tile_index(toff, kb, R, k));
-    load_tile(Sb, tiles + tile_index(toff, kb, C, k));
     if (t < NB) {
         T di = dinv[roff + (long long)k * NB + t];
         sd[t] = di != T(0) ? T(1) / di : T(0);
     }
+    load_tile(Sa, tiles + tile_index(toff, kb, R, k));
+    const T* lb = tiles + tile_index(toff, kb, C, k);
     __syncthreads();
-#pragma unroll 8
-    for (int kk = 0; kk < NB; ++kk) {
-        T a = Sa[r][kk] * sd[kk];
+    for (int x = t; x < NB2; x += TPB) Sb[x / NB][x % NB] = lb[x] * sd[x % NB];   // L_Ck D_k
+    __syncthreads();
+    const int kk0 = max(0, NB * (R - k) - b_[i]);      // columns of L_Rk before it are zero
+    // a warp has rows r .. r + 3; of a diagonal tile the column groups beyond them are not stored
+    const int nq = R == C ? (4 * (t >> 5) + 3) / 8 + 1 : 4;
+    if (nq == 4) {
+#pragma unroll 4
+        for (int kk = kk0; kk < NB; ++kk) {
+            const T a = Sa[r][kk];
 #pragma unroll
-        for (int q = 0; q < 4; ++q) acc[q] -= a * Sb[c0 + 8 * q][kk];
+            for (int q = 0; q < 4; ++q) acc[q] -= a * Sb[c0 + 8 * q][kk];
+        }
+    } else {
+        for (int kk = kk0; kk < NB; ++kk) {
+            const T a = Sa[r][kk];
+            acc[0] -= a * Sb[c0][kk];
+            if (nq > 1) acc[1] -= a * Sb[c0 + 8][kk];
+            if (nq > 2) acc[2] -= a * Sb[c0 + 16][kk];
+        }
     }
 #pragma unroll
     for (int q = 0; q < 4; ++q) dst[r * NB + c0 + 8 * q] = acc[q];
@@ -1958,22 +2022,23 @@ void tile_factor(TileBatch& tb, double reg_tol, cudaStream_t s) {
     for (int v : tb.kb) maxkb = std::max(maxkb, v);
     bool dense = tb.max_K >= 3;
     for (int i = 0; i < tb.P && dense; ++i) dense = tb.kb[i] >= tb.K[i] - 1;
-    if (dense) {
+    if (dense || !tb.prec) {
         auto run = [&](auto* tl, auto* dv) {
             using T = std::remove_pointer_t<decltype(tl)>;
             k_save_diag<T><<<tb.P, TPB, 0, s>>>(tl, dv, tb.d_kb.p, tb.d_K.p, tb.d_toff.p, tb.d_roff.p, tb.d_status.p,
                                                tb.d_nreg.p);
             MSDD_LAUNCH_CHECK();
             for (int k = 0; k < tb.max_K; ++k) {
-                k_rl_diag<T><<<tb.P, TPB, 0, s>>>(tl, dv, tb.d_n.p, tb.d_kb.p, tb.d_K.p, tb.d_toff.p, tb.d_roff.p,
+                k_rl_diag<T><<<tb.P, 128, 0, s>>>(tl, dv, tb.d_n.p, tb.d_kb.p, tb.d_K.p, tb.d_toff.p, tb.d_roff.p,
                                                  tb.d_status.p, tb.d_nreg.p, reg_tol, k);
                 MSDD_LAUNCH_CHECK();
-                const int m = tb.max_K - 1 - k;
-                if (m == 0) break;
-                k_rl_panel<T><<<dim3(tb.P, m), TPB, 0, s>>>(tl, dv, tb.d_kb.p, tb.d_K.p, tb.d_toff.p, tb.d_roff.p, k);
+                const int m = std::min(maxkb, tb.max_K - 1 - k);
+                if (m == 0) continue;
+                k_rl_panel<T><<<dim3(tb.P, m), TPB, 0, s>>>(tl, dv, tb.d_kb.p, tb.d_K.p, tb.d_b.p, tb.d_toff.p,
+                                                           tb.d_roff.p, k);
                 MSDD_LAUNCH_CHECK();
-                k_rl_update<T><<<dim3(tb.P, m * (m + 1) / 2), TPB, 0, s>>>(tl, dv, tb.d_kb.p, tb.d_K.p, tb.d_toff.p,
-                                                                         tb.d_roff.p, k);
+                k_rl_update<T><<<dim3(tb.P, m * (m + 1) / 2), TPB, 0, s>>>(tl, dv, tb.d_kb.p, tb.d_K.p, tb.d_b.p,
+                                                                         tb.d_toff.p, tb.d_roff.p, k);
                 MSDD_LAUNCH_CHECK();
             }
         };
@@ -2004,12 +2069,8 @@ void tile_factor(TileBatch& tb, double reg_tol, cudaStream_t s) {
             return;
         }
     }
-    if (tb.prec)
-        k_tile_factor<float><<<tb.P, TPB, 0, s>>>(tb.tiles_f.p, tb.dinv_f.p, tb.d_n.p, tb.d_kb.p, tb.d_K.p,
-                                                 tb.d_toff.p, tb.d_roff.p, tb.d_status.p, tb.d_nreg.p, reg_tol);
-    else
-        k_tile_factor<double><<<tb.P, TPB, 0, s>>>(tb.tiles_d.p, tb.dinv_d.p, tb.d_n.p, tb.d_kb.p, tb.d_K.p,
-                                                  tb.d_toff.p, tb.d_roff.p, tb.d_status.p, tb.d_nreg.p, reg_tol);
+    k_tile_factor<float><<<tb.P, TPB, 0, s>>>(tb.tiles_f.p, tb.dinv_f.p, tb.d_n.p, tb.d_kb.p, tb.d_K.p, tb.d_toff.p,
+                                             tb.d_roff.p, tb.d_status.p, tb.d_nreg.p, reg_tol);
     MSDD_LAUNCH_CHECK();
 }
 
