@@ -6,8 +6,6 @@ namespace msdd {
 
 namespace {
 
-constexpr int COMBINE_NT = 1024;
-
 __global__ void k_block_sum(const SumItem* __restrict__ items, const long long* __restrict__ contrib,
                             const double* __restrict__ G, double* __restrict__ dst) {
     const SumItem it = items[blockIdx.x];
@@ -116,64 +114,88 @@ __global__ void k_dense_shift(const double* __restrict__ A, double* __restrict__
     }
 }
 
-// One CTA of 512 threads per fine subdomain; templated on the dimension so
-// that node coordinates and box bounds stay in registers.
+// global unknown of row rr of a Dirichlet box (rr < box size)
 template <int D>
-__global__ void __launch_bounds__(512) k_fine_gather_restrict(
-    Geom g, const ProbBox* __restrict__ fine, const long long* __restrict__ droff, const int* __restrict__ dK,
-    const double* __restrict__ r, double* __restrict__ rhs, const double* __restrict__ Phi,
-    const long long* __restrict__ phioff, int ldphi, const int* __restrict__ m_, const long long* __restrict__ c1off,
-    double* __restrict__ r1, const int* __restrict__ done) {
-    __shared__ double red[PMAX][16];
-    if (done && *done) return;
-    const int j = blockIdx.x;
-    int dlo[3], wd[3];
-    int n = 1;
+__device__ __forceinline__ int dirichlet_unknown(const Geom& g, const int* dlo, const int* wd, int rr) {
+    int u = 0, stride = 1;
 #pragma unroll
-    for (int d = 0; d < 3; ++d) {
-        dlo[d] = d < D ? fine[j].dlo[d] : 0;
-        const int hi = d < D ? fine[j].dhi[d] : 0;
-        wd[d] = hi >= dlo[d] ? hi - dlo[d] + 1 : 0;
-        if (d < D) n *= wd[d];
+    for (int d = 0; d < D; ++d) {
+        const int q = d + 1 < D ? rr / wd[d] : 0;
+        const int x = d + 1 < D ? rr - q * wd[d] : rr;
+        u += (dlo[d] + x - g.ulo[d]) * stride;
+        stride *= g.ushape[d];
+        rr = q;
+    }
+    return u;
+}
+
+// rhs_j = r on the Dirichlet box of j, zero on padding rows
+template <int D>
+__global__ void __launch_bounds__(256) k_fine_gather(Geom g, const ProbBox* __restrict__ fine,
+                                                     const long long* __restrict__ droff, const int* __restrict__ dK,
+                                                     const double* __restrict__ r, double* __restrict__ rhs,
+                                                     const int* __restrict__ done) {
+    if (done && *done) return;
+    const int j = blockIdx.y;
+    int dlo[D], wd[D], n = 1;
+#pragma unroll
+    for (int d = 0; d < D; ++d) {
+        dlo[d] = fine[j].dlo[d];
+        wd[d] = fine[j].dhi[d] - dlo[d] + 1;
+        n *= wd[d];
     }
     const int rows = dK[j] * NB;
-    const int m = m_[j];
-    const int t = threadIdx.x;
-    const int lane = t & 31, warp = t >> 5;
-    double acc[PMAX];
+    for (int rr = blockIdx.x * 256 + threadIdx.x; rr < rows; rr += gridDim.x * 256)
+        rhs[droff[j] + rr] = rr < n ? r[dirichlet_unknown<D>(g, dlo, wd, rr)] : 0.0;
+}
+
+// r1[c1off_j + k] = Phi_j^T r on the box of j: one CTA per fine subdomain,
+// neighbouring threads on neighbouring entries of Phi (thread = column
+// t % ldphi of every (512 / ldphi)-th row), so that Phi is read in whole lines
+// and no FP64 shuffle sums are needed: the row lanes are summed in shared
+// memory.  (A row per thread with a shuffle tree per column took 41 us at
+// 512^2 together with the gather; FP64 pipe and strided reads.)
+constexpr int FR_T = 512;
+template <int D>
+__global__ void __launch_bounds__(FR_T) k_fine_restrict(Geom g, const ProbBox* __restrict__ fine,
+                                                        const double* __restrict__ r, const double* __restrict__ Phi,
+                                                        const long long* __restrict__ phioff, int ldphi,
+                                                        const int* __restrict__ m_, const long long* __restrict__ c1off,
+                                                        double* __restrict__ r1, const int* __restrict__ done) {
+    __shared__ double red[FR_T];
+    if (done && *done) return;
+    const int j = blockIdx.x;
+    int dlo[D], wd[D], n = 1;
 #pragma unroll
-    for (int k = 0; k < PMAX; ++k) acc[k] = 0.0;
-    for (int rr = t; rr < rows; rr += blockDim.x) {
-        double v = 0.0;
-        if (rr < n) {
-            int rem = rr;
-            long long u = 0, stride = 1;
-#pragma unroll
-            for (int d = 0; d < D; ++d) {
-                const int xd = dlo[d] + rem % wd[d];
-                rem /= wd[d];
-                u += (xd - g.ulo[d]) * stride;
-                stride *= g.ushape[d];
-            }
-            v = r[u];
-            const double* ph = Phi + phioff[j] + (long long)rr * ldphi;
-#pragma unroll
-            for (int k = 0; k < PMAX; ++k)
-                if (k < m) acc[k] += ph[k] * v;
+    for (int d = 0; d < D; ++d) {
+        dlo[d] = fine[j].dlo[d];
+        wd[d] = fine[j].dhi[d] - dlo[d] + 1;
+        n *= wd[d];
+    }
+    const int m = m_[j], t = threadIdx.x, k = t % ldphi, rl = t / ldphi, lanes = FR_T / ldphi;
+    double a0 = 0.0, a1 = 0.0;
+    if (k < m && rl < lanes) {
+        const double* ph = Phi + phioff[j] + k;
+        int rr = rl;
+        for (; rr + lanes < n; rr += 2 * lanes) {
+            a0 = fma(ph[(long long)rr * ldphi], r[dirichlet_unknown<D>(g, dlo, wd, rr)], a0);
+            a1 = fma(ph[(long long)(rr + lanes) * ldphi], r[dirichlet_unknown<D>(g, dlo, wd, rr + lanes)], a1);
         }
-        rhs[droff[j] + rr] = v;
+        if (rr < n) a0 = fma(ph[(long long)rr * ldphi], r[dirichlet_unknown<D>(g, dlo, wd, rr)], a0);
     }
-#pragma unroll
-    for (int k = 0; k < PMAX; ++k) {
-        if (k >= m) break;
-        double v = acc[k];
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        if (lane == 0) red[k][warp] = v;
-    }
+    red[t] = a0 + a1;
+    __syncthreads();
+    // eight partial sums per column, then one
+    const int g8 = t / ldphi;
+    double s = 0.0;
+    if (k < m && g8 < 8)
+        for (int l = g8; l < lanes; l += 8) s += red[l * ldphi + k];
+    __syncthreads();
+    if (k < m && g8 < 8) red[g8 * ldphi + k] = s;
     __syncthreads();
     if (t < m) {
         double v = 0.0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) v += red[t][w];
+        for (int l = 0; l < min(8, lanes); ++l) v += red[l * ldphi + t];
         r1[c1off[j] + t] = v;
     }
 }
@@ -183,13 +205,13 @@ __global__ void __launch_bounds__(512) k_fine_gather_restrict(
 // subdomains' box bounds stay in registers.  32-bit coordinate divisions
 // (the set-up rejects 2^31 unknowns or more).
 template <int D>
-__global__ void __launch_bounds__(COMBINE_NT, 1) k_fine_combine(
+__global__ void __launch_bounds__(PCG_NT) k_fine_combine(
     Geom g, CombineMaps cm, const ProbBox* __restrict__ fine, const long long* __restrict__ droff,
     const double* __restrict__ y, const double* __restrict__ Phi, const long long* __restrict__ phioff, int ldphi,
     const int* __restrict__ m_, const long long* __restrict__ c1off, const double* __restrict__ z1,
     double* __restrict__ z, const double* __restrict__ r, double* __restrict__ partial, long long nun,
     const int* __restrict__ done, int mode, PcgScalars* sc, int fin) {
-    __shared__ double red[COMBINE_NT];
+    __shared__ double red[PCG_NT];
     if (done && *done) return;
     double part = 0.0;
     for (long long u = blockIdx.x * (long long)blockDim.x + threadIdx.x; u < nun; u += (long long)gridDim.x * blockDim.x) {
@@ -222,7 +244,16 @@ __global__ void __launch_bounds__(COMBINE_NT, 1) k_fine_combine(
                         const int m = m_[j];
                         const double* ph = Phi + phioff[j] + (long long)loc * ldphi;
                         const double* zz = z1 + c1off[j];
-                        for (int k = 0; k < m; ++k) v += ph[k] * zz[k];
+                        // pairs: Phi rows start on 16 bytes (ldphi is even)
+                        double v1 = 0.0;
+                        int k = 0;
+                        for (; k + 1 < m; k += 2) {
+                            const double2 a = *reinterpret_cast<const double2*>(ph + k);
+                            v = fma(a.x, zz[k], v);
+                            v1 = fma(a.y, zz[k + 1], v1);
+                        }
+                        if (k < m) v = fma(ph[k], zz[k], v);
+                        v += v1;
                     }
                     acc += v;
                     ++ncov;
@@ -234,14 +265,9 @@ __global__ void __launch_bounds__(COMBINE_NT, 1) k_fine_combine(
         if (partial) part += acc * r[u];
     }
     if (!partial) return;
-    red[threadIdx.x] = part;
-    __syncthreads();
-    for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-        if (threadIdx.x < s) red[threadIdx.x] += red[threadIdx.x + s];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) partial[blockIdx.x] = red[0];
-    if (sc) pcg_last_block(sc, fin, partial);
+    part = pcg_block_sum(part, red);
+    if (threadIdx.x == 0) partial[blockIdx.x] = part;
+    if (sc) pcg_last_block(sc, fin, partial, red);
 }
 
 __global__ void k_segment_copy(const long long* __restrict__ so, const long long* __restrict__ dof,
@@ -296,17 +322,23 @@ void gemm_batched(const GemmItem* d_items, int nitems, int transA, int transB, d
     MSDD_LAUNCH_CHECK();
 }
 
-void fine_gather_restrict(const Geom& g, const ProbBox* d_fine, const long long* d_droff, const int* d_K,
-                          const double* r, double* rhs, const double* Phi, const long long* d_phioff, int ldphi,
-                          const int* d_m, const long long* d_c1off, double* r1, int P, const int* done,
-                          cudaStream_t s) {
+void fine_gather(const Geom& g, const ProbBox* d_fine, const long long* d_droff, const int* d_K, int max_K,
+                 const double* r, double* rhs, int P, const int* done, cudaStream_t s) {
+    if (P == 0) return;
+    const dim3 grid(ceil_div((long long)max_K * NB, 256), P);
+    if (g.dim == 3) k_fine_gather<3><<<grid, 256, 0, s>>>(g, d_fine, d_droff, d_K, r, rhs, done);
+    else k_fine_gather<2><<<grid, 256, 0, s>>>(g, d_fine, d_droff, d_K, r, rhs, done);
+    MSDD_LAUNCH_CHECK();
+}
+
+void fine_restrict(const Geom& g, const ProbBox* d_fine, const double* r, const double* Phi, const long long* d_phioff,
+                   int ldphi, const int* d_m, const long long* d_c1off, double* r1, int P, const int* done,
+                   cudaStream_t s) {
     if (P == 0) return;
     if (g.dim == 3)
-        k_fine_gather_restrict<3><<<P, 512, 0, s>>>(g, d_fine, d_droff, d_K, r, rhs, Phi, d_phioff, ldphi, d_m, d_c1off, r1,
-                                             done);
+        k_fine_restrict<3><<<P, FR_T, 0, s>>>(g, d_fine, r, Phi, d_phioff, ldphi, d_m, d_c1off, r1, done);
     else
-        k_fine_gather_restrict<2><<<P, 512, 0, s>>>(g, d_fine, d_droff, d_K, r, rhs, Phi, d_phioff, ldphi, d_m, d_c1off, r1,
-                                             done);
+        k_fine_restrict<2><<<P, FR_T, 0, s>>>(g, d_fine, r, Phi, d_phioff, ldphi, d_m, d_c1off, r1, done);
     MSDD_LAUNCH_CHECK();
 }
 
@@ -325,10 +357,10 @@ void fine_combine_mode(const Geom& g, const CombineMaps& cm, const ProbBox* d_fi
     long long nun = (long long)g.ushape[0] * g.ushape[1] * (g.dim == 3 ? g.ushape[2] : 1);
     if (!partial) sc = nullptr;                      // no partials, nothing to finish
     if (g.dim == 3)
-        k_fine_combine<3><<<nblocks, COMBINE_NT, 0, s>>>(g, cm, d_fine, d_droff, y, Phi, d_phioff, ldphi, d_m, d_c1off,
+        k_fine_combine<3><<<nblocks, PCG_NT, 0, s>>>(g, cm, d_fine, d_droff, y, Phi, d_phioff, ldphi, d_m, d_c1off,
                                                          z1, z, r, partial, nun, done, mode, sc, fin);
     else
-        k_fine_combine<2><<<nblocks, COMBINE_NT, 0, s>>>(g, cm, d_fine, d_droff, y, Phi, d_phioff, ldphi, d_m, d_c1off,
+        k_fine_combine<2><<<nblocks, PCG_NT, 0, s>>>(g, cm, d_fine, d_droff, y, Phi, d_phioff, ldphi, d_m, d_c1off,
                                                          z1, z, r, partial, nun, done, mode, sc, fin);
     MSDD_LAUNCH_CHECK();
 }
@@ -341,7 +373,8 @@ void segment_copy(const long long* d_src_off, const long long* d_dst_off, const 
     MSDD_LAUNCH_CHECK();
 }
 
-int dot_blocks(long long n) { return (int)std::max(1u, std::min(ceil_div(n, 1024), 152u * 4)); }
+// one unknown a thread up to eight blocks an SM
+int dot_blocks(long long n) { return (int)std::max(1u, std::min(ceil_div(n, PCG_NT), 152u * 8)); }
 
 void dot_partial(const double* x, const double* y, long long n, double* partial, int nblocks, cudaStream_t s) {
     k_dot_partial<<<nblocks, 256, 0, s>>>(x, y, n, partial);

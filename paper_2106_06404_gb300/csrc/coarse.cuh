@@ -40,12 +40,14 @@ void dense_shift(const double* Abar, double* Kd, const long long* d_aoff, const 
                  double sigma, int P, int nmax, cudaStream_t s);
 
 // ---- preconditioner / CG vector kernels
-// Fine Dirichlet gather and coarse restriction: rhs_j = r on the Dirichlet box
-// of j (solve-buffer layout), r1[c1off_j + k] = Phi_j^T rhs_j.
-void fine_gather_restrict(const Geom& g, const ProbBox* d_fine, const long long* d_droff, const int* d_K,
-                          const double* r, double* rhs, const double* Phi, const long long* d_phioff, int ldphi,
-                          const int* d_m, const long long* d_c1off, double* r1, int P, const int* done,
-                          cudaStream_t s);
+// Fine Dirichlet gather: rhs_j = r on the Dirichlet box of j (solve-buffer
+// layout; max_K the largest number of tile rows).
+void fine_gather(const Geom& g, const ProbBox* d_fine, const long long* d_droff, const int* d_K, int max_K,
+                 const double* r, double* rhs, int P, const int* done, cudaStream_t s);
+// Coarse restriction: r1[c1off_j + k] = Phi_j^T r on the Dirichlet box of j.
+void fine_restrict(const Geom& g, const ProbBox* d_fine, const double* r, const double* Phi, const long long* d_phioff,
+                   int ldphi, const int* d_m, const long long* d_c1off, double* r1, int P, const int* done,
+                   cudaStream_t s);
 
 // Per-axis lookup of fine subdomains whose Dirichlet range holds a coordinate.
 struct CombineMaps {

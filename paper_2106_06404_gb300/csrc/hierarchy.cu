@@ -664,7 +664,7 @@ void Hierarchy::build_fine() {
         stats.subdomains[L] = Pf;
     }
     d_fm = upload_vec(fm, st);
-    ldphi = std::max(1, spec.nev_max);
+    ldphi = (spec.nev_max + 1) / 2 * 2;              // even: rows of Phi start on 16 bytes
     phioff.resize(Pf);
     long long tot = 0;
     for (int j = 0; j < Pf; ++j) {
@@ -1195,11 +1195,11 @@ void Hierarchy::build_coarse() {
 
 void Hierarchy::apply_prec(const double* rr, double* zz, const int* gdone, PcgScalars* fin_sc) {
     double* r1 = levels == 2 ? r0buf.p : v1.p;
-    fine_gather_restrict(g, d_fboxes.p, fdir.d_roff.p, fdir.d_K.p, rr, frhs.p, Phi.p, d_phioff.p, ldphi, d_fm.p,
-                         d_c1off.p, r1, Pf, gdone, st);
-    // the coarse chain runs on a second stream, concurrently with the fine solves
+    // the coarse chain, restriction included, runs on a second stream, concurrently with the fine solves
     MSDD_CUDA(cudaEventRecord(ev_fork, st));
     MSDD_CUDA(cudaStreamWaitEvent(st2, ev_fork, 0));
+    fine_gather(g, d_fboxes.p, fdir.d_roff.p, fdir.d_K.p, fdir.max_K, rr, frhs.p, Pf, gdone, st);
+    fine_restrict(g, d_fboxes.p, rr, Phi.p, d_phioff.p, ldphi, d_fm.p, d_c1off.p, r1, Pf, gdone, st2);
     const double* zc;
     if (levels == 2) {
         gemv_batched(d_gemm_y0.p, 1, 0, 1.0, A0inv.p, r0buf.p, 0.0, y0buf.p, (int)n0, st2, gdone);
@@ -1331,15 +1331,13 @@ void Hierarchy::apply_hybrid(const double* rr, double* zz, const int* done) {
         a.m = (int)n1; a.n = 1; a.k = (int)n1;
         d_gemm_a1 = upload_vec(std::vector<GemmItem>{a}, st);
     }
-    fine_gather_restrict(g, d_fboxes.p, fdir.d_roff.p, fdir.d_K.p, rr, frhs.p, Phi.p, d_phioff.p, ldphi, d_fm.p,
-                         d_c1off.p, r1, Pf, done, st);
+    fine_gather(g, d_fboxes.p, fdir.d_roff.p, fdir.d_K.p, fdir.max_K, rr, frhs.p, Pf, done, st);
     tile_solve(fdir, frhs.p, 1, 1, nullptr, st, done);
     fine_combine_mode(g, cmaps, d_fboxes.p, fdir.d_roff.p, frhs.p, Phi.p, d_phioff.p, ldphi, d_fm.p, d_c1off.p, r1,
                       zz, rr, nullptr, nblocks, done, COMB_Y | COMB_RAS, st);
     spmv_stencil_dot(g, stencil.p, zz, hyb_q.p, partial.p, nblocks, done, st);
     vec_sub(rr, hyb_q.p, hyb_t.p, nun, st, done);                           // t = r - A z
-    fine_gather_restrict(g, d_fboxes.p, fdir.d_roff.p, fdir.d_K.p, hyb_t.p, frhs.p, Phi.p, d_phioff.p, ldphi, d_fm.p,
-                         d_c1off.p, r1, Pf, done, st);                      // r1 = Phi^T t
+    fine_restrict(g, d_fboxes.p, hyb_t.p, Phi.p, d_phioff.p, ldphi, d_fm.p, d_c1off.p, r1, Pf, done, st);   // Phi^T t
     const double* zc;
     if (levels == 2) {
         gemv_batched(d_gemm_y0.p, 1, 0, 1.0, A0inv.p, r0buf.p, 0.0, y0buf.p, (int)n0, st, done);

@@ -13,9 +13,9 @@ __device__ double sum_partials(const double* partial, int nblocks) {
     return v;
 }
 
-__global__ void __launch_bounds__(1024) k_start(const double* __restrict__ b, double* __restrict__ x, double* __restrict__ r, long long n,
+__global__ void __launch_bounds__(PCG_NT) k_start(const double* __restrict__ b, double* __restrict__ x, double* __restrict__ r, long long n,
                         double* __restrict__ partial) {
-    __shared__ double red[1024];
+    __shared__ double red[PCG_NT];
     double part = 0.0;
     for (long long u = blockIdx.x * (long long)blockDim.x + threadIdx.x; u < n; u += (long long)gridDim.x * blockDim.x) {
         double v = b[u];
@@ -23,13 +23,8 @@ __global__ void __launch_bounds__(1024) k_start(const double* __restrict__ b, do
         x[u] = 0.0;
         part += v * v;
     }
-    red[threadIdx.x] = part;
-    __syncthreads();
-    for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-        if (threadIdx.x < s) red[threadIdx.x] += red[threadIdx.x + s];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) partial[blockIdx.x] = red[0];
+    part = pcg_block_sum(part, red);
+    if (threadIdx.x == 0) partial[blockIdx.x] = part;
 }
 
 __global__ void k_fin_bb(PcgScalars* sc, const double* __restrict__ partial, int nblocks, double tol, int maxit) {
@@ -57,10 +52,10 @@ __global__ void k_copy(const double* __restrict__ z, double* __restrict__ p, lon
 
 
 // fin = PCG_FIN_RR: the last block applies the r.r test itself
-__global__ void __launch_bounds__(1024) k_axpy(PcgScalars* sc, double* __restrict__ x, double* __restrict__ r,
+__global__ void __launch_bounds__(PCG_NT) k_axpy(PcgScalars* sc, double* __restrict__ x, double* __restrict__ r,
                        const double* __restrict__ p, const double* __restrict__ q, long long n,
                        double* __restrict__ partial, int fin) {
-    __shared__ double red[1024];
+    __shared__ double red[PCG_NT];
     if (sc->done) return;
     const double a = sc->alpha;
     double part = 0.0;
@@ -70,14 +65,9 @@ __global__ void __launch_bounds__(1024) k_axpy(PcgScalars* sc, double* __restric
         r[u] = rv;
         part += rv * rv;
     }
-    red[threadIdx.x] = part;
-    __syncthreads();
-    for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-        if (threadIdx.x < s) red[threadIdx.x] += red[threadIdx.x + s];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) partial[blockIdx.x] = red[0];
-    if (fin) pcg_last_block(sc, fin, partial);
+    part = pcg_block_sum(part, red);
+    if (threadIdx.x == 0) partial[blockIdx.x] = part;
+    if (fin) pcg_last_block(sc, fin, partial, red);
 }
 
 
@@ -225,7 +215,7 @@ void vec_sub(const double* a, const double* b, double* c, long long n, cudaStrea
 }
 
 void pcg_start(const double* b, double* x, double* r, long long n, double* partial, int nblocks, cudaStream_t s) {
-    k_start<<<nblocks, 1024, 0, s>>>(b, x, r, n, partial);
+    k_start<<<nblocks, PCG_NT, 0, s>>>(b, x, r, n, partial);
     MSDD_LAUNCH_CHECK();
 }
 void pcg_fin_bb(PcgScalars* sc, const double* partial, int nblocks, double tol, int maxit, cudaStream_t s) {
@@ -241,7 +231,7 @@ void pcg_fin_rho0(PcgScalars* sc, const double* partial, int nblocks, const doub
 }
 void pcg_axpy(PcgScalars* sc, double* x, double* r, const double* p, const double* q, long long n, double* partial,
               int nblocks, cudaStream_t s, bool fuse_rr) {
-    k_axpy<<<nblocks, 1024, 0, s>>>(sc, x, r, p, q, n, partial, fuse_rr ? PCG_FIN_RR : PCG_FIN_NONE);
+    k_axpy<<<nblocks, PCG_NT, 0, s>>>(sc, x, r, p, q, n, partial, fuse_rr ? PCG_FIN_RR : PCG_FIN_NONE);
     MSDD_LAUNCH_CHECK();
 }
 void pcg_update_p(PcgScalars* sc, const double* z, double* p, long long n, cudaStream_t s) {

@@ -42,21 +42,43 @@ __device__ __forceinline__ void pcg_fin_apply(PcgScalars* sc, int fin, double v)
         sc->rho = v;
     }
 }
+// Blocks of the kernels that carry a dot product: 256 threads, so that small
+// problems still give every SM several blocks and the sum over a block takes
+// three barriers and five shuffles (FP64 additions are what it costs: the tree
+// issues 12 of them a block, shuffles alone 40).  At 1024 threads a block the
+// 512^2 kernels had 1.7 blocks an SM and ten barriers each.
+constexpr int PCG_NT = 256;
+// sum of v over the block, valid in thread 0; red: PCG_NT doubles of shared
+// memory, free again after the next barrier
+__device__ __forceinline__ double pcg_block_sum(double v, double* red) {
+    const int t = threadIdx.x;
+    red[t] = v;
+    __syncthreads();
+    if (t < 128) red[t] += red[t + 128];
+    __syncthreads();
+    if (t < 64) red[t] += red[t + 64];
+    __syncthreads();
+    if (t < 32) {
+        v = red[t] + red[t + 32];
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    }
+    return v;
+}
 // Called by every thread of every block once thread 0 has stored
 // partial[blockIdx.x]: the last block to arrive sums the gridDim.x partials
-// (one warp, lane-strided then a fixed shuffle tree: a fixed order, so the
-// result does not depend on which block arrives last) and applies `fin`.
-__device__ __forceinline__ void pcg_last_block(PcgScalars* sc, int fin, const double* partial) {
+// (thread-strided, then the block sum: a fixed order, so the result does not
+// depend on which block arrives last) and applies `fin`.
+__device__ __forceinline__ void pcg_last_block(PcgScalars* sc, int fin, const double* partial, double* red) {
     __shared__ int s_last;
     __threadfence();
     __syncthreads();
     if (threadIdx.x == 0) s_last = atomicAdd(&sc->ticket, 1u) == gridDim.x - 1;
     __syncthreads();
-    if (!s_last || threadIdx.x >= 32) return;
+    if (!s_last) return;
     __threadfence();
     double v = 0.0;
-    for (int k = threadIdx.x; k < (int)gridDim.x; k += 32) v += __ldcg(partial + k);
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    for (int k = threadIdx.x; k < (int)gridDim.x; k += PCG_NT) v += __ldcg(partial + k);
+    v = pcg_block_sum(v, red);
     if (threadIdx.x == 0) {
         pcg_fin_apply(sc, fin, v);
         sc->ticket = 0u;

@@ -602,43 +602,39 @@ __global__ void k_global_stencil(Geom g, double* __restrict__ S, long long nun) 
     }
 }
 
-// q = A p from the stored stencil (one thread per unknown, neighbours of an
-// x-row are contiguous), plus partial sums of p.q.
 // q = S p over the unknowns with the stored 3^D-point stencil, and block
 // partial sums of p.q.  Every neighbour index is clamped into [0, nun): a
 // neighbour outside the unknown box has coefficient exactly 0 in S, so its
-// term adds nothing and the loads need no branch.  1024 threads a block
-// (the grid is the dot-product block count, a few blocks per SM).
+// term adds nothing and the loads need no branch.  Indices fit 32 bits (the
+// set-up rejects 2^31 unknowns or more).  The FP64 pipe (3^D + 1 operations an
+// unknown) and the launch bound it.
 template <int D>
-__global__ void __launch_bounds__(1024) k_spmv_stencil_dot(Geom g, const double* __restrict__ S,
-                                                           const double* __restrict__ p, double* __restrict__ q,
-                                                           long long nun, double* __restrict__ partial,
-                                                           const int* __restrict__ done, PcgScalars* sc, int fin) {
-    __shared__ double red[1024];
+__global__ void __launch_bounds__(PCG_NT) k_spmv_stencil_dot(Geom g, const double* __restrict__ S,
+                                                             const double* __restrict__ p, double* __restrict__ q,
+                                                             int nun, double* __restrict__ partial,
+                                                             const int* __restrict__ done, PcgScalars* sc, int fin) {
+    __shared__ double red[PCG_NT];
     if (done && *done) return;
     constexpr int NOFF = D == 3 ? 27 : 9;
-    const long long sy = g.ushape[0], sz = (long long)g.ushape[0] * g.ushape[1];
+    const int sy = g.ushape[0], sz = g.ushape[0] * g.ushape[1];
     double part = 0.0;
-    for (long long u = blockIdx.x * (long long)blockDim.x + threadIdx.x; u < nun; u += (long long)gridDim.x * blockDim.x) {
-        double acc = 0.0;
+    for (int u = blockIdx.x * PCG_NT + threadIdx.x; u < nun; u += gridDim.x * PCG_NT) {
+        double a0 = 0.0, a1 = 0.0;
 #pragma unroll
         for (int oi = 0; oi < NOFF; ++oi) {
             const double c = S[(long long)oi * nun + u];
-            long long v = u + (oi % 3 - 1) + ((oi / 3) % 3 - 1) * sy + (D == 3 ? (oi / 9 - 1) * sz : 0);
-            v = v < 0 ? 0 : (v >= nun ? nun - 1 : v);
-            acc += c * p[v];
+            int v = u + (oi % 3 - 1) + ((oi / 3) % 3 - 1) * sy + (D == 3 ? (oi / 9 - 1) * sz : 0);
+            v = min(max(v, 0), nun - 1);
+            if (oi & 1) a1 = fma(c, p[v], a1);
+            else a0 = fma(c, p[v], a0);
         }
+        const double acc = a0 + a1;
         q[u] = acc;
-        part += acc * p[u];
+        part = fma(acc, p[u], part);
     }
-    red[threadIdx.x] = part;
-    __syncthreads();
-    for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-        if (threadIdx.x < s) red[threadIdx.x] += red[threadIdx.x + s];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) partial[blockIdx.x] = red[0];
-    if (sc) pcg_last_block(sc, fin, partial);
+    part = pcg_block_sum(part, red);
+    if (threadIdx.x == 0) partial[blockIdx.x] = part;
+    if (sc) pcg_last_block(sc, fin, partial, red);
 }
 
 __global__ void k_apply_global(Geom g, const double* __restrict__ x, double* __restrict__ y, long long nun) {
@@ -805,9 +801,9 @@ void spmv_stencil_dot(const Geom& g, const double* S, const double* p, double* q
                       const int* done, cudaStream_t s, PcgScalars* sc, int fin) {
     long long nun = (long long)g.ushape[0] * g.ushape[1] * (g.dim == 3 ? g.ushape[2] : 1);
     if (g.dim == 3)
-        k_spmv_stencil_dot<3><<<nblocks, 1024, 0, s>>>(g, S, p, q, nun, partial, done, sc, fin);
+        k_spmv_stencil_dot<3><<<nblocks, PCG_NT, 0, s>>>(g, S, p, q, (int)nun, partial, done, sc, fin);
     else
-        k_spmv_stencil_dot<2><<<nblocks, 1024, 0, s>>>(g, S, p, q, nun, partial, done, sc, fin);
+        k_spmv_stencil_dot<2><<<nblocks, PCG_NT, 0, s>>>(g, S, p, q, (int)nun, partial, done, sc, fin);
     MSDD_LAUNCH_CHECK();
 }
 
