@@ -1834,6 +1834,201 @@ void launch_band_split(const TileBatch& tb, const CUtensorMap& tm, double* X, cu
     MSDD_LAUNCH_CHECK();
 }
 
+// ---- one right-hand side, kb <= 2, FP32 (the PCG local solves of 2D boxes)
+// The solve is a chain of 2 K dependent steps, z_R = T_R (x_R - L_{R,R-1}
+// z_{R-1} - L_{R,R-2} z_{R-2}) forward, and a step's 64 multiply-adds a row are
+// a small part of it: with four warps sharing each step, the barriers, shuffle
+// sums and copy instructions around them took 1400 cycles.  Here one warp does
+// a step alone (lane = row, its rows of T and L_{R,R-1} in registers, the 32
+// values of z_{R-1} and of the right-hand side broadcast through shared
+// memory: 133 + 126 cycles), and four warps take turns: while one runs its
+// step, the others wait for the tiles of their next ones, load their rows into
+// registers (some 600 cycles, off the chain) and take the far tile's part off
+// the right-hand side.  Warps hand over in pairs (named barriers: z_R is
+// announced to the warps of the next two steps).  (One warp doing all of it was
+// no faster than four sharing a step, a warp issues in order; a barrier of all
+// four a step made each wait for the slowest load; a fifth warp issuing every
+// copy took 830 cycles a step for it.)  Each warp streams the tiles of its own
+// steps by TMA, two turns (eight steps) ahead; of the far tile, whose columns
+// before 64 - b are zero, only the 8-column boxes that hold nonzeros are copied
+// (at b = 38 a step moves 9 of 12 KB).  Every wait is bounded; after a timeout
+// (recorded in g_wait_timeouts) the chain runs to its end without waiting for
+// tiles, and each warp waits (bounded) for its copies in flight.
+// Measured: 256 problems of n = 1369, b = 38 with cold caches 60 -> 53 us (DRAM
+// from there on), with the factors in L2 59 -> 32 us; 128 of them 57 -> 29 us.
+constexpr int S1W_W = 4, S1W_NST = 2 * S1W_W;
+__device__ __forceinline__ void tma_load_cols8(void* dst, const CUtensorMap* map, int col, int row,
+                                               unsigned long long* bar) {
+    asm volatile(
+        "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];\n" ::"r"(
+            smem_u32(dst)),
+        "l"(map), "r"(col), "r"(row), "r"(smem_u32(bar))
+        : "memory");
+}
+// first 8-column group of the far tile (R, R - 2) that holds nonzeros
+__host__ __device__ inline int s1w_group0(int b) { return b >= 64 ? 0 : (64 - b) >> 3; }
+
+__global__ void __launch_bounds__(32 * S1W_W) k_tile_solve1_warp(
+    const __grid_constant__ CUtensorMap tmt, const __grid_constant__ CUtensorMap tmc, const float* __restrict__ dinv,
+    const int* __restrict__ kb_, const int* __restrict__ K_, const int* __restrict__ b_,
+    const long long* __restrict__ toff_, const long long* __restrict__ roff_, double* __restrict__ X,
+    const int* __restrict__ gdone, int nbox)
+{
+    constexpr int NTC = 32 * S1W_W;
+    extern __shared__ unsigned char smem_raw[];
+    unsigned char* base = smem_raw + ((1024 - (smem_u32(smem_raw) & 1023)) & 1023);
+    const int stage_floats = 2 * NB2 + nbox * 8 * NB;      // T, near tile, far tile's boxes
+    float* St = reinterpret_cast<float*>(base);
+    float* Fr = St + (size_t)S1W_NST * stage_floats;         // [S1W_W][boxes] far boxes of the step each warp prepares
+    float* Ac = Fr + (size_t)S1W_W * nbox * 8 * NB;          // [32]
+    float* zs = Ac + NB;                                     // [K * 32]
+    __shared__ unsigned long long full[S1W_NST];
+    __shared__ int s_abort;
+    if (gdone && *gdone) return;
+    const int i = blockIdx.x;
+    const int kb = kb_[i], K = K_[i], bw = b_[i];
+    if (kb > 2 || K == 0) return;                            // never launched so (host dispatch)
+    const long long toff = toff_[i], roff = roff_[i];
+    const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
+    const int g0 = s1w_group0(bw), nb = kb == 2 ? min(nbox, 4 - g0) : 0;
+    if (t == 0) {
+        s_abort = 0;
+        for (int s = 0; s < S1W_NST; ++s) mbar_init(&full[s], 1);
+        fence_mbar_init();
+    }
+    for (int e = t; e < K * NB; e += NTC) zs[e] = f64_to_f32(X[roff + e]);
+    __syncthreads();
+    auto give_up = [&]() {
+        if (atomicExch(&s_abort, 1) == 0) atomicAdd(&g_wait_timeouts, 1);
+    };
+    const int total = 2 * K;
+
+    // turn u of a warp is step 4 u + warp, its tiles go to stage 2 warp + (u & 1)
+    auto stage = [&](int u) { return 2 * warp + (u & 1); };
+    auto issue = [&](int u) {                                // one lane issues a step's copies
+        const int it = S1W_W * u + warp;
+        if (lane != 0 || it >= total) return;
+        const bool fwd = it < K;
+        const int R = fwd ? it : total - 1 - it, nd = min(kb, fwd ? R : K - 1 - R), st = stage(u);
+        float* dst = St + (size_t)st * stage_floats;
+        mbar_expect_tx(&full[st], (1 + (nd > 0)) * NB2 * 4 + (nd > 1 ? nb * 8 * NB * 4 : 0));
+        tma_load_tile(dst, &tmt, (int)(tile_index(toff, kb, R, R) / NB), &full[st]);
+        if (nd > 0) {
+            const long long ti = fwd ? tile_index(toff, kb, R, R - 1) : tile_index(toff, kb, R + 1, R);
+            tma_load_tile(dst + NB2, &tmt, (int)(ti / NB), &full[st]);
+        }
+        if (nd > 1) {
+            const long long ti = fwd ? tile_index(toff, kb, R, R - 2) : tile_index(toff, kb, R + 2, R);
+            for (int q = 0; q < nb; ++q)
+                tma_load_cols8(dst + 2 * NB2 + q * 8 * NB, &tmc, 8 * (g0 + q), (int)(ti / NB), &full[st]);
+        }
+    };
+    issue(0);
+    issue(1);
+
+    // ---------------- the chain warps, lane = row (column in the backward sweep)
+    auto announce = [&](int id) { asm volatile("bar.arrive %0, 64;\n" ::"r"(id) : "memory"); };
+    auto await = [&](int id) { asm volatile("bar.sync %0, 64;\n" ::"r"(id) : "memory"); };
+    float* far = Fr + (size_t)warp * nbox * 8 * NB;
+    float l[NB], tr[NB], xfar = 0.f, dv = 1.f;               // near tile's and T's row, the far tile's part, D^{-1}
+    // the rows of step `it` (turn u) into registers, its far boxes to this warp's copy, the next copies into its stage
+    auto fetch = [&](int it, int u) -> bool {
+        const int st = stage(u);
+        const bool fwd = it < K;
+        const int R = fwd ? it : total - 1 - it, nd = min(kb, fwd ? R : K - 1 - R);
+        if (!fwd) dv = dinv[roff + (long long)R * NB + lane];
+        if (*(volatile int*)&s_abort) return false;          // the chain ends without the tiles
+        if (!mbar_wait_bounded(&full[st], (u >> 1) & 1u)) { give_up(); return false; }
+        const float *T = St + (size_t)st * stage_floats, *L = T + NB2, *F = L + NB2;
+        if (fwd) {
+#pragma unroll
+            for (int g = 0; g < 8; ++g) {
+                const float4 a = *reinterpret_cast<const float4*>(T + lane * NB + ((g ^ (lane & 7)) << 2));
+                tr[4 * g] = a.x; tr[4 * g + 1] = a.y; tr[4 * g + 2] = a.z; tr[4 * g + 3] = a.w;
+                const float4 c = *reinterpret_cast<const float4*>(L + lane * NB + ((g ^ (lane & 7)) << 2));
+                l[4 * g] = c.x; l[4 * g + 1] = c.y; l[4 * g + 2] = c.z; l[4 * g + 3] = c.w;
+            }
+        } else {
+#pragma unroll
+            for (int k = 0; k < NB; ++k) {
+                tr[k] = T[swz(k, lane)];
+                l[k] = L[swz(k, lane)];
+            }
+        }
+        if (nd == 0)                                         // (no near tile: the stage holds an older one)
+#pragma unroll
+            for (int k = 0; k < NB; ++k) l[k] = 0.f;
+        if (nd > 1)
+            for (int e = lane; e < nb * 2 * NB; e += 32)
+                *reinterpret_cast<float4*>(far + 4 * e) = *reinterpret_cast<const float4*>(F + 4 * e);
+        __syncwarp();
+        issue(u + 2);
+        return true;
+    };
+    // the far tile's product of step `it` (z of step it - 2 is there)
+    auto far_part = [&](int it) {
+        const bool fwd = it < K;
+        const int R = fwd ? it : total - 1 - it, nd = min(kb, fwd ? R : K - 1 - R);
+        xfar = 0.f;
+        if (nd < 2) return;
+        if (fwd) {
+            for (int q = 0; q < nb; ++q) {
+                const float4 a = *reinterpret_cast<const float4*>(far + q * 8 * NB + lane * 8);
+                const float4 c = *reinterpret_cast<const float4*>(far + q * 8 * NB + lane * 8 + 4);
+                const float4 u = *reinterpret_cast<const float4*>(zs + (R - 2) * NB + 8 * (g0 + q));
+                const float4 v = *reinterpret_cast<const float4*>(zs + (R - 2) * NB + 8 * (g0 + q) + 4);
+                xfar += (fmaf(a.x, u.x, fmaf(a.y, u.y, fmaf(a.z, u.z, a.w * u.w)))) +
+                        (fmaf(c.x, v.x, fmaf(c.y, v.y, fmaf(c.z, v.z, c.w * v.w))));
+            }
+        } else if ((lane >> 3) >= g0 && (lane >> 3) - g0 < nb) {
+            const float* f = far + ((lane >> 3) - g0) * 8 * NB + (lane & 7);
+            const float* z = zs + (R + 2) * NB;
+            const int kend = min(NB, bw - 31);               // rows of the far tile with nonzeros
+            float s1 = 0.f;
+            int k = 0;
+            for (; k + 1 < kend; k += 2) {
+                xfar = fmaf(f[k * 8], z[k], xfar);
+                s1 = fmaf(f[k * 8 + 8], z[k + 1], s1);
+            }
+            if (k < kend) xfar = fmaf(f[k * 8], z[k], xfar);
+            xfar += s1;
+        }
+    };
+    auto dot = [&](const float (&a)[NB], const float* v) {   // sum_k a[k] v[k], v broadcast from shared memory
+        float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
+#pragma unroll
+        for (int g = 0; g < 8; ++g) {
+            const float4 x = *reinterpret_cast<const float4*>(v + 4 * g);
+            s0 = fmaf(a[4 * g], x.x, s0); s1 = fmaf(a[4 * g + 1], x.y, s1);
+            s2 = fmaf(a[4 * g + 2], x.z, s2); s3 = fmaf(a[4 * g + 3], x.w, s3);
+        }
+        return (s0 + s1) + (s2 + s3);
+    };
+#pragma unroll
+    for (int k = 0; k < NB; ++k) { l[k] = 0.f; tr[k] = 0.f; }
+    int u = 0, landed = 0;                                   // turn; turns whose copies have been waited for
+    for (int it = warp; it < total; it += S1W_W, ++u) {
+        const bool fwd = it < K;
+        const int R = fwd ? it : total - 1 - it, other = fwd ? max(R - 1, 0) : min(R + 1, K - 1);
+        if (fetch(it, u)) landed = u + 1;
+        if (it >= 2) await(1 + ((it - 2) & 3));              // z of step it - 2
+        far_part(it);
+        if (it >= 1) await(5 + ((it - 1) & 3));              // z of step it - 1
+        const float x = fmaf(dv, zs[R * NB + lane], -xfar);  // (dv = 1 forward)
+        Ac[lane] = x - dot(l, zs + other * NB);
+        __syncwarp();
+        const float z = dot(tr, Ac);
+        zs[R * NB + lane] = z;
+        __syncwarp();
+        if (it + 1 < total) announce(5 + warp);
+        if (it + 2 < total) announce(1 + warp);
+    }
+    for (int v = landed; v < landed + 2 && S1W_W * v + warp < total; ++v)     // after a timeout only
+        mbar_wait_bounded(&full[stage(v)], (v >> 1) & 1u);
+    asm volatile("bar.sync 9, %0;\n" ::"r"(NTC) : "memory");
+    for (int e = t; e < K * NB; e += NTC) X[roff + e] = f32_to_f64(zs[e]);
+}
+
 using EncodeTiledFn = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
                                    const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
                                    CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
@@ -1860,6 +2055,19 @@ bool encode_tile_map(const float* base, long long elems, CUtensorMap* m) {
     const cuuint32_t estr[2] = {1, 1};
     return enc(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, (void*)base, dims, strides, box, estr,
                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+// [elems / 32][32] FP32 view, boxes of 8 columns x 32 rows, plain layout.
+bool encode_cols8_map(const float* base, long long elems, CUtensorMap* m) {
+    EncodeTiledFn enc = encode_tiled();
+    if (!enc || !base || elems <= 0) return false;
+    const cuuint64_t dims[2] = {(cuuint64_t)NB, (cuuint64_t)(elems / NB)};
+    const cuuint64_t strides[1] = {(cuuint64_t)NB * sizeof(float)};
+    const cuuint32_t box[2] = {8, (cuuint32_t)NB};
+    const cuuint32_t estr[2] = {1, 1};
+    return enc(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, (void*)base, dims, strides, box, estr,
+               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_NONE,
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
@@ -2092,19 +2300,27 @@ void tile_solve(const TileBatch& tb, double* X, int ldx, int ncols, const int* s
     if (ncols == 1 && ldx == 1 && skip == nullptr) {
         int maxkb = 0;
         for (int v : tb.kb) maxkb = std::max(maxkb, v);
-        const size_t zt = (size_t)tb.max_K * NB * (tb.prec ? sizeof(float) : sizeof(double));
-        const size_t ring_bytes = (tb.prec ? (maxkb <= 1 ? solve1_ring_bytes<float, 1>() : solve1_ring_bytes<float, 2>())
-                                           : (maxkb <= 1 ? solve1_ring_bytes<double, 1>() : solve1_ring_bytes<double, 2>())) + zt;
-        if (maxkb <= 2 && ring_bytes <= 200 * 1024) {
-            if (tb.prec) {
-                auto k = maxkb <= 1 ? k_tile_solve1<float, 1> : k_tile_solve1<float, 2>;
-                raise_smem_limit(k, ring_bytes);
-                k<<<tb.P, S1T, ring_bytes, s>>>(tb.tiles_f.p, tb.dinv_f.p, tb.d_kb.p, tb.d_K.p, tb.d_toff.p, tb.d_roff.p, X, gdone);
-            } else {
-                auto k = maxkb <= 1 ? k_tile_solve1<double, 1> : k_tile_solve1<double, 2>;
-                raise_smem_limit(k, ring_bytes);
-                k<<<tb.P, S1T, ring_bytes, s>>>(tb.tiles_d.p, tb.dinv_d.p, tb.d_kb.p, tb.d_K.p, tb.d_toff.p, tb.d_roff.p, X, gdone);
+        if (tb.prec && maxkb <= 2) {
+            const CUtensorMap* tm = tile_tensor_map(tb);
+            alignas(64) CUtensorMap tc;
+            int nbox = 0;
+            for (int i = 0; i < tb.P; ++i)
+                if (tb.kb[i] == 2) nbox = std::max(nbox, 4 - s1w_group0(tb.b[i]));
+            const size_t bytes = 1024 + sizeof(float) * ((size_t)S1W_NST * (2 * NB2 + nbox * 8 * NB) +
+                                                         (size_t)S1W_W * nbox * 8 * NB + NB + (size_t)tb.max_K * NB);
+            if (tm && bytes <= 200 * 1024 && encode_cols8_map(tb.tiles_f.p, tb.total_tile_elems, &tc)) {
+                raise_smem_limit(k_tile_solve1_warp, bytes);
+                k_tile_solve1_warp<<<tb.P, 32 * S1W_W, bytes, s>>>(*tm, tc, tb.dinv_f.p, tb.d_kb.p, tb.d_K.p, tb.d_b.p,
+                                                          tb.d_toff.p, tb.d_roff.p, X, gdone, nbox);
+                MSDD_LAUNCH_CHECK();
+                return;
             }
+        }
+        const size_t ring_bytes = (maxkb <= 1 ? solve1_ring_bytes<double, 1>() : solve1_ring_bytes<double, 2>()) + zbytes;
+        if (!tb.prec && maxkb <= 2 && ring_bytes <= 200 * 1024) {
+            auto k = maxkb <= 1 ? k_tile_solve1<double, 1> : k_tile_solve1<double, 2>;
+            raise_smem_limit(k, ring_bytes);
+            k<<<tb.P, S1T, ring_bytes, s>>>(tb.tiles_d.p, tb.dinv_d.p, tb.d_kb.p, tb.d_K.p, tb.d_toff.p, tb.d_roff.p, X, gdone);
             MSDD_LAUNCH_CHECK();
             return;
         }
@@ -2117,7 +2333,7 @@ void tile_solve(const TileBatch& tb, double* X, int ldx, int ncols, const int* s
                 return;
             }
         }
-        if (maxkb > 2 && zbytes <= 160 * 1024) {
+        if ((maxkb > 2 || tb.prec) && zbytes <= 160 * 1024) {
             if (zbytes > 48 * 1024) {
                 raise_smem_limit(k_tile_solve1_dense<float>, zbytes);
                 raise_smem_limit(k_tile_solve1_dense<double>, zbytes);
