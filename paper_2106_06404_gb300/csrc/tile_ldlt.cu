@@ -1630,11 +1630,17 @@ void launch_band_ks(const TileBatch& tb, const CUtensorMap& tm, int maxkb, XT* X
     MSDD_LAUNCH_CHECK();
 }
 
-// Column groups of 4 J <= 20 columns, as even as they come: J from the count.
+// Column groups of 4 J <= 20 columns, as even as they come; fewer columns a CTA
+// while that still leaves every CTA an SM of its own (the tiles are then read
+// by several CTAs, but a step's products and loads are shared out): 48 problems
+// of n = 3600, b = 226, 16 columns 737 us in one group, 556 us in two, 24 of
+// them 703 us in one, 478 us in four.
 template <typename XT>
 void solve_band_ks(const TileBatch& tb, const CUtensorMap& tm, int maxkb, XT* X, int ldx, int ncols, const int* skip,
                    cudaStream_t s, const int* gdone) {
-    const int chunks = (ncols + 19) / 20, J = (ncols + 4 * chunks - 1) / (4 * chunks);
+    int chunks = (ncols + 19) / 20, J = (ncols + 4 * chunks - 1) / (4 * chunks);
+    while (J > 1 && (long long)tb.P * ((ncols + 4 * (J - 1) - 1) / (4 * (J - 1))) <= 152) --J;
+    chunks = (ncols + 4 * J - 1) / (4 * J);
     auto go = [&](auto nw) {
         constexpr int NW = decltype(nw)::value;
         switch (J) {
