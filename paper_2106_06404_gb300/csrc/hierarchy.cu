@@ -764,9 +764,12 @@ void Hierarchy::build_coarse() {
     std::vector<GramItem> gitems;
     std::vector<long long> gpatch;       // patch index of each item
     long long gtot = 0;
+    std::vector<GramItem> gram_items;    // one per unordered pair: the kernel writes both blocks
     for (size_t k = 0; k < patches.size(); ++k) {
-        for (int j : patches[k].mem)
-            for (int jj : patches[k].mem) {
+        const std::vector<int>& mem = patches[k].mem;
+        for (size_t a = 0; a < mem.size(); ++a)
+            for (size_t b = a; b < mem.size(); ++b) {
+                const int j = mem[a], jj = mem[b];
                 if (fm[j] == 0 || fm[jj] == 0) continue;
                 GramItem it;
                 for (int d = 0; d < 3; ++d) { it.elo[d] = patches[k].elo[d]; it.ehi[d] = patches[k].ehi[d]; }
@@ -774,13 +777,25 @@ void Hierarchy::build_coarse() {
                 it.jj = jj;
                 it.goff = gtot;
                 gtot += (long long)fm[j] * fm[jj];
+                it.goff_t = -1;
+                if (j != jj) {
+                    it.goff_t = gtot;
+                    gtot += (long long)fm[j] * fm[jj];
+                }
                 gitems.push_back(it);
                 gpatch.push_back((long long)k);
+                gram_items.push_back(it);
+                if (j != jj) {
+                    std::swap(it.j, it.jj);
+                    it.goff = it.goff_t;
+                    gitems.push_back(it);
+                    gpatch.push_back((long long)k);
+                }
             }
     }
-    DevBuf<GramItem> d_gitems = upload_vec(gitems, st);
+    DevBuf<GramItem> d_gitems = upload_vec(gram_items, st);
     DevBuf<double> G(std::max<long long>(gtot, 1));
-    patch_gram(g, d_fboxes.p, Phi.p, d_phioff.p, ldphi, d_fm.p, d_gitems.p, (int)gitems.size(), G.p, st);
+    patch_gram(g, d_fboxes.p, Phi.p, d_phioff.p, ldphi, d_fm.p, d_gitems.p, (int)gram_items.size(), G.p, st);
 
     // ---- Galerkin matrix of level L-1: block (j, jj) = sum over patches holding both
     std::map<std::pair<int, int>, std::vector<long long>> pairc;

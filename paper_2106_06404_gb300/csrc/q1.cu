@@ -835,77 +835,128 @@ void make_coarse_basis(const Geom& g, const ProbBox* d_boxes, const int* d_count
 namespace msdd {
 namespace {
 
-constexpr int GCH = 16;   // elements staged per chunk in patch_gram
-
+// G = Phi_j^T A_patch Phi_jj for the patch operator A_patch (the elements of
+// the item's box), and its transpose for the pair (jj, j): one CTA per
+// unordered pair of a patch.  Nodes of the patch in chunks of GN: the 3^D
+// stencil coefficients of the patch operator at each node (a warp on one
+// offset of 32 nodes, so that the reference matrices in constant memory are
+// read uniformly), then Y = A_patch Phi_jj on the chunk, then the m_j x m_jj
+// product.  The FP64 pipe bounds it: per node 3^D m + m^2 operations and the
+// coefficients.  Going by elements (2^D x 2^D element matrices, evaluated again
+// for every column, for both orders of a pair) took 8-10 times the operations:
+// with the rest of the coarse assembly 86 -> 28 ms on the 96^3 composite, 9.4 ->
+// 6.8 ms at 1000^2.
+constexpr int GN = 32;
+template <int D>
 __global__ void __launch_bounds__(256) k_patch_gram(Geom g, const ProbBox* __restrict__ fine,
                                                     const double* __restrict__ Phi, const long long* __restrict__ phioff,
                                                     int ldphi, const int* __restrict__ m_,
                                                     const GramItem* __restrict__ items, double* __restrict__ G) {
+    constexpr int NOFF = D == 3 ? 27 : 9;
     extern __shared__ double sm[];
     const GramItem it = items[blockIdx.x];
-    const int nloc = 1 << g.dim;
     const int mj = m_[it.j], mjj = m_[it.jj];
     if (mj == 0 || mjj == 0) return;
+    double* S = sm;                                    // [NOFF][GN]
+    double* Pj = S + NOFF * GN;                        // [GN][ldphi]
+    double* Y = Pj + GN * ldphi;                       // [GN][ldphi]
+    int* base = reinterpret_cast<int*>(Y + GN * ldphi);  // [GN] row of the node in box jj (its neighbours: by offset)
     const ProbBox bj = fine[it.j], bjj = fine[it.jj];
-    double* Pj = sm;
-    double* Pjj = Pj + GCH * nloc * ldphi;
-    double* Tm = Pjj + GCH * nloc * ldphi;
-    int w[3] = {1, 1, 1};
-    long long ne = 1;
-    for (int d = 0; d < g.dim; ++d) { w[d] = it.ehi[d] - it.elo[d]; ne *= w[d]; }
+    int w[3] = {1, 1, 1}, n = 1, wj[3] = {1, 1, 1}, wjj[3] = {1, 1, 1};
+#pragma unroll
+    for (int d = 0; d < D; ++d) {
+        w[d] = it.ehi[d] - it.elo[d] + 1;              // nodes of the patch's closure
+        n *= w[d];
+        wj[d] = bj.dhi[d] - bj.dlo[d] + 1;
+        wjj[d] = bjj.dhi[d] - bjj.dlo[d] + 1;
+    }
     const int t = threadIdx.x;
-    double acc[4] = {0, 0, 0, 0};
     const long long pj = phioff[it.j], pjj = phioff[it.jj];
-    for (long long c0 = 0; c0 < ne; c0 += GCH) {
+    auto coords = [&](int node, int* x) {
+        x[0] = x[1] = x[2] = 0;
+#pragma unroll
+        for (int d = 0; d < D; ++d) {
+            const int q = node / w[d];
+            x[d] = it.elo[d] + node - q * w[d];
+            node = q;
+        }
+    };
+    double acc[4] = {0, 0, 0, 0};
+    for (int c0 = 0; c0 < n; c0 += GN) {
+        const int nc = min(GN, n - c0);
         __syncthreads();
-        for (int e = t; e < GCH * nloc; e += blockDim.x) {
-            long long el = c0 + e / nloc;
-            int a = e % nloc;
-            bool ok = el < ne;
-            int x[3] = {0, 0, 0};
-            if (ok) {
-                long long rem = el;
-                for (int d = 0; d < g.dim; ++d) {
-                    x[d] = it.elo[d] + (int)(rem % w[d]) + ((a >> d) & 1);
-                    rem /= w[d];
+        // coefficients, zero where the node is outside box j or the neighbour outside box jj
+        for (int e = t; e < NOFF * GN; e += 256) {
+            const int oi = e / GN, r = e % GN;
+            double v = 0.0;
+            if (r < nc) {
+                int x[3];
+                coords(c0 + r, x);
+                const int o[3] = {oi % 3 - 1, (oi / 3) % 3 - 1, D == 3 ? oi / 9 - 1 : 0};
+                const int y[3] = {x[0] + o[0], x[1] + o[1], x[2] + o[2]};
+                if (in_box(bj.dlo, bj.dhi, x, D) && in_box(bjj.dlo, bjj.dhi, y, D))
+                    v = stencil_coef(g, it.elo, it.ehi, x, o);
+                if (oi == 0) {
+                    int rb = 0;
+#pragma unroll
+                    for (int d = D - 1; d >= 0; --d) rb = rb * wjj[d] + (x[d] - bjj.dlo[d]);
+                    base[r] = rb;
                 }
             }
-            bool inj = ok && in_box(bj.dlo, bj.dhi, x, g.dim);
-            bool injj = ok && in_box(bjj.dlo, bjj.dhi, x, g.dim);
-            int rj = inj ? box_index(bj.dlo, bj.dhi, x, g.dim) : 0;
-            int rjj = injj ? box_index(bjj.dlo, bjj.dhi, x, g.dim) : 0;
-            for (int k = 0; k < mj; ++k) Pj[e * ldphi + k] = inj ? Phi[pj + (long long)rj * ldphi + k] : 0.0;
-            for (int k = 0; k < mjj; ++k) Pjj[e * ldphi + k] = injj ? Phi[pjj + (long long)rjj * ldphi + k] : 0.0;
+            S[e] = v;
+        }
+        for (int e = t; e < GN * mj; e += 256) {
+            const int r = e / mj, k = e % mj;
+            double v = 0.0;
+            if (r < nc) {
+                int x[3];
+                coords(c0 + r, x);
+                if (in_box(bj.dlo, bj.dhi, x, D)) {
+                    int rb = 0;
+#pragma unroll
+                    for (int d = D - 1; d >= 0; --d) rb = rb * wj[d] + (x[d] - bj.dlo[d]);
+                    v = Phi[pj + (long long)rb * ldphi + k];
+                }
+            }
+            Pj[r * ldphi + k] = v;
         }
         __syncthreads();
-        for (int e = t; e < GCH * nloc * mjj; e += blockDim.x) {
-            int elc = e / (nloc * mjj), a = (e / mjj) % nloc, kk = e % mjj;
-            long long el = c0 + elc;
-            double v = 0.0;
-            if (el < ne) {
-                long long rem = el;
-                int l[3] = {0, 0, 0};
-                for (int d = 0; d < g.dim; ++d) { l[d] = it.elo[d] + (int)(rem % w[d]); rem /= w[d]; }
-                long long E = l[0] + (long long)g.n[0] * (l[1] + (long long)g.n[1] * l[2]);
-                for (int b = 0; b < nloc; ++b) v += elem_entry(g, E, a, b) * Pjj[(elc * nloc + b) * ldphi + kk];
+        for (int e = t; e < GN * mjj; e += 256) {
+            const int r = e / mjj, k = e % mjj;
+            double v0 = 0.0, v1 = 0.0;
+#pragma unroll
+            for (int oi = 0; oi < NOFF; ++oi) {
+                const double c = S[oi * GN + r];
+                if (c == 0.0) continue;
+                const int q = base[r] + (oi % 3 - 1) + wjj[0] * (((oi / 3) % 3 - 1) + (D == 3 ? wjj[1] * (oi / 9 - 1) : 0));
+                const double f = Phi[pjj + (long long)q * ldphi + k];
+                if (oi & 1) v1 = fma(c, f, v1);
+                else v0 = fma(c, f, v0);
             }
-            Tm[(elc * nloc + a) * ldphi + kk] = v;
+            Y[r * ldphi + k] = v0 + v1;
         }
         __syncthreads();
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
-            int e = t + q * blockDim.x;
+            const int e = t + q * 256;
             if (e >= mj * mjj) break;
-            int k = e / mjj, kk = e % mjj;
-            double s = 0.0;
-            for (int ea = 0; ea < GCH * nloc; ++ea) s += Pj[ea * ldphi + k] * Tm[ea * ldphi + kk];
-            acc[q] += s;
+            const int k = e / mjj, kk = e % mjj;
+            double s0 = 0.0, s1 = 0.0;
+            int r = 0;
+            for (; r + 1 < nc; r += 2) {
+                s0 = fma(Pj[r * ldphi + k], Y[r * ldphi + kk], s0);
+                s1 = fma(Pj[(r + 1) * ldphi + k], Y[(r + 1) * ldphi + kk], s1);
+            }
+            if (r < nc) s0 = fma(Pj[r * ldphi + k], Y[r * ldphi + kk], s0);
+            acc[q] += s0 + s1;
         }
     }
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
-        int e = t + q * blockDim.x;
-        if (e < mj * mjj) G[it.goff + e] = acc[q];
+        const int e = t + q * 256;
+        if (e >= mj * mjj) break;
+        G[it.goff + e] = acc[q];
+        if (it.goff_t >= 0) G[it.goff_t + (long long)(e % mjj) * mj + e / mjj] = acc[q];
     }
 }
 
@@ -950,9 +1001,9 @@ __global__ void k_apply_global_dot(Geom g, const double* __restrict__ x, double*
 void patch_gram(const Geom& g, const ProbBox* d_fine, const double* Phi, const long long* d_phioff, int ldphi,
                 const int* d_m, const GramItem* d_items, int nitems, double* G, cudaStream_t s) {
     if (nitems == 0) return;
-    size_t smem = (size_t)3 * GCH * (1 << g.dim) * ldphi * sizeof(double);
-    if (smem > 48 * 1024) raise_smem_limit(k_patch_gram, smem);
-    k_patch_gram<<<nitems, 256, smem, s>>>(g, d_fine, Phi, d_phioff, ldphi, d_m, d_items, G);
+    const size_t smem = sizeof(double) * ((size_t)(g.dim == 3 ? 27 : 9) * GN + 2 * (size_t)GN * ldphi) + sizeof(int) * GN;
+    if (g.dim == 3) k_patch_gram<3><<<nitems, 256, smem, s>>>(g, d_fine, Phi, d_phioff, ldphi, d_m, d_items, G);
+    else k_patch_gram<2><<<nitems, 256, smem, s>>>(g, d_fine, Phi, d_phioff, ldphi, d_m, d_items, G);
     MSDD_LAUNCH_CHECK();
 }
 

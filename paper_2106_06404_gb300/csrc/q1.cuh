@@ -161,7 +161,8 @@ void make_coarse_basis(const Geom& g, const ProbBox* d_boxes, const int* d_count
 struct GramItem {
     int elo[3], ehi[3];
     int j, jj;
-    long long goff;
+    long long goff;      // block (j, jj), row-major m_j x m_jj
+    long long goff_t;    // block (jj, j), its transpose; -1 for j == jj
 };
 void patch_gram(const Geom& g, const ProbBox* d_fine, const double* Phi, const long long* d_phioff, int ldphi,
                 const int* d_m, const GramItem* d_items, int nitems, double* G, cudaStream_t s);
