@@ -274,15 +274,6 @@ __global__ void __launch_bounds__(TPB) k_tile_solve(
 }
 
 
-// ------------------------------------------------------------------ solve, one right-hand side
-// The PCG local solves.  One CTA of 128 threads per matrix; the whole local
-// vector lives in shared memory.  Forward sweep: thread (row r = t/4, chunk
-// t%4) reads 8 contiguous entries of row r of each tile (coalesced) and the 4
-// partial sums of a row are combined by warp shuffles.  Backward sweep uses
-// the transposed tiles: thread (column c = lane, rows 8*warp..) reads tile
-// rows contiguously across the warp, partial sums of the 4 warps are combined
-// in shared memory.  For band matrices (kb <= KBP) the tiles of step R+1 are
-// loaded into registers while step R computes.
 // ------------------------------------------------------------------ factor, right-looking
 // Dense batches (coarse-level matrices) and FP64 bands are factored one tile
 // column k per launch triple, so that many CTAs share each step instead of
@@ -635,130 +626,8 @@ __global__ void __launch_bounds__(FB_T) k_tile_factor_band32(
 
 constexpr int S1T = 128;
 
-constexpr int S1_STAGES = 4;
-
-template <typename T, int KBP>
-constexpr size_t solve1_ring_bytes() { return sizeof(T) * (size_t)S1_STAGES * (KBP + 1) * NB2; }
-
-template <typename T, int KBP>
-__global__ void __launch_bounds__(S1T) k_tile_solve1(
-    const T* __restrict__ tiles, const T* __restrict__ dinv, const int* __restrict__ kb_, const int* __restrict__ K_,
-    const long long* __restrict__ toff_, const long long* __restrict__ roff_, double* __restrict__ X,
-    const int* __restrict__ gdone)
-{
-    // The tiles of step R + S1_STAGES - 1 are copied into a shared ring with
-    // cp.async while step R computes; zs holds the whole local vector.
-    constexpr int NST = S1_STAGES;
-    extern __shared__ __align__(16) unsigned char zs_raw[];
-    T* ring = reinterpret_cast<T*>(zs_raw);                       // [NST][KBP + 1][32 * 32]
-    T* zs = ring + (size_t)NST * (KBP + 1) * NB2;                 // [K * 32]
-    __shared__ T accs[NB];
-    __shared__ T part[S1T / 32][NB + 1];
-    if (gdone && *gdone) return;
-    const int i = blockIdx.x;
-    const int kb = kb_[i], K = K_[i];
-    const long long toff = toff_[i], roff = roff_[i];
-    const int t = threadIdx.x;
-    auto stage = [&](int st, int d) { return ring + ((size_t)st * (KBP + 1) + d) * NB2; };
-    auto issue = [&](int st, int R, bool fwd) {
-        if (R >= 0 && R < K) {
-            for (int d = 0; d <= KBP; ++d) {
-                const int other = fwd ? R - d : R + d;
-                if (d > kb || other < 0 || other >= K) continue;
-                const T* src = tiles + (fwd ? tile_index(toff, kb, R, other) : tile_index(toff, kb, other, R));
-                T* dst = stage(st, d);
-                constexpr int PER = 16 / (int)sizeof(T);
-                for (int ch = t; ch < NB2 / PER; ch += S1T) cp_async16(dst + ch * PER, src + ch * PER);
-            }
-        }
-        cp_async_commit();
-    };
-    for (int k = 0; k < NST - 1; ++k) issue(k, k, true);
-    for (int e = t; e < K * NB; e += S1T) zs[e] = from_f64<T>(X[roff + e]);
-
-    // forward: z_R = T_R (x_R - sum_{J<R} L_RJ z_J); thread (row r = t/4,
-    // columns c0..c0+7) with the 4 partial sums of a row combined by shuffles
-    {
-        const int r = t >> 2, c0 = (t & 3) * 8;
-        for (int R = 0; R < K; ++R) {
-            const int st = R % NST;
-            cp_async_wait_n<NST - 2>();
-            __syncthreads();
-            issue((R + NST - 1) % NST, R + NST - 1, true);
-            T acc = T(0);
-#pragma unroll
-            for (int d = 1; d <= KBP; ++d) {
-                if (d > kb || R - d < 0) continue;
-                const T* lt = stage(st, d) + r * NB + c0;
-                const T* zj = zs + (R - d) * NB + c0;
-#pragma unroll
-                for (int q = 0; q < 8; ++q) acc += lt[q] * zj[q];
-            }
-            acc += __shfl_xor_sync(0xffffffffu, acc, 1);
-            acc += __shfl_xor_sync(0xffffffffu, acc, 2);
-            if ((t & 3) == 0) accs[r] = zs[R * NB + r] - acc;
-            __syncthreads();
-            const T* tt = stage(st, 0) + r * NB + c0;
-            T s = T(0);
-#pragma unroll
-            for (int q = 0; q < 8; ++q) s += tt[q] * accs[c0 + q];
-            s += __shfl_xor_sync(0xffffffffu, s, 1);
-            s += __shfl_xor_sync(0xffffffffu, s, 2);
-            if ((t & 3) == 0) zs[R * NB + r] = s;
-        }
-    }
-    cp_async_wait_n<0>();
-    __syncthreads();
-    for (int k = 0; k < NST - 1; ++k) issue(k, K - 1 - k, false);
-    for (int e = t; e < K * NB; e += S1T) zs[e] *= dinv[roff + e];
-    // backward: x_R = T_R^T (D_R^{-1} z_R - sum_{I>R} L_IR^T x_I); thread
-    // (column = lane, rows k0..k0+7 of the tile), warps combined in shared memory
-    {
-        const int lane = t & 31, warp = t >> 5, k0 = warp * 8;
-        for (int R = K - 1, it = 0; R >= 0; --R, ++it) {
-            const int st = it % NST;
-            cp_async_wait_n<NST - 2>();
-            __syncthreads();
-            issue((it + NST - 1) % NST, R - (NST - 1), false);
-            T s = T(0);
-#pragma unroll
-            for (int d = 1; d <= KBP; ++d) {
-                if (d > kb || R + d >= K) continue;
-                const T* lt = stage(st, d) + k0 * NB + lane;
-                const T* xi = zs + (R + d) * NB + k0;
-#pragma unroll
-                for (int q = 0; q < 8; ++q) s += lt[q * NB] * xi[q];
-            }
-            part[warp][lane] = s;
-            __syncthreads();
-            if (warp == 0) {
-                T v = T(0);
-#pragma unroll
-                for (int w = 0; w < S1T / 32; ++w) v += part[w][lane];
-                accs[lane] = zs[R * NB + lane] - v;
-            }
-            __syncthreads();
-            const T* tt = stage(st, 0) + k0 * NB + lane;
-            T s2 = T(0);
-#pragma unroll
-            for (int q = 0; q < 8; ++q) s2 += tt[q * NB] * accs[k0 + q];
-            part[warp][lane] = s2;
-            __syncthreads();
-            if (warp == 0) {
-                T v = T(0);
-#pragma unroll
-                for (int w = 0; w < S1T / 32; ++w) v += part[w][lane];
-                zs[R * NB + lane] = v;
-            }
-        }
-    }
-    cp_async_wait_n<0>();
-    __syncthreads();
-    for (int e = t; e < K * NB; e += S1T) X[roff + e] = to_f64(zs[e]);
-}
-
-// One right-hand side, any kb (dense coarse matrices): tiles are read as
-// needed without prefetch; same thread mappings as above.
+// One right-hand side where the streamed kernels below do not fit (very wide
+// bands, dense matrices): tiles are read as needed without prefetch.
 template <typename T>
 __global__ void __launch_bounds__(S1T) k_tile_solve1_dense(
     const T* __restrict__ tiles, const T* __restrict__ dinv, const int* __restrict__ kb_, const int* __restrict__ K_,
@@ -1863,7 +1732,8 @@ void launch_band_split(const TileBatch& tb, const CUtensorMap& tm, double* X, cu
 // Measured: 256 problems of n = 1369, b = 38 with cold caches 60 -> 53 us (DRAM
 // from there on), with the factors in L2 59 -> 32 us; 128 of them 57 -> 29 us.
 constexpr int S1W_W = 4, S1W_NST = 2 * S1W_W;
-__device__ __forceinline__ void tma_load_cols8(void* dst, const CUtensorMap* map, int col, int row,
+// the box of a tile map at (col, row)
+__device__ __forceinline__ void tma_load_box(void* dst, const CUtensorMap* map, int col, int row,
                                                unsigned long long* bar) {
     asm volatile(
         "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];\n" ::"r"(
@@ -1926,7 +1796,7 @@ __global__ void __launch_bounds__(32 * S1W_W) k_tile_solve1_warp(
         if (nd > 1) {
             const long long ti = fwd ? tile_index(toff, kb, R, R - 2) : tile_index(toff, kb, R + 2, R);
             for (int q = 0; q < nb; ++q)
-                tma_load_cols8(dst + 2 * NB2 + q * 8 * NB, &tmc, 8 * (g0 + q), (int)(ti / NB), &full[st]);
+                tma_load_box(dst + 2 * NB2 + q * 8 * NB, &tmc, 8 * (g0 + q), (int)(ti / NB), &full[st]);
         }
     };
     issue(0);
@@ -2035,6 +1905,187 @@ __global__ void __launch_bounds__(32 * S1W_W) k_tile_solve1_warp(
     for (int e = t; e < K * NB; e += NTC) X[roff + e] = f32_to_f64(zs[e]);
 }
 
+// ---- one right-hand side, FP64 bands (the local solves of the plain form)
+// A DFMA holds a scheduler's FP64 pipe for some 67 cycles whatever its active
+// lanes, so a step's products are spread over four warps (four pipes) by k:
+// warp w multiplies columns 8 w .. 8 w + 7 of every tile, lane = row, and the
+// partial sums are exchanged through shared memory.  Warp w then sums and
+// finishes exactly the rows 8 w .. 8 w + 7 that it multiplies next, as its
+// k-slice of T_R and of the next step's nearest tile: two barriers and two
+// two-level sums a step, where every lane group of a row summing its own part
+// with each product took 3700 cycles a step at kb = 2.  The columns of the
+// outermost tile that lie in the band are dealt out singly.  A fifth warp
+// streams the tiles by TMA in halves of 16 columns (128-byte swizzle), of the
+// outermost tile only the halves that hold nonzeros.  Waits and time-outs as in
+// k_tile_solve_band_ks.
+// Measured (warm L2): 144 problems of n = 1296, b = 37 147 -> 125 us, 27 of
+// n = 1728, b = 157 331 -> 295 us.
+constexpr int S1D_W = 4, S1D_HALF = NB * 16;           // doubles of a half tile
+__host__ __device__ constexpr size_t s1d_bytes(int S, int nst, int K) {
+    return 1024 + sizeof(double) * ((size_t)nst * S * NB2 + 2 * S1D_W * NB + NB + (size_t)K * NB);
+}
+
+__global__ void __launch_bounds__(32 * (S1D_W + 1)) k_tile_solve1_f64(
+    const __grid_constant__ CUtensorMap tmt, const double* __restrict__ dinv, const int* __restrict__ kb_,
+    const int* __restrict__ K_, const int* __restrict__ b_, const long long* __restrict__ toff_,
+    const long long* __restrict__ roff_, double* __restrict__ X, const int* __restrict__ gdone, int S, int nst)
+{
+    extern __shared__ unsigned char smem_raw[];
+    unsigned char* base = smem_raw + ((1024 - (smem_u32(smem_raw) & 1023)) & 1023);
+    double* St = reinterpret_cast<double*>(base);            // [nst][S][2][32][16]
+    double* P1 = St + (size_t)nst * S * NB2;                 // [4][32] partial sums
+    double* P2 = P1 + S1D_W * NB;
+    double* Ac = P2 + S1D_W * NB;                            // [32]
+    double* zs = Ac + NB;                                    // [K * 32]
+    __shared__ unsigned long long full[4], empty[4];
+    __shared__ int s_abort, s_stop;
+    if (gdone && *gdone) return;
+    const int i = blockIdx.x;
+    const int kb = kb_[i], K = K_[i], bw = b_[i];
+    if (kb >= S || K == 0) return;                           // never launched so (host dispatch)
+    const long long toff = toff_[i], roff = roff_[i];
+    const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
+    const int k_out = max(0, NB * kb - bw);                  // columns of the outermost tile before it are zero
+    const int h_out = k_out >> 4;                            // its first half with nonzeros
+    if (t == 0) {
+        s_abort = 0;
+        s_stop = 0;
+        for (int s = 0; s < nst; ++s) {
+            mbar_init(&full[s], 1);
+            mbar_init(&empty[s], S1D_W);
+        }
+        fence_mbar_init();
+    }
+    for (int e = t; e < K * NB; e += 32 * (S1D_W + 1)) zs[e] = X[roff + e];
+    __syncthreads();
+    auto give_up = [&]() {
+        if (atomicExch(&s_abort, 1) == 0) atomicAdd(&g_wait_timeouts, 1);
+    };
+    const int total = 2 * K;
+
+    if (warp == S1D_W) {
+        // ---------------- producer: one lane issues every copy
+        if (lane == 0) {
+            unsigned pending = 0, par = 0, ph = 0;
+            int st = 0;
+            for (int it = 0; it < total; ++it) {
+                if (it >= nst) {
+                    if (!mbar_wait_bounded(&empty[st], ((ph >> st) & 1u) ^ 1u)) { give_up(); break; }
+                    pending &= ~(1u << st);
+                }
+                if (*(volatile int*)&s_abort) break;
+                const bool fwd = it < K;
+                const int R = fwd ? it : total - 1 - it, nd = min(kb, fwd ? R : K - 1 - R);
+                const int skipped = nd == kb && kb > 0 ? h_out : 0;
+                double* dst = St + (size_t)st * S * NB2;
+                mbar_expect_tx(&full[st], (2 * (nd + 1) - skipped) * S1D_HALF * 8);
+                for (int d = nd; d >= 0; --d) {
+                    const long long ti = fwd ? tile_index(toff, kb, R, R - d) : tile_index(toff, kb, R + d, R);
+                    for (int h = d == kb && kb > 0 ? h_out : 0; h < 2; ++h)
+                        tma_load_box(dst + (size_t)d * NB2 + h * S1D_HALF, &tmt, 16 * h, (int)(ti / NB), &full[st]);
+                }
+                pending |= 1u << st;
+                par = (par & ~(1u << st)) | (((ph >> st) & 1u) << st);
+                ph ^= 1u << st;
+                st = st + 1 == nst ? 0 : st + 1;
+            }
+            // after an abort, copies still in flight must land before the CTA exits
+            if (*(volatile int*)&s_abort)
+                for (int s = 0; s < nst; ++s)
+                    if (pending & (1u << s)) mbar_wait_bounded(&full[s], (par >> s) & 1u);
+        }
+        return;
+    }
+
+    // ---------------- consumer warps
+    auto consumers_sync = [&]() { asm volatile("bar.sync 1, %0;\n" ::"r"(32 * S1D_W) : "memory"); };
+    // a0 += columns 8 w .. 8 w + 7 (rows, backward) of a tile times v[8 w ..]: lane = row (column).  One chain: a
+    // dependent DFMA starts as soon as the pipe is free
+    double a0;
+    auto slice = [&](const double* T, const double* v, bool fwd) {
+        const double2* vv = reinterpret_cast<const double2*>(v + 8 * warp);
+        if (fwd) {
+            const double* Tr = T + (warp >> 1) * S1D_HALF + lane * 16;
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                const double2 l = *reinterpret_cast<const double2*>(Tr + (((4 * (warp & 1) + c) ^ (lane & 7)) << 1));
+                const double2 x = vv[c];
+                a0 = fma(l.x, x.x, a0);
+                a0 = fma(l.y, x.y, a0);
+            }
+        } else {
+            const double* Tc = T + (lane >> 4) * S1D_HALF + (lane & 1);
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                const int k = 8 * warp + 2 * c;
+                const double2 x = vv[c];
+                a0 = fma(Tc[k * 16 + ((((lane >> 1) & 7) ^ (k & 7)) << 1)], x.x, a0);
+                a0 = fma(Tc[(k + 1) * 16 + ((((lane >> 1) & 7) ^ ((k + 1) & 7)) << 1)], x.y, a0);
+            }
+        }
+    };
+    const int row = 8 * warp + (lane >> 2), part = lane & 3;  // the slice's row that this lane helps to sum
+    auto sum4 = [&](const double* P) {
+        double v = P[part * NB + row];
+        v += __shfl_xor_sync(0xffffffffu, v, 1);
+        v += __shfl_xor_sync(0xffffffffu, v, 2);
+        return v;
+    };
+    int st = 0;
+    unsigned ph = 0;
+    for (int it = 0; it < total; ++it) {
+        const bool fwd = it < K;
+        const int R = fwd ? it : total - 1 - it, sg = fwd ? -1 : 1, nd = min(kb, fwd ? R : K - 1 - R);
+        const double dv = fwd ? 1.0 : dinv[roff + (long long)R * NB + row];
+        const double* tiles = St + (size_t)st * S * NB2;
+        const bool ok = mbar_wait_bounded(&full[st], (ph >> st) & 1u);
+        if (!ok) give_up();
+        a0 = 0.0;
+        if (ok) {
+            for (int d = 2; d <= nd; ++d) {
+                const double *T = tiles + (size_t)d * NB2, *z = zs + (R + sg * d) * NB;
+                if (d < kb) {
+                    slice(T, z, fwd);
+                } else if (fwd) {                            // columns k_out .. 31, dealt out
+                    for (int k = k_out + warp; k < NB; k += S1D_W)
+                        a0 = fma(T[(k >> 4) * S1D_HALF + lane * 16 + ((((k >> 1) & 7) ^ (lane & 7)) << 1) + (k & 1)],
+                                 z[k], a0);
+                } else if (lane >> 4 >= h_out) {             // rows 0 .. 31 - k_out, dealt out
+                    for (int k = warp; k < NB - k_out; k += S1D_W)
+                        a0 = fma(T[(lane >> 4) * S1D_HALF + k * 16 + ((((lane >> 1) & 7) ^ (k & 7)) << 1) + (lane & 1)],
+                                 z[k], a0);
+                }
+            }
+            if (nd > 0) {
+                // (kb = 1: the halves that were not copied hold zeros of the band)
+                const double *T = tiles + NB2, *z = zs + (R + sg) * NB;
+                if (kb > 1) slice(T, z, fwd);
+                else if (fwd ? (warp >> 1) >= h_out : (lane >> 4) >= h_out) slice(T, z, fwd);
+            }
+        }
+        P1[warp * NB + lane] = a0;
+        consumers_sync();                                    // every partial sum is in P1
+        const double y = fma(dv, zs[R * NB + row], -sum4(P1));
+        if (part == 0) Ac[row] = y;
+        __syncwarp();
+        a0 = 0.0;
+        if (ok) slice(tiles, Ac, fwd);
+        P2[warp * NB + lane] = a0;
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&empty[st]);
+        if (t == 0) *(volatile int*)&s_stop = *(volatile int*)&s_abort;
+        consumers_sync();                                    // every partial of the solution is in P2
+        if (*(volatile int*)&s_stop) break;                  // sampled once: every warp leaves after this step
+        const double z = sum4(P2);
+        if (part == 0) zs[R * NB + row] = z;
+        __syncwarp();
+        ph ^= 1u << st;
+        st = st + 1 == nst ? 0 : st + 1;
+    }
+    consumers_sync();
+    for (int e = t; e < K * NB; e += 32 * S1D_W) X[roff + e] = zs[e];
+}
+
 using EncodeTiledFn = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
                                    const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
                                    CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
@@ -2064,17 +2115,17 @@ bool encode_tile_map(const float* base, long long elems, CUtensorMap* m) {
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// [elems / 32][32] FP32 view, boxes of 8 columns x 32 rows, plain layout.
-bool encode_cols8_map(const float* base, long long elems, CUtensorMap* m) {
+// [elems / 32][32] view, boxes of `cols` columns x 32 rows.
+bool encode_box_map(const void* base, CUtensorMapDataType type, size_t esize, long long elems, int cols,
+                    CUtensorMapSwizzle swizzle, CUtensorMap* m) {
     EncodeTiledFn enc = encode_tiled();
     if (!enc || !base || elems <= 0) return false;
     const cuuint64_t dims[2] = {(cuuint64_t)NB, (cuuint64_t)(elems / NB)};
-    const cuuint64_t strides[1] = {(cuuint64_t)NB * sizeof(float)};
-    const cuuint32_t box[2] = {8, (cuuint32_t)NB};
+    const cuuint64_t strides[1] = {(cuuint64_t)NB * esize};
+    const cuuint32_t box[2] = {(cuuint32_t)cols, (cuuint32_t)NB};
     const cuuint32_t estr[2] = {1, 1};
-    return enc(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, (void*)base, dims, strides, box, estr,
-               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_NONE,
-               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+    return enc(m, type, 2, (void*)base, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle,
+               CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
 // The tile descriptor of an FP32 batch (built once per tiles_f allocation).
@@ -2314,7 +2365,8 @@ void tile_solve(const TileBatch& tb, double* X, int ldx, int ncols, const int* s
                 if (tb.kb[i] == 2) nbox = std::max(nbox, 4 - s1w_group0(tb.b[i]));
             const size_t bytes = 1024 + sizeof(float) * ((size_t)S1W_NST * (2 * NB2 + nbox * 8 * NB) +
                                                          (size_t)S1W_W * nbox * 8 * NB + NB + (size_t)tb.max_K * NB);
-            if (tm && bytes <= 200 * 1024 && encode_cols8_map(tb.tiles_f.p, tb.total_tile_elems, &tc)) {
+            if (tm && bytes <= 200 * 1024 && encode_box_map(tb.tiles_f.p, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, tb.total_tile_elems, 8,
+                                                              CU_TENSOR_MAP_SWIZZLE_NONE, &tc)) {
                 raise_smem_limit(k_tile_solve1_warp, bytes);
                 k_tile_solve1_warp<<<tb.P, 32 * S1W_W, bytes, s>>>(*tm, tc, tb.dinv_f.p, tb.d_kb.p, tb.d_K.p, tb.d_b.p,
                                                           tb.d_toff.p, tb.d_roff.p, X, gdone, nbox);
@@ -2322,13 +2374,20 @@ void tile_solve(const TileBatch& tb, double* X, int ldx, int ncols, const int* s
                 return;
             }
         }
-        const size_t ring_bytes = (maxkb <= 1 ? solve1_ring_bytes<double, 1>() : solve1_ring_bytes<double, 2>()) + zbytes;
-        if (!tb.prec && maxkb <= 2 && ring_bytes <= 200 * 1024) {
-            auto k = maxkb <= 1 ? k_tile_solve1<double, 1> : k_tile_solve1<double, 2>;
-            raise_smem_limit(k, ring_bytes);
-            k<<<tb.P, S1T, ring_bytes, s>>>(tb.tiles_d.p, tb.dinv_d.p, tb.d_kb.p, tb.d_K.p, tb.d_toff.p, tb.d_roff.p, X, gdone);
-            MSDD_LAUNCH_CHECK();
-            return;
+        if (!tb.prec) {
+            int nst = 4;
+            while (nst > 2 && s1d_bytes(maxkb + 1, nst, tb.max_K) > 200 * 1024) --nst;
+            const size_t bytes = s1d_bytes(maxkb + 1, nst, tb.max_K);
+            alignas(64) CUtensorMap tm;
+            if (bytes <= 226 * 1024 && encode_box_map(tb.tiles_d.p, CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 8,
+                                                      tb.total_tile_elems, 16, CU_TENSOR_MAP_SWIZZLE_128B, &tm)) {
+                raise_smem_limit(k_tile_solve1_f64, bytes);
+                k_tile_solve1_f64<<<tb.P, 32 * (S1D_W + 1), bytes, s>>>(tm, tb.dinv_d.p, tb.d_kb.p, tb.d_K.p, tb.d_b.p,
+                                                                       tb.d_toff.p, tb.d_roff.p, X, gdone, maxkb + 1,
+                                                                       nst);
+                MSDD_LAUNCH_CHECK();
+                return;
+            }
         }
         if (tb.prec && maxkb > 2 && maxkb <= 12) {
             // wide bands, one right-hand side (PCG local solves of 3D boxes):
@@ -2339,7 +2398,7 @@ void tile_solve(const TileBatch& tb, double* X, int ldx, int ncols, const int* s
                 return;
             }
         }
-        if ((maxkb > 2 || tb.prec) && zbytes <= 160 * 1024) {
+        if (zbytes <= 160 * 1024) {
             if (zbytes > 48 * 1024) {
                 raise_smem_limit(k_tile_solve1_dense<float>, zbytes);
                 raise_smem_limit(k_tile_solve1_dense<double>, zbytes);
