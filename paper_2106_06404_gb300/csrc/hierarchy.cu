@@ -16,7 +16,6 @@
 #include <chrono>
 #include <cmath>
 #include <cstring>
-#include <map>
 
 namespace msdd {
 
@@ -798,23 +797,51 @@ void Hierarchy::build_coarse() {
     patch_gram(g, d_fboxes.p, Phi.p, d_phioff.p, ldphi, d_fm.p, d_gitems.p, (int)gram_items.size(), G.p, st);
 
     // ---- Galerkin matrix of level L-1: block (j, jj) = sum over patches holding both
-    std::map<std::pair<int, int>, std::vector<long long>> pairc;
-    for (size_t k = 0; k < gitems.size(); ++k) pairc[{gitems[k].j, gitems[k].jj}].push_back(gitems[k].goff);
-    {
-        std::vector<SumItem> si;
-        std::vector<long long> contrib;
-        for (auto& kv : pairc) {
-            int j = kv.first.first, jj = kv.first.second;
+    // (pairs grouped by counting on j and small sorts on jj: ordered maps took
+    // 4.4 of 9.4 ms of the coarse assembly at 1000^2)
+    struct PairRef {
+        int j, jj;
+        long long goff;
+    };
+    std::vector<PairRef> sorted;
+    std::vector<int> cnt;
+    auto group_pairs = [&](std::vector<PairRef>& v) {         // by (j, jj), equal pairs in their order
+        cnt.assign(Pf + 1, 0);
+        for (const PairRef& r : v) ++cnt[r.j + 1];
+        for (int j = 0; j < Pf; ++j) cnt[j + 1] += cnt[j];
+        sorted.resize(v.size());
+        for (const PairRef& r : v) sorted[cnt[r.j]++] = r;     // cnt[j]: end of j's segment afterwards
+        v.swap(sorted);
+        for (int j = 0, at = 0; j < Pf; at = cnt[j], ++j)
+            std::stable_sort(v.begin() + at, v.begin() + cnt[j],
+                             [](const PairRef& x, const PairRef& y) { return x.jj < y.jj; });
+    };
+    // one SumItem per pair, placed by place(j, jj, item), from grouped pairs
+    auto sum_items = [&](const std::vector<PairRef>& v, auto place, std::vector<SumItem>& si,
+                         std::vector<long long>& contrib) {
+        for (size_t k = 0; k < v.size();) {
+            const int j = v[k].j, jj = v[k].jj;
             SumItem it;
-            it.doff = c1off[j] * n1 + c1off[jj];
-            it.ld = (int)n1;
             it.rows = fm[j];
             it.cols = fm[jj];
+            place(j, jj, it);
             it.cbeg = (int)contrib.size();
-            for (long long c : kv.second) contrib.push_back(c);
+            for (; k < v.size() && v[k].j == j && v[k].jj == jj; ++k) contrib.push_back(v[k].goff);
             it.cend = (int)contrib.size();
             si.push_back(it);
         }
+    };
+    {
+        std::vector<PairRef> pairs;
+        pairs.reserve(gitems.size());
+        for (const GramItem& it : gitems) pairs.push_back({it.j, it.jj, it.goff});
+        group_pairs(pairs);
+        std::vector<SumItem> si;
+        std::vector<long long> contrib;
+        sum_items(pairs, [&](int j, int jj, SumItem& it) {
+            it.doff = c1off[j] * n1 + c1off[jj];
+            it.ld = (int)n1;
+        }, si, contrib);
         A1.alloc(n1 * n1);
         A1.zero(st);
         DevBuf<SumItem> d_si = upload_vec(si, st);
@@ -931,29 +958,28 @@ void Hierarchy::build_coarse() {
     {
         std::vector<SumItem> si;
         std::vector<long long> contrib;
-        for (int i = 0; i < Pm; ++i) {
-            std::map<std::pair<int, int>, std::vector<long long>> pc;
-            for (size_t k = 0; k < gitems.size(); ++k) {
-                int j = gitems[k].j, jj = gitems[k].jj;
-                if (genoff[i][j] < 0 || genoff[i][jj] < 0) continue;
-                bool touches = false;
+        // the pairs of a patch go to every group that owns one of its subdomains
+        std::vector<int> owner(Pf, -1), touched;
+        for (int i = 0; i < Pm; ++i)
+            for (int j : members[i]) owner[j] = i;
+        std::vector<std::vector<PairRef>> pc(Pm);
+        for (size_t k = 0; k < gitems.size(); ++k) {
+            if (k == 0 || gpatch[k] != gpatch[k - 1]) {
+                touched.clear();
                 for (int mbr : patches[gpatch[k]].mem)
-                    if (isown[i][mbr]) { touches = true; break; }
-                if (!touches) continue;
-                pc[{j, jj}].push_back(gitems[k].goff);
+                    if (std::find(touched.begin(), touched.end(), owner[mbr]) == touched.end())
+                        touched.push_back(owner[mbr]);
             }
-            for (auto& kv : pc) {
-                int j = kv.first.first, jj = kv.first.second;
-                SumItem it;
+            for (int i : touched)
+                if (genoff[i][gitems[k].j] >= 0 && genoff[i][gitems[k].jj] >= 0)
+                    pc[i].push_back({gitems[k].j, gitems[k].jj, gitems[k].goff});
+        }
+        for (int i = 0; i < Pm; ++i) {
+            group_pairs(pc[i]);
+            sum_items(pc[i], [&](int j, int jj, SumItem& it) {
                 it.doff = aoff[i] + (long long)genoff[i][j] * ngen[i] + genoff[i][jj];
                 it.ld = ngen[i];
-                it.rows = fm[j];
-                it.cols = fm[jj];
-                it.cbeg = (int)contrib.size();
-                for (long long c : kv.second) contrib.push_back(c);
-                it.cend = (int)contrib.size();
-                si.push_back(it);
-            }
+            }, si, contrib);
         }
         DevBuf<SumItem> d_si = upload_vec(si, st);
         DevBuf<long long> d_contrib = upload_vec(contrib, st);
