@@ -395,6 +395,20 @@ __device__ void block_jacobi(T (*S)[LD], T (*V)[LD], int q, T rel_tol, T floor_r
     __shared__ int sa[2][PMAX / 2], sb[2][PMAX / 2], sr[2][PMAX / 2];
     __shared__ double s_scale;
     const int t = threadIdx.x, h = q / 2;
+    // this thread's share of a step, the same in every step: 2 x 2 blocks of S
+    // (pair j rows, pair jj columns), then entries (row j, pair jj) of V; the
+    // index divisions took a third of a step
+    constexpr int NI = (PMAX / 2 * (PMAX / 2) + PMAX * PMAX / 2 + TPB - 1) / TPB;
+    const int nblk = h * h, nitem = nblk + q * h;
+    int ij[NI], ijj[NI];
+#pragma unroll
+    for (int z = 0; z < NI; ++z) {
+        const int e = t + z * TPB, e2 = e < nblk ? e : e - nblk;
+        ij[z] = e2 / h;
+        ijj[z] = e2 % h;
+    }
+    // circle method: position 0 fixed, the others rotate by one a step (a sweep is a full turn)
+    int pa = t - 1, pb = q - 2 - t;
     for (int e = t; e < q * q; e += TPB) V[e / q][e % q] = (e / q == e % q) ? T(1) : T(0);
     if (t < 32) {
         double m = 0.0;
@@ -418,10 +432,9 @@ __device__ void block_jacobi(T (*S)[LD], T (*V)[LD], int q, T rel_tol, T floor_r
         for (int step = 0; step < q - 1; ++step, par ^= 1) {
             int rot = 0;
             if (t < h) {
-                // circle method: position 0 fixed, the others rotate
-                int pos1 = t, pos2 = q - 1 - t;
-                int a = pos1 == 0 ? 0 : 1 + (pos1 - 1 + step) % (q - 1);
-                int b = 1 + (pos2 - 1 + step) % (q - 1);
+                int a = t == 0 ? 0 : 1 + pa, b = 1 + pb;
+                pa = pa + 1 == q - 1 ? 0 : pa + 1;
+                pb = pb + 1 == q - 1 ? 0 : pb + 1;
                 if (a > b) { int tmp = a; a = b; b = tmp; }
                 T c = T(1), s = T(0);
                 rot = pair_active<T>(S[a][a], S[b][b], S[a][b], rel_tol, floor_abs) ? 1 : 0;
@@ -430,10 +443,11 @@ __device__ void block_jacobi(T (*S)[LD], T (*V)[LD], int q, T rel_tol, T floor_r
             }
             // (integer flags: FP64 comparisons would occupy the narrow FP64 pipe)
             if (!__syncthreads_or(rot)) continue;
-            const int nblk = h * h;
-            for (int e = t; e < nblk + q * h; e += TPB) {
+#pragma unroll
+            for (int z = 0; z < NI; ++z) {
+                const int e = t + z * TPB, j = ij[z], jj = ijj[z];
+                if (e >= nitem) break;
                 if (e < nblk) {
-                    const int j = e / h, jj = e % h;
                     if (!(sr[par][j] | sr[par][jj])) continue;
                     const T sj = ss[par][j], sjj = ss[par][jj];
                     const T cj = sc[par][j], cjj = sc[par][jj];
@@ -446,14 +460,13 @@ __device__ void block_jacobi(T (*S)[LD], T (*V)[LD], int q, T rel_tol, T floor_r
                     if (sizeof(T) == 4 && j == jj) { n12 = T(0); n21 = T(0); }        // exact angle: annihilated
                     S[x1][y1] = n11; S[x1][y2] = n12; S[x2][y1] = n21; S[x2][y2] = n22;
                 } else {
-                    const int e2 = e - nblk, k = e2 / h, jj = e2 % h;
                     if (!sr[par][jj]) continue;
                     const T sjj = ss[par][jj];
                     const T cjj = sc[par][jj];
                     const int y1 = sa[par][jj], y2 = sb[par][jj];
-                    const T u = V[k][y1], v = V[k][y2];
-                    V[k][y1] = cjj * u - sjj * v;
-                    V[k][y2] = sjj * u + cjj * v;
+                    const T u = V[j][y1], v = V[j][y2];
+                    V[j][y1] = cjj * u - sjj * v;
+                    V[j][y2] = sjj * u + cjj * v;
                 }
             }
             __syncthreads();
@@ -550,6 +563,148 @@ __device__ __forceinline__ void smem_gemm_f(float (*D)[LD], const float (*E)[LD]
     }
 }
 
+// One warp: FP32 Cholesky M = R^T R (upper R) of the symmetric q x q matrix in
+// G (overwritten) and U = R^{-T}, lower triangular, zero above (q <= PB).  Lane
+// b holds column b in registers and exchanges a row of R through G per step: 3
+// to 4 thousand cycles where rows in shared memory with run-time loops took 11
+// (q = 10) to 29 (q = 20) thousand.  Returns whether every pivot exceeds 1e-3.
+template <int PB>
+__device__ bool chol_inverse_warp(float (*G)[LD], float (*U)[LD], int q) {
+    const int b = threadIdx.x & 31;
+    float g[PB], rinv[PB], x[PB];
+#pragma unroll
+    for (int a = 0; a < PB; ++a) g[a] = a < q && b < q ? G[a][b] : (a == b ? 1.f : 0.f);
+    __syncwarp();
+    bool ok = true;
+#pragma unroll
+    for (int k = 0; k < PB; ++k) {
+        const float piv = __shfl_sync(0xffffffffu, g[k], k);
+        ok = ok && piv > 1e-3f;
+        float r = rsqrtf(fmaxf(piv, 1e-30f));
+        r = r * fmaf(-0.5f * piv * r, r, 1.5f);
+        rinv[k] = r;
+        const float u = b >= k ? g[k] * r : 0.f;               // R[k][b]
+        G[k][b] = u;
+        __syncwarp();
+#pragma unroll
+        for (int a = k + 1; a < PB; ++a) g[a] = fmaf(-G[k][a], u, g[a]);
+    }
+    // column b of R^{-1}, from the last row up
+#pragma unroll
+    for (int a = 0; a < PB; ++a) x[a] = a == b ? 1.f : 0.f;
+#pragma unroll
+    for (int j = PB - 1; j >= 0; --j) {
+        x[j] *= rinv[j];
+#pragma unroll
+        for (int a = 0; a < j; ++a) x[a] = fmaf(-G[a][j], x[j], x[a]);
+    }
+    if (b < q)
+#pragma unroll
+        for (int a = 0; a < PB; ++a)
+            if (a < q) U[b][a] = x[a];                         // zero for a > b
+    return ok;
+}
+
+// max over the rows of sum_b |K_ab| for K in V, as a float, to every thread
+__device__ float row_sum_norm(const double (*V)[LD], int q, int* s_max) {
+    const int t = threadIdx.x;
+    if (t == 0) *s_max = 0;
+    __syncthreads();
+    if (t < q) {
+        float v = 0.f;
+        for (int b = 0; b < q; ++b) v += fabsf(f64_to_f32(V[t][b]));
+        atomicMax(s_max, v != v ? 0x7f800000 : __float_as_int(v));
+    }
+    __syncthreads();
+    const float v = __int_as_float(*s_max);
+    __syncthreads();
+    return v;
+}
+
+// Diagonalises the nearly diagonal symmetric A (off-diagonals ~1e-6 of the
+// diagonal, from an FP32 eigen-decomposition) and applies the rotation to Z:
+// all Jacobi angles t_ab of A at once, K antisymmetric with K_ab = t_ab,
+// Q = I + K + K^2 / 2, whose orthogonality error is K^4 / 4: rounding for
+// |K| <= 2e-4, else one Newton-Schulz step Q <- Q (3 I - Q^T Q) / 2 squares it.
+// Z <- Z Q, A <- Q^T A Q, until no pair is active by the test of block_jacobi
+// (usually one step of four to six q x q products; a Jacobi sweep, q - 1 steps
+// with rotations of every pair on the FP64 pipe, took 42 (q = 10) to 95 (q =
+// 20) thousand cycles of 125 to 260).  Angles beyond 0.02 (clustered pairs) are
+// left to block_jacobi: false, with A and Z consistent.
+__device__ bool rotate_all(double (*A)[LD], double (*Z)[LD], double (*V)[LD], double (*T)[LD], double (*L)[LD], int q,
+                           double rel_tol, double floor_rel) {
+    __shared__ int s_max;
+    __shared__ float s_scale;
+    const int t = threadIdx.x;
+    for (int step = 0; step < 4; ++step) {
+        if (t < 32) {
+            float m = 0.f;
+            for (int k = t; k < q; k += 32) m = fmaxf(m, fabsf(f64_to_f32(A[k][k])));
+            for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+            if (t == 0) s_scale = m;
+        }
+        __syncthreads();
+        const float rt = (float)rel_tol, fl = fmaxf((float)floor_rel * s_scale, 1e-37f);
+        for (int e = t; e < q * q; e += TPB) {
+            const int a = e / q, b = e % q;
+            if (a > b) continue;
+            float k = 0.f;
+            if (a < b) {
+                const float off = f64_to_f32(A[a][b]);
+                if (pair_active_f(f64_to_f32(A[a][a]), f64_to_f32(A[b][b]), off, rt, fl)) {
+                    const float th = f64_to_f32(A[b][b] - A[a][a]) / (2.f * off);
+                    k = copysignf(1.f, th) / (fabsf(th) + sqrtf(fmaf(th, th, 1.f)));
+                    if (!(fabsf(th) <= 1e15f)) k = 0.5f / th;
+                }
+            }
+            V[a][b] = f32_to_f64(k);
+            V[b][a] = f32_to_f64(-k);
+        }
+        __syncthreads();
+        const float nrm = row_sum_norm(V, q, &s_max);
+        if (nrm == 0.f) return true;
+        if (!(nrm <= 0.02f)) return false;
+        smem_gemm(T, V, V, q, false);                    // K^2
+        __syncthreads();
+        for (int e = t; e < q * q; e += TPB) {
+            const int a = e / q, b = e % q;
+            T[a][b] = fma(0.5, T[a][b], V[a][b] + (a == b ? 1.0 : 0.0));
+        }
+        __syncthreads();
+        const double (*Q)[LD] = T;
+        if (nrm > 2e-4f) {
+            smem_gemm(V, T, T, q, true);                 // Q^T Q
+            __syncthreads();
+            for (int e = t; e < q * q; e += TPB) {
+                const int a = e / q, b = e % q;
+                V[a][b] = fma(-0.5, V[a][b], a == b ? 1.5 : 0.0);
+            }
+            __syncthreads();
+            smem_gemm(L, T, V, q, false);
+            __syncthreads();
+            Q = L;
+        }
+        smem_gemm(V, Z, Q, q, false);                    // Z Q
+        __syncthreads();
+        for (int e = t; e < q * q; e += TPB) Z[e / q][e % q] = V[e / q][e % q];
+        __syncthreads();
+        smem_gemm(V, A, Q, q, false);                    // A Q
+        __syncthreads();
+        smem_gemm(A, Q, V, q, true);                     // Q^T A Q
+        __syncthreads();
+        for (int e = t; e < q * q; e += TPB) {
+            const int a = e / q, b = e % q;
+            if (a < b) {
+                const double v = 0.5 * (A[a][b] + A[b][a]);
+                A[a][b] = v;
+                A[b][a] = v;
+            }
+        }
+        __syncthreads();
+    }
+    return false;
+}
+
 // Rayleigh-Ritz for a well-conditioned scaled pencil (Hs, Ms), FP32 first:
 //   1. FP32 Cholesky Ms = L L^T and U = L^{-1} (warp 0), G = U Hs U^T and its
 //      FP32 Jacobi eigenvectors V; Z = U^T V (so Z^T Ms Z ~ I, Z^T Hs Z ~
@@ -557,16 +712,15 @@ __device__ __forceinline__ void smem_gemm_f(float (*D)[LD], const float (*E)[LD]
 //   2. FP64: Z <- Z P with P = I - E/2 + 3 E^2/8, E = Z^T Ms Z - I (the
 //      second-order inverse square root of I + E: the error drops from |E|
 //      to O(|E|^3)), repeated while |E| > 2e-6 (at most 3 times);
-//   3. FP64 Jacobi on A = Z^T Hs Z (nearly diagonal), Z <- Z Q.
-// Every serial chain runs in FP32 and the FP64 work is seven or so q x q
-// products plus the finishing Jacobi steps.  Returns false (nothing of L and
+//   3. A = Z^T Hs Z is nearly diagonal: rotate_all, or FP64 Jacobi where pairs
+//      are clustered, Z <- Z Q.
+// Every serial chain runs in FP32 and the FP64 work is ten or so q x q products.  Returns false (nothing of L and
 // T changed but a unit dummy pivot) when an FP32 pivot is below 1e-3 or
 // |E| > 0.05: the caller then takes the FP64 Cholesky path.  On success S
 // holds theta on its diagonal and T the coefficients C' (rows scaled by D
 // later).  L = Ms, T = Hs on entry (zero padded to q); S, V, U scratch.
 __device__ bool rr_fast(double (*S)[LD], double (*V)[LD], double (*L)[LD], double (*T)[LD], double (*U)[LD], int p,
                         int q) {
-    __shared__ float linv32[PMAX];
     __shared__ int s_fail32, s_emax;
     const int t = threadIdx.x;
     float (*L32)[LD] = reinterpret_cast<float (*)[LD]>(&U[0][0]);
@@ -584,44 +738,12 @@ __device__ bool rr_fast(double (*S)[LD], double (*V)[LD], double (*L)[LD], doubl
     }
     __syncthreads();
     if (t < 32) {
-        const int lane = t;
-        int fail = 0;
-        for (int k = 0; k < q; ++k) {
-            const float d = L32[k][k];
-            float r = 0.f, lkk = 0.f;
-            if (d > 1e-3f) {
-                r = rsqrtf(d);
-                r = r * fmaf(-0.5f * d * r, r, 1.5f);
-                lkk = d * r;
-            } else {
-                fail = 1;
-            }
-            __syncwarp();
-            if (lane == k) { L32[k][k] = lkk; linv32[k] = r; }
-            if (lane > k && lane < q) L32[lane][k] *= r;
-            __syncwarp();
-            if (lane > k && lane < q)
-                for (int b = k + 1; b <= lane; ++b) L32[lane][b] = fmaf(-L32[lane][k], L32[b][k], L32[lane][b]);
-            __syncwarp();
-        }
-        if (lane < q) {
-            const int c = lane;
-            for (int r = 0; r < q; ++r) {
-                float v = 0.f;
-                if (r >= c) {
-                    float a0 = (r == c) ? 1.f : 0.f, a1 = 0.f;
-                    int j = c;
-                    for (; j + 1 < r; j += 2) {
-                        a0 = fmaf(-L32[r][j], U32[j][c], a0);
-                        a1 = fmaf(-L32[r][j + 1], U32[j + 1][c], a1);
-                    }
-                    if (j < r) a0 = fmaf(-L32[r][j], U32[j][c], a0);
-                    v = (a0 + a1) * linv32[r];
-                }
-                U32[r][c] = v;
-            }
-        }
-        if (lane == 0) { s_fail32 = fail; s_emax = 0; }
+        bool good;
+        if (q <= 12) good = chol_inverse_warp<12>(L32, U32, q);
+        else if (q <= 16) good = chol_inverse_warp<16>(L32, U32, q);
+        else if (q <= 20) good = chol_inverse_warp<20>(L32, U32, q);
+        else good = chol_inverse_warp<32>(L32, U32, q);
+        if (t == 0) { s_fail32 = good ? 0 : 1; s_emax = 0; }
     }
     __syncthreads();
     if (s_fail32) return false;
@@ -697,9 +819,13 @@ __device__ bool rr_fast(double (*S)[LD], double (*V)[LD], double (*L)[LD], doubl
         }
     }
     __syncthreads();
-    block_jacobi<double>(U, V, q, 1e-10, 1e-15, 8);
-    __syncthreads();
-    smem_gemm(T, S, V, q, false);                        // C' = Z Q
+    if (rotate_all(U, S, V, T, L, q, 1e-10, 1e-15)) {    // C' = Z, rotated in place
+        for (int e = t; e < q * q; e += TPB) T[e / q][e % q] = S[e / q][e % q];
+    } else {
+        block_jacobi<double>(U, V, q, 1e-10, 1e-15, 8);
+        __syncthreads();
+        smem_gemm(T, S, V, q, false);                    // C' = Z Q
+    }
     __syncthreads();
     for (int e = t; e < q * q; e += TPB) S[e / q][e % q] = U[e / q][e % q];
     __syncthreads();
