@@ -145,8 +145,8 @@ void run_eig(GevpBatch& g, const EigParams& ep, Apply apply, Solve solve, BApply
             const double n = v.K.n[i], b = v.K.b[i], p = v.p[i];
             am[k].pm = std::max(am[k].pm, v.p[i]);
             // factor band read by both sweeps; right-hand sides read once and
-            // solutions written once (FP64)
-            am[k].sb0 += 2.0 * n * (b + 1) * fsz + 2.0 * n * p * 8.0;
+            // solutions written once, in the factors' type
+            am[k].sb0 += 2.0 * n * (b + 1) * fsz + 2.0 * n * p * fsz;
             am[k].sf0 += 4.0 * n * b * p;
             am[k].vec_n += n * p;
         }
