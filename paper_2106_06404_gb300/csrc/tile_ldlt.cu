@@ -406,7 +406,8 @@ __global__ void __launch_bounds__(TPB) k_rl_panel(T* __restrict__ tiles, const T
     for (int q = 0; q < 4; ++q) dst[r * NB + c0 + 8 * q] = out[q] * sd[c0 + 8 * q];
 }
 
-// grid.y enumerates the tiles (R, C), k < C <= R <= k + kb, row by row
+// grid.y, continued in grid.z beyond its 65535 blocks (kb > 361), enumerates
+// the tiles (R, C), k < C <= R <= k + kb, row by row
 template <typename T>
 __global__ void __launch_bounds__(TPB) k_rl_update(T* __restrict__ tiles, const T* __restrict__ dinv,
                                                    const int* __restrict__ kb_, const int* __restrict__ K_,
@@ -417,7 +418,7 @@ __global__ void __launch_bounds__(TPB) k_rl_update(T* __restrict__ tiles, const 
     __shared__ T sd[NB];
     const int i = blockIdx.x;
     const int K = K_[i], kb = kb_[i];
-    int e = blockIdx.y, R = k + 1;
+    int e = blockIdx.y + blockIdx.z * gridDim.y, R = k + 1;
     while (R < K && e >= R - k) { e -= R - k; ++R; }
     if (R >= K || R - k > kb) return;
     const int C = k + 1 + e;
@@ -2302,8 +2303,9 @@ void tile_factor(TileBatch& tb, double reg_tol, cudaStream_t s) {
                 k_rl_panel<T><<<dim3(tb.P, m), TPB, 0, s>>>(tl, dv, tb.d_kb.p, tb.d_K.p, tb.d_b.p, tb.d_toff.p,
                                                            tb.d_roff.p, k);
                 MSDD_LAUNCH_CHECK();
-                k_rl_update<T><<<dim3(tb.P, m * (m + 1) / 2), TPB, 0, s>>>(tl, dv, tb.d_kb.p, tb.d_K.p, tb.d_b.p,
-                                                                         tb.d_toff.p, tb.d_roff.p, k);
+                const int nt = m * (m + 1) / 2, ny = std::min(nt, 65535);
+                k_rl_update<T><<<dim3(tb.P, ny, (nt + ny - 1) / ny), TPB, 0, s>>>(
+                    tl, dv, tb.d_kb.p, tb.d_K.p, tb.d_b.p, tb.d_toff.p, tb.d_roff.p, k);
                 MSDD_LAUNCH_CHECK();
             }
         };
