@@ -218,7 +218,10 @@ void raise_smem_limit(const void* func, size_t bytes) {
     std::lock_guard<std::mutex> lk(mu);
     size_t& cur = limit[std::make_pair(current_device(), func)];
     if (bytes <= cur) return;
-    if (bytes > 48 * 1024)
+    cudaFuncAttributes a;
+    MSDD_CUDA(cudaFuncGetAttributes(&a, func));
+    // the 48 KB that need no attribute hold the kernel's static arrays too
+    if (bytes + a.sharedSizeBytes > 48 * 1024)
         MSDD_CUDA(cudaFuncSetAttribute(func, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
     cur = bytes;
 }

@@ -2401,10 +2401,8 @@ void tile_solve(const TileBatch& tb, double* X, int ldx, int ncols, const int* s
             }
         }
         if (zbytes <= 160 * 1024) {
-            if (zbytes > 48 * 1024) {
-                raise_smem_limit(k_tile_solve1_dense<float>, zbytes);
-                raise_smem_limit(k_tile_solve1_dense<double>, zbytes);
-            }
+            raise_smem_limit(k_tile_solve1_dense<float>, zbytes);
+            raise_smem_limit(k_tile_solve1_dense<double>, zbytes);
             if (tb.prec) k_tile_solve1_dense<float><<<tb.P, S1T, zbytes, s>>>(tb.tiles_f.p, tb.dinv_f.p, tb.d_kb.p, tb.d_K.p, tb.d_toff.p, tb.d_roff.p, X, gdone);
             else k_tile_solve1_dense<double><<<tb.P, S1T, zbytes, s>>>(tb.tiles_d.p, tb.dinv_d.p, tb.d_kb.p, tb.d_K.p, tb.d_toff.p, tb.d_roff.p, X, gdone);
             MSDD_LAUNCH_CHECK();
