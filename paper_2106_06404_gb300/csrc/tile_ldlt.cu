@@ -1136,6 +1136,24 @@ __global__ void __launch_bounds__(TF_NT) k_tile_factor_tc(
     if (t == 0) { status[i] = s_status; nreg[i] = s_nreg; }
 }
 
+template <int C>
+__device__ __forceinline__ void ws_ld(const float* p, float (&v)[C]) {
+    if constexpr (C == 4) {
+        const float4 x = *reinterpret_cast<const float4*>(p);
+        v[0] = x.x; v[1] = x.y; v[2] = x.z; v[3] = x.w;
+    } else if constexpr (C == 2) {
+        const float2 x = *reinterpret_cast<const float2*>(p);
+        v[0] = x.x; v[1] = x.y;
+    } else {
+        v[0] = *p;
+    }
+}
+template <int C>
+__device__ __forceinline__ void ws_st(float* p, const float (&v)[C]) {
+    if constexpr (C == 4) *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]);
+    else if constexpr (C == 2) *reinterpret_cast<float2*>(p) = make_float2(v[0], v[1]);
+    else *p = v[0];
+}
 // element (row, col) of a 128-byte-swizzled 32 x 32 FP32 tile
 __device__ __forceinline__ int swz(int row, int col) { return row * NB + ((((col >> 2) ^ (row & 7))) << 2) + (col & 3); }
 
@@ -1152,10 +1170,12 @@ __device__ __forceinline__ void ws_row_product(const float* tile, const float* V
     }
 #pragma unroll
     for (int k = K0; k < K1; ++k) {
+        float v[C];
+        ws_ld<C>(V + k * C, v);
 #pragma unroll
         for (int c = 0; c < C; ++c) {
-            if (SIGN > 0) acc[c] += l[k - K0] * V[k * C + c];
-            else acc[c] -= l[k - K0] * V[k * C + c];
+            if (SIGN > 0) acc[c] += l[k - K0] * v[c];
+            else acc[c] -= l[k - K0] * v[c];
         }
     }
 }
@@ -1167,12 +1187,115 @@ __device__ __forceinline__ void ws_col_product(const float* tile, const float* V
     for (int k = 0; k < K1; ++k) l[k] = tile[swz(k, lane)];
 #pragma unroll
     for (int k = 0; k < K1; ++k) {
+        float v[C];
+        ws_ld<C>(V + k * C, v);
 #pragma unroll
         for (int c = 0; c < C; ++c) {
-            if (SIGN > 0) acc[c] += l[k] * V[k * C + c];
-            else acc[c] -= l[k] * V[k * C + c];
+            if (SIGN > 0) acc[c] += l[k] * v[c];
+            else acc[c] -= l[k] * v[c];
         }
     }
+}
+
+// Wide-band forms of the two products: the loads are volatile shared
+// loads issued eight k at a time ahead of their products (the compiler keeps
+// their order), with two partial sums per column.  With 13 tiles a step the
+// products dominate and this ordering is 2-12% faster; with 3 tiles the
+// plain forms above are.
+__device__ __forceinline__ float4 lds4_ordered(const float* p) {
+    float4 r;
+    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];\n"
+                 : "=f"(r.x), "=f"(r.y), "=f"(r.z), "=f"(r.w)
+                 : "r"(smem_u32(p)));
+    return r;
+}
+__device__ __forceinline__ float lds1_ordered(const float* p) {
+    float r;
+    asm volatile("ld.shared.f32 %0, [%1];\n" : "=f"(r) : "r"(smem_u32(p)));
+    return r;
+}
+__device__ __forceinline__ float2 lds2_ordered(const float* p) {
+    float2 r;
+    asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];\n" : "=f"(r.x), "=f"(r.y) : "r"(smem_u32(p)));
+    return r;
+}
+template <int C>
+__device__ __forceinline__ void ws_ld_ordered(const float* p, float (&v)[C]) {
+    if constexpr (C == 4) {
+        const float4 x = lds4_ordered(p);
+        v[0] = x.x; v[1] = x.y; v[2] = x.z; v[3] = x.w;
+    } else if constexpr (C == 2) {
+        const float2 x = lds2_ordered(p);
+        v[0] = x.x; v[1] = x.y;
+    } else {
+        ws_ld<C>(p, v);
+    }
+}
+template <int C, int K0, int K1, int SIGN>
+__device__ __forceinline__ void ws_row_product_wide(const float* tile, const float* V, int lane, float (&acc)[C]) {
+    constexpr int NK = K1 - K0;
+    static_assert(NK % 8 == 0, "k range in multiples of 8");
+    float l[NK];
+#pragma unroll
+    for (int g = K0 / 4; g < K1 / 4; ++g) {
+        const float4 x = lds4_ordered(tile + lane * NB + ((g ^ (lane & 7)) << 2));
+        l[4 * g - K0] = x.x; l[4 * g - K0 + 1] = x.y; l[4 * g - K0 + 2] = x.z; l[4 * g - K0 + 3] = x.w;
+    }
+    float a0[C], a1[C];
+#pragma unroll
+    for (int c = 0; c < C; ++c) { a0[c] = acc[c]; a1[c] = 0.f; }
+#pragma unroll
+    for (int k8 = 0; k8 < NK; k8 += 8) {
+        float v[8][C];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) ws_ld_ordered<C>(V + (K0 + k8 + k) * C, v[k]);
+#pragma unroll
+        for (int k = 0; k < 8; k += 2)
+#pragma unroll
+            for (int c = 0; c < C; ++c) {
+                if (SIGN > 0) { a0[c] += l[k8 + k] * v[k][c]; a1[c] += l[k8 + k + 1] * v[k + 1][c]; }
+                else { a0[c] -= l[k8 + k] * v[k][c]; a1[c] -= l[k8 + k + 1] * v[k + 1][c]; }
+            }
+    }
+#pragma unroll
+    for (int c = 0; c < C; ++c) acc[c] = a0[c] + a1[c];
+}
+template <int C, int K1, int SIGN>
+__device__ __forceinline__ void ws_col_product_wide(const float* tile, const float* V, int lane, float (&acc)[C]) {
+    static_assert(K1 % 8 == 0, "k range in multiples of 8");
+    float l[K1];
+#pragma unroll
+    for (int k = 0; k < K1; ++k) l[k] = lds1_ordered(tile + swz(k, lane));
+    float a0[C], a1[C];
+#pragma unroll
+    for (int c = 0; c < C; ++c) { a0[c] = acc[c]; a1[c] = 0.f; }
+#pragma unroll
+    for (int k8 = 0; k8 < K1; k8 += 8) {
+        float v[8][C];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) ws_ld_ordered<C>(V + (k8 + k) * C, v[k]);
+#pragma unroll
+        for (int k = 0; k < 8; k += 2)
+#pragma unroll
+            for (int c = 0; c < C; ++c) {
+                if (SIGN > 0) { a0[c] += l[k8 + k] * v[k][c]; a1[c] += l[k8 + k + 1] * v[k + 1][c]; }
+                else { a0[c] -= l[k8 + k] * v[k][c]; a1[c] -= l[k8 + k + 1] * v[k + 1][c]; }
+            }
+    }
+#pragma unroll
+    for (int c = 0; c < C; ++c) acc[c] = a0[c] + a1[c];
+}
+// the form a configuration uses: ordered for wide bands (more than 2 tiles)
+// with 2 or 4 columns a warp (the configurations that were measured)
+template <bool WIDE, int C, int K0, int K1, int SIGN>
+__device__ __forceinline__ void ws_rowp(const float* tile, const float* V, int lane, float (&acc)[C]) {
+    if constexpr (WIDE) ws_row_product_wide<C, K0, K1, SIGN>(tile, V, lane, acc);
+    else ws_row_product<C, K0, K1, SIGN>(tile, V, lane, acc);
+}
+template <bool WIDE, int C, int K1, int SIGN>
+__device__ __forceinline__ void ws_colp(const float* tile, const float* V, int lane, float (&acc)[C]) {
+    if constexpr (WIDE) ws_col_product_wide<C, K1, SIGN>(tile, V, lane, acc);
+    else ws_col_product<C, K1, SIGN>(tile, V, lane, acc);
 }
 
 __device__ __forceinline__ void mbar_arrive(unsigned long long* bar) {
@@ -1211,8 +1334,7 @@ __device__ __forceinline__ float as_f32(double x) { return f64_to_f32(x); }
 __device__ __forceinline__ float as_f32(float x) { return x; }
 constexpr int KS_LD = 40;        // column stride of the exchange blocks: 16-byte reads of 4 columns or 8 row groups are conflict-free
 
-template <int NW, int J>
-constexpr size_t band_ks_smem(int S, int nst) {
+constexpr size_t band_ks_smem(int NW, int J, int S, int nst) {
     return 1024 + (size_t)nst * S * NB2 * 4 + 16 * (size_t)nst + sizeof(float) * (size_t)(2 * NW + S + 1) * 4 * J * KS_LD;
 }
 
@@ -1483,16 +1605,235 @@ __global__ void __launch_bounds__(32 * (NW + 1)) k_tile_solve_band_ks(
     }
 }
 
+// ---- the FP32 band solve of several right-hand sides (kb <= 12), a warp per
+// few columns.  No block barrier sits on the sweeps' chain: each of W consumer
+// warps owns C right-hand-side columns and all 32 rows of a tile row (lane =
+// row), so a step's data exchange is warp-internal (__syncwarp).  Producer
+// warp, bounded waits and time-outs as in k_tile_solve_band_ks.  Each lane
+// prefetches its own row of the right-hand sides with cp.async, XD steps ahead
+// (X rows start on 16 bytes: host dispatch).  Column k of tile L_{R,R-d} can be
+// nonzero only where 32 d + r - k <= b (the band), so the forward products
+// start at k = 32 d - b and the backward ones stop at k = b - 32 d + 31.
+template <int KBP, int W, int C, int NST, int XD, typename XT>
+struct BandWs {
+    // The backward sweep's first right-hand side read from X (block K-1-S,
+    // written by forward step K-1-S) is issued XD - 1 steps ahead, at step
+    // K - XD + 1: it must come after that write, so XD <= S + 1 = KBP + 2.
+    static_assert(XD <= KBP + 2, "X prefetch deeper than the solution ring allows");
+    static constexpr int SLOTS = KBP + 1;            // tiles per step; also the solution ring per warp
+    static constexpr int NT = 32 * (W + 1);
+    static constexpr int COLS = W * C;
+    static constexpr size_t stage_bytes = (size_t)SLOTS * NB2 * sizeof(float);
+    static constexpr size_t warp_bytes =
+        sizeof(float) * ((size_t)SLOTS * NB * C + (size_t)NB * C) + sizeof(XT) * (size_t)XD * NB * C;
+    static constexpr size_t smem_bytes =
+        1024 + (size_t)NST * stage_bytes + (size_t)NST * NB * sizeof(float) + 16 * (size_t)NST + (size_t)W * warp_bytes;
+};
+
+// Half-bandwidth b at most KBP tiles (kb <= KBP); a step needs the diagonal
+// tile and kb off-diagonal tiles, and z_{R-1} .. z_{R-kb} (forward) or
+// x_{R+1} .. x_{R+kb} (backward) from the warp's ring of KBP + 1 solution
+// blocks.  When the backward sweep starts, the ring still holds z_R for the
+// last KBP + 1 rows, so only the rows before those are read back from X.
+template <int KBP, int W, int C, int NST, int XD, typename XT>
+__global__ void __launch_bounds__(32 * (W + 1)) k_tile_solve_band_ws(
+    const __grid_constant__ CUtensorMap tmt, const float* __restrict__ dinv, const int* __restrict__ kb_,
+    const int* __restrict__ K_, const int* __restrict__ b_, const long long* __restrict__ toff_,
+    const long long* __restrict__ roff_, XT* Xall, int ldx, int ncols_all,
+    const int* __restrict__ skip, const int* __restrict__ gdone)
+{
+    using Cfg = BandWs<KBP, W, C, NST, XD, XT>;
+    constexpr int S = Cfg::SLOTS;
+    static_assert(C == 2 || C == 4, "2 or 4 columns per warp");
+    extern __shared__ unsigned char smem_raw[];
+    unsigned char* base = smem_raw + ((1024 - (smem_u32(smem_raw) & 1023)) & 1023);
+    float* St = reinterpret_cast<float*>(base);                                        // [NST][S][32*32]
+    float* Sd = St + (size_t)NST * S * NB2;                                            // [NST][32]
+    unsigned long long* full = reinterpret_cast<unsigned long long*>(Sd + (size_t)NST * NB);
+    unsigned long long* empty = full + NST;
+    unsigned char* wbase = reinterpret_cast<unsigned char*>(empty + NST);
+    __shared__ int s_abort;
+
+    const int i = blockIdx.x;
+    if (skip && skip[i]) return;
+    if (gdone && *gdone) return;
+    const int kb = kb_[i], K = K_[i], bw = b_[i];
+    if (kb > KBP) return;                            // never launched so (host dispatch)
+    const long long toff = toff_[i], roff = roff_[i];
+    const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
+    if (t == 0) {
+        s_abort = 0;
+        for (int s = 0; s < NST; ++s) {
+            mbar_init(&full[s], 1);
+            mbar_init(&empty[s], W);
+        }
+        fence_mbar_init();
+    }
+    __syncthreads();
+    auto stile = [&](int st, int slot) { return St + (size_t)(st * S + slot) * NB2; };
+    auto give_up = [&]() {
+        if (atomicExch(&s_abort, 1) == 0) atomicAdd(&g_wait_timeouts, 1);
+    };
+    const int total = 2 * K;                         // steps of both sweeps
+
+    if (warp == W) {
+        // ---------------- producer: one lane issues every copy
+        if (lane == 0) {
+            unsigned pending = 0, par = 0;           // stages with copies in flight, their phase parity
+            for (int it = 0; it < total; ++it) {
+                const int st = it % NST;
+                if (it >= NST) {
+                    if (!mbar_wait_bounded(&empty[st], ((it / NST) - 1) & 1u)) { give_up(); break; }
+                    pending &= ~(1u << st);
+                }
+                if (*(volatile int*)&s_abort) break;
+                const bool fwd = it < K;
+                const int R = fwd ? it : total - 1 - it;
+                int nt = 1;
+                for (int d = 1; d <= kb; ++d) {
+                    const int o = fwd ? R - d : R + d;
+                    if (o >= 0 && o < K) ++nt;
+                }
+                mbar_expect_tx(&full[st], nt * NB2 * 4 + (fwd ? 0 : NB * 4));
+                tma_load_tile(stile(st, 0), &tmt, (int)(tile_index(toff, kb, R, R) / NB), &full[st]);
+                for (int d = 1; d <= kb; ++d) {
+                    const int o = fwd ? R - d : R + d;
+                    if (o < 0 || o >= K) continue;
+                    const long long ti = fwd ? tile_index(toff, kb, R, o) : tile_index(toff, kb, o, R);
+                    tma_load_tile(stile(st, d), &tmt, (int)(ti / NB), &full[st]);
+                }
+                if (!fwd) bulk_load(Sd + st * NB, dinv + roff + (long long)R * NB, NB * 4, &full[st]);
+                pending |= 1u << st;
+                par = (par & ~(1u << st)) | (((unsigned)(it / NST) & 1u) << st);
+            }
+            // after an abort, copies still in flight must land before the CTA exits
+            if (*(volatile int*)&s_abort)
+                for (int s = 0; s < NST; ++s)
+                    if (pending & (1u << s)) mbar_wait_bounded(&full[s], (par >> s) & 1u);
+        }
+        return;
+    }
+
+    // ---------------- consumer warp: columns [c_lo, c_lo + nc)
+    const int c_lo = blockIdx.y * Cfg::COLS + warp * C;
+    const int nc = max(0, min(C, ncols_all - c_lo));
+    float* Zr = reinterpret_cast<float*>(wbase + (size_t)warp * Cfg::warp_bytes);     // [S][32][C]
+    float* Acc = Zr + (size_t)S * NB * C;                                               // [32][C]
+    XT* Xs = reinterpret_cast<XT*>(Acc + (size_t)NB * C);                      // [XD][32][C]
+    XT* X = Xall + c_lo;
+    // loads of this lane's row: index q < K: forward step q (row q); q >= K:
+    // backward row K - 1 - S - (q - K) (backward steps s >= S)
+    const int nload = K + max(0, K - S);
+    auto issue_load = [&](int q) {
+        if (q < nload && nc > 0) {
+            if (q >= K) __threadfence_block();       // rows written by this lane in the forward sweep
+            const int R = q < K ? q : K - 1 - S - (q - K);
+            const XT* src = X + (roff + (long long)R * NB + lane) * ldx;
+            XT* dst = Xs + ((size_t)(q % XD) * NB + lane) * C;
+            if constexpr (C * sizeof(XT) == 8) {
+                asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(smem_u32(dst)), "l"(src));
+            } else {
+                cp_async16(dst, src);
+                if (C * sizeof(XT) == 32 && nc > 2) cp_async16(dst + 2, src + 2);
+            }
+        }
+        cp_async_commit();
+    };
+    for (int q = 0; q < XD - 1; ++q) issue_load(q);
+    int q_next = XD - 1, q_use = 0;
+    for (int it = 0; it < total; ++it) {
+        const int st = it % NST;
+        const bool fwd = it < K;
+        const int R = fwd ? it : total - 1 - it;
+        float acc[C];
+        // right-hand side of this step (own row)
+        if (fwd || (it - K) >= S) {
+            issue_load(q_next++);
+            cp_async_wait_n<XD - 1>();
+            const XT* xs = Xs + ((size_t)(q_use % XD) * NB + lane) * C;
+#pragma unroll
+            for (int c = 0; c < C; ++c) acc[c] = c < nc ? as_f32(xs[c]) : 0.f;
+            ++q_use;
+        } else {
+            ws_ld<C>(Zr + ((size_t)(R % S) * NB + lane) * C, acc);
+        }
+        if (!mbar_wait_bounded(&full[st], (it / NST) & 1u)) { give_up(); break; }
+        if (nc > 0) {
+            if (!fwd) {
+                const float dr = Sd[st * NB + lane];
+#pragma unroll
+                for (int c = 0; c < C; ++c) acc[c] *= dr;
+            }
+            for (int d = 1; d <= kb; ++d) {
+                const int o = fwd ? R - d : R + d;
+                if (o < 0 || o >= K) continue;
+                const float* L = stile(st, d);
+                const float* Z = Zr + (size_t)(o % S) * NB * C;
+                if (fwd) {
+                    // acc -= L_{R,o}[lane][k] z_o[k]; nonzero only for k >= 32 d - b
+                    const int k0 = NB * d - bw;
+                    if (k0 >= 24) ws_rowp<(KBP > 2 && C >= 2), C, 24, 32, -1>(L, Z, lane, acc);
+                    else if (k0 >= 16) ws_rowp<(KBP > 2 && C >= 2), C, 16, 32, -1>(L, Z, lane, acc);
+                    else ws_rowp<(KBP > 2 && C >= 2), C, 0, 32, -1>(L, Z, lane, acc);
+                } else {
+                    // acc -= L_{o,R}[k][lane] x_o[k]; nonzero only for k <= b - 32 d + 31
+                    const int kend = bw - NB * d + NB;
+                    if (kend <= 8) ws_colp<(KBP > 2 && C >= 2), C, 8, -1>(L, Z, lane, acc);
+                    else if (kend <= 16) ws_colp<(KBP > 2 && C >= 2), C, 16, -1>(L, Z, lane, acc);
+                    else ws_colp<(KBP > 2 && C >= 2), C, 32, -1>(L, Z, lane, acc);
+                }
+            }
+            ws_st<C>(Acc + lane * C, acc);
+            __syncwarp();
+            const float* T = stile(st, 0);
+            float out[C];
+#pragma unroll
+            for (int c = 0; c < C; ++c) out[c] = 0.f;
+            if (fwd) ws_rowp<(KBP > 2 && C >= 2), C, 0, 32, 1>(T, Acc, lane, out);
+            else ws_colp<(KBP > 2 && C >= 2), C, 32, 1>(T, Acc, lane, out);
+            __syncwarp();                                   // Acc reads done before the next step's writes
+            ws_st<C>(Zr + ((size_t)(R % S) * NB + lane) * C, out);
+            XT* xw = X + (roff + (long long)R * NB + lane) * ldx;
+#pragma unroll
+            for (int c = 0; c < C; ++c)
+                if (c < nc) {
+                    if constexpr (sizeof(XT) == 8) xw[c] = f32_to_f64(out[c]);
+                    else xw[c] = out[c];
+                }
+        }
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&empty[st]);
+    }
+    cp_async_wait_n<0>();
+}
+
+// Launch of k_tile_solve_band_ws for one configuration.
+template <int KBP, int W, int C, int NST, int XD, typename XT>
+void launch_band_ws(const TileBatch& tb, const CUtensorMap& tm, XT* X, int ldx, int ncols, const int* skip,
+                    cudaStream_t s, const int* gdone) {
+    using Cfg = BandWs<KBP, W, C, NST, XD, XT>;
+    static_assert(Cfg::smem_bytes <= 227 * 1024, "shared memory per CTA");
+    auto kern = k_tile_solve_band_ws<KBP, W, C, NST, XD, XT>;
+    raise_smem_limit(kern, Cfg::smem_bytes);
+    kern<<<dim3(tb.P, (ncols + Cfg::COLS - 1) / Cfg::COLS), Cfg::NT, Cfg::smem_bytes, s>>>(
+        tm, tb.dinv_f.p, tb.d_kb.p, tb.d_K.p, tb.d_b.p, tb.d_toff.p, tb.d_roff.p, X, ldx, ncols, skip, gdone);
+    MSDD_LAUNCH_CHECK();
+}
+
+// stages of k_tile_solve_band_ks: up to four, with two CTAs an SM where that leaves at least two
+int band_ks_stages(int NW, int J, int S) {
+    const size_t half = 112 * 1024, full = 226 * 1024;
+    const size_t limit = band_ks_smem(NW, J, S, 2) <= half ? half : full;
+    int nst = 4;
+    while (nst > 2 && band_ks_smem(NW, J, S, nst) > limit) --nst;
+    return nst;
+}
+
 template <int NW, int J, typename XT>
 void launch_band_ks(const TileBatch& tb, const CUtensorMap& tm, int maxkb, XT* X, int ldx, int ncols, int chunks,
                     const int* skip, cudaStream_t s, const int* gdone) {
-    const int S = maxkb + 1;
-    // stages: up to four, with two CTAs an SM where that leaves at least two
-    const size_t half = 112 * 1024, full = 226 * 1024;
-    const size_t limit = band_ks_smem<NW, J>(S, 2) <= half ? half : full;
-    int nst = 4;
-    while (nst > 2 && band_ks_smem<NW, J>(S, nst) > limit) --nst;
-    const size_t b = band_ks_smem<NW, J>(S, nst);
+    const int S = maxkb + 1, nst = band_ks_stages(NW, J, S);
+    const size_t b = band_ks_smem(NW, J, S, nst);
     auto kern = k_tile_solve_band_ks<NW, J, XT>;
     raise_smem_limit(kern, b);
     kern<<<dim3(tb.P, chunks), 32 * (NW + 1), b, s>>>(tm, tb.dinv_f.p, tb.d_kb.p, tb.d_K.p, tb.d_b.p, tb.d_toff.p,
@@ -1500,28 +1841,73 @@ void launch_band_ks(const TileBatch& tb, const CUtensorMap& tm, int maxkb, XT* X
     MSDD_LAUNCH_CHECK();
 }
 
-// Column groups of 4 J <= 20 columns, as even as they come; fewer columns a CTA
-// while that still leaves every CTA an SM of its own (the tiles are then read
-// by several CTAs, but a step's products and loads are shared out): 48 problems
-// of n = 3600, b = 226, 16 columns 737 us in one group, 556 us in two, 24 of
-// them 703 us in one, 478 us in four.
+// FP32 factors, several columns, kb <= 12.
+//
+// k_tile_solve_band_ks takes column groups of 4 J <= 20 columns, as even as
+// they come; fewer columns a CTA while that still leaves every CTA an SM of its
+// own (the tiles are then read by several CTAs, but a step's products and loads
+// are shared out).  Four consumer warps, eight where a step's tiles outweigh the
+// exchange of the partial sums: wide bands with one group of columns or with
+// five, and J >= 4 beside an FP64 X (whose conversions take four warps' registers).
+// k_tile_solve_band_ws takes 16 (kb <= 2) or 20 columns a CTA, two and one CTA an SM.
+//
+// Which one: the kernel that takes fewer rounds of CTAs over the SMs; in a tie
+// the column split for kb <= 2 (its step has no block barrier), but the k split
+// at kb = 2 where its CTAs have an SM each and at most 8 columns; for kb >= 3 the
+// k split from 11 (FP32 X) or 15 (FP64 X) columns on, where a warp's run over
+// the step's tiles is longer than the exchange.  Measured, us a launch with cold
+// L2, n = 1500, column split / k split, FP32 X unless said:
+//   kb 1, 128 problems, 12 columns 70 / 103; 500, 8 columns 154 / 140;
+//   kb 2, 128, 16: 107 / 121; 300, 20: 226 / 187; 8, 8: 101 / 97;
+//   kb 3, 72, 8: 109 / 119; 72, 16: 138 / 121; 300, 8: 214 / 150;
+//   kb 12, 48, 16: 341 / 279; 128, 16 with FP64 X 365 / 324; 128, 6 with FP64 X 287 / 343.
+// Over 2320 such cells (b 5 to 380, 1 to 961 problems, 2 to 32 columns, both types)
+// the choice takes 1.1% more than the faster kernel on average, 29% at most.  The k
+// split alone, with eight warps from kb = 3, took 16% more, 85% at most, and was
+// the slower one in 1301 of them (through the band API, b = 100, 8 problems of
+// 5000, 8 columns: 0.54 -> 0.70 ms).
 template <typename XT>
-void solve_band_ks(const TileBatch& tb, const CUtensorMap& tm, int maxkb, XT* X, int ldx, int ncols, const int* skip,
-                   cudaStream_t s, const int* gdone) {
+void solve_band_f32(const TileBatch& tb, const CUtensorMap& tm, int maxkb, XT* X, int ldx, int ncols, const int* skip,
+                    cudaStream_t s, const int* gdone) {
+    constexpr int SMS = 152;
+    constexpr bool F64X = sizeof(XT) == 8;
     int chunks = (ncols + 19) / 20, J = (ncols + 4 * chunks - 1) / (4 * chunks);
-    while (J > 1 && (long long)tb.P * ((ncols + 4 * (J - 1) - 1) / (4 * (J - 1))) <= 152) --J;
+    while (J > 1 && (long long)tb.P * ((ncols + 4 * (J - 1) - 1) / (4 * (J - 1))) <= SMS) --J;
     chunks = (ncols + 4 * J - 1) / (4 * J);
+    const long long ctas = (long long)tb.P * chunks;
+    const bool own_sm = ctas <= SMS;
+    const int NW = maxkb <= 2 ? 4
+                   : F64X && J >= 4 ? 8
+                   : maxkb <= 6 ? (J == 5 && own_sm && maxkb > 4 ? 8 : 4)
+                   : J == 1 || J == 5 ? 8 : 4;
+    const size_t bytes = band_ks_smem(NW, J, maxkb + 1, band_ks_stages(NW, J, maxkb + 1));
+    const long long ks_rounds = ceil_div(ctas, SMS * std::max<long long>(1, 227 * 1024 / (bytes + 1024)));
+    const int ws_cols = maxkb <= 2 ? 16 : 20;
+    const long long ws_rounds = ceil_div((long long)tb.P * ((ncols + ws_cols - 1) / ws_cols), maxkb <= 2 ? 2 * SMS : SMS);
+    bool ks;
+    if (maxkb <= 2)
+        ks = ks_rounds != ws_rounds ? ks_rounds < ws_rounds : maxkb == 2 && ((own_sm && J <= 2) || (!F64X && ncols > 28));
+    else if (F64X && J >= 4 && maxkb <= 6)
+        ks = false;
+    else
+        ks = ks_rounds < ws_rounds || (ncols > (F64X ? 14 : 10) && (J < 5 || maxkb > 4));
+    const bool aligned = ldx * sizeof(XT) % 16 == 0 && (uintptr_t)X % 16 == 0;
+    if (!ks && aligned) {
+        if (maxkb <= 2) launch_band_ws<2, 4, 4, 6, 4>(tb, tm, X, ldx, ncols, skip, s, gdone);
+        else launch_band_ws<12, 10, 2, 2, 4>(tb, tm, X, ldx, ncols, skip, s, gdone);
+        return;
+    }
     auto go = [&](auto nw) {
-        constexpr int NW = decltype(nw)::value;
+        constexpr int W = decltype(nw)::value;
         switch (J) {
-            case 1: launch_band_ks<NW, 1>(tb, tm, maxkb, X, ldx, ncols, chunks, skip, s, gdone); break;
-            case 2: launch_band_ks<NW, 2>(tb, tm, maxkb, X, ldx, ncols, chunks, skip, s, gdone); break;
-            case 3: launch_band_ks<NW, 3>(tb, tm, maxkb, X, ldx, ncols, chunks, skip, s, gdone); break;
-            case 4: launch_band_ks<NW, 4>(tb, tm, maxkb, X, ldx, ncols, chunks, skip, s, gdone); break;
-            default: launch_band_ks<NW, 5>(tb, tm, maxkb, X, ldx, ncols, chunks, skip, s, gdone); break;
+            case 1: launch_band_ks<W, 1>(tb, tm, maxkb, X, ldx, ncols, chunks, skip, s, gdone); break;
+            case 2: launch_band_ks<W, 2>(tb, tm, maxkb, X, ldx, ncols, chunks, skip, s, gdone); break;
+            case 3: launch_band_ks<W, 3>(tb, tm, maxkb, X, ldx, ncols, chunks, skip, s, gdone); break;
+            case 4: launch_band_ks<W, 4>(tb, tm, maxkb, X, ldx, ncols, chunks, skip, s, gdone); break;
+            default: launch_band_ks<W, 5>(tb, tm, maxkb, X, ldx, ncols, chunks, skip, s, gdone); break;
         }
     };
-    if (maxkb <= 2) go(std::integral_constant<int, 4>{});
+    if (NW == 4) go(std::integral_constant<int, 4>{});
     else go(std::integral_constant<int, 8>{});
 }
 
@@ -2146,7 +2532,7 @@ void solve_f32(const TileBatch& tb, XT* X, int ldx, int ncols, const int* skip, 
     for (int v : tb.kb) maxkb = std::max(maxkb, v);
     const CUtensorMap* tm = maxkb <= 12 ? tile_tensor_map(tb) : nullptr;
     if (tm) {
-        solve_band_ks(tb, *tm, maxkb, X, ldx, ncols, skip, s, gdone);
+        solve_band_f32(tb, *tm, maxkb, X, ldx, ncols, skip, s, gdone);
         return;
     }
     k_tile_solve<float, XT><<<dim3(tb.P, (ncols + NB - 1) / NB), TPB, 0, s>>>(
