@@ -2111,14 +2111,14 @@ void launch_band_split(const TileBatch& tb, const CUtensorMap& tm, double* X, cu
 // no faster than four sharing a step, a warp issues in order; a barrier of all
 // four a step made each wait for the slowest load; a fifth warp issuing every
 // copy took 830 cycles a step for it.)  Each warp streams the tiles of its own
-// steps by TMA, two turns (eight steps) ahead; of the far tile, whose columns
+// steps by TMA, D turns (4 D steps) ahead; of the far tile, whose columns
 // before 64 - b are zero, only the 8-column boxes that hold nonzeros are copied
 // (at b = 38 a step moves 9 of 12 KB).  Every wait is bounded; after a timeout
 // (recorded in g_wait_timeouts) the chain runs to its end without waiting for
 // tiles, and each warp waits (bounded) for its copies in flight.
 // Measured: 256 problems of n = 1369, b = 38 with cold caches 60 -> 53 us (DRAM
 // from there on), with the factors in L2 59 -> 32 us; 128 of them 57 -> 29 us.
-constexpr int S1W_W = 4, S1W_NST = 2 * S1W_W;
+constexpr int S1W_W = 4;
 // the box of a tile map at (col, row)
 __device__ __forceinline__ void tma_load_box(void* dst, const CUtensorMap* map, int col, int row,
                                                unsigned long long* bar) {
@@ -2131,21 +2131,27 @@ __device__ __forceinline__ void tma_load_box(void* dst, const CUtensorMap* map, 
 // first 8-column group of the far tile (R, R - 2) that holds nonzeros
 __host__ __device__ inline int s1w_group0(int b) { return b >= 64 ? 0 : (64 - b) >> 3; }
 
+constexpr size_t s1w_bytes(int D, int nbox, int K) {
+    return 1024 + sizeof(float) * ((size_t)D * S1W_W * (2 * NB2 + nbox * 8 * NB) + (size_t)S1W_W * nbox * 8 * NB + NB +
+                                   (size_t)K * NB);
+}
+
+template <int D>
 __global__ void __launch_bounds__(32 * S1W_W) k_tile_solve1_warp(
     const __grid_constant__ CUtensorMap tmt, const __grid_constant__ CUtensorMap tmc, const float* __restrict__ dinv,
     const int* __restrict__ kb_, const int* __restrict__ K_, const int* __restrict__ b_,
     const long long* __restrict__ toff_, const long long* __restrict__ roff_, double* __restrict__ X,
     const int* __restrict__ gdone, int nbox)
 {
-    constexpr int NTC = 32 * S1W_W;
+    constexpr int NTC = 32 * S1W_W, NST = D * S1W_W;
     extern __shared__ unsigned char smem_raw[];
     unsigned char* base = smem_raw + ((1024 - (smem_u32(smem_raw) & 1023)) & 1023);
     const int stage_floats = 2 * NB2 + nbox * 8 * NB;      // T, near tile, far tile's boxes
     float* St = reinterpret_cast<float*>(base);
-    float* Fr = St + (size_t)S1W_NST * stage_floats;         // [S1W_W][boxes] far boxes of the step each warp prepares
+    float* Fr = St + (size_t)NST * stage_floats;         // [S1W_W][boxes] far boxes of the step each warp prepares
     float* Ac = Fr + (size_t)S1W_W * nbox * 8 * NB;          // [32]
     float* zs = Ac + NB;                                     // [K * 32]
-    __shared__ unsigned long long full[S1W_NST];
+    __shared__ unsigned long long full[NST];
     __shared__ int s_abort;
     if (gdone && *gdone) return;
     const int i = blockIdx.x;
@@ -2156,7 +2162,7 @@ __global__ void __launch_bounds__(32 * S1W_W) k_tile_solve1_warp(
     const int g0 = s1w_group0(bw), nb = kb == 2 ? min(nbox, 4 - g0) : 0;
     if (t == 0) {
         s_abort = 0;
-        for (int s = 0; s < S1W_NST; ++s) mbar_init(&full[s], 1);
+        for (int s = 0; s < NST; ++s) mbar_init(&full[s], 1);
         fence_mbar_init();
     }
     for (int e = t; e < K * NB; e += NTC) zs[e] = f64_to_f32(X[roff + e]);
@@ -2166,8 +2172,8 @@ __global__ void __launch_bounds__(32 * S1W_W) k_tile_solve1_warp(
     };
     const int total = 2 * K;
 
-    // turn u of a warp is step 4 u + warp, its tiles go to stage 2 warp + (u & 1)
-    auto stage = [&](int u) { return 2 * warp + (u & 1); };
+    // turn u of a warp is step 4 u + warp, its tiles go to stage D warp + u % D
+    auto stage = [&](int u) { return D * warp + u % D; };
     auto issue = [&](int u) {                                // one lane issues a step's copies
         const int it = S1W_W * u + warp;
         if (lane != 0 || it >= total) return;
@@ -2186,8 +2192,7 @@ __global__ void __launch_bounds__(32 * S1W_W) k_tile_solve1_warp(
                 tma_load_box(dst + 2 * NB2 + q * 8 * NB, &tmc, 8 * (g0 + q), (int)(ti / NB), &full[st]);
         }
     };
-    issue(0);
-    issue(1);
+    for (int u = 0; u < D; ++u) issue(u);
 
     // ---------------- the chain warps, lane = row (column in the backward sweep)
     auto announce = [&](int id) { asm volatile("bar.arrive %0, 64;\n" ::"r"(id) : "memory"); };
@@ -2201,7 +2206,7 @@ __global__ void __launch_bounds__(32 * S1W_W) k_tile_solve1_warp(
         const int R = fwd ? it : total - 1 - it, nd = min(kb, fwd ? R : K - 1 - R);
         if (!fwd) dv = dinv[roff + (long long)R * NB + lane];
         if (*(volatile int*)&s_abort) return false;          // the chain ends without the tiles
-        if (!mbar_wait_bounded(&full[st], (u >> 1) & 1u)) { give_up(); return false; }
+        if (!mbar_wait_bounded(&full[st], (u / D) & 1u)) { give_up(); return false; }
         const float *T = St + (size_t)st * stage_floats, *L = T + NB2, *F = L + NB2;
         if (fwd) {
 #pragma unroll
@@ -2225,7 +2230,7 @@ __global__ void __launch_bounds__(32 * S1W_W) k_tile_solve1_warp(
             for (int e = lane; e < nb * 2 * NB; e += 32)
                 *reinterpret_cast<float4*>(far + 4 * e) = *reinterpret_cast<const float4*>(F + 4 * e);
         __syncwarp();
-        issue(u + 2);
+        issue(u + D);
         return true;
     };
     // the far tile's product of step `it` (z of step it - 2 is there)
@@ -2286,8 +2291,8 @@ __global__ void __launch_bounds__(32 * S1W_W) k_tile_solve1_warp(
         if (it + 1 < total) announce(5 + warp);
         if (it + 2 < total) announce(1 + warp);
     }
-    for (int v = landed; v < landed + 2 && S1W_W * v + warp < total; ++v)     // after a timeout only
-        mbar_wait_bounded(&full[stage(v)], (v >> 1) & 1u);
+    for (int v = landed; v < landed + D && S1W_W * v + warp < total; ++v)     // after a timeout only
+        mbar_wait_bounded(&full[stage(v)], (v / D) & 1u);
     asm volatile("bar.sync 9, %0;\n" ::"r"(NTC) : "memory");
     for (int e = t; e < K * NB; e += NTC) X[roff + e] = f32_to_f64(zs[e]);
 }
@@ -2751,13 +2756,18 @@ void tile_solve(const TileBatch& tb, double* X, int ldx, int ncols, const int* s
             int nbox = 0;
             for (int i = 0; i < tb.P; ++i)
                 if (tb.kb[i] == 2) nbox = std::max(nbox, 4 - s1w_group0(tb.b[i]));
-            const size_t bytes = 1024 + sizeof(float) * ((size_t)S1W_NST * (2 * NB2 + nbox * 8 * NB) +
-                                                         (size_t)S1W_W * nbox * 8 * NB + NB + (size_t)tb.max_K * NB);
-            if (tm && bytes <= 200 * 1024 && encode_box_map(tb.tiles_f.p, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, tb.total_tile_elems, 8,
-                                                              CU_TENSOR_MAP_SWIZZLE_NONE, &tc)) {
-                raise_smem_limit(k_tile_solve1_warp, bytes);
-                k_tile_solve1_warp<<<tb.P, 32 * S1W_W, bytes, s>>>(*tm, tc, tb.dinv_f.p, tb.d_kb.p, tb.d_K.p, tb.d_b.p,
-                                                          tb.d_toff.p, tb.d_roff.p, X, gdone, nbox);
+            // one turn ahead where two do not fit beside the vector (n = 38500, b = 38: 3.4 ms without the ring, 0.73 with
+            // it), and where two leave one CTA an SM to more CTAs than SMs (n = 1369, b = 60, 256 problems: 126 -> 103 us)
+            const size_t deep = s1w_bytes(2, nbox, tb.max_K);
+            const int D = deep <= (tb.P > 152 ? 112 : 226) * 1024 ? 2 : 1;
+            const size_t bytes = s1w_bytes(D, nbox, tb.max_K);
+            if (tm && bytes <= 226 * 1024 &&
+                encode_box_map(tb.tiles_f.p, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, tb.total_tile_elems, 8,
+                               CU_TENSOR_MAP_SWIZZLE_NONE, &tc)) {
+                auto kern = D == 2 ? k_tile_solve1_warp<2> : k_tile_solve1_warp<1>;
+                raise_smem_limit(kern, bytes);
+                kern<<<tb.P, 32 * S1W_W, bytes, s>>>(*tm, tc, tb.dinv_f.p, tb.d_kb.p, tb.d_K.p, tb.d_b.p,
+                                                     tb.d_toff.p, tb.d_roff.p, X, gdone, nbox);
                 MSDD_LAUNCH_CHECK();
                 return;
             }
