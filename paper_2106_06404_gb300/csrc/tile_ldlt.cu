@@ -628,7 +628,8 @@ __global__ void __launch_bounds__(FB_T) k_tile_factor_band32(
 constexpr int S1T = 128;
 
 // One right-hand side where the streamed kernels below do not fit (very wide
-// bands, dense matrices): tiles are read as needed without prefetch.
+// bands, dense matrices) or keep too few CTAs on an SM (large batches of wide FP64
+// bands): tiles are read as needed without prefetch.
 template <typename T>
 __global__ void __launch_bounds__(S1T) k_tile_solve1_dense(
     const T* __restrict__ tiles, const T* __restrict__ dinv, const int* __restrict__ kb_, const int* __restrict__ K_,
@@ -2309,7 +2310,9 @@ __global__ void __launch_bounds__(32 * S1W_W) k_tile_solve1_warp(
 // outermost tile that lie in the band are dealt out singly.  A fifth warp
 // streams the tiles by TMA in halves of 16 columns (128-byte swizzle), of the
 // outermost tile only the halves that hold nonzeros.  Waits and time-outs as in
-// k_tile_solve_band_ks.
+// k_tile_solve_band_ks.  Ring and vector share 226 KB: at two stages of kb + 1
+// tiles, n <= 24,400 at kb = 1, 12,100 at kb = 7, 8,000 at kb = 9, 3,900 at kb = 11,
+// 1,900 at kb = 12; beyond, and for wide bands in large batches, k_tile_solve1_dense.
 // Measured (warm L2): 144 problems of n = 1296, b = 37 147 -> 125 us, 27 of
 // n = 1728, b = 157 331 -> 295 us.
 constexpr int S1D_W = 4, S1D_HALF = NB * 16;           // doubles of a half tile
@@ -2776,9 +2779,15 @@ void tile_solve(const TileBatch& tb, double* X, int ldx, int ncols, const int* s
             int nst = 4;
             while (nst > 2 && s1d_bytes(maxkb + 1, nst, tb.max_K) > 200 * 1024) --nst;
             const size_t bytes = s1d_bytes(maxkb + 1, nst, tb.max_K);
+            // wide bands: while the ring's CTAs (one an SM mostly) take at most two rounds over the SMs; many small CTAs
+            // without a ring hide the tiles' latency better in more (b = 157, n = 1369: 152 problems 526 -> 278 us, 300
+            // 575 -> 504, but 700 894 -> 1181; b = 100, n = 441, 700 problems 254 -> 334)
+            const bool ring = maxkb <= 2 || zbytes > 160 * 1024 ||
+                              tb.P <= 2 * 152 * (int)std::max<size_t>(1, 227 * 1024 / (bytes + 1024));
             alignas(64) CUtensorMap tm;
-            if (bytes <= 226 * 1024 && encode_box_map(tb.tiles_d.p, CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 8,
-                                                      tb.total_tile_elems, 16, CU_TENSOR_MAP_SWIZZLE_128B, &tm)) {
+            if (ring && bytes <= 226 * 1024 &&
+                encode_box_map(tb.tiles_d.p, CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 8, tb.total_tile_elems, 16,
+                               CU_TENSOR_MAP_SWIZZLE_128B, &tm)) {
                 raise_smem_limit(k_tile_solve1_f64, bytes);
                 k_tile_solve1_f64<<<tb.P, 32 * (S1D_W + 1), bytes, s>>>(tm, tb.dinv_d.p, tb.d_kb.p, tb.d_K.p, tb.d_b.p,
                                                                        tb.d_toff.p, tb.d_roff.p, X, gdone, maxkb + 1,
