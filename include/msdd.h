@@ -113,9 +113,10 @@ typedef struct msdd_options {
     int profile;         /* 1: time every kernel family with CUDA events (see msdd_stats.prof);
                             2: only the band-solve families (*_solve): two events per band solve
                             instead of ~500 intervals per set-up, for timing runs */
-    int fp32_start_iters;/* precision 1: most fine-level FP32 subspace iterations (FP32 B apply
-                            and solve, Euclidean CholQR) before the FP64 iterations (default
-                            20); a subdomain ends earlier where its spectrum needs fewer */
+    int fp32_start_iters;/* precision 1: fine-level FP32 subspace iterations (FP32 B apply and
+                            solve, Euclidean CholQR) before the FP64 iterations (default 20).
+                            Under the default a subdomain ends earlier where its spectrum
+                            needs fewer; any other number is run in full by every subdomain */
     const double* warm_start; /* device, may be NULL (default): start vectors of the fine-level
                             subspace iteration, rows = the fine subdomains' Neumann-box nodes
                             (subdomain order, each box lexicographic, x fastest) and warm_cols
@@ -167,7 +168,8 @@ typedef struct msdd_stats {
     msdd_kernel_prof prof[MSDD_MAX_PROF];     /* accumulated over set-up and solves */
     long long eig_iters_total[MSDD_MAX_LEVELS]; /* subspace iterations summed over the level's
                                                  subdomains (FP64 phase; the fine FP32 start
-                                                 phase adds up to fp32_start_iters each) */
+                                                 phase adds fp32_start_iters each, the
+                                                 default at most) */
 } msdd_stats;
 
 typedef struct msdd_hierarchy msdd_hierarchy;   /* opaque, library-owned */

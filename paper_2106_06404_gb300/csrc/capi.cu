@@ -169,7 +169,7 @@ msdd_status msdd_default_options(msdd_options* opt) {
     opt->seed = 12345;
     opt->stream = nullptr;
     opt->profile = 0;
-    opt->fp32_start_iters = 20;
+    opt->fp32_start_iters = msdd::START_ITERS;
     opt->warm_start = nullptr;
     opt->warm_cols = 0;
     return MSDD_OK;

@@ -1314,7 +1314,8 @@ __device__ float cholqr_warp(float (*G)[PMAX + 4], float* dinv, int p, float* __
 // Chebyshev step grows mu_w by x + sqrt(x^2 - 1), x = 2 mu_w / c - 1, against
 // the damped ones; START_GAIN in all takes the block to FP32 accuracy, where
 // further FP32 steps no longer save FP64 ones.  Rounded up to a few stops
-// (start_stop); at most the caller's number.  Fine eigensolve at 20 and at the
+// (start_stop).  Only the default number of iterations is cut short so; a
+// number that the caller chose is run in full.  Fine eigensolve at 20 and at the
 // chosen steps: 512^2 8.8 and 7.0 ms (10-13 steps, the same five FP64
 // iterations), 1000^2 26.8 and 20.7, 50x44x38 22.1 and 16.4 ms; the 96^3
 // composite keeps its 20 (147 ms), where 13 cost six more FP64 iterations
@@ -1343,7 +1344,7 @@ __global__ void __launch_bounds__(G32_T) k_gram_cholqr32(const float* __restrict
                                                          double* __restrict__ cheb, const int* __restrict__ n_,
                                                          const long long* __restrict__ roff_,
                                                          const int* __restrict__ p_, int gsplit,
-                                                         unsigned* __restrict__ ticket, int it, float mu_eta, int nev,
+                                                         unsigned* __restrict__ ticket, int it, int early, float mu_eta, int nev,
                                                          int* __restrict__ sdone, int* __restrict__ sstop,
                                                          int* __restrict__ smax) {
     __shared__ float red[G32_T][17];
@@ -1439,7 +1440,7 @@ __global__ void __launch_bounds__(G32_T) k_gram_cholqr32(const float* __restrict
         for (int o = 16; o > 0; o >>= 1) rmin = fminf(rmin, __shfl_xor_sync(0xffffffffu, rmin, o));
         const float c = (float)CHEB_CUT * rmin;
         if (t == 0) cheb[i] = c;
-        if (it == START_SETTLE - 1) {
+        if (early && it == START_SETTLE - 1) {
             const int stop = start_stop(start_steps(rkk, c, p, nev, mu_eta));
             if (t == 0) {
                 sstop[i] = stop;
@@ -1722,12 +1723,12 @@ void eig_start32(GevpBatch& g, float* W, cudaStream_t s) {
     MSDD_LAUNCH_CHECK();
 }
 
-void eig_cholqr32(GevpBatch& g, const EigParams& ep, int it, EigForm mode, const float* SX, const float* X,
-                  const float* Q, float* V, cudaStream_t s) {
+void eig_cholqr32(GevpBatch& g, const EigParams& ep, int it, EigForm mode, bool early, const float* SX,
+                  const float* X, const float* Q, float* V, cudaStream_t s) {
     // the FP64 Gram partials and coefficients are free in this phase and hold the FP32 ones
     k_gram_cholqr32<<<dim3(g.P, g.gsplit), G32_T, 0, s>>>(SX, X, Q, V, mode, g.ldw, reinterpret_cast<float*>(g.Hp.p),
                                                           reinterpret_cast<float*>(g.C.p), g.cheb.p, g.K.d_n.p,
-                                                          g.K.d_roff.p, g.d_p.p, g.gsplit, g.ticket.p, it,
+                                                          g.K.d_roff.p, g.d_p.p, g.gsplit, g.ticket.p, it, early ? 1 : 0,
                                                           (float)(1.0 / (ep.eta + ep.sigma)), ep.nev_max, g.sdone.p,
                                                           g.sstop.p, g.smax.p);
     MSDD_LAUNCH_CHECK();

@@ -81,15 +81,16 @@ void eig_form_y(GevpBatch& g, double sigma, EigForm mode, cudaStream_t s);
 // and C (FP32, in the buffer of g.C) with V C an orthonormal basis of span(V)
 // by Euclidean CholQR; X <- W C of the problems that end after `steps`
 // iterations (last: or later).  The first START_SETTLE iterations are power
-// steps and every eighth after them; after the settling part sstop holds each
-// problem's number of iterations, one of the stops of start_stop.
+// steps and every eighth after them; with `early`, after the settling part sstop
+// holds each problem's number of iterations, one of the stops of start_stop.
 constexpr int START_SETTLE = 6;
+constexpr int START_ITERS = 20;   // the default number of iterations, under which a problem may end earlier
 __host__ __device__ inline int start_stop(int steps) {
     return steps <= 10 ? 10 : steps <= 13 ? 13 : 1 << 20;
 }
 void eig_start32(GevpBatch& g, float* W, cudaStream_t s);
-void eig_cholqr32(GevpBatch& g, const EigParams& ep, int it, EigForm mode, const float* SX, const float* X,
-                  const float* Q, float* V, cudaStream_t s);
+void eig_cholqr32(GevpBatch& g, const EigParams& ep, int it, EigForm mode, bool early, const float* SX,
+                  const float* X, const float* Q, float* V, cudaStream_t s);
 void eig_update32(GevpBatch& g, const float* W, int steps, bool last, cudaStream_t s);
 // The same with the K^+-norm residual partial sums of X.
 void eig_form_y_knorm(GevpBatch& g, double sigma, EigForm mode, cudaStream_t s);

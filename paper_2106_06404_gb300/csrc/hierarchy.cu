@@ -159,20 +159,21 @@ void run_eig(GevpBatch& g, const EigParams& ep, Apply apply, Solve solve, BApply
     // alone decides convergence.  The damped interval comes from the last power
     // step, so the first six are power steps (the block has to settle) and
     // every eighth after them renews it: 20 such steps leave a 1400-point model
-    // spectrum 2-5 FP64 iterations, 20 power steps 9-14.  Each problem ends
-    // after the iterations that its spectrum needs (start_steps); the host
-    // reads the largest number while the iterations up to the first stop are
-    // still running.
+    // spectrum 2-5 FP64 iterations, 20 power steps 9-14.  Under the default
+    // number each problem ends after the iterations that its spectrum needs
+    // (start_steps); the host reads the largest of them while the iterations up
+    // to the first stop are still running.  Any other number is run in full.
     DevBuf<float> wb(fp32_iters > 0 ? 3 * g.W32.n : 0);
     float *vb = wb.p, *sb = g.W32.p, *xb = wb.p + g.W32.n, *qb = wb.p + 2 * g.W32.n;    // V, S X, X, Q
     auto start_mode = [](int it) {
         const int j = (it - START_SETTLE) % 8;
         return it < START_SETTLE || j == 7 ? FORM_FIRST : j == 0 ? FORM_CHEB1 : FORM_CHEB;
     };
+    const bool early = fp32_iters == START_ITERS;
     for (int k = 0; k < G && fp32_iters > 0; ++k) eig_start32(gv[k], vb, gs[k]);
     for (int it = 0; it < fp32_iters; ++it) {
         const EigForm mode = start_mode(it);
-        if (it == start_stop(0)) {
+        if (early && it == start_stop(0)) {
             int most = 0;
             for (int k = 0; k < G; ++k) {
                 MSDD_CUDA(cudaEventSynchronize(ev_smax[k]));
@@ -195,10 +196,10 @@ void run_eig(GevpBatch& g, const EigParams& ep, Apply apply, Solve solve, BApply
                 MSDD_CUDA(cudaStreamWaitEvent(gs[1], ev_off, 0));
             }
             prof.begin(tag + "_fp32_start_other", gs[k]);
-            eig_cholqr32(v, ep, it, mode, sb, xb, qb, vb, gs[k]);
-            if (it + 1 == fp32_iters || it + 1 == start_stop(it + 1))
+            eig_cholqr32(v, ep, it, mode, early, sb, xb, qb, vb, gs[k]);
+            if (it + 1 == fp32_iters || (early && it + 1 == start_stop(it + 1)))
                 eig_update32(v, mode == FORM_FIRST ? sb : vb, it + 1, it + 1 == fp32_iters, gs[k]);
-            if (it + 1 == START_SETTLE && fp32_iters > START_SETTLE) {
+            if (early && it + 1 == START_SETTLE) {
                 MSDD_CUDA(cudaMemcpyAsync(&h_act[4 + k], v.smax.p, sizeof(int), cudaMemcpyDeviceToHost, gs[k]));
                 MSDD_CUDA(cudaEventRecord(ev_smax[k], gs[k]));
             }
