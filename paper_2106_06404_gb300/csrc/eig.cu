@@ -1588,11 +1588,17 @@ __global__ void k_load_start(double* __restrict__ X, const double* __restrict__ 
 
 }  // namespace
 
-void GevpBatch::alloc(cudaStream_t s) {
+void GevpBatch::alloc(cudaStream_t s, bool fused) {
     P = K.P;
     d_p.upload(p, s);
     size_t rows = (size_t)K.total_rows;
-    for (DevBuf<double>* b : {&X, &AX, &BX, &Y, &AY, &BY, &Q}) { b->alloc(rows * ldx); b->zero(s); }
+    for (DevBuf<double>* b : {&X, &AX, &BX, &Y, &AY, &BY}) { b->alloc(rows * ldx); b->zero(s); }
+    if (fused) {
+        Q = AX.view(0, AX.n);
+    } else {
+        Q.alloc(rows * ldx);
+        Q.zero(s);
+    }
     if (K.prec) {
         int pm = 1;
         for (int v : p) pm = std::max(pm, v);

@@ -34,7 +34,9 @@ struct GevpBatch {
     int ldw = PMAX;
     DevBuf<int> sdone, sstop, smax;   // FP32 start phase: ended, its iterations; per group the largest of them
     DevBuf<unsigned> ticket;          // per problem: row ranges of the FP32 Gram that are done
-    DevBuf<double> Q;                              // the block before X in its basis (Chebyshev recurrence)
+    // the block before X in its basis (Chebyshev recurrence); where AX and BX are only needed by the first iteration
+    // (`fused` of alloc: the operator is applied afresh), a view of AX
+    DevBuf<double> Q;
     DevBuf<double> cheb;                           // per problem: end of the damped interval of S = K^{-1} B, 0 unknown
     DevBuf<double> H, M, C, theta, res;            // per problem PMAX^2 / PMAX
     int gsplit = 1;                                // row splits of the Gram products
@@ -46,7 +48,7 @@ struct GevpBatch {
     DevBuf<int> n_active;
     int nblk_max = 0;
     bool knorm = false;           // residual measured in the K^+-norm (coarse levels)
-    void alloc(cudaStream_t s);
+    void alloc(cudaStream_t s, bool fused = false);
     // Non-owning view of problems [p0, p0 + np) with its own active counter
     // (group < 2): per-problem arrays offset, block vectors shared (they are
     // addressed by absolute row offsets).

@@ -163,14 +163,21 @@ void run_eig(GevpBatch& g, const EigParams& ep, Apply apply, Solve solve, BApply
     // number each problem ends after the iterations that its spectrum needs
     // (start_steps); the host reads the largest of them while the iterations up
     // to the first stop are still running.  Any other number is run in full.
-    DevBuf<float> wb(fp32_iters > 0 ? 3 * g.W32.n : 0);
-    float *vb = wb.p, *sb = g.W32.p, *xb = wb.p + g.W32.n, *qb = wb.p + 2 * g.W32.n;    // V, S X, X, Q
+    // V, X and Q lie in Y, AY and BY, which the FP64 phase writes before it reads them; each group's
+    // (rows of ldw floats) inside its own rows (of ldx doubles) of these, since the groups' phases overlap.
+    struct Start32 { float *v, *s, *x, *q; };       // V, S X, X, Q
+    std::vector<Start32> b32(G);
+    for (int k = 0; k < G; ++k) {
+        const long long r0 = g.K.roff[gp0[k]];
+        auto rows_in = [&](const DevBuf<double>& b) { return reinterpret_cast<float*>(b.p + r0 * g.ldx) - r0 * g.ldw; };
+        b32[k] = {rows_in(g.Y), g.W32.p, rows_in(g.AY), rows_in(g.BY)};
+    }
     auto start_mode = [](int it) {
         const int j = (it - START_SETTLE) % 8;
         return it < START_SETTLE || j == 7 ? FORM_FIRST : j == 0 ? FORM_CHEB1 : FORM_CHEB;
     };
     const bool early = fp32_iters == START_ITERS;
-    for (int k = 0; k < G && fp32_iters > 0; ++k) eig_start32(gv[k], vb, gs[k]);
+    for (int k = 0; k < G && fp32_iters > 0; ++k) eig_start32(gv[k], b32[k].v, gs[k]);
     for (int it = 0; it < fp32_iters; ++it) {
         const EigForm mode = start_mode(it);
         if (early && it == start_stop(0)) {
@@ -184,28 +191,29 @@ void run_eig(GevpBatch& g, const EigParams& ep, Apply apply, Solve solve, BApply
         }
         for (int k = 0; k < G; ++k) {
             GevpBatch& v = gv[k];
+            Start32& b = b32[k];
             prof.begin(tag + "_fp32_start_other", gs[k]);
-            bapply32(v, gp0[k], vb, sb, it == 0 ? nullptr : reinterpret_cast<const float*>(v.C.p),
-                     mode == FORM_FIRST ? nullptr : xb, mode == FORM_CHEB ? qb : nullptr, gs[k]);
+            bapply32(v, gp0[k], b.v, b.s, it == 0 ? nullptr : reinterpret_cast<const float*>(v.C.p),
+                     mode == FORM_FIRST ? nullptr : b.x, mode == FORM_CHEB ? b.q : nullptr, gs[k]);
             prof.end(gs[k], 0.0, 0.0);
             prof.begin(tag + "_solve", gs[k]);
-            solve(v, gp0[k], am[k].pm, sb, (const int*)v.sdone.p, gs[k]);
+            solve(v, gp0[k], am[k].pm, b.s, (const int*)v.sdone.p, gs[k]);
             prof.end(gs[k], am[k].sb0, am[k].sf0);
             if (G == 2 && k == 0 && it == 0) {
                 MSDD_CUDA(cudaEventRecord(ev_off, gs[0]));        // the second half starts one solve later
                 MSDD_CUDA(cudaStreamWaitEvent(gs[1], ev_off, 0));
             }
             prof.begin(tag + "_fp32_start_other", gs[k]);
-            eig_cholqr32(v, ep, it, mode, early, sb, xb, qb, vb, gs[k]);
+            eig_cholqr32(v, ep, it, mode, early, b.s, b.x, b.q, b.v, gs[k]);
             if (it + 1 == fp32_iters || (early && it + 1 == start_stop(it + 1)))
-                eig_update32(v, mode == FORM_FIRST ? sb : vb, it + 1, it + 1 == fp32_iters, gs[k]);
+                eig_update32(v, mode == FORM_FIRST ? b.s : b.v, it + 1, it + 1 == fp32_iters, gs[k]);
             if (early && it + 1 == START_SETTLE) {
                 MSDD_CUDA(cudaMemcpyAsync(&h_act[4 + k], v.smax.p, sizeof(int), cudaMemcpyDeviceToHost, gs[k]));
                 MSDD_CUDA(cudaEventRecord(ev_smax[k], gs[k]));
             }
             prof.end(gs[k], 0.0, 0.0);
+            if (mode == FORM_FIRST) std::swap(b.v, b.s);              // V is S X itself
         }
-        if (mode == FORM_FIRST) std::swap(vb, sb);                // V is S X itself
     }
     std::vector<int> active(G), iter(G, 0);
     for (int k = 0; k < G; ++k) {
@@ -404,7 +412,7 @@ std::vector<ProbBox> make_fine_boxes(const Geom& g, const msdd_decomp& dec) {
 size_t Hierarchy::device_bytes() const {
     size_t b = 0;
     b += fdir.bytes() + fge.K.bytes() + cdir.bytes() + mdir.bytes() + mge.K.bytes();
-    b += (fge.X.n + fge.AX.n + fge.BX.n + fge.Y.n + fge.AY.n + fge.BY.n + fge.W.n + fge.Q.n) * 8 + fge.W32.n * 4;
+    b += (fge.X.n + fge.AX.n + fge.BX.n + fge.Y.n + fge.AY.n + fge.BY.n + fge.W.n) * 8 + fge.W32.n * 4;   // (fge.Q is a view)
     b += (mge.X.n + mge.AX.n + mge.BX.n + mge.Y.n + mge.AY.n + mge.BY.n + mge.W.n + mge.Q.n) * 8;
     b += (Phi.n + A1.n + Abar_m.n + K_m.n + Zb.n + Tm.n + A0.n + frhs.n + v1.n + r0buf.n) * 8;
     b += (Minv.n + A0inv.n + y0buf.n + z1t.n) * 8;
@@ -604,7 +612,7 @@ void Hierarchy::build_fine() {
     fge.ldx = PMAX;
     fge.p.resize(Pf);
     for (int j = 0; j < Pf; ++j) fge.p[j] = std::min(block_p, nN[j]);
-    fge.alloc(st);
+    fge.alloc(st, true);
     EigParams ep;
     ep.sigma = opt.sigma;
     ep.tol = opt.eig_tol;
