@@ -605,26 +605,25 @@ __global__ void k_global_stencil(Geom g, double* __restrict__ S, long long nun) 
 // q = S p over the unknowns with the stored 3^D-point stencil, and block
 // partial sums of p.q.  Every neighbour index is clamped into [0, nun): a
 // neighbour outside the unknown box has coefficient exactly 0 in S, so its
-// term adds nothing and the loads need no branch.  Indices fit 32 bits (the
-// set-up rejects 2^31 unknowns or more).  The FP64 pipe (3^D + 1 operations an
+// term adds nothing and the loads need no branch.  Indices are unsigned 32-bit
+// numbers (the set-up rejects 2^31 unknowns or more).  The FP64 pipe (3^D + 1 operations an
 // unknown) and the launch bound it.
 template <int D>
 __global__ void __launch_bounds__(PCG_NT) k_spmv_stencil_dot(Geom g, const double* __restrict__ S,
                                                              const double* __restrict__ p, double* __restrict__ q,
-                                                             int nun, double* __restrict__ partial,
+                                                             unsigned nun, double* __restrict__ partial,
                                                              const int* __restrict__ done, PcgScalars* sc, int fin) {
     __shared__ double red[PCG_NT];
     if (done && *done) return;
     constexpr int NOFF = D == 3 ? 27 : 9;
-    const int sy = g.ushape[0], sz = g.ushape[0] * g.ushape[1];
+    const unsigned sy = g.ushape[0], sz = sy * (unsigned)g.ushape[1];
     double part = 0.0;
-    for (int u = blockIdx.x * PCG_NT + threadIdx.x; u < nun; u += gridDim.x * PCG_NT) {
+    for (UnknownIndex u = blockIdx.x * PCG_NT + threadIdx.x; u < nun; u += gridDim.x * PCG_NT) {
         double a0 = 0.0, a1 = 0.0;
 #pragma unroll
         for (int oi = 0; oi < NOFF; ++oi) {
             const double c = S[(long long)oi * nun + u];
-            int v = u + (oi % 3 - 1) + ((oi / 3) % 3 - 1) * sy + (D == 3 ? (oi / 9 - 1) * sz : 0);
-            v = min(max(v, 0), nun - 1);
+            const unsigned v = stencil_neighbour(u, stencil_offset(oi, D, sy, sz), nun);
             if (oi & 1) a1 = fma(c, p[v], a1);
             else a0 = fma(c, p[v], a0);
         }
@@ -801,9 +800,9 @@ void spmv_stencil_dot(const Geom& g, const double* S, const double* p, double* q
                       const int* done, cudaStream_t s, PcgScalars* sc, int fin) {
     long long nun = (long long)g.ushape[0] * g.ushape[1] * (g.dim == 3 ? g.ushape[2] : 1);
     if (g.dim == 3)
-        k_spmv_stencil_dot<3><<<nblocks, PCG_NT, 0, s>>>(g, S, p, q, (int)nun, partial, done, sc, fin);
+        k_spmv_stencil_dot<3><<<nblocks, PCG_NT, 0, s>>>(g, S, p, q, (unsigned)nun, partial, done, sc, fin);
     else
-        k_spmv_stencil_dot<2><<<nblocks, PCG_NT, 0, s>>>(g, S, p, q, (int)nun, partial, done, sc, fin);
+        k_spmv_stencil_dot<2><<<nblocks, PCG_NT, 0, s>>>(g, S, p, q, (unsigned)nun, partial, done, sc, fin);
     MSDD_LAUNCH_CHECK();
 }
 

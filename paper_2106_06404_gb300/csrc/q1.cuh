@@ -131,6 +131,20 @@ void apply_local_b32(const LocalStencil& ls, const ProbBox* d_boxes, int dim, co
                      const float* W, float* Wout, int ldw, const float* C, float* X, float* Q,
                      const int* skip, cudaStream_t s);
 
+// Loop counter over the unknowns (fewer than 2^31) in steps of a grid: as a signed
+// number it would wrap in the step past the last unknown.
+using UnknownIndex = unsigned;
+// Linear index of neighbour oi of unknown u (row length sy, plane size sz), in
+// [0, nun) whatever the offset: modulo 2^32 it is exact for every neighbour inside
+// the unknown box (nun < 2^31); outside, where the coefficient is 0, any index does.
+__host__ __device__ constexpr unsigned stencil_offset(int oi, int dim, unsigned sy, unsigned sz) {
+    return (unsigned)(oi % 3 - 1) + (unsigned)((oi / 3) % 3 - 1) * sy + (dim == 3 ? (unsigned)(oi / 9 - 1) * sz : 0u);
+}
+__host__ __device__ constexpr unsigned stencil_neighbour(unsigned u, unsigned offset, unsigned nun) {
+    const unsigned v = u + offset, last = nun - 1u;
+    return v < last ? v : last;
+}
+
 // Stored 3^d-point stencil of the global operator: S[o * n + u] = A(u, u + o),
 // offsets o lexicographic (x fastest) in {-1, 0, 1}^d, zero where u + o is
 // not an unknown.  n * 3^d doubles.
