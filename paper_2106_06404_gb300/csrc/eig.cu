@@ -26,7 +26,8 @@ __global__ void k_init(double* __restrict__ X, const int* __restrict__ n_, const
                        const long long* __restrict__ roff_, const int* __restrict__ p_, int ldx,
                        unsigned long long seed, int* __restrict__ done, int* __restrict__ iters,
                        double* __restrict__ theta, double* __restrict__ best, int* __restrict__ best_it,
-                       int* __restrict__ sdone, int* __restrict__ sstop, int* __restrict__ smax) {
+                       int* __restrict__ sdone, int* __restrict__ sstop, int* __restrict__ smax,
+                       int* __restrict__ m_, double* __restrict__ res) {
     const int i = blockIdx.y;
     const int n = n_[i], p = p_[i];
     const long long rows = (long long)K_[i] * NB;
@@ -42,9 +43,11 @@ __global__ void k_init(double* __restrict__ X, const int* __restrict__ n_, const
     }
     if (blockIdx.x == 0 && threadIdx.x < PMAX) {
         theta[i * PMAX + threadIdx.x] = 0.0;
+        res[i * PMAX + threadIdx.x] = 1e300;               // until a convergence test
         if (threadIdx.x == 0) {
             done[i] = (n == 0 || p == 0) ? 1 : 0;
             iters[i] = 0;
+            m_[i] = 0;
             sdone[i] = done[i];
             sstop[i] = 1 << 20;
             if (i < 2) smax[i] = 0;
@@ -1219,6 +1222,16 @@ __global__ void k_check(const double* __restrict__ partial, const double* __rest
                best_it);
 }
 
+// m of the running problems from their Ritz values
+__global__ void k_select(const double* __restrict__ theta, const int* __restrict__ p_, double eta, int nev_max,
+                         const int* __restrict__ done, int* __restrict__ m_, int P) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= P || done[i]) return;
+    int count = 0;
+    for (int k = 0; k < p_[i]; ++k) count += theta[i * PMAX + k] < eta ? 1 : 0;
+    m_[i] = min(count, nev_max);
+}
+
 __global__ void k_check_knorm(const double* __restrict__ partial, const double* __restrict__ theta,
                               double* __restrict__ res, const int* __restrict__ K_, const int* __restrict__ p_,
                               int nblk_max, double sigma, double tol, double eta, int nev_max, int it, int maxit,
@@ -1684,7 +1697,7 @@ void eig_init(GevpBatch& g, unsigned long long seed, cudaStream_t s) {
     if (g.P == 0) return;
     dim3 grid(32, g.P);
     k_init<<<grid, 256, 0, s>>>(g.X.p, g.K.d_n.p, g.K.d_K.p, g.K.d_roff.p, g.d_p.p, g.ldx, seed, g.done.p, g.iters.p,
-                                g.theta.p, g.best.p, g.best_it.p, g.sdone.p, g.sstop.p, g.smax.p);
+                                g.theta.p, g.best.p, g.best_it.p, g.sdone.p, g.sstop.p, g.smax.p, g.m.p, g.res.p);
     MSDD_LAUNCH_CHECK();
 }
 
@@ -1714,6 +1727,11 @@ void eig_form_y_knorm(GevpBatch& g, double sigma, EigForm mode, cudaStream_t s) 
     dim3 grid(g.nblk_max, g.P);
     k_form_y_knorm<<<grid, TPB, 0, s>>>(g.Y.p, g.X.p, g.W.p, g.AX.p, g.BX.p, g.Q.p, g.cheb.p, mode, g.theta.p, g.K.d_n.p, g.K.d_K.p,
                                         g.K.d_roff.p, g.d_p.p, g.ldx, sigma, g.partial.p, g.nblk_max, g.done.p);
+    MSDD_LAUNCH_CHECK();
+}
+
+void eig_select(GevpBatch& g, const EigParams& ep, cudaStream_t s) {
+    k_select<<<ceil_div(g.P, 128), 128, 0, s>>>(g.theta.p, g.d_p.p, ep.eta, ep.nev_max, g.done.p, g.m.p, g.P);
     MSDD_LAUNCH_CHECK();
 }
 

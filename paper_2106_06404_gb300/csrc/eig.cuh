@@ -107,7 +107,9 @@ void eig_update(GevpBatch& g, bool want_q, cudaStream_t s);
 // X = Y C only: with a cheap operator (stored stencils) AX and BX are applied
 // afresh, together with the next right-hand side (apply_local_rhs).
 void eig_update_x(GevpBatch& g, bool want_q, cudaStream_t s);
-// Residuals, selection count m = min(nev_max, #{theta < eta}), convergence flags.
+// Selection count m = min(nev_max, #{theta < eta}) of the running problems.
+void eig_select(GevpBatch& g, const EigParams& ep, cudaStream_t s);
+// Residuals, selection count m, convergence flags.
 void eig_check(GevpBatch& g, const EigParams& ep, int it, cudaStream_t s);
 
 // Dense operators for the coarse levels: Abar dense (problem i at aoff[i],

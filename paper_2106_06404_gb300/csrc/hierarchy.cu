@@ -318,7 +318,9 @@ void run_eig(GevpBatch& g, const EigParams& ep, Apply apply, Solve solve, BApply
     int left = 0;
     for (int k = 0; k < G; ++k) left += active[k];
     if (g.knorm && left > 0) {
-        // eig_maxit reached: the last updated pairs are kept and marked unconverged
+        // eig_maxit reached: the last updated pairs are kept and marked unconverged (after one iteration no test has
+        // counted them yet)
+        if (ep.maxit == 1) eig_select(g, ep, st);
         std::vector<int> dn = g.done.download(st);
         for (int& v : dn)
             if (v == 0) v = 2;
