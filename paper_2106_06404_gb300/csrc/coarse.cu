@@ -374,7 +374,7 @@ void segment_copy(const long long* d_src_off, const long long* d_dst_off, const 
 }
 
 // one unknown a thread up to eight blocks an SM
-int dot_blocks(long long n) { return (int)std::max(1u, std::min(ceil_div(n, PCG_NT), 152u * 8)); }
+int dot_blocks(long long n) { return (int)std::max(1u, std::min(ceil_div(n, PCG_NT), NUM_SMS * 8u)); }
 
 void dot_partial(const double* x, const double* y, long long n, double* partial, int nblocks, cudaStream_t s) {
     k_dot_partial<<<nblocks, 256, 0, s>>>(x, y, n, partial);

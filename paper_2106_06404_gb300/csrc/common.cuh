@@ -15,6 +15,8 @@ constexpr int NB = 32;
 constexpr int NB2 = NB * NB;
 // Maximum block size of the subspace iteration (columns of X, Y).
 constexpr int PMAX = 32;
+// streaming multiprocessors of a GB300 (two dies of 76): the rules that spread work over the chip count in them
+constexpr int NUM_SMS = 152;
 // rows per block of the eigensolver's residual partial sums: entry
 // ((i * nblk_max + blk) * 2 + {0, 1}) * PMAX + c holds, for rows
 // [32 blk, 32 blk + 32) of problem i and column c, sum |AX - theta BX|^2 and

@@ -16,10 +16,11 @@ constexpr int ROWBLK = EIG_ROWBLK;
 // Ritz value mu_p of the block bounds it from above once the block has settled
 // and is below mu_p's limit before that (Ritz values grow), where a smaller
 // interval only damps less.  0.95 of it rather than all of it, so that the
-// last wanted pair still grows against the interval when the block holds no
-// guard columns (block_p = nev_max): 12 pairs of a 1400-point model spectrum
-// in a block of 12 took 95 plain steps, 31 at 0.95, over 100 at 1; in a block
-// of 16, 48, 19 and 17.
+// last wanted pair still grows against the interval in the smallest block that
+// a caller may ask for, one guard column: of four model spectra of some 1400
+// points the slowest took 122 plain steps there, 41 at 0.9, 28 at 0.95 and 31 at
+// 1.  With the default four guard columns the same four took 51 / 15 / 54 / 51
+// plain steps, 21 / 11 / 22 / 20 at 0.95 and 18 / 10 / 19 / 19 at 1.
 constexpr double CHEB_CUT = 0.95;
 
 __global__ void k_init(double* __restrict__ X, const int* __restrict__ n_, const int* __restrict__ K_,

@@ -6,12 +6,15 @@
 // the non-defectiveness lemma of Section 3.3).
 //
 // One iteration for every unconverged problem i (X B-orthonormal Ritz vectors
-// with Ritz values theta, AX = Abar X, BX = B X):
+// with Ritz values theta, AX = Abar X, BX = B X, S = K^{-1} B):
 //   W = BX - (AX + sigma BX) diag(mu),      mu_k = 1 / (theta_k + sigma)
-//   W <- K^{-1} W        (tile LDL^T solve, FP64 or FP32 factors)
-//   Y = X diag(mu) + W   (= K^{-1} B X when the solve is exact)
+//   W <- K^{-1} W        (tile LDL^T solve, FP64 or FP32 factors), so that S X = X diag(mu) + W
+//   Y = the Chebyshev step of S X, X and Q (the block before X in the basis of
+//       X) that damps [0, c], c = 0.95 times the smallest Ritz value of S in
+//       the block; the first iteration Y = S X
 //   AY, BY; H = Y^T AY, M = Y^T BY (FP64); Rayleigh-Ritz H c = theta M c
-//   X = Y C, AX = AY C, BX = BY C; residuals |AX_k - theta_k BX_k| / ((theta_k + sigma) |BX_k|).
+//   Q = X C, X = Y C, AX = AY C, BX = BY C (with a cheap operator X and Q only, AX
+//       and BX afresh); residuals |AX_k - theta_k BX_k| / ((theta_k + sigma) |BX_k|).
 // The residual form lets an inexact (lower precision) K^{-1} still converge
 // to the FP64 eigenpairs: its fixed point does not depend on the solve.
 #pragma once

@@ -1309,19 +1309,19 @@ __device__ __forceinline__ void mbar_arrive(unsigned long long* bar) {
 //
 // A solve is a chain of 2 K dependent steps of one CTA; a step's products
 // are (kb + 1) tiles of 32 x 32 by 4 J columns.  Letting every warp run over
-// all tiles for columns of its own makes each tile element travel from shared
-// memory once per warp (LSU bound: the earlier form took 3350 cycles a step
-// at kb = 2, 9700 at kb = 12).  Here the NW consumer warps split the k index
-// instead, so that every tile element is read once: a warp takes groups of
-// four k and accumulates all 32 rows x 4 J columns in registers (lane = 8 row
-// groups x 4 column groups, 4 rows x J columns each: 4 + J wide loads per
-// 16 J FMA).  The partial sums are exchanged through shared memory: warp w
-// sums and finishes the 32 / NW rows of its slice, which are exactly the rows
-// it then multiplies as its k-slice of T_R, and of the next step's nearest
-// tile.  Two barriers of the consumer warps a step.  128 problems of n = 1369,
-// b = 38, 16 columns: 134.6 -> 110.8 us a launch (with X in FP32); 108 of
-// n = 6859, b = 381, 20 columns: 2113 -> 1571 us.  Still bound by shared
-// memory: 4 + J 16-byte loads, four LSU cycles each, feed 16 J FMA.
+// all tiles for columns of its own (k_tile_solve_band_ws below) makes each tile
+// element travel from shared memory once per warp.  Here the NW consumer warps
+// split the k index instead, so that every tile element is read once: a warp
+// takes groups of four k and accumulates all 32 rows x 4 J columns in registers
+// (lane = 8 row groups x 4 column groups, 4 rows x J columns each: 4 + J wide
+// loads per 16 J FMA).  The partial sums are exchanged through shared memory:
+// warp w sums and finishes the 32 / NW rows of its slice, which are exactly the
+// rows it then multiplies as its k-slice of T_R, and of the next step's nearest
+// tile.  The exchange costs two barriers of the consumer warps a step, which
+// pays where a step has many tiles or columns (solve_band_f32 has the line): of
+// 128 problems of n = 1500, b = 380, 20 columns, FP32 X 400 -> 324 us a launch;
+// of 128 with b = 38, 16 columns 107 -> 121.  Still bound by shared memory: 4 + J
+// 16-byte loads, four LSU cycles each, feed 16 J FMA.
 //
 // A producer warp streams the tiles of each step by TMA (128-byte swizzle,
 // ring of nst stages of S = maxkb + 1 tiles, "full" mbarriers by byte count,
@@ -1870,21 +1870,20 @@ void launch_band_ks(const TileBatch& tb, const CUtensorMap& tm, int maxkb, XT* X
 template <typename XT>
 void solve_band_f32(const TileBatch& tb, const CUtensorMap& tm, int maxkb, XT* X, int ldx, int ncols, const int* skip,
                     cudaStream_t s, const int* gdone) {
-    constexpr int SMS = 152;
     constexpr bool F64X = sizeof(XT) == 8;
     int chunks = (ncols + 19) / 20, J = (ncols + 4 * chunks - 1) / (4 * chunks);
-    while (J > 1 && (long long)tb.P * ((ncols + 4 * (J - 1) - 1) / (4 * (J - 1))) <= SMS) --J;
+    while (J > 1 && (long long)tb.P * ((ncols + 4 * (J - 1) - 1) / (4 * (J - 1))) <= NUM_SMS) --J;
     chunks = (ncols + 4 * J - 1) / (4 * J);
     const long long ctas = (long long)tb.P * chunks;
-    const bool own_sm = ctas <= SMS;
+    const bool own_sm = ctas <= NUM_SMS;
     const int NW = maxkb <= 2 ? 4
                    : F64X && J >= 4 ? 8
                    : maxkb <= 6 ? (J == 5 && own_sm && maxkb > 4 ? 8 : 4)
                    : J == 1 || J == 5 ? 8 : 4;
     const size_t bytes = band_ks_smem(NW, J, maxkb + 1, band_ks_stages(NW, J, maxkb + 1));
-    const long long ks_rounds = ceil_div(ctas, SMS * std::max<long long>(1, 227 * 1024 / (bytes + 1024)));
+    const long long ks_rounds = ceil_div(ctas, NUM_SMS * std::max<long long>(1, 227 * 1024 / (bytes + 1024)));
     const int ws_cols = maxkb <= 2 ? 16 : 20;
-    const long long ws_rounds = ceil_div((long long)tb.P * ((ncols + ws_cols - 1) / ws_cols), maxkb <= 2 ? 2 * SMS : SMS);
+    const long long ws_rounds = ceil_div((long long)tb.P * ((ncols + ws_cols - 1) / ws_cols), maxkb <= 2 ? 2 * NUM_SMS : NUM_SMS);
     bool ks;
     if (maxkb <= 2)
         ks = ks_rounds != ws_rounds ? ks_rounds < ws_rounds : maxkb == 2 && ((own_sm && J <= 2) || (!F64X && ncols > 28));
@@ -2762,7 +2761,7 @@ void tile_solve(const TileBatch& tb, double* X, int ldx, int ncols, const int* s
             // one turn ahead where two do not fit beside the vector (n = 38500, b = 38: 3.4 ms without the ring, 0.73 with
             // it), and where two leave one CTA an SM to more CTAs than SMs (n = 1369, b = 60, 256 problems: 126 -> 103 us)
             const size_t deep = s1w_bytes(2, nbox, tb.max_K);
-            const int D = deep <= (tb.P > 152 ? 112 : 226) * 1024 ? 2 : 1;
+            const int D = deep <= (tb.P > NUM_SMS ? 112 : 226) * 1024 ? 2 : 1;
             const size_t bytes = s1w_bytes(D, nbox, tb.max_K);
             if (tm && bytes <= 226 * 1024 &&
                 encode_box_map(tb.tiles_f.p, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, tb.total_tile_elems, 8,
@@ -2783,7 +2782,7 @@ void tile_solve(const TileBatch& tb, double* X, int ldx, int ncols, const int* s
             // without a ring hide the tiles' latency better in more (b = 157, n = 1369: 152 problems 526 -> 278 us, 300
             // 575 -> 504, but 700 894 -> 1181; b = 100, n = 441, 700 problems 254 -> 334)
             const bool ring = maxkb <= 2 || zbytes > 160 * 1024 ||
-                              tb.P <= 2 * 152 * (int)std::max<size_t>(1, 227 * 1024 / (bytes + 1024));
+                              tb.P <= 2 * NUM_SMS * (int)std::max<size_t>(1, 227 * 1024 / (bytes + 1024));
             alignas(64) CUtensorMap tm;
             if (ring && bytes <= 226 * 1024 &&
                 encode_box_map(tb.tiles_d.p, CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 8, tb.total_tile_elems, 16,

@@ -82,8 +82,9 @@ void mirror_lower(const TileBatch& tb, const double* E, int lde, int maxn, const
 // E (total_rows x lde) <- per problem the identity of order n[i] (zero elsewhere).
 void tile_identity(const TileBatch& tb, double* E, int lde, cudaStream_t s);
 // Solve K X = B in place.  X is double, row-major, problem i rows at
-// (roff[i] + r) * ldx, columns 0..ncols-1 (any ncols <= ldx; blocks of 32
-// columns go to separate CTAs).  `skip` (device, per problem, may be
+// (roff[i] + r) * ldx, columns 0..ncols-1 (any ncols <= ldx; groups of at most
+// 20 columns with FP32 factors, 4, 2 or 1 with FP64 ones go to separate CTAs, of
+// 32 in the generic kernel).  `skip` (device, per problem, may be
 // null) skips problems whose flag is non-zero; `gdone` (device, may be null)
 // skips everything when non-zero.
 void tile_solve(const TileBatch& tb, double* X, int ldx, int ncols, const int* skip, cudaStream_t s,

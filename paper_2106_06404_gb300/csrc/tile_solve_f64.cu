@@ -197,13 +197,13 @@ void launch_f64(const TileBatch& tb, int maxkb, double* X, int ldx, int ncols, c
     MSDD_LAUNCH_CHECK();
 }
 
-// Columns per CTA: 4 while that gives 1.5 CTAs for each of the 152 SMs, else
+// Columns per CTA: 4 while that gives 1.5 CTAs for each SM, else
 // 2 or 1 (fewer columns cost shuffles and tile reads, idle SMs cost more).
 // 0: the solution ring does not fit shared memory (dense problems beyond
 // 21,000 rows).
 int f64_columns(const TileBatch& tb, int maxkb, int ncols) {
     for (int c : {4, 2, 1})
-        if ((c == 1 || (c <= ncols && (long long)tb.P * ((ncols + c - 1) / c) >= 228)) && f6_bytes(maxkb, c) <= F6_MAX)
+        if ((c == 1 || (c <= ncols && (long long)tb.P * ((ncols + c - 1) / c) >= 3 * NUM_SMS / 2)) && f6_bytes(maxkb, c) <= F6_MAX)
             return c;
     return 0;
 }
