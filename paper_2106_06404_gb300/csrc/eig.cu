@@ -994,7 +994,10 @@ __global__ void __launch_bounds__(TPB) k_rayleigh_ritz(const double* __restrict_
         for (int k = 0; k < p; ++k) r += th[k] > 0.0 ? 1 : 0;
     }
 sorted_output:
-    // sort eigenvalues ascending; apply D to rows of C
+    // sort eigenvalues ascending; apply D to rows of C.  A NaN counts as a dropped
+    // column: every position of perm is written whatever the pencil holds
+    if (t < p && !(S[t][t] < 1e300)) S[t][t] = 1e300;
+    __syncthreads();
     if (t < p) {
         double v = S[t][t];
         int rk = 0;
