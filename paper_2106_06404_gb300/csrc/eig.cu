@@ -22,6 +22,22 @@ constexpr int ROWBLK = EIG_ROWBLK;
 // 1.  With the default four guard columns the same four took 51 / 15 / 54 / 51
 // plain steps, 21 / 11 / 22 / 20 at 0.95 and 18 / 10 / 19 / 19 at 1.
 constexpr double CHEB_CUT = 0.95;
+// A block that spans more than the range of B (small subdomains, generating
+// systems) holds Ritz values of S that are rounding errors, 1e-19 and less; an
+// interval that short would scale the wanted columns by its inverse, out of the
+// double-float products' range and past the accuracy of the others.  The interval
+// therefore ends no earlier than at CHEB_FLOOR of the largest Ritz value (a step
+// then grows it by 4e6 at most), or at half of mu at eta where that is lower: a
+// wanted pair is not damped (down to 1e-12 of the largest, below which S does not
+// resolve any).  Blocks whose Ritz values lie within six orders, all of the usual
+// ones, are not affected.
+constexpr double CHEB_FLOOR = 1e-6;
+template <typename T>
+__device__ __forceinline__ T cheb_end(T c, T mu_max, T mu_eta) {        // c: CHEB_CUT mu_min
+    const T f = T(CHEB_FLOOR) * mu_max, h = T(0.5) * mu_eta, r = T(1e-12) * mu_max;
+    const T low = f < h ? f : h > r ? h : r;
+    return c > low ? c : low;
+}
 
 __global__ void k_init(double* __restrict__ X, const int* __restrict__ n_, const int* __restrict__ K_,
                        const long long* __restrict__ roff_, const int* __restrict__ p_, int ldx,
@@ -848,7 +864,7 @@ __device__ bool rr_fast(double (*S)[LD], double (*V)[LD], double (*L)[LD], doubl
 __global__ void __launch_bounds__(TPB) k_rayleigh_ritz(const double* __restrict__ Hp, const double* __restrict__ Mp,
                                                        int gsplit, double* __restrict__ H, double* __restrict__ M,
                                                        double* __restrict__ C, double* __restrict__ theta,
-                                                       double* __restrict__ cheb, double sigma,
+                                                       double* __restrict__ cheb, double sigma, double eta,
                                                        const int* __restrict__ p_, int* __restrict__ rank,
                                                        const int* __restrict__ done) {
     __shared__ double S[PMAX][LD], V[PMAX][LD], L[PMAX][LD], T[PMAX][LD], U[PMAX][LD];
@@ -1018,11 +1034,12 @@ sorted_output:
     }
     if (t == 0) {
         rank[i] = r;
-        // damped interval [0, CHEB_CUT mu_min]: mu_min the smallest finite Ritz value of S = K^{-1} B in the block
+        // damped interval: mu_min the smallest finite Ritz value of S = K^{-1} B in the block
         int k = p - 1;
         while (k > 0 && !(S[perm[k]][perm[k]] < 1e299)) --k;
         const double th = S[perm[k]][perm[k]] + sigma;
-        cheb[i] = th > 0.0 && th < 1e299 ? CHEB_CUT / th : 0.0;
+        const double th0 = S[perm[0]][perm[0]] + sigma;
+        cheb[i] = th0 > 0.0 && th < 1e299 ? cheb_end(CHEB_CUT / th, 1.0 / th0, 1.0 / (eta + sigma)) : 0.0;
     }
 }
 
@@ -1453,9 +1470,12 @@ __global__ void __launch_bounds__(G32_T) k_gram_cholqr32(const float* __restrict
     else if (ldw <= 20) rkk = cholqr_warp<20>(G, dinv, p, Ci);
     else rkk = cholqr_warp<32>(G, dinv, p, Ci);
     if (mode == FORM_FIRST) {
-        float rmin = rkk;
-        for (int o = 16; o > 0; o >>= 1) rmin = fminf(rmin, __shfl_xor_sync(0xffffffffu, rmin, o));
-        const float c = (float)CHEB_CUT * rmin;
+        float rmin = rkk, rmax = t < p ? rkk : 0.f;
+        for (int o = 16; o > 0; o >>= 1) {
+            rmin = fminf(rmin, __shfl_xor_sync(0xffffffffu, rmin, o));
+            rmax = fmaxf(rmax, __shfl_xor_sync(0xffffffffu, rmax, o));
+        }
+        const float c = rmin > 0.f ? cheb_end((float)CHEB_CUT * rmin, rmax, mu_eta) : 0.f;
         if (t == 0) cheb[i] = c;
         if (early && it == START_SETTLE - 1) {
             const int stop = start_stop(start_steps(rkk, c, p, nev, mu_eta));
@@ -1780,8 +1800,8 @@ void eig_gram(GevpBatch& g, cudaStream_t s) {
     MSDD_LAUNCH_CHECK();
 }
 
-void eig_rayleigh_ritz(GevpBatch& g, double sigma, cudaStream_t s) {
-    k_rayleigh_ritz<<<g.P, TPB, 0, s>>>(g.Hp.p, g.Mp.p, g.gsplit, g.H.p, g.M.p, g.C.p, g.theta.p, g.cheb.p, sigma,
+void eig_rayleigh_ritz(GevpBatch& g, const EigParams& ep, cudaStream_t s) {
+    k_rayleigh_ritz<<<g.P, TPB, 0, s>>>(g.Hp.p, g.Mp.p, g.gsplit, g.H.p, g.M.p, g.C.p, g.theta.p, g.cheb.p, ep.sigma, ep.eta,
                                         g.d_p.p, g.rank.p, g.done.p);
     MSDD_LAUNCH_CHECK();
 }
