@@ -23,21 +23,15 @@ constexpr int ROWBLK = EIG_ROWBLK;
 // plain steps, 21 / 11 / 22 / 20 at 0.95 and 18 / 10 / 19 / 19 at 1.
 constexpr double CHEB_CUT = 0.95;
 // A block that spans more than the range of B (small subdomains, generating
-// systems) holds Ritz values of S that are rounding errors, 1e-19 and less; an
-// interval that short would scale the wanted columns by its inverse, out of the
-// double-float products' range and past the accuracy of the others.  The interval
-// therefore ends no earlier than at CHEB_FLOOR of the largest Ritz value (a step
-// then grows it by 4e6 at most), or at half of mu at eta where that is lower: a
-// wanted pair is not damped (down to 1e-12 of the largest, below which S does not
-// resolve any).  Blocks whose Ritz values lie within six orders, all of the usual
-// ones, are not affected.
-constexpr double CHEB_FLOOR = 1e-6;
-template <typename T>
-__device__ __forceinline__ T cheb_end(T c, T mu_max, T mu_eta) {        // c: CHEB_CUT mu_min
-    const T f = T(CHEB_FLOOR) * mu_max, h = T(0.5) * mu_eta, r = T(1e-12) * mu_max;
-    const T low = f < h ? f : h > r ? h : r;
-    return c > low ? c : low;
-}
+// systems) has columns without a B-norm of their own: normalised in it they are
+// rounding errors times up to 1e9, with Ritz values of any size.  S takes them to
+// nothing, but a Chebyshev polynomial is 1 at zero, and Q carries them into the
+// other columns.  Where the scaled Gram matrix has a pivot below this, or the Ritz
+// values of S lie further apart than CHEB_RANGE, the next step is the plain one (Y
+// = S X), and the first one after it starts the recurrence anew.  The blocks of
+// subdomains larger than a few dozen nodes stay well away from both.
+constexpr double CHEB_PIVOT = 1e-9;
+constexpr double CHEB_RANGE = 1e6, CHEB_RANGE32 = 1e5;      // (FP32 start phase)
 
 __global__ void k_init(double* __restrict__ X, const int* __restrict__ n_, const int* __restrict__ K_,
                        const long long* __restrict__ roff_, const int* __restrict__ p_, int ldx,
@@ -105,14 +99,16 @@ __global__ void k_form_rhs(WT* __restrict__ W, int ldw, const double* __restrict
 // the Chebyshev recurrence in x = (S - e) / e on the damped interval [0, 2 e],
 //   Y = 2 x X - Q  (FORM_CHEB), the first step of it Y = x X  (FORM_CHEB1),
 // where Q is the block before X in the basis of X.  FORM_FIRST: Y = W (the
-// block W = S X itself).  2 e = cheb[i] (0: no interval known, plain step).
+// block W = S X itself).  2 e = |cheb[i]| (0: plain step; negative: the step
+// before was a plain one, so this is the first of the recurrence whatever mode says).
 __device__ __forceinline__ void cheb_coef(int mode, double cc, double mu, double& a, double& w, double& q) {
     if (mode == FORM_FIRST) { a = 0.0; w = 1.0; q = 0.0; return; }
-    if (!(cc > 0.0)) { a = mu; w = 1.0; q = 0.0; return; }
-    const double e = 0.5 * cc;
-    w = (mode == FORM_CHEB ? 2.0 : 1.0) / e;
+    if (!(fabs(cc) > 0.0)) { a = mu; w = 1.0; q = 0.0; return; }
+    const bool on = mode == FORM_CHEB && cc > 0.0;
+    const double e = 0.5 * fabs(cc);
+    w = (on ? 2.0 : 1.0) / e;
     a = w * (mu - e);
-    q = mode == FORM_CHEB ? -1.0 : 0.0;
+    q = on ? -1.0 : 0.0;
 }
 
 template <typename WT>
@@ -864,13 +860,13 @@ __device__ bool rr_fast(double (*S)[LD], double (*V)[LD], double (*L)[LD], doubl
 __global__ void __launch_bounds__(TPB) k_rayleigh_ritz(const double* __restrict__ Hp, const double* __restrict__ Mp,
                                                        int gsplit, double* __restrict__ H, double* __restrict__ M,
                                                        double* __restrict__ C, double* __restrict__ theta,
-                                                       double* __restrict__ cheb, double sigma, double eta,
+                                                       double* __restrict__ cheb, double sigma,
                                                        const int* __restrict__ p_, int* __restrict__ rank,
                                                        const int* __restrict__ done) {
     __shared__ double S[PMAX][LD], V[PMAX][LD], L[PMAX][LD], T[PMAX][LD], U[PMAX][LD];
     __shared__ double dsc[PMAX], th[PMAX], linv[PMAX];
     __shared__ int perm[PMAX];
-    __shared__ int s_fail, s_zero;
+    __shared__ int s_fail, s_zero, s_deficient;
     const int i = blockIdx.x;
     if (done[i]) return;
     const int p = p_[i];
@@ -891,7 +887,7 @@ __global__ void __launch_bounds__(TPB) k_rayleigh_ritz(const double* __restrict_
     }
     const double* Hi = Hw;
     const double* Mi = Mw;
-    if (t == 0) s_zero = 0;
+    if (t == 0) { s_zero = 0; s_deficient = 0; }
     __syncthreads();
     if (t < PMAX) {
         double mkk = t < p ? Mi[t * PMAX + t] : 0.0;
@@ -921,6 +917,7 @@ __global__ void __launch_bounds__(TPB) k_rayleigh_ritz(const double* __restrict_
         for (int k = 0; k < p; ++k) {
             const double d = L[k][k];
             double lkk = 0.0, r = 0.0;
+            if (lane == 0 && (dsc[k] == 0.0 || !(d > CHEB_PIVOT))) s_deficient = 1;
             if (dsc[k] != 0.0) {
                 if (d > 1e-13) { r = rsqrt_nr(d); lkk = d * r; }
                 else fail = 1;
@@ -1039,7 +1036,9 @@ sorted_output:
         while (k > 0 && !(S[perm[k]][perm[k]] < 1e299)) --k;
         const double th = S[perm[k]][perm[k]] + sigma;
         const double th0 = S[perm[0]][perm[0]] + sigma;
-        cheb[i] = th0 > 0.0 && th < 1e299 ? cheb_end(CHEB_CUT / th, 1.0 / th0, 1.0 / (eta + sigma)) : 0.0;
+        const bool ok = !s_deficient && th0 > 0.0 && th < 1e299 && th <= CHEB_RANGE * th0;
+        const double c = ok ? CHEB_CUT / th : 0.0;
+        cheb[i] = cheb[i] == 0.0 ? -c : c;
     }
 }
 
@@ -1475,7 +1474,7 @@ __global__ void __launch_bounds__(G32_T) k_gram_cholqr32(const float* __restrict
             rmin = fminf(rmin, __shfl_xor_sync(0xffffffffu, rmin, o));
             rmax = fmaxf(rmax, __shfl_xor_sync(0xffffffffu, rmax, o));
         }
-        const float c = rmin > 0.f ? cheb_end((float)CHEB_CUT * rmin, rmax, mu_eta) : 0.f;
+        const float c = rmin * (float)CHEB_RANGE32 >= rmax ? (float)CHEB_CUT * rmin : 0.f;
         if (t == 0) cheb[i] = c;
         if (early && it == START_SETTLE - 1) {
             const int stop = start_stop(start_steps(rkk, c, p, nev, mu_eta));
@@ -1800,8 +1799,8 @@ void eig_gram(GevpBatch& g, cudaStream_t s) {
     MSDD_LAUNCH_CHECK();
 }
 
-void eig_rayleigh_ritz(GevpBatch& g, const EigParams& ep, cudaStream_t s) {
-    k_rayleigh_ritz<<<g.P, TPB, 0, s>>>(g.Hp.p, g.Mp.p, g.gsplit, g.H.p, g.M.p, g.C.p, g.theta.p, g.cheb.p, ep.sigma, ep.eta,
+void eig_rayleigh_ritz(GevpBatch& g, double sigma, cudaStream_t s) {
+    k_rayleigh_ritz<<<g.P, TPB, 0, s>>>(g.Hp.p, g.Mp.p, g.gsplit, g.H.p, g.M.p, g.C.p, g.theta.p, g.cheb.p, sigma,
                                         g.d_p.p, g.rank.p, g.done.p);
     MSDD_LAUNCH_CHECK();
 }

@@ -11,7 +11,8 @@
 //   W <- K^{-1} W        (tile LDL^T solve, FP64 or FP32 factors), so that S X = X diag(mu) + W
 //   Y = the Chebyshev step of S X, X and Q (the block before X in the basis of
 //       X) that damps [0, c], c = 0.95 times the smallest Ritz value of S in
-//       the block (at least 1e-6 of the largest); the first iteration Y = S X
+//       the block; the first iteration, and blocks that span more than the
+//       range of B, Y = S X
 //   AY, BY; H = Y^T AY, M = Y^T BY (FP64); Rayleigh-Ritz H c = theta M c
 //   Q = X C, X = Y C, AX = AY C, BX = BY C (with a cheap operator X and Q only, AX
 //       and BX afresh); residuals |AX_k - theta_k BX_k| / ((theta_k + sigma) |BX_k|).
@@ -40,7 +41,8 @@ struct GevpBatch {
     // the block before X in its basis (Chebyshev recurrence); where AX and BX are only needed by the first iteration
     // (`fused` of alloc: the operator is applied afresh), a view of AX
     DevBuf<double> Q;
-    DevBuf<double> cheb;                           // per problem: end of the damped interval of S = K^{-1} B, 0 unknown
+    // per problem: end of the damped interval of S = K^{-1} B; 0: plain step next; negative: the step before was plain
+    DevBuf<double> cheb;
     DevBuf<double> H, M, C, theta, res;            // per problem PMAX^2 / PMAX
     int gsplit = 1;                                // row splits of the Gram products
     DevBuf<double> Hp, Mp;                         // per (problem, split) PMAX^2 partial Grams
@@ -104,7 +106,7 @@ void eig_check_knorm(GevpBatch& g, const EigParams& ep, int it, cudaStream_t s);
 // H = Y^T AY, M = Y^T BY.
 void eig_gram(GevpBatch& g, cudaStream_t s);
 // Rayleigh-Ritz: theta ascending, C with C^T M C = I; the next damped interval.
-void eig_rayleigh_ritz(GevpBatch& g, const EigParams& ep, cudaStream_t s);
+void eig_rayleigh_ritz(GevpBatch& g, double sigma, cudaStream_t s);
 // X = Y C, AX = AY C, BX = BY C, residual partial sums; want_q: Q = (old X) C.
 void eig_update(GevpBatch& g, bool want_q, cudaStream_t s);
 // X = Y C only: with a cheap operator (stored stencils) AX and BX are applied

@@ -250,7 +250,7 @@ void run_eig(GevpBatch& g, const EigParams& ep, Apply apply, Solve solve, BApply
         eig_gram(v, s);
         prof.end(s, 3.0 * am[k].vec_n * 8.0 * fr, 2.0 * am[k].vec_n * (am[k].pm + 1) * fr);
         prof.begin(tag + "_rayleigh_ritz", s);
-        eig_rayleigh_ritz(v, ep, s);
+        eig_rayleigh_ritz(v, ep.sigma, s);
         prof.end(s, 0.0, 0.0);
         if (fused) {
             prof.begin(tag + "_update", s);
