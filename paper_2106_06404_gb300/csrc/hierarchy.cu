@@ -69,9 +69,8 @@ int sum_nreg(const TileBatch& tb, cudaStream_t s) {
 }
 
 // Dense (pseudo-)inverse of every factorised FP64 problem of a tile batch:
-// out[ooff[i] + r * ld[i] + c] = (K_i^+)[r][c] for r, c < n[i].  The lower
-// triangle is solved for, one CTA per (problem, few columns), so the whole
-// GPU works on it, and mirrored.
+// out[ooff[i] + r * ld[i] + c] = (K_i^+)[r][c] for r, c < n[i], solved for column
+// by column, one CTA per (problem, few columns), so the whole GPU works on it.
 void dense_inverse(const TileBatch& tb, double* out, const std::vector<long long>& ooff, const std::vector<int>& ld,
                    cudaStream_t st) {
     int maxn = 0;
@@ -84,7 +83,7 @@ void dense_inverse(const TileBatch& tb, double* out, const std::vector<long long
     }
     DevBuf<long long> d_ooff = upload_vec(ooff, st);
     DevBuf<int> d_ld = upload_vec(ld, st);
-    mirror_lower(tb, E.p, lde, maxn, d_ooff.p, d_ld.p, out, st);
+    copy_squares(tb, E.p, lde, maxn, d_ooff.p, d_ld.p, out, st);
     MSDD_CUDA(cudaStreamSynchronize(st));
 }
 

@@ -73,11 +73,10 @@ void tile_factor(TileBatch& tb, double reg_tol, cudaStream_t s);
 bool tile_solve_f64(const TileBatch& tb, double* X, int ldx, int ncols, const int* skip, cudaStream_t s,
                     const int* gdone);
 // E (total_rows x lde, lde >= ncols) <- columns 0 .. ncols - 1 of every
-// problem's inverse, the tile rows from each column's own on (the lower
-// triangle and the diagonal tiles); false as above.
+// problem's inverse (columns beyond its order are left alone); false as above.
 bool tile_inverse_f64(const TileBatch& tb, double* E, int lde, int ncols, cudaStream_t s);
-// out[ooff[i] + r * ld[i] + c] for r, c < n[i] from the lower triangle of E.
-void mirror_lower(const TileBatch& tb, const double* E, int lde, int maxn, const long long* d_ooff, const int* d_ld,
+// out[ooff[i] + r * ld[i] + c] = row r, column c of problem i in E for r, c < n[i].
+void copy_squares(const TileBatch& tb, const double* E, int lde, int maxn, const long long* d_ooff, const int* d_ld,
                   double* out, cudaStream_t s);
 // E (total_rows x lde) <- per problem the identity of order n[i] (zero elsewhere).
 void tile_identity(const TileBatch& tb, double* E, int lde, cudaStream_t s);

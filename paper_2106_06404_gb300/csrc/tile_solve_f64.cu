@@ -32,13 +32,15 @@ constexpr int F6_NST = 4;       // tiles in flight (8 KB each)
 // Measured (GB300): 14 columns of 27 problems of n = 1452..1872, b = 133..157
 // 8.75 -> 0.75 ms a launch against one CTA of full tiles a problem; 16 columns
 // of 72 problems of n ~ 1300, b = 36 1.28 -> 0.54 ms; dense inverses of 27
-// matrices of order ~1000 and their copy 26 ms less in the 96^3 set-up.
+// matrices of order ~1000 and their copy about 20 ms less in the 96^3 set-up.
 //
-// INV: the right-hand sides are the identity columns c_lo .. c_lo + C - 1
-// (X is not read); z_R = 0 above the first of them, so both sweeps run over
-// the tile rows from there on and the rows above are left alone: the inverse
-// is symmetric and the caller mirrors it (a third of the products of n
-// full solves).
+// INV: the right-hand sides are the identity columns c_lo .. c_lo + C - 1 (X is
+// not read); z_R = 0 above the first of them, so the forward sweep starts there
+// (three quarters of the products of n full solves).  The backward sweep runs over
+// all rows: taking the upper triangle from the other columns, by symmetry, leaves
+// columns whose errors belong to different solves, and K times such a column is off
+// by the condition number: eigensolves of near-dependent generating systems then
+// stalled at residuals around 1 where they reach 1e-4.
 template <int C, bool INV>
 __global__ void __launch_bounds__(F6_T) k_tile_solve_f64(
     const double* __restrict__ tiles, const double* __restrict__ dinv, const int* __restrict__ n_,
@@ -69,7 +71,7 @@ __global__ void __launch_bounds__(F6_T) k_tile_solve_f64(
     // the tiles of a sweep, one after the other: (R, d) with d = dmax .. 1
     // (off-diagonal, far to near) and then 0 (T_R)
     auto issue = [&](int st, int R, int d, bool fwd) {
-        if (R >= R0 && R < K) {
+        if (R >= (fwd ? R0 : 0) && R < K) {
             const double* src = tiles + (fwd ? tile_index(toff, kb, R, R - d) : tile_index(toff, kb, R + d, R));
             double* dst = ring + st * NB2;
 #pragma unroll
@@ -93,17 +95,17 @@ __global__ void __launch_bounds__(F6_T) k_tile_solve_f64(
         };
         for (int k = 0; k < F6_NST - 1; ++k) issue_next();
         auto load_x = [&](int R) -> double {
-            if (R < R0 || R >= K) return 0.0;
+            if (R < R0 || R >= K) return 0.0;        // (backward, above R0: z_R = 0)
             const int row = R * NB + r;
             if (INV && fwd) return (row == c_lo + c && row < n) ? 1.0 : 0.0;
             return owner ? X[(roff + row) * ldx] : 0.0;
         };
         double xnext = load_x(Rbeg), dnext = fwd ? 0.0 : dinv[roff + Rbeg * NB + r];
         int st = 0;
-        for (int R = Rbeg; R >= R0 && R < K; R += step) {
+        for (int R = Rbeg; R >= (fwd ? R0 : 0) && R < K; R += step) {
             const double xr = fwd ? xnext : dnext * xnext;
             xnext = load_x(R + step);                           // one step ahead
-            if (!fwd && R > R0) dnext = dinv[roff + (R - 1) * NB + r];
+            if (!fwd && R > 0) dnext = dinv[roff + (R - 1) * NB + r];
             double a0 = 0.0, a1 = 0.0;
             for (int d = dmax(R); d >= 0; --d) {
                 cp_async_wait_n<F6_NST - 2>();
@@ -159,28 +161,15 @@ __global__ void __launch_bounds__(F6_T) k_tile_solve_f64(
     }
 }
 
-// out_i[r][c] = E[r][c] on and below the diagonal, mirrored above it
-__global__ void k_mirror_lower(const double* __restrict__ E, int lde, const int* __restrict__ n_,
+__global__ void k_copy_squares(const double* __restrict__ E, int lde, const int* __restrict__ n_,
                                const long long* __restrict__ roff_, const long long* __restrict__ ooff,
                                const int* __restrict__ ldo, double* __restrict__ out) {
-    __shared__ double s[NB][NB + 1];
-    const int i = blockIdx.z, n = n_[i];
-    const int bi = blockIdx.y, bj = blockIdx.x;
-    if (bj > bi || bi * NB >= n) return;
+    const int i = blockIdx.x, n = n_[i], r1 = min(n, (int)(blockIdx.y + 1) * NB);
     const double* Ei = E + roff_[i] * lde;
     double* o = out + ooff[i];
-    const int ld = ldo[i], x = threadIdx.x & 31;
-    for (int y = threadIdx.x >> 5; y < NB; y += 8) {
-        const int rr = bi * NB + y, cc = bj * NB + x;
-        const double v = rr < n && cc <= rr ? Ei[(long long)rr * lde + cc] : 0.0;
-        s[y][x] = v;
-        if (rr < n && cc <= rr) o[(long long)rr * ld + cc] = v;
-    }
-    __syncthreads();
-    for (int y = threadIdx.x >> 5; y < NB; y += 8) {
-        const int rr = bj * NB + y, cc = bi * NB + x;           // the transposed position
-        if (cc < n && rr < cc) o[(long long)rr * ld + cc] = s[x][y];
-    }
+    const int ld = ldo[i];
+    for (int r = blockIdx.y * NB + (threadIdx.x >> 5); r < r1; r += 8)
+        for (int c = threadIdx.x & 31; c < n; c += 32) o[(long long)r * ld + c] = Ei[(long long)r * lde + c];
 }
 
 size_t f6_bytes(int maxkb, int C) { return sizeof(double) * ((size_t)F6_NST * NB2 + (size_t)(maxkb + 1) * NB * C); }
@@ -231,11 +220,10 @@ bool tile_inverse_f64(const TileBatch& tb, double* E, int lde, int ncols, cudaSt
     return solve_f64<true>(tb, E, lde, ncols, nullptr, s, nullptr);
 }
 
-void mirror_lower(const TileBatch& tb, const double* E, int lde, int maxn, const long long* d_ooff, const int* d_ld,
+void copy_squares(const TileBatch& tb, const double* E, int lde, int maxn, const long long* d_ooff, const int* d_ld,
                   double* out, cudaStream_t s) {
-    if (tb.P == 0 || maxn == 0) return;
-    const unsigned nb = ceil_div(maxn, NB);
-    k_mirror_lower<<<dim3(nb, nb, tb.P), 256, 0, s>>>(E, lde, tb.d_n.p, tb.d_roff.p, d_ooff, d_ld, out);
+    if (tb.P == 0 || maxn <= 0) return;
+    k_copy_squares<<<dim3(tb.P, (maxn + NB - 1) / NB), 256, 0, s>>>(E, lde, tb.d_n.p, tb.d_roff.p, d_ooff, d_ld, out);
     MSDD_LAUNCH_CHECK();
 }
 
